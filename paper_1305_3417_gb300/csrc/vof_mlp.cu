@@ -24,7 +24,6 @@ constexpr int IN = VOF_MLP_IN, K0 = 48, HID = VOF_MLP_HID, OUT = VOF_MLP_OUT, OU
 constexpr int OW1 = 0, OB1 = OW1 + IN * HID, OW2 = OB1 + HID, OB2 = OW2 + HID * HID, OW3 = OB2 + HID,
               OB3 = OW3 + HID * OUT, NPARAM = OB3 + OUT;
 static_assert(NPARAM == VOF_MLP_NPARAM, "parameter count");
-constexpr int CHUNK = 512;  // samples per weight-gradient partial
 
 using bf = unsigned short;
 
@@ -83,16 +82,14 @@ __global__ void k_mlp_features(DevMesh m, const double *__restrict__ alpha, cons
 }
 
 // ---------------------------------------------------------------- weights
-// BF16 copies of the FP32 master weights, zero padded: W1 [K0 x HID] and its
-// transpose, W2 [HID x HID] and transpose, W3 [HID x OUTP] and transpose
-__global__ void k_mlp_pack(const float *p, bf *W1, bf *W1t, bf *W2, bf *W2t, bf *W3, bf *W3t)
+// BF16 copies of the FP32 master weights, zero padded: W1 [K0 x HID] transposed,
+// W2 [HID x HID] and transpose, W3 [HID x OUTP] and transpose
+__global__ void k_mlp_pack(const float *p, bf *W1t, bf *W2, bf *W2t, bf *W3, bf *W3t)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < K0 * HID) {
         const int k = i / HID, j = i % HID;
-        const bf v = k < IN ? to_bf(p[OW1 + k * HID + j]) : (bf)0;
-        W1[k * HID + j] = v;
-        W1t[j * K0 + k] = v;
+        W1t[j * K0 + k] = k < IN ? to_bf(p[OW1 + k * HID + j]) : (bf)0;
     }
     if (i < HID * HID) {
         const int k = i / HID, j = i % HID;
@@ -108,175 +105,273 @@ __global__ void k_mlp_pack(const float *p, bf *W1, bf *W1t, bf *W2, bf *W2t, bf 
     }
 }
 
-__global__ void k_mlp_input(const float *feat, int ncap, const int *ndev, bf *X0)
-{
-    const int n = ndev ? min(*ndev, ncap) : ncap;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n * K0; i += gridDim.x * blockDim.x) {
-        const int r = i / K0, k = i % K0;
-        X0[i] = k < IN ? to_bf(feat[(size_t)r * IN + k]) : (bf)0;
-    }
-}
-
-// ---------------------------------------------------------------- layers
-// C [n x M] = A [n x K] . B [K x M] with A row-major BF16 (rows >= n read as
-// 0) and B given as Bt [M x K] row-major.  One warp per 16 rows.  mode 0:
-// Z = C + bias (FP32) and H = BF16(ReLU(Z)); mode 1: Y = C + bias (FP32);
-// mode 2 (backward through a hidden layer): G = C * (Zf > 0) written as BF16.
-template <int K, int M, int MODE>
-__device__ __forceinline__ void mlp_gemm_tile(const bf *A, const bf *Bt, const float *bias, int n, int r0, int g, int t,
-                                              float *Zout, bf *Hout, const float *Zf)
-{
-    float acc[M / 8][4];
-#pragma unroll
-    for (int j = 0; j < M / 8; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.0f;
-    auto ld = [&](int r, int k) -> bf { return r < n ? A[(size_t)r * K + k] : (bf)0; };
-#pragma unroll
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        const uint32_t a0 = pk(ld(r0 + g, k0 + 2 * t), ld(r0 + g, k0 + 2 * t + 1));
-        const uint32_t a1 = pk(ld(r0 + g + 8, k0 + 2 * t), ld(r0 + g + 8, k0 + 2 * t + 1));
-        const uint32_t a2 = pk(ld(r0 + g, k0 + 2 * t + 8), ld(r0 + g, k0 + 2 * t + 9));
-        const uint32_t a3 = pk(ld(r0 + g + 8, k0 + 2 * t + 8), ld(r0 + g + 8, k0 + 2 * t + 9));
-#pragma unroll
-        for (int j = 0; j < M / 8; ++j) {
-            const bf *bt = Bt + (size_t)(8 * j + g) * K + k0 + 2 * t;
-            mma16816(acc[j], a0, a1, a2, a3, pk(bt[0], bt[1]), pk(bt[8], bt[9]));
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < M / 8; ++j)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int r = r0 + g + (e >= 2 ? 8 : 0), col = 8 * j + 2 * t + (e & 1);
-            if (r >= n) continue;
-            const size_t o = (size_t)r * M + col;
-            if (MODE == 0) {
-                const float z = acc[j][e] + bias[col];
-                Zout[o] = z;
-                Hout[o] = to_bf(fmaxf(z, 0.0f));
-            } else if (MODE == 1) {
-                Zout[o] = acc[j][e] + (col < OUT ? bias[col] : 0.0f);
-            } else {
-                const float gz = Zf[o] > 0.0f ? acc[j][e] : 0.0f;
-                Zout[o] = gz;
-                Hout[o] = to_bf(gz);
-            }
-        }
-}
-
-template <int K, int M, int MODE>
-__global__ void k_mlp_gemm(const bf *A, const bf *Bt, const float *bias, int ncap, const int *ndev, float *Zout,
-                           bf *Hout, const float *Zf)
-{
-    const int n = ndev ? min(*ndev, ncap) : ncap;
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    for (int r0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 16; r0 < n; r0 += ((gridDim.x * blockDim.x) >> 5) * 16)
-        mlp_gemm_tile<K, M, MODE>(A, Bt, bias, n, r0, g, t, Zout, Hout, Zf);
-}
-
-// output gradient of the mean squared error: dY = 2 (Y - T) / n (FP32 and
-// BF16, padded columns 0) and per-block partial losses
-__global__ void k_mlp_dy(const float *Y, const float *T, int n, float *dYf, bf *dYb, float *lpart)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    float l = 0.0f;
-    if (i < n * OUTP) {
-        const int r = i / OUTP, j = i % OUTP;
-        float d = 0.0f;
-        if (j < OUT) {
-            const float e = Y[i] - T[(size_t)r * OUT + j];
-            l = e * e;
-            d = 2.0f * e / (float)n;
-        }
-        dYf[i] = d;
-        dYb[i] = to_bf(d);
-    }
-    l = vofd::warp_sum((double)l);
-    __shared__ float sh[8];
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = l;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float s = 0.0f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh[w];
-        lpart[blockIdx.x] = s;
-    }
-}
-
-// weight gradient partials: P[chunk] [K x M] = A[chunk]^T . D[chunk] over CHUNK
-// samples (A [n x K], D [n x M], both BF16 row-major); one warp per 16 x 8
-// output tile and chunk
-template <int K, int M>
-__global__ void k_mlp_wgrad(const bf *A, const bf *D, int n, float *P)
-{
-    const int lane = threadIdx.x & 31;
-    const int tile = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    constexpr int TM = M / 8, NT = (K / 16) * TM;
-    if (tile >= NT) return;
-    const int k0 = (tile / TM) * 16, m0 = (tile % TM) * 8, ch = blockIdx.y;
-    const int g = lane >> 2, t = lane & 3;
-    const int s0 = ch * CHUNK, s1 = min(n, s0 + CHUNK);
-    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    auto la = [&](int r, int s) -> bf { return s < s1 ? A[(size_t)s * K + k0 + r] : (bf)0; };  // A^T (r, s)
-    auto ld = [&](int s, int c) -> bf { return s < s1 ? D[(size_t)s * M + m0 + c] : (bf)0; };
-    for (int sb = s0; sb < s1; sb += 16) {
-        const uint32_t a0 = pk(la(g, sb + 2 * t), la(g, sb + 2 * t + 1));
-        const uint32_t a1 = pk(la(g + 8, sb + 2 * t), la(g + 8, sb + 2 * t + 1));
-        const uint32_t a2 = pk(la(g, sb + 2 * t + 8), la(g, sb + 2 * t + 9));
-        const uint32_t a3 = pk(la(g + 8, sb + 2 * t + 8), la(g + 8, sb + 2 * t + 9));
-        const uint32_t b0 = pk(ld(sb + 2 * t, g), ld(sb + 2 * t + 1, g));
-        const uint32_t b1 = pk(ld(sb + 2 * t + 8, g), ld(sb + 2 * t + 9, g));
-        mma16816(acc, a0, a1, a2, a3, b0, b1);
-    }
-    float *o = P + (size_t)ch * K * M;
-    o[(k0 + g) * M + m0 + 2 * t] = acc[0];
-    o[(k0 + g) * M + m0 + 2 * t + 1] = acc[1];
-    o[(k0 + g + 8) * M + m0 + 2 * t] = acc[2];
-    o[(k0 + g + 8) * M + m0 + 2 * t + 1] = acc[3];
-}
-
-// bias gradient partials: per chunk, column sums of the FP32 upstream gradient
-__global__ void k_mlp_bgrad(const float *G, int n, int M, float *P)
-{
-    const int ch = blockIdx.x, col = threadIdx.x;
-    if (col >= M) return;
-    const int s0 = ch * CHUNK, s1 = min(n, s0 + CHUNK);
-    float s = 0.0f;
-    for (int r = s0; r < s1; ++r) s += G[(size_t)r * M + col];
-    P[(size_t)ch * M + col] = s;
-}
-
-// sums the chunk partials in chunk order into the flat gradient, then Adam
-struct GradPtrs {
-    const float *pw1, *pw2, *pw3, *pb1, *pb2, *pb3, *lpart;
-    int nch, nlb;
+// ---------------------------------------------------- forward and backward
+// One kernel for the network's whole pass over a tile of 64 samples (four
+// warps, 16 samples each), the layers chained through registers: the
+// accumulators of two 8-column tiles are the next layer's 16-column operand,
+// forward and backward.  GRAD: the operands of the weight gradients
+// (activations and BF16 upstream gradients) go to shared memory transposed,
+// [column][sample], so that a pair of samples is one 32-bit operand load, and
+// the block's 60 weight-gradient tiles (16 x 8) stay in registers over all the
+// tiles that the block takes; a block writes one partial gradient in the flat
+// parameter layout.  Rows of 72 (56, 24) 16-bit values: conflict-free operand
+// loads.  Bound by latency (a few hundred small mma per tile on one SM): a tile
+// of 64 samples spreads a batch of 4096 over 64 SMs.  Against one kernel per
+// layer and per gradient with everything through global memory (13 launches,
+// the weight gradients read with 16-bit loads): 4096 samples 251 -> 56 us a
+// gradient call with its loss.
+constexpr int TILE = 64, GT = 128, LT = TILE + 8, L1 = K0 + 8, L2 = HID + 8, L3 = OUTP + 8;
+struct MlpShared {
+    bf W1t[HID * L1], W2t[HID * L2], W2[HID * L2], W3t[8 * L2], W3[HID * L3];
+    bf X[TILE * L1];
+    bf XT[K0 * LT], H1T[HID * LT], H2T[HID * LT], D1T[HID * LT], D2T[HID * LT], DYT[8 * LT];
+    float b1[HID], b2[HID], b3[8];
+    float red[4][2 * HID + 8];
+    double loss[4];
+};
+struct MlpWeights {
+    const float *p;
+    const bf *W1t, *W2, *W2t, *W3, *W3t;
 };
 
-__global__ void k_mlp_reduce(GradPtrs q, float *grad, float *loss)
+__device__ __forceinline__ uint32_t ld2(const bf *q) { return *reinterpret_cast<const uint32_t *>(q); }
+
+template <bool GRAD>
+__global__ void __launch_bounds__(GT) k_mlp_pass(MlpWeights w, const float *__restrict__ feat,
+                                                 const float *__restrict__ target, int n, float *out, float *part,
+                                                 double *lpart)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    extern __shared__ __align__(16) unsigned char mlp_smem[];
+    MlpShared &sh = *reinterpret_cast<MlpShared *>(mlp_smem);
+    const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5, g = lane >> 2, t = lane & 3;
+    // weights: rows of the packed copies, two values a load
+    auto rows = [&](bf *dst, const bf *src, int nr, int len, int ld) {
+        for (int i = tid; i < nr * (len / 2); i += GT) {
+            const int r = i / (len / 2), c = 2 * (i % (len / 2));
+            *reinterpret_cast<uint32_t *>(dst + r * ld + c) = ld2(src + r * len + c);
+        }
+    };
+    rows(sh.W1t, w.W1t, HID, K0, L1);
+    rows(sh.W2t, w.W2t, HID, HID, L2);
+    rows(sh.W3t, w.W3t, 8, HID, L2);
+    if (GRAD) {
+        rows(sh.W2, w.W2, HID, HID, L2);
+        rows(sh.W3, w.W3, HID, OUTP, L3);
+    }
+    for (int i = tid; i < HID; i += GT) { sh.b1[i] = w.p[OB1 + i]; sh.b2[i] = w.p[OB2 + i]; }
+    if (tid < 8) sh.b3[tid] = tid < OUT ? w.p[OB3 + tid] : 0.0f;
+
+    float wacc[15][4];           // weight-gradient tiles wp, wp + 4, ...: 24 of W1, 32 of W2, 4 of W3
+    float s1[8][2], s2[8][2], s3[2] = {0.0f, 0.0f};  // bias gradients: column sums over this thread's rows
+    double loss = 0.0;
+    if (GRAD) {
+#pragma unroll
+        for (int i = 0; i < 15; ++i) wacc[i][0] = wacc[i][1] = wacc[i][2] = wacc[i][3] = 0.0f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s1[j][0] = s1[j][1] = s2[j][0] = s2[j][1] = 0.0f;
+    }
+    const int ntile = (n + TILE - 1) / TILE;
+    for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+        const int r00 = tile * TILE;
+        // features to BF16, zero beyond the batch and beyond the 33 columns
+        for (int i = tid; i < TILE * K0; i += GT) {
+            const int r = i / K0, k = i % K0;
+            const bf v = (k < IN && r00 + r < n) ? to_bf(feat[(size_t)(r00 + r) * IN + k]) : (bf)0;
+            sh.X[r * L1 + k] = v;
+            if (GRAD) sh.XT[k * LT + r] = v;
+        }
+        __syncthreads();
+        const int ra = 16 * wp + g, rb = ra + 8;  // this thread's rows of the tile
+        float h[8][4];
+        // bias and ReLU of a layer's accumulators: the next layer's operand
+        // pairs (first row, second row) per 8-column tile, and the ReLU's mask
+        auto relu = [&](const float *bias, uint32_t (&pa)[8], uint32_t (&pb)[8], uint32_t &mask, bf *HT) {
+            mask = 0u;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int c = 8 * j + 2 * t;
+                const float z0 = h[j][0] + bias[c], z1 = h[j][1] + bias[c + 1], z2 = h[j][2] + bias[c],
+                            z3 = h[j][3] + bias[c + 1];
+                mask |= (z0 > 0.0f ? 1u : 0u) << (4 * j) | (z1 > 0.0f ? 2u : 0u) << (4 * j) |
+                        (z2 > 0.0f ? 4u : 0u) << (4 * j) | (z3 > 0.0f ? 8u : 0u) << (4 * j);
+                const bf v0 = to_bf(fmaxf(z0, 0.0f)), v1 = to_bf(fmaxf(z1, 0.0f)), v2 = to_bf(fmaxf(z2, 0.0f)),
+                         v3 = to_bf(fmaxf(z3, 0.0f));
+                pa[j] = pk(v0, v1);
+                pb[j] = pk(v2, v3);
+                if (GRAD) {
+                    HT[c * LT + ra] = v0; HT[(c + 1) * LT + ra] = v1;
+                    HT[c * LT + rb] = v2; HT[(c + 1) * LT + rb] = v3;
+                }
+            }
+        };
+        auto zero = [&]() {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) h[j][0] = h[j][1] = h[j][2] = h[j][3] = 0.0f;
+        };
+        uint32_t pa[8], pb[8], m1, m2;
+        // layer 1
+        zero();
+#pragma unroll
+        for (int k0 = 0; k0 < K0; k0 += 16) {
+            const bf *xa = sh.X + ra * L1 + k0 + 2 * t, *xb = sh.X + rb * L1 + k0 + 2 * t;
+            const uint32_t a0 = ld2(xa), a1 = ld2(xb), a2 = ld2(xa + 8), a3 = ld2(xb + 8);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const bf *bt = sh.W1t + (8 * j + g) * L1 + k0 + 2 * t;
+                mma16816(h[j], a0, a1, a2, a3, ld2(bt), ld2(bt + 8));
+            }
+        }
+        relu(sh.b1, pa, pb, m1, sh.H1T);
+        // layer 2
+        zero();
+#pragma unroll
+        for (int kk = 0; kk < HID / 16; ++kk)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const bf *bt = sh.W2t + (8 * j + g) * L2 + 16 * kk + 2 * t;
+                mma16816(h[j], pa[2 * kk], pb[2 * kk], pa[2 * kk + 1], pb[2 * kk + 1], ld2(bt), ld2(bt + 8));
+            }
+        relu(sh.b2, pa, pb, m2, sh.H2T);
+        // output layer (columns 0..7, of which 0..3 exist)
+        float y[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int kk = 0; kk < HID / 16; ++kk) {
+            const bf *bt = sh.W3t + g * L2 + 16 * kk + 2 * t;
+            mma16816(y, pa[2 * kk], pb[2 * kk], pa[2 * kk + 1], pb[2 * kk + 1], ld2(bt), ld2(bt + 8));
+        }
+        if constexpr (!GRAD) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int r = r00 + (e < 2 ? ra : rb), c = 2 * t + (e & 1);
+                if (r < n && c < OUT) out[(size_t)r * OUT + c] = y[e] + sh.b3[c];
+            }
+        } else {
+        // gradient of the mean squared error: 2 (Y - T) / n
+        bf db[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int r = r00 + (e < 2 ? ra : rb), c = 2 * t + (e & 1);
+            float d = 0.0f;
+            if (r < n && c < OUT) {
+                const float er = y[e] + sh.b3[c] - target[(size_t)r * OUT + c];
+                const float l = er * er;
+                loss += (double)l;
+                d = 2.0f * er / (float)n;
+            }
+            db[e] = to_bf(d);
+            s3[e & 1] += d;
+            sh.DYT[c * LT + (e < 2 ? ra : rb)] = db[e];
+        }
+        // back through a layer: accumulators masked by the ReLU, their column
+        // sums, and the next operand pairs
+        auto back = [&](uint32_t mask, float (&s)[8][2], bf *DT) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int c = 8 * j + 2 * t;
+                const float d0 = mask >> (4 * j) & 1u ? h[j][0] : 0.0f, d1 = mask >> (4 * j) & 2u ? h[j][1] : 0.0f,
+                            d2 = mask >> (4 * j) & 4u ? h[j][2] : 0.0f, d3 = mask >> (4 * j) & 8u ? h[j][3] : 0.0f;
+                s[j][0] += d0 + d2;
+                s[j][1] += d1 + d3;
+                const bf v0 = to_bf(d0), v1 = to_bf(d1), v2 = to_bf(d2), v3 = to_bf(d3);
+                pa[j] = pk(v0, v1);
+                pb[j] = pk(v2, v3);
+                DT[c * LT + ra] = v0; DT[(c + 1) * LT + ra] = v1;
+                DT[c * LT + rb] = v2; DT[(c + 1) * LT + rb] = v3;
+            }
+        };
+        zero();
+        {
+            const uint32_t a0 = pk(db[0], db[1]), a1 = pk(db[2], db[3]);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) mma16816(h[j], a0, a1, 0u, 0u, ld2(sh.W3 + (8 * j + g) * L3 + 2 * t), 0u);
+        }
+        back(m2, s2, sh.D2T);
+        zero();
+#pragma unroll
+        for (int kk = 0; kk < HID / 16; ++kk)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const bf *bt = sh.W2 + (8 * j + g) * L2 + 16 * kk + 2 * t;
+                mma16816(h[j], pa[2 * kk], pb[2 * kk], pa[2 * kk + 1], pb[2 * kk + 1], ld2(bt), ld2(bt + 8));
+            }
+        back(m1, s1, sh.D1T);
+        __syncthreads();
+        // weight gradients of the tile: A^T . D over its 64 samples
+        auto wtile = [&](float (&acc)[4], const bf *AT, const bf *DT, int k0, int c0) {
+#pragma unroll
+            for (int sb = 0; sb < TILE; sb += 16) {
+                const bf *a = AT + (k0 + g) * LT + sb + 2 * t, *d = DT + (c0 + g) * LT + sb + 2 * t;
+                mma16816(acc, ld2(a), ld2(a + 8 * LT), ld2(a + 8), ld2(a + 8 * LT + 8), ld2(d), ld2(d + 8));
+            }
+        };
+#pragma unroll
+        for (int i = 0; i < 6; ++i) wtile(wacc[i], sh.XT, sh.D1T, 16 * ((wp + 4 * i) / 8), 8 * ((wp + 4 * i) % 8));
+#pragma unroll
+        for (int i = 0; i < 8; ++i) wtile(wacc[6 + i], sh.H1T, sh.D2T, 16 * ((wp + 4 * i) / 8), 8 * ((wp + 4 * i) % 8));
+        wtile(wacc[14], sh.H2T, sh.DYT, 16 * wp, 0);
+        }
+        __syncthreads();  // every operand read before the next tile
+    }
+    if (!GRAD) return;
+    float *o = part + (size_t)blockIdx.x * NPARAM;
+    auto put = [&](int base, int ld, int k, int c, int kmax, int cmax, const float (&acc)[4]) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int kk = k + g + (e >= 2 ? 8 : 0), cc = c + 2 * t + (e & 1);
+            if (kk < kmax && cc < cmax) o[base + kk * ld + cc] = acc[e];
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < 6; ++i) put(OW1, HID, 16 * ((wp + 4 * i) / 8), 8 * ((wp + 4 * i) % 8), IN, HID, wacc[i]);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) put(OW2, HID, 16 * ((wp + 4 * i) / 8), 8 * ((wp + 4 * i) % 8), HID, HID, wacc[6 + i]);
+    put(OW3, OUT, 16 * wp, 0, HID, OUT, wacc[14]);
+    // bias gradients: over the rows of a warp (lanes of one t), then the warps
+    auto rsum = [&](float v) {
+#pragma unroll
+        for (int x = 4; x < 32; x <<= 1) v += __shfl_xor_sync(0xffffffffu, v, x);
+        return v;
+    };
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const float v1 = rsum(s1[j][e]), v2 = rsum(s2[j][e]);
+            if (g == 0) { sh.red[wp][8 * j + 2 * t + e] = v1; sh.red[wp][HID + 8 * j + 2 * t + e] = v2; }
+        }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const float v = rsum(s3[e]);
+        if (g == 0) sh.red[wp][2 * HID + 2 * t + e] = v;
+    }
+    loss = vofd::warp_sum(loss);
+    if (lane == 0) sh.loss[wp] = loss;
+    __syncthreads();
+    for (int i = tid; i < 2 * HID + OUT; i += GT) {
+        const float v = (sh.red[0][i] + sh.red[1][i]) + (sh.red[2][i] + sh.red[3][i]);
+        o[i < HID ? OB1 + i : i < 2 * HID ? OB2 + (i - HID) : OB3 + (i - 2 * HID)] = v;
+    }
+    if (tid == 0) lpart[blockIdx.x] = (sh.loss[0] + sh.loss[1]) + (sh.loss[2] + sh.loss[3]);
+}
+
+// sums the blocks' partials in block order into the flat gradient (and the
+// caller's copy of it), and the squared errors into *loss (host memory)
+constexpr int RED_T = 64;
+__global__ void __launch_bounds__(RED_T) k_mlp_reduce(const float *__restrict__ part, const double *__restrict__ lpart,
+                                                      int nb, float *grad, float *copy, float *loss)
+{
+    const int i = blockIdx.x * RED_T + threadIdx.x;
     if (i < NPARAM) {
         float s = 0.0f;
-        if (i < OB1) {
-            const int k = i / HID, j = i % HID;
-            for (int c = 0; c < q.nch; ++c) s += q.pw1[(size_t)c * K0 * HID + k * HID + j];
-        } else if (i < OW2) {
-            for (int c = 0; c < q.nch; ++c) s += q.pb1[(size_t)c * HID + (i - OB1)];
-        } else if (i < OB2) {
-            const int k = (i - OW2) / HID, j = (i - OW2) % HID;
-            for (int c = 0; c < q.nch; ++c) s += q.pw2[(size_t)c * HID * HID + k * HID + j];
-        } else if (i < OW3) {
-            for (int c = 0; c < q.nch; ++c) s += q.pb2[(size_t)c * HID + (i - OB2)];
-        } else if (i < OB3) {
-            const int k = (i - OW3) / OUT, j = (i - OW3) % OUT;
-            for (int c = 0; c < q.nch; ++c) s += q.pw3[(size_t)c * HID * OUTP + k * OUTP + j];
-        } else {
-            for (int c = 0; c < q.nch; ++c) s += q.pb3[(size_t)c * OUTP + (i - OB3)];
-        }
+#pragma unroll 8
+        for (int b = 0; b < nb; ++b) s += part[(size_t)b * NPARAM + i];
         grad[i] = s;
+        if (copy) copy[i] = s;
     }
     if (i == 0 && loss) {
-        float s = 0.0f;
-        for (int b = 0; b < q.nlb; ++b) s += q.lpart[b];
-        *loss = s;  // sum of squared errors; the host divides by n
+        double s = 0.0;
+        for (int b = 0; b < nb; ++b) s += lpart[b];
+        *loss = (float)s;  // sum of squared errors; the host divides by n
     }
 }
 
@@ -411,12 +506,12 @@ inline int cdiv(long a, long b) { return (int)((a + b - 1) / b); }
 }  // namespace
 
 struct vof_mlp {
-    int device, max_batch, nch, adam_t;
+    int device, max_batch, nblk, adam_t;   // nblk: blocks (partial gradients) of a pass at most
     float *p, *grad, *m1, *m2;
-    bf *W1, *W1t, *W2, *W2t, *W3, *W3t;
-    bf *X0, *H1, *H2, *dYb, *dZ2b, *dZ1b;
-    float *Z1, *Z2, *Y, *dYf, *dZ2f, *dZ1f, *lpart, *loss;
-    float *pw1, *pw2, *pw3, *pb1, *pb2, *pb3;
+    bf *W1t, *W2, *W2t, *W3, *W3t;
+    float *part;
+    double *lpart;
+    float *h_loss;                         // pinned host memory that the device writes
     std::vector<void *> bufs;
 };
 
@@ -434,39 +529,29 @@ T *mlp_alloc(vof_mlp *q, size_t n, bool *ok)
     return nullptr;
 }
 
-// rows: n, or min(*ndev, n) when ndev is given (a device-side count)
-int mlp_forward(vof_mlp *q, const float *feat, int n, const int *ndev, cudaStream_t s)
+MlpWeights mlp_weights(const vof_mlp *q) { return MlpWeights{q->p, q->W1t, q->W2, q->W2t, q->W3, q->W3t}; }
+
+int mlp_forward(vof_mlp *q, const float *feat, int n, float *out, cudaStream_t s)
 {
-    const int blocks = std::min(cdiv(n, 64), 1024);
-    k_mlp_input<<<std::min(cdiv((long)n * K0, 256), 2048), 256, 0, s>>>(feat, n, ndev, q->X0);
-    k_mlp_gemm<K0, HID, 0><<<blocks, 128, 0, s>>>(q->X0, q->W1t, q->p + OB1, n, ndev, q->Z1, q->H1, nullptr);
-    k_mlp_gemm<HID, HID, 0><<<blocks, 128, 0, s>>>(q->H1, q->W2t, q->p + OB2, n, ndev, q->Z2, q->H2, nullptr);
-    k_mlp_gemm<HID, OUTP, 1><<<blocks, 128, 0, s>>>(q->H2, q->W3t, q->p + OB3, n, ndev, q->Y, nullptr, nullptr);
+    k_mlp_pass<false><<<std::min(cdiv(n, TILE), q->nblk), GT, sizeof(MlpShared), s>>>(mlp_weights(q), feat, nullptr, n,
+                                                                                      out, nullptr, nullptr);
     return cudaGetLastError() == cudaSuccess ? VOF_OK : VOF_ERR_CUDA;
 }
 
-int mlp_backward(vof_mlp *q, const float *target, int n, cudaStream_t s)
+// forward and backward: the flat gradient into q->grad (and copy, if given),
+// the sum of squared errors into q->h_loss if wanted
+int mlp_gradient(vof_mlp *q, const float *feat, const float *target, int n, float *copy, bool want_loss, cudaStream_t s)
 {
-    const int nlb = cdiv((long)n * OUTP, 256), nch = cdiv(n, CHUNK), blocks = std::min(cdiv(n, 64), 1024);
-    k_mlp_dy<<<nlb, 256, 0, s>>>(q->Y, target, n, q->dYf, q->dYb, q->lpart);
-    // through layer 3 and 2: dZ = (dY . W^T) masked by the pre-activation
-    k_mlp_gemm<OUTP, HID, 2><<<blocks, 128, 0, s>>>(q->dYb, q->W3, nullptr, n, nullptr, q->dZ2f, q->dZ2b, q->Z2);
-    k_mlp_gemm<HID, HID, 2><<<blocks, 128, 0, s>>>(q->dZ2b, q->W2, nullptr, n, nullptr, q->dZ1f, q->dZ1b, q->Z1);
-    // weight and bias gradients per chunk
-    k_mlp_wgrad<HID, OUTP><<<dim3(cdiv((HID / 16) * (OUTP / 8), 4), nch), 128, 0, s>>>(q->H2, q->dYb, n, q->pw3);
-    k_mlp_wgrad<HID, HID><<<dim3(cdiv((HID / 16) * (HID / 8), 4), nch), 128, 0, s>>>(q->H1, q->dZ2b, n, q->pw2);
-    k_mlp_wgrad<K0, HID><<<dim3(cdiv((K0 / 16) * (HID / 8), 4), nch), 128, 0, s>>>(q->X0, q->dZ1b, n, q->pw1);
-    k_mlp_bgrad<<<nch, 64, 0, s>>>(q->dYf, n, OUTP, q->pb3);
-    k_mlp_bgrad<<<nch, 64, 0, s>>>(q->dZ2f, n, HID, q->pb2);
-    k_mlp_bgrad<<<nch, 64, 0, s>>>(q->dZ1f, n, HID, q->pb1);
-    GradPtrs g{q->pw1, q->pw2, q->pw3, q->pb1, q->pb2, q->pb3, q->lpart, nch, nlb};
-    k_mlp_reduce<<<cdiv(NPARAM, 256), 256, 0, s>>>(g, q->grad, q->loss);
+    const int nb = std::min(cdiv(n, TILE), q->nblk);
+    k_mlp_pass<true><<<nb, GT, sizeof(MlpShared), s>>>(mlp_weights(q), feat, target, n, nullptr, q->part, q->lpart);
+    k_mlp_reduce<<<cdiv(NPARAM, RED_T), RED_T, 0, s>>>(q->part, q->lpart, nb, q->grad, copy,
+                                                       want_loss ? q->h_loss : nullptr);
     return cudaGetLastError() == cudaSuccess ? VOF_OK : VOF_ERR_CUDA;
 }
 
 int mlp_pack(vof_mlp *q, cudaStream_t s)
 {
-    k_mlp_pack<<<cdiv(HID * HID, 256), 256, 0, s>>>(q->p, q->W1, q->W1t, q->W2, q->W2t, q->W3, q->W3t);
+    k_mlp_pack<<<cdiv(HID * HID, 256), 256, 0, s>>>(q->p, q->W1t, q->W2, q->W2t, q->W3, q->W3t);
     return cudaGetLastError() == cudaSuccess ? VOF_OK : VOF_ERR_CUDA;
 }
 
@@ -499,39 +584,26 @@ int vof_mlp_create(int max_batch, const float *params, int device, vof_mlp **out
     if (!q) return VOF_ERR_CUDA;
     q->device = device;
     q->max_batch = max_batch;
-    q->nch = cdiv(max_batch, CHUNK);
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    q->nblk = std::min(cdiv(max_batch, TILE), std::max(sms, 1));  // a block per SM at most: its shared memory
     bool ok = true;
-    const size_t B = max_batch;
     q->p = mlp_alloc<float>(q, NPARAM, &ok);
     q->grad = mlp_alloc<float>(q, NPARAM, &ok);
     q->m1 = mlp_alloc<float>(q, NPARAM, &ok);
     q->m2 = mlp_alloc<float>(q, NPARAM, &ok);
-    q->W1 = mlp_alloc<bf>(q, K0 * HID, &ok);
     q->W1t = mlp_alloc<bf>(q, K0 * HID, &ok);
     q->W2 = mlp_alloc<bf>(q, HID * HID, &ok);
     q->W2t = mlp_alloc<bf>(q, HID * HID, &ok);
     q->W3 = mlp_alloc<bf>(q, HID * OUTP, &ok);
     q->W3t = mlp_alloc<bf>(q, HID * OUTP, &ok);
-    q->X0 = mlp_alloc<bf>(q, B * K0, &ok);
-    q->H1 = mlp_alloc<bf>(q, B * HID, &ok);
-    q->H2 = mlp_alloc<bf>(q, B * HID, &ok);
-    q->dYb = mlp_alloc<bf>(q, B * OUTP, &ok);
-    q->dZ2b = mlp_alloc<bf>(q, B * HID, &ok);
-    q->dZ1b = mlp_alloc<bf>(q, B * HID, &ok);
-    q->Z1 = mlp_alloc<float>(q, B * HID, &ok);
-    q->Z2 = mlp_alloc<float>(q, B * HID, &ok);
-    q->Y = mlp_alloc<float>(q, B * OUTP, &ok);
-    q->dYf = mlp_alloc<float>(q, B * OUTP, &ok);
-    q->dZ2f = mlp_alloc<float>(q, B * HID, &ok);
-    q->dZ1f = mlp_alloc<float>(q, B * HID, &ok);
-    q->lpart = mlp_alloc<float>(q, cdiv((long)B * OUTP, 256), &ok);
-    q->loss = mlp_alloc<float>(q, 1, &ok);
-    q->pw1 = mlp_alloc<float>(q, (size_t)q->nch * K0 * HID, &ok);
-    q->pw2 = mlp_alloc<float>(q, (size_t)q->nch * HID * HID, &ok);
-    q->pw3 = mlp_alloc<float>(q, (size_t)q->nch * HID * OUTP, &ok);
-    q->pb1 = mlp_alloc<float>(q, (size_t)q->nch * HID, &ok);
-    q->pb2 = mlp_alloc<float>(q, (size_t)q->nch * HID, &ok);
-    q->pb3 = mlp_alloc<float>(q, (size_t)q->nch * OUTP, &ok);
+    q->part = mlp_alloc<float>(q, (size_t)q->nblk * NPARAM, &ok);
+    q->lpart = mlp_alloc<double>(q, q->nblk, &ok);
+    ok = ok && cudaMallocHost(&q->h_loss, sizeof(float)) == cudaSuccess &&
+         cudaFuncSetAttribute(k_mlp_pass<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(MlpShared)) ==
+             cudaSuccess &&
+         cudaFuncSetAttribute(k_mlp_pass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(MlpShared)) ==
+             cudaSuccess;
     ok = ok && cudaMemcpy(q->p, params, sizeof(float) * NPARAM, cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemset(q->m1, 0, sizeof(float) * NPARAM) == cudaSuccess &&
          cudaMemset(q->m2, 0, sizeof(float) * NPARAM) == cudaSuccess && mlp_pack(q, 0) == VOF_OK &&
@@ -546,6 +618,7 @@ void vof_mlp_destroy(vof_mlp *q)
     if (!q) return;
     cudaSetDevice(q->device);
     for (void *p : q->bufs) cudaFree(p);
+    if (q->h_loss) cudaFreeHost(q->h_loss);
     delete q;
 }
 
@@ -571,11 +644,7 @@ int vof_mlp_forward(vof_mlp *q, const float *feat, int n, float *out, void *stre
 {
     if (!q || !feat || !out || n < 1 || n > q->max_batch) return VOF_ERR_INVALID_ARG;
     if (cudaSetDevice(q->device) != cudaSuccess) return VOF_ERR_CUDA;
-    cudaStream_t s = (cudaStream_t)stream;
-    int r = mlp_forward(q, feat, n, nullptr, s);
-    if (r) return r;
-    return cudaMemcpy2DAsync(out, OUT * sizeof(float), q->Y, OUTP * sizeof(float), OUT * sizeof(float), n,
-                             cudaMemcpyDeviceToDevice, s) == cudaSuccess ? VOF_OK : VOF_ERR_CUDA;
+    return mlp_forward(q, feat, n, out, (cudaStream_t)stream);
 }
 
 int vof_mlp_gradient(vof_mlp *q, const float *feat, const float *target, int n, float *grad, float *loss,
@@ -584,17 +653,11 @@ int vof_mlp_gradient(vof_mlp *q, const float *feat, const float *target, int n, 
     if (!q || !feat || !target || n < 1 || n > q->max_batch) return VOF_ERR_INVALID_ARG;
     if (cudaSetDevice(q->device) != cudaSuccess) return VOF_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
-    int r = mlp_forward(q, feat, n, nullptr, s);
-    if (!r) r = mlp_backward(q, target, n, s);
+    const int r = mlp_gradient(q, feat, target, n, grad, loss != nullptr, s);
     if (r) return r;
-    if (grad && cudaMemcpyAsync(grad, q->grad, sizeof(float) * NPARAM, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-        return VOF_ERR_CUDA;
     if (loss) {
-        float l = 0.0f;
-        if (cudaMemcpyAsync(&l, q->loss, sizeof(float), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess)
-            return VOF_ERR_CUDA;
-        *loss = l / (float)n;
+        if (cudaStreamSynchronize(s) != cudaSuccess) return VOF_ERR_CUDA;
+        *loss = *static_cast<volatile float *>(q->h_loss) / (float)n;
     }
     return VOF_OK;
 }
