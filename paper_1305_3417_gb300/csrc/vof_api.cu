@@ -450,17 +450,13 @@ int vof_create(const vof_mesh *mesh, const vof_options *opt, vof_ctx **out)
     c->precision = opt ? opt->precision : VOF_FP64;
     {
         const int kmax = *std::max_element(ktet.begin(), ktet.end());
-        // lanes per cell in the reconstruction: narrow groups (several cells
-        // a warp) for the mixed form's few, short FP32 iterations; in the FP64
-        // form the groups of a warp would run their long Alg. 1 iterations
-        // one after another, so hexahedra keep a warp each there
-        if (c->precision == VOF_MIXED) {
-            c->rc_g = kmax <= 4 ? 4 : kmax <= 24 ? 8 : 32;
-            c->rc_k = kmax <= 4 ? 1 : kmax <= 16 ? 2 : kmax <= 24 ? 3 : kmax <= 64 ? 2 : 3;
-        } else {
-            c->rc_g = kmax <= 16 ? 8 : 32;
-            c->rc_k = kmax <= 64 ? 2 : 3;
-        }
+        // lanes per cell in the reconstruction, and tetrahedra per lane: in
+        // the mixed form several cells share a warp where they are small (few
+        // FP64 instructions each); the FP64 form's Alg. 1 takes up to 50
+        // iterations, which cells sharing a warp would wait for one another in
+        if (kmax <= 4) { c->rc_g = 4; c->rc_k = 1; }
+        else if (kmax <= 24 && c->precision == VOF_MIXED) { c->rc_g = 8; c->rc_k = kmax <= 16 ? 2 : 3; }
+        else { c->rc_g = 32; c->rc_k = kmax <= 32 ? 1 : kmax <= 64 ? 2 : 3; }
     }
     c->bound = opt ? (opt->bound != 0) : 1;
     int err = 0;
@@ -498,6 +494,7 @@ int vof_create(const vof_mesh *mesh, const vof_options *opt, vof_ctx **out)
     m.cent = dev_copy(c, cent.data(), cent.size(), &err);
     m.ctptr = dev_copy(c, ctptr.data(), ctptr.size(), &err);
     m.ctet = dev_copy(c, ctet.data(), ctet.size(), &err);
+    m.ctvol = dev_alloc<double>(c, ctet.size(), &err);
     m.pcode = nullptr; m.scode = nullptr; m.fimg = nullptr;
     m.fkey = m.fpts;
     m.cflux = m.cface;

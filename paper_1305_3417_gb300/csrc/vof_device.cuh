@@ -125,6 +125,16 @@ __device__ __forceinline__ bool lt_neg(double a, double t)
     x.hi &= 0x7fffffff;
     return neg && !bits_le(x, dbits(t));
 }
+// a > b for any signs: the bit patterns made monotone by flipping the
+// magnitude bits of negative values (-0 then orders just below +0)
+__device__ __forceinline__ bool gt_bits(double a, double b)
+{
+    DBits x = dbits(a), y = dbits(b);
+    const int sx = x.hi >> 31, sy = y.hi >> 31;
+    x.hi ^= sx & 0x7fffffff; x.lo ^= (unsigned)sx;
+    y.hi ^= sy & 0x7fffffff; y.lo ^= (unsigned)sy;
+    return !bits_le(x, y);
+}
 // a is +0 or -0
 __device__ __forceinline__ bool is_zero(double a)
 {

@@ -37,6 +37,7 @@ struct DevMesh {
     const int2 *cent;
     const int *ctptr;
     const int4 *ctet;
+    const double *ctvol;         // volume of each cell tetrahedron
     // Periodic meshes (null otherwise, with fkey == fpts and cflux == cface):
     // translation code per (point, cell) entry and per stencil entry, (i+1) +
     // 3(j+1) + 9(k+1) for i L0 + j L1 + k L2 (13: none); the period vectors; the

@@ -47,7 +47,7 @@ __global__ void k_face_geom(DevMesh m, double *cf, double *sf, double *nagc)
     st3(sf, m.nf, f, S);
 }
 
-__global__ void k_cell_geom(DevMesh m, double *cc, double *vc, double *cbox, unsigned *bad)
+__global__ void k_cell_geom(DevMesh m, double *cc, double *vc, double *cbox, double *ctvol, unsigned *bad)
 {
     int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= m.nc) return;
@@ -61,6 +61,7 @@ __global__ void k_cell_geom(DevMesh m, double *cc, double *vc, double *cbox, uns
     }
     V3 ctr = s * (1.0 / (p1 - p0));
     double V = 0.0;
+    int k0 = m.ctptr[c];
     for (int k = m.cptr[c]; k < m.cptr[c + 1]; ++k) {
         int code = m.cface[k], f = code >> 1;
         int n = m.fptr[f + 1] - m.fptr[f], nt = n == 3 ? 1 : n;
@@ -69,6 +70,7 @@ __global__ void k_cell_geom(DevMesh m, double *cc, double *vc, double *cbox, uns
             face_tri(m, f, t, code & 1, a, b, e);
             double v = tvol(ctr, a, b, e);
             if (!(v > 0.0)) atomicOr(bad, 1u);
+            ctvol[k0++] = v;  // (faces and fan triangles in the order of ctet)
             V += v;
         }
     }
@@ -149,318 +151,454 @@ __global__ void k_point_velocity(DevMesh m, const double *__restrict__ Uc, doubl
 }
 
 // ===================================================== reconstruction (A1-A3)
-// one warp per cell: NAG gradient over the (face, point) entries of the cell,
-// then Alg. 1 with the fill function summed over the cell tetrahedra, one or
-// two per lane, each a closed-form cut fraction of its sorted projections.
+// G lanes per cell: NAG gradient over the (face, point) entries of the cell,
+// then the plane offset, the fill function summed over the cell tetrahedra, KL
+// or fewer per lane, each a closed-form cut fraction of its sorted projections.
+//
+// Bound by the FP64 pipe, which issues one warp instruction in 16 cycles on
+// this part whatever the number of active lanes: what counts is FP64 warp
+// instructions per cell.  So several cells share a warp, every order and
+// threshold test is taken on the integer pipe from the bit patterns, the
+// tetrahedra's volumes come from the context, and the fill is evaluated
+// without branches and with few divisions (below).
 
-// Reciprocal for the fill of the mixed positioning: the correctly rounded FP32
-// reciprocal for R = float (the FP32 stage only brings the residual to 1e-5);
-// for R = double the FP32 reciprocal refined by one Newton-Raphson step
-// r <- r + r (1 - x r) in FP64, whose relative error is about the square of
-// the FP32 one (~4e-15), with exact division where x is outside the FP32
-// range.  The FP64 pipe of this part runs at 1/64 of the FP32 rate: this is a
-// conversion pair and two FMAs in place of a full FP64 division.
+// Reciprocal in FP64 without a full division: the FP32 reciprocal refined by
+// one Newton-Raphson step r <- r + r (1 - x r) in FP64, whose relative error is
+// about the square of the FP32 one (~4e-15), with exact division where x is
+// outside the FP32 range: a conversion pair and two FMAs.
 __device__ __noinline__ double exact_rcp(double x) { return 1.0 / x; }
-template <class R> __device__ __forceinline__ R mx_rcp(R x);
-template <> __device__ __forceinline__ float mx_rcp<float>(float x) { return __frcp_rn(x); }
-template <> __device__ __forceinline__ double mx_rcp<double>(double x)
+__device__ __forceinline__ double mx_rcp(double x)
 {
     const float r0 = __frcp_rn((float)x);
     if (!isfinite(r0) || r0 == 0.0f) return exact_rcp(x);
     const double r = (double)r0;
     return fma(r, fma(-x, r, 1.0), r);
 }
-
-// Cut fraction of a tetrahedron with sorted projections h0..h3 below level d,
-// and its derivative in d (the cut area over the volume): the same closed form
-// as frac_below, differentiated piece by piece.
-template <class R>
-__device__ __forceinline__ R frac_below_dd(R h0, R h1, R h2, R h3, R d, R &df)
+// refined once more: FP64 accuracy (the last place may differ)
+__device__ __forceinline__ double full_rcp(double x)
 {
-    df = R(0);
-    if (d <= h0) return R(0);
-    if (d >= h3) return R(1);
-    if (d <= h1) {
-        const R x = d - h0, p = mx_rcp<R>((h1 - h0) * (h2 - h0) * (h3 - h0));
-        df = R(3) * x * x * p;
-        return x * x * x * p;
-    }
-    if (d >= h2) {
-        const R y = h3 - d, q = mx_rcp<R>((h3 - h0) * (h3 - h1) * (h3 - h2));
-        df = R(3) * y * y * q;
-        return R(1) - y * y * y * q;
-    }
-    const R ra = mx_rcp<R>(h2 - h0), rb = mx_rcp<R>(h3 - h0), rc = mx_rcp<R>(h2 - h1), re = mx_rcp<R>(h3 - h1);
-    const R a = (d - h0) * ra, b = (d - h0) * rb, c = (d - h1) * rc, e = (d - h1) * re;
-    df = ra * b + a * rb + ra * (R(1) - b) * e - a * rb * e + a * (R(1) - b) * re - ra * c * e +
-         (R(1) - a) * rc * e + (R(1) - a) * c * re;
-    return a * b + a * (R(1) - b) * e + (R(1) - a) * c * e;
+    const double r = mx_rcp(x), t = fma(r, fma(-x, r, 1.0), r);
+    return isfinite(t) ? t : r;
+}
+__device__ __forceinline__ int hiword(double x) { return __double2hiint(x); }
+
+// Cut fraction of a tetrahedron with sorted projections h0..h3 below a level:
+// one vertex below: the product of three edge fractions; one above: one minus
+// such a product; two and two: ab + a(1-b)e + (1-a)ce.  The reciprocals of the
+// projection differences are formed once (r10 = 1/(h1-h0), ra = 1/(h2-h0),
+// rb = 1/(h3-h0), rc = 1/(h2-h1), re = 1/(h3-h1), r32 = 1/(h3-h2)), all three
+// forms are evaluated and one is selected by the signs of the level's distances
+// to the vertices: 21 FP64 instructions a tetrahedron, where the branches, taken
+// one after another by the lanes of a warp, with their divisions were over 200.
+// (A difference of zero makes an infinite reciprocal only in a form that is not
+// selected.)
+struct FillTet { double h0, h1, h2, h3, r10, ra, rb, rc, re, r32; };
+
+__device__ __forceinline__ double fill_below(const FillTet &q, double d)
+{
+    const double u = d - q.h0, v = d - q.h1, z = q.h2 - d, y = q.h3 - d;
+    const double a = u * q.ra, b = u * q.rb, c = v * q.rc, e = v * q.re;
+    const double ab = a * b;
+    const double mid = fma(fma(-a, c, c), e, fma(fma(-a, b, a), e, ab));
+    const double low = (u * q.r10) * ab;
+    const double top = 1.0 - (y * q.r32) * (y * q.re) * (y * q.rb);
+    double f = hiword(v) <= 0 ? low : hiword(z) <= 0 ? top : mid;
+    f = hiword(y) <= 0 ? 1.0 : f;
+    return hiword(u) <= 0 ? 0.0 : f;
 }
 
-// MIXED: cells with 1e-4 < alpha < 1 - 1e-4 are positioned by safeguarded
-// Newton steps on the fill, whose derivative is the cut area: first in FP32
-// on projections relative to the cell centre while the residual is above 1e-5
-// (FP32 rounding of the fill is ~1e-7), then in FP64 to the 1e-13 stop; a
-// step that leaves the bracket is replaced by bisection.  Cells within 1e-4
-// of 0 or 1 take FP64 Newton from the corner estimate.  The plain FP64 form
-// follows Alg. 1 (secant; bisection once the secant leaves the bracket or
-// has not converged in POS_SECANT_MAX steps).
-// G lanes per cell: 32, or 8 where every cell has at most 16 tetrahedra (a
-// tetrahedral mesh: four cells per warp); reductions over the cell's lanes
-template <bool LIST, bool MIXED, int G, int KL, bool COUNT>
-__global__ void __launch_bounds__(128, KL == 3 ? 4 : 5) k_reconstruct(DevMesh m, const double *__restrict__ alpha,
-                                                     const double *__restrict__ palpha, const int *list,
-                                                     const int *count, double *nout, double *dout,
-                                                     uint8_t *fout, int *itout, int *maxit, unsigned *status,
-                                                     const float *__restrict__ s0, int s0cap, int *next,
-                                                     unsigned long long *work, const double *__restrict__ gin)
+// the same in FP32 with its derivative (the cut area over the volume)
+struct FillTetF { float h0, h1, h2, h3, r10, ra, rb, rc, re, r32; };
+
+__device__ __forceinline__ float fill_below(const FillTetF &q, float d, float &df)
 {
-    // fill evaluations per cell tetrahedron (FP64, FP32), counted by the
-    // cell's first lane and added once per thread at the end
-    unsigned long long nf64 = 0, nf32 = 0;
+    const float u = d - q.h0, v = d - q.h1, z = q.h2 - d, y = q.h3 - d;
+    const float a = u * q.ra, b = u * q.rb, c = v * q.rc, e = v * q.re;
+    const float ab = a * b, b1 = 1.0f - b, a1 = 1.0f - a;
+    const float mid = ab + a * b1 * e + a1 * c * e;
+    const float dmid = q.ra * b + a * q.rb + q.ra * b1 * e - a * q.rb * e + a * b1 * q.re - q.ra * c * e +
+                       a1 * q.rc * e + a1 * c * q.re;
+    const float lx = q.r10 * ab, tx = (y * q.re) * (y * q.rb) * q.r32;
+    const float low = u * lx, top = 1.0f - y * tx;
+    float f = v <= 0.0f ? low : z <= 0.0f ? top : mid;
+    df = v <= 0.0f ? 3.0f * lx : z <= 0.0f ? 3.0f * tx : dmid;
+    if (y <= 0.0f) { f = 1.0f; df = 0.0f; }
+    if (u <= 0.0f) { f = 0.0f; df = 0.0f; }
+    return f;
+}
+
+// The fill in FP64 with its three derivatives (between two vertex projections
+// it is a cubic, so these give it exactly up to the next one); gap is lowered
+// to the high word of the least distance of the level to a projection.
+__device__ __forceinline__ void fill_taylor(const double h[4], double d, double F[4], int &gap)
+{
+    const double u = d - h[0], v = d - h[1], z = h[2] - d, y = h[3] - d;
+    gap = min(min(gap, hiword(u) & 0x7fffffff), hiword(v) & 0x7fffffff);
+    gap = min(min(gap, hiword(z) & 0x7fffffff), hiword(y) & 0x7fffffff);
+    F[0] = F[1] = F[2] = F[3] = 0.0;
+    if (hiword(u) <= 0) return;
+    if (hiword(y) <= 0) { F[0] = 1.0; return; }
+    const double d20 = h[2] - h[0], d30 = h[3] - h[0], d31 = h[3] - h[1];
+    const bool low = hiword(v) <= 0;
+    if (low || hiword(z) <= 0) {
+        // k w^3 from the lowest vertex, or one minus that from the highest
+        const double w = low ? u : y;
+        const double k = mx_rcp(d30 * (low ? (h[1] - h[0]) * d20 : d31 * (h[3] - h[2])));
+        const double kw = k * w, kww = kw * w;
+        F[0] = low ? kww * w : fma(-kww, w, 1.0);
+        F[1] = 3.0 * kww;
+        F[2] = (low ? 6.0 : -6.0) * kw;
+        F[3] = 6.0 * k;
+        return;
+    }
+    const double ra = mx_rcp(d20), rb = mx_rcp(d30), rc = mx_rcp(h[2] - h[1]), re = mx_rcp(d31);
+    const double a = u * ra, b = u * rb, c = v * rc, e = v * re;
+    // f = ab + ae + ce - ae (b + c)
+    const double s = b + c, rs = rb + rc, ae = a * e, dae = fma(ra, e, a * re), rae = ra * re;
+    F[0] = fma(-ae, s, fma(a, b, fma(c, e, ae)));
+    F[1] = fma(-ae, rs, fma(-dae, s, fma(ra, b, fma(a, rb, fma(rc, e, fma(c, re, dae))))));
+    F[2] = 2.0 * fma(-rae, s, fma(-dae, rs, fma(ra, rb, fma(rc, re, rae))));
+    F[3] = -6.0 * rae * rs;
+}
+
+struct RcCell {
+    int fl, it, it32;
+    V3 n;
+    double d;
+};
+
+// The plane of interface cell c (eps < a = alpha[c] < 1 - eps).
+//
+// MIXED: the offset is measured from the end of the cell's extent that is
+// nearer in volume (target t = a from below, or 1 - a from above), so that
+// cells near 0 and 1 keep their relative precision: safeguarded Newton steps on
+// the fill in FP32 until its residual is within 1e-5 t (ten times its
+// rounding) and one more, then one FP64 evaluation with derivatives, on whose
+// cubic the offset is finished when the step stays short of the next vertex
+// projection (nearly always: the FP32 offset is good to about 1e-6); else
+// safeguarded FP64 Newton steps to the same 1e-13 stop.  (With FP64 Newton
+// steps of value and slope there were 2.4 evaluations per cell, up to 14 near 0
+// and 1.)  FP64 form: Alg. 1 (secant; bisection once the secant leaves the
+// bracket or has not converged in POS_SECANT_MAX steps).
+// guess: a start sg (fraction of the extent from below) is given.
+template <bool MIXED, int G, int KL>
+__device__ __forceinline__ RcCell rc_cell(const DevMesh &m, const double *__restrict__ alpha,
+                                          const double *__restrict__ palpha, const double *__restrict__ gin, int c,
+                                          double a, bool guess, float sg, unsigned *status)
+{
     const int lane = threadIdx.x & (G - 1);
     const unsigned tm = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (threadIdx.x & 31 & ~(G - 1));
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) / G;
-    const int nwarps = (gridDim.x * blockDim.x) / G;
     auto tsum = [&](double v) {
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(tm, v, o);
         return v;
     };
-    auto tmin = [&](double v) {
+    RcCell r{VOF_INTERFACE, 0, 0, mk(0, 0, 0), 0.0};
+    const double V = m.vc[c];
+    const int t0 = __ldg(m.ctptr + c), nt = __ldg(m.ctptr + c + 1) - t0;
+    // ---- NAG gradient: lane j handles the j-th (face, point) entry
+    // (a given gradient instead, times V: the generalised LSQ one)
+    V3 g = mk(0, 0, 0);
+    if (gin) {
+        if (lane == 0) g = ld3(gin, m.nc, c) * V;
+    } else
+    for (int j = __ldg(m.ceptr + c) + lane, e1 = __ldg(m.ceptr + c + 1); j < e1; j += G) {
+        const int2 en = __ldg(m.cent + j);  // {fpts slot, face code}
+        const int f = en.y >> 1, p = __ldg(m.fpts + en.x);
+        double ap = 0.0;  // Eq. idwpointphi (precomputed per point when palpha is given)
+        if (palpha) ap = __ldg(palpha + p);
+        else
+            for (int q = __ldg(m.pptr + p); q < __ldg(m.pptr + p + 1); ++q)
+                ap += __ldg(m.pw + q) * __ldg(alpha + __ldg(m.pcell + q));
+        double w = __ldg(m.nagc + en.x) * ap;
+        if (en.y & 1) w = -w;  // Eq. own-nei: the neighbour sees -S_f
+        g = g + ld3(m.sf, m.nf, f) * w;
+    }
+    // g = G / V; the cell is oriented where |g| V^(1/3) > 1e-12, taken
+    // as |G|^6 > 1e-72 V^4 (no cube root, square root or division)
+    g = mk(tsum(g.x), tsum(g.y), tsum(g.z));
+    const double g2 = dot(g, g);
+    if (!(g2 * g2 * g2 > 1e-72 * (V * V) * (V * V))) return r;
+    const V3 nn = r.n = g * -rsqrt(g2);  // points out of the phase
+    r.fl |= VOF_ORIENTED;
+    // ---- cell tetrahedra (c_c, outward face triangle), lanes j, j + G, ...:
+    // sorted projections and volumes (0: no tetrahedron)
+    const double ec = dot(nn, ld3(m.cc, m.nc, c));
+    double h[KL][4], vk[KL];
+    double lo = 1e300, hi = -1e300;
 #pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(tm, v, o));
-        return v;
-    };
-    auto tmax = [&](double v) {
+    for (int s = 0; s < KL; ++s) {
+        vk[s] = 0.0;
+        h[s][0] = h[s][1] = h[s][2] = h[s][3] = 0.0;
+        if (lane + G * s >= nt) continue;
+        const int4 te = __ldg(m.ctet + t0 + lane + G * s);  // {face code, slot a, slot b, slot c or -1}
+        vk[s] = __ldg(m.ctvol + t0 + lane + G * s);
+        const V3 p1 = ldP(m, __ldg(m.fpts + te.y)), p2 = ldP(m, __ldg(m.fpts + te.z));
+        const V3 p0 = te.w >= 0 ? ldP(m, __ldg(m.fpts + te.w)) : ld3(m.cf, m.nf, te.x >> 1);
+        double e0 = ec, e1 = dot(nn, p0), e2 = dot(nn, p1), e3 = dot(nn, p2), t;
+#define RC_CS(p, q) if (gt_bits(p, q)) { t = p; p = q; q = t; }
+        RC_CS(e0, e1) RC_CS(e2, e3) RC_CS(e0, e2) RC_CS(e1, e3) RC_CS(e1, e2)
+#undef RC_CS
+        h[s][0] = e0; h[s][1] = e1; h[s][2] = e2; h[s][3] = e3;
+        if (gt_bits(lo, e0)) lo = e0;
+        if (gt_bits(e3, hi)) hi = e3;
+    }
 #pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(tm, v, o));
-        return v;
-    };
-    const int total = LIST ? *count : m.nc;
+    for (int o = G / 2; o > 0; o >>= 1) {
+        const double l2 = __shfl_xor_sync(tm, lo, o), h2 = __shfl_xor_sync(tm, hi, o);
+        if (gt_bits(lo, l2)) lo = l2;
+        if (gt_bits(h2, hi)) hi = h2;
+    }
+    const double dmin = lo, dmax = hi, range = dmax - dmin, rV = 1.0 / V;
+    int it = 0;
+    if constexpr (MIXED) {
+        const bool up = gt_pos(a, 0.5);  // measured from above
+        const double tgt = up ? 1.0 - a : a;
+        FillTetF q[KL];
+        float vf[KL];
+        const float rr = __frcp_rn((float)range), tf = (float)tgt;
+#pragma unroll
+        for (int s = 0; s < KL; ++s) {
+            if (up) {
+                const double x0 = dmax - h[s][3], x1 = dmax - h[s][2], x2 = dmax - h[s][1], x3 = dmax - h[s][0];
+                h[s][0] = x0; h[s][1] = x1; h[s][2] = x2; h[s][3] = x3;
+            } else {
+                h[s][0] -= dmin; h[s][1] -= dmin; h[s][2] -= dmin; h[s][3] -= dmin;
+            }
+            // in units of the extent; volumes as fractions of the cell's
+            const float f0 = (float)h[s][0] * rr, f1 = (float)h[s][1] * rr, f2 = (float)h[s][2] * rr,
+                        f3 = (float)h[s][3] * rr;
+            q[s] = FillTetF{f0, f1, f2, f3, __fdividef(1.0f, f1 - f0), __fdividef(1.0f, f2 - f0),
+                            __fdividef(1.0f, f3 - f0), __fdividef(1.0f, f2 - f1), __fdividef(1.0f, f3 - f1),
+                            __fdividef(1.0f, f3 - f2)};
+            vf[s] = (float)(vk[s] * rV);
+        }
+        // start: the fraction itself (or the learned offset), the corner
+        // estimate t^(1/3) within 1e-4 of 0 or 1
+        float A = 0.0f, B = 1.0f, x;
+        if (tf > 1e-4f) x = guess ? (up ? 1.0f - sg : sg) : tf;
+        else x = cbrtf(tf);
+        while (it < POS_MAXIT) {
+            float part = 0.0f, dpart = 0.0f;
+#pragma unroll
+            for (int s = 0; s < KL; ++s)
+                if (vf[s] > 0.0f) {
+                    float df;
+                    part += vf[s] * fill_below(q[s], x, df);
+                    dpart += vf[s] * df;
+                }
+#pragma unroll
+            for (int o = G / 2; o > 0; o >>= 1) {
+                part += __shfl_xor_sync(tm, part, o);
+                dpart += __shfl_xor_sync(tm, dpart, o);
+            }
+            ++it;
+            const float gf = part - tf;
+            const bool sure = fabsf(gf) > 1e-5f * tf;
+            if (sure) {
+                if (gf < 0.0f) A = x; else B = x;
+            }
+            float xn = x - __fdividef(gf, dpart);
+            if (!(xn > A && xn < B)) xn = 0.5f * (A + B);
+            if (!(xn > A && xn < B)) break;  // bracket at FP32 resolution
+            x = xn;
+            if (!sure) break;
+        }
+        r.it32 = it;
+        double X = (double)x * range, lo64 = (double)A * range, hi64 = (double)B * range;
+        while (it < POS_MAXIT) {
+            double S[4] = {0.0, 0.0, 0.0, 0.0};
+            int gap = 0x7fffffff;
+#pragma unroll
+            for (int s = 0; s < KL; ++s)
+                if (vf[s] > 0.0f) {
+                    double F[4];
+                    fill_taylor(h[s], X, F, gap);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) S[k] = fma(vk[s], F[k], S[k]);
+                }
+#pragma unroll
+            for (int o = G / 2; o > 0; o >>= 1) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) S[k] += __shfl_xor_sync(tm, S[k], o);
+                gap = min(gap, __shfl_xor_sync(tm, gap, o));
+            }
+            ++it;
+            const double gx = fma(S[0], rV, -tgt);
+            if (le_pos(fabs(gx), POS_TOL)) break;
+            if (hiword(gx) < 0) lo64 = X; else hi64 = X;
+            if (hi64 - lo64 <= 1e-15 * range) break;
+            // chord steps on the cubic gx + f1 s + f2 s^2 + f3 s^3 (the slope
+            // sets the rate only: an FP32 reciprocal of it)
+            const double f1 = S[1] * rV, f2 = S[2] * (0.5 * rV), f3 = S[3] * ((1.0 / 6.0) * rV);
+            const double k1 = (double)__frcp_rn((float)f1);
+            const double s1 = -gx * k1;
+            auto cubic = [&](double s) { return fma(fma(fma(f3, s, f2), s, f1), s, gx); };
+            const double s2 = fma(-cubic(s1), k1, s1);
+            const double xn = X + s2;
+            if ((hiword(s2) & 0x7fffffff) < gap && le_pos(fabs(cubic(s2)), POS_TOL) && xn > lo64 && xn < hi64) {
+                X = xn;
+                break;
+            }
+            X += s1;
+            if (!(X > lo64 && X < hi64)) X = 0.5 * (lo64 + hi64);
+        }
+        r.d = up ? dmax - X : dmin + X;
+    } else {
+        FillTet q[KL];
+#pragma unroll
+        for (int s = 0; s < KL; ++s) {
+            const double d10 = h[s][1] - h[s][0], d20 = h[s][2] - h[s][0], d30 = h[s][3] - h[s][0];
+            const double d21 = h[s][2] - h[s][1], d31 = h[s][3] - h[s][1], d32 = h[s][3] - h[s][2];
+            q[s] = FillTet{h[s][0], h[s][1], h[s][2], h[s][3], full_rcp(d10), full_rcp(d20), full_rcp(d30),
+                           full_rcp(d21), full_rcp(d31), full_rcp(d32)};
+        }
+        double A = dmin, B = dmax, x0 = A, g0 = -a, x1 = B, g1 = 1.0 - a, gx = 0.0, x = 0.0;
+        const double btol = 1e-15 * range;
+        bool bisect = false;
+        while (it < POS_MAXIT) {
+            if (it >= POS_SECANT_MAX) bisect = true;
+            if (!bisect) {
+                x = x1 - g1 * (x1 - x0) * mx_rcp(g1 - g0);
+                if (!(gt_bits(x, A) && gt_bits(B, x))) bisect = true;
+            }
+            if (bisect) x = 0.5 * (A + B);
+            double part = 0.0;
+#pragma unroll
+            for (int s = 0; s < KL; ++s)
+                if (hiword(vk[s]) > 0) part = fma(vk[s], fill_below(q[s], x), part);
+            gx = fma(tsum(part), rV, -a);
+            ++it;
+            if (hiword(gx) < 0) A = x; else B = x;
+            x0 = x1; g0 = g1; x1 = x; g1 = gx;
+            if (le_pos(fabs(gx), POS_TOL)) break;
+            if (!gt_bits(B - A, btol)) break;
+        }
+        r.d = x;
+    }
+    if (it >= POS_MAXIT && lane == 0) atomicOr(status, VOF_ST_POS_NOT_CONVERGED);
+    r.it = it;
+    return r;
+}
+
+struct RcArgs {
+    const double *alpha, *palpha, *gin;  // palpha, gin: may be null
+    double *n, *d;
+    uint8_t *flags;
+    int *iters;                  // or null
+    unsigned *status;
+    unsigned long long *work;    // counting variant
+};
+
+constexpr int RC_THREADS = 128;
+// blocks per SM (96 registers a thread, 128 with more tetrahedra per lane)
+template <int KL> constexpr int rc_resident() { return KL == 1 ? 5 : 4; }
+
+// fill evaluations per cell tetrahedron (FP64, FP32), counted by a cell's first lane
+template <int G, bool COUNT>
+struct RcCount {
+    unsigned nf64 = 0, nf32 = 0;
+    __device__ __forceinline__ void add(const DevMesh &m, int c, const RcCell &r)
+    {
+        if (!COUNT || (threadIdx.x & (G - 1))) return;
+        const unsigned nte = __ldg(m.ctptr + c + 1) - __ldg(m.ctptr + c);
+        nf32 += r.it32 * nte;
+        nf64 += (r.it - r.it32) * nte;
+    }
+    __device__ __forceinline__ void flush(unsigned long long *work)
+    {
+        if (!COUNT) return;
+        const unsigned r64 = __reduce_add_sync(0xffffffffu, nf64);
+        const unsigned r32 = __reduce_add_sync(0xffffffffu, nf32);
+        if ((threadIdx.x & 31) == 0) {
+            work_add1(work, WK_FILL64, r64);
+            work_add1(work, WK_FILL32, r32);
+        }
+    }
+};
+
+// The listed cells; with a counter a lane group takes its next cell as it
+// finishes one (cells differ in positioning iterations), else static striding.
+template <bool MIXED, int G, int KL, bool COUNT>
+__global__ void __launch_bounds__(RC_THREADS, rc_resident<KL>())
+k_reconstruct(DevMesh m, RcArgs q, const int *list, const int *count, int *maxit, const float *__restrict__ s0,
+              int s0cap, int *next)
+{
+    const int lane = threadIdx.x & (G - 1);
+    const unsigned tm = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (threadIdx.x & 31 & ~(G - 1));
+    const int group = (blockIdx.x * blockDim.x + threadIdx.x) / G, ngroups = (gridDim.x * blockDim.x) / G;
+    const int total = *count;
     const double eps = m.eps;
-    // LIST with a counter: a lane group takes its next cell as it finishes one
-    // (cells differ in positioning iterations); else static striding
-    const bool dyn = LIST && next != nullptr;
+    RcCount<G, COUNT> wk;
     auto take = [&]() {
         int v = 0;
         if (lane == 0) v = atomicAdd(next, 1);
         return __shfl_sync(tm, v, 0, G);
     };
-    for (int item = dyn ? take() : warp; item < total; item = dyn ? take() : item + nwarps) {
-        const int c = LIST ? list[item] : item;
-        const double a = alpha[c];
-        uint8_t fl = 0;
-        V3 nn = mk(0, 0, 0);
-        double dd = 0.0;
-        int it = 0;
-        if (a >= 1.0 - eps) fl = VOF_FULL;
-        else if (a > eps) {
-            fl = VOF_INTERFACE;
-            const double V = m.vc[c];
-            // ---- NAG gradient: lane j handles the j-th (face, point) entry
-            // (a given gradient instead, times V: the generalised LSQ one)
-            V3 g = mk(0, 0, 0);
-            if (gin) {
-                if (lane == 0) g = ld3(gin, m.nc, c) * V;
-            } else
-            for (int j = __ldg(m.ceptr + c) + lane, e1 = __ldg(m.ceptr + c + 1); j < e1; j += G) {
-                const int2 en = __ldg(m.cent + j);  // {fpts slot, face code}
-                const int f = en.y >> 1, p = __ldg(m.fpts + en.x);
-                double ap = 0.0;  // Eq. idwpointphi (precomputed per point when palpha is given)
-                if (palpha) ap = __ldg(palpha + p);
-                else
-                    for (int q = __ldg(m.pptr + p); q < __ldg(m.pptr + p + 1); ++q)
-                        ap += __ldg(m.pw + q) * __ldg(alpha + __ldg(m.pcell + q));
-                double w = __ldg(m.nagc + en.x) * ap;
-                if (en.y & 1) w = -w;  // Eq. own-nei: the neighbour sees -S_f
-                g = g + ld3(m.sf, m.nf, f) * w;
-            }
-            // g = G / V; the cell is oriented where |g| V^(1/3) > 1e-12, taken
-            // as |G|^6 > 1e-72 V^4 (no cube root, square root or division)
-            g = mk(tsum(g.x), tsum(g.y), tsum(g.z));
-            const double g2 = dot(g, g);
-            if (g2 * g2 * g2 > 1e-72 * (V * V) * (V * V)) {
-                nn = g * -rsqrt(g2);  // points out of the phase
-                fl |= VOF_ORIENTED;
-                // ---- cell tetrahedra (c_c, outward face triangle), lanes j, j+32
-                const V3 ctr = ld3(m.cc, m.nc, c);
-                double h[KL][4], vk[KL];
-                float hf[KL][4], vkf[KL];
-                const double href = dot(nn, ctr);
-                double lo = 1e300, hi = -1e300;
-#pragma unroll
-                for (int s = 0; s < KL; ++s) {
-                    vk[s] = 0.0;
-                    h[s][0] = h[s][1] = h[s][2] = h[s][3] = 0.0;
-                    vkf[s] = 0.0f;
-                    hf[s][0] = hf[s][1] = hf[s][2] = hf[s][3] = 0.0f;
-                    const int tj = __ldg(m.ctptr + c) + lane + G * s;
-                    if (tj >= __ldg(m.ctptr + c + 1)) continue;
-                    const int4 te = __ldg(m.ctet + tj);  // {face code, slot a, slot b, slot c or -1}
-                    V3 t0, t1, t2;
-                    if (te.w >= 0) {
-                        t0 = ldP(m, __ldg(m.fpts + te.y)); t1 = ldP(m, __ldg(m.fpts + te.z)); t2 = ldP(m, __ldg(m.fpts + te.w));
-                    } else {
-                        t0 = ld3(m.cf, m.nf, te.x >> 1); t1 = ldP(m, __ldg(m.fpts + te.y)); t2 = ldP(m, __ldg(m.fpts + te.z));
-                    }
-                    if (te.x & 1) { V3 q = t1; t1 = t2; t2 = q; }
-                    vk[s] = fabs(tvol(ctr, t0, t1, t2));
-                    double e0 = dot(nn, ctr), e1 = dot(nn, t0), e2 = dot(nn, t1), e3 = dot(nn, t2);
-                    sort4(e0, e1, e2, e3);
-                    h[s][0] = e0; h[s][1] = e1; h[s][2] = e2; h[s][3] = e3;
-                    if (MIXED) {
-                        hf[s][0] = (float)(e0 - href); hf[s][1] = (float)(e1 - href);
-                        hf[s][2] = (float)(e2 - href); hf[s][3] = (float)(e3 - href);
-                        vkf[s] = (float)vk[s];
-                    }
-                    lo = fmin(lo, e0);
-                    hi = fmax(hi, e3);
-                }
-                const double dmin = tmin(lo), dmax = tmax(hi);
-                double x = 0.0;
-                int it32 = 0;
-                if (MIXED && a > 1e-4 && a < 1.0 - 1e-4) {
-                    // ---- FP32 Newton, relative to the cell centre's projection
-                    const float Vf = (float)V, af = (float)a, rVf = __frcp_rn(Vf);
-                    float Ar = (float)(dmin - href), Br = (float)(dmax - href);
-                    // start: the learned offset where one is given, else alpha
-                    const float sg = (s0 && item < s0cap) ? s0[item] : af;
-                    float xr = Ar + sg * (Br - Ar);
-                    int near = 0;
-                    while (it < POS_MAXIT) {
-                        float part = 0.0f, dpart = 0.0f;
-#pragma unroll
-                        for (int s = 0; s < KL; ++s)
-                            if (vkf[s] > 0.0f) {
-                                float df;
-                                part += vkf[s] * frac_below_dd(hf[s][0], hf[s][1], hf[s][2], hf[s][3], xr, df);
-                                dpart += vkf[s] * df;
-                            }
-#pragma unroll
-                        for (int o = G / 2; o > 0; o >>= 1) {
-                            part += __shfl_xor_sync(tm, part, o);
-                            dpart += __shfl_xor_sync(tm, dpart, o);
-                        }
-                        ++it;
-                        const float gf = part * rVf - af;
-                        // below 1e-5 the FP32 sign is not reliable: the bracket takes
-                        // no update from it, and after two more Newton steps (down to
-                        // the FP32 rounding of the fill) FP64 takes over
-                        const bool sure = fabsf(gf) > 1e-5f;
-                        if (sure) {
-                            if (gf < 0.0f) Ar = xr; else Br = xr;
-                        }
-                        float xn = xr - gf * Vf * __frcp_rn(dpart);
-                        if (!(xn > Ar && xn < Br)) xn = 0.5f * (Ar + Br);
-                        if (!(xn > Ar && xn < Br)) break;  // bracket at FP32 resolution
-                        xr = xn;
-                        if (!sure && ++near >= 2) break;
-                    }
-                    // ---- FP64 Newton from there
-                    it32 = it;
-                    const double rV = 1.0 / V;
-                    double A = href + (double)Ar, B = href + (double)Br;
-                    x = href + (double)xr;
-                    while (it < POS_MAXIT) {
-                        double part = 0.0, dpart = 0.0;
-#pragma unroll
-                        for (int s = 0; s < KL; ++s)
-                            if (vk[s] > 0.0) {
-                                double df;
-                                part += vk[s] * frac_below_dd(h[s][0], h[s][1], h[s][2], h[s][3], x, df);
-                                dpart += vk[s] * df;
-                            }
-                        const double gx = tsum(part) * rV - a;
-                        dpart = tsum(dpart);
-                        ++it;
-                        if (fabs(gx) <= POS_TOL) break;
-                        if (gx < 0) A = x; else B = x;
-                        if (B - A <= 1e-15 * (dmax - dmin)) break;
-                        // the slope only sets the rate, not the root: an FP32
-                        // reciprocal of it (a step that leaves the bracket, or is
-                        // NaN, is replaced by bisection)
-                        double xn = x - gx * V * (double)__frcp_rn((float)dpart);
-                        if (!(xn > A && xn < B)) xn = 0.5 * (A + B);
-                        x = xn;
-                    }
-                } else if (MIXED) {
-                    // ---- alpha within 1e-4 of 0 or 1: FP64 Newton from the corner
-                    // estimate (near an end the fill grows like the cube of the
-                    // distance from the extreme vertex)
-                    double A = dmin, B = dmax;
-                    const double rV = 1.0 / V;
-                    x = a < 0.5 ? dmin + (dmax - dmin) * cbrt(a) : dmax - (dmax - dmin) * cbrt(1.0 - a);
-                    while (it < POS_MAXIT) {
-                        double part = 0.0, dpart = 0.0;
-#pragma unroll
-                        for (int s = 0; s < KL; ++s)
-                            if (vk[s] > 0.0) {
-                                double df;
-                                part += vk[s] * frac_below_dd(h[s][0], h[s][1], h[s][2], h[s][3], x, df);
-                                dpart += vk[s] * df;
-                            }
-                        const double gx = tsum(part) * rV - a;
-                        dpart = tsum(dpart);
-                        ++it;
-                        if (fabs(gx) <= POS_TOL) break;
-                        if (gx < 0) A = x; else B = x;
-                        if (B - A <= 1e-15 * (dmax - dmin)) break;
-                        // the slope only sets the rate, not the root: an FP32
-                        // reciprocal of it (a step that leaves the bracket, or is
-                        // NaN, is replaced by bisection)
-                        double xn = x - gx * V * (double)__frcp_rn((float)dpart);
-                        if (!(xn > A && xn < B)) xn = 0.5 * (A + B);
-                        x = xn;
-                    }
-                } else {
-                    // ---- Alg. 1: secant, bisection once the secant leaves the
-                    // bracket or has stalled for POS_SECANT_MAX steps
-                    double A = dmin, B = dmax, x0 = A, g0 = -a, x1 = B, g1 = 1.0 - a, gx = 0.0;
-                    bool bisect = false;
-                    while (it < POS_MAXIT) {
-                        if (it >= POS_SECANT_MAX) bisect = true;
-                        if (!bisect) {
-                            x = x1 - g1 * (x1 - x0) / (g1 - g0);
-                            if (!(x > A && x < B)) bisect = true;
-                        }
-                        if (bisect) x = 0.5 * (A + B);
-                        double part = 0.0;
-#pragma unroll
-                        for (int s = 0; s < KL; ++s)
-                            if (vk[s] > 0.0) part += vk[s] * frac_below(h[s][0], h[s][1], h[s][2], h[s][3], x);
-                        gx = tsum(part) / V - a;
-                        ++it;
-                        if (gx < 0) A = x; else B = x;
-                        x0 = x1; g0 = g1; x1 = x; g1 = gx;
-                        if (fabs(gx) <= POS_TOL) break;
-                        if (B - A <= 1e-15 * (dmax - dmin)) break;
-                    }
-                }
-                if (it >= POS_MAXIT && lane == 0) atomicOr(status, VOF_ST_POS_NOT_CONVERGED);
-                if (COUNT && lane == 0) {
-                    const unsigned nte = __ldg(m.ctptr + c + 1) - __ldg(m.ctptr + c);
-                    nf32 += (unsigned long long)it32 * nte;
-                    nf64 += (unsigned long long)(it - it32) * nte;
-                }
-                dd = x;
-            }
+    for (int item = next ? take() : group; item < total; item = next ? take() : item + ngroups) {
+        const int c = list[item];
+        const double a = q.alpha[c];
+        RcCell r{a >= 1.0 - eps ? (int)VOF_FULL : 0, 0, 0, mk(0, 0, 0), 0.0};
+        if (a > eps && a < 1.0 - eps) {
+            const bool guess = s0 && item < s0cap;
+            r = rc_cell<MIXED, G, KL>(m, q.alpha, q.palpha, q.gin, c, a, guess, guess ? s0[item] : 0.0f, q.status);
+            wk.add(m, c, r);
         }
         if (lane == 0) {
-            if (nout) st3(nout, m.nc, c, nn);
-            if (dout) dout[c] = dd;
-            if (fout) fout[c] = fl;
-            if (itout) itout[c] = it;
-            if (maxit && it > 0) atomicMax(maxit, it);
+            st3(q.n, m.nc, c, r.n);
+            q.d[c] = r.d;
+            q.flags[c] = (uint8_t)r.fl;
+            if (q.iters) q.iters[c] = r.it;
+            if (maxit && r.it > 0) atomicMax(maxit, r.it);
         }
     }
-    if (!COUNT) return;
-    const unsigned r64 = __reduce_add_sync(0xffffffffu, (unsigned)nf64);
-    const unsigned r32 = __reduce_add_sync(0xffffffffu, (unsigned)nf32);
-    if ((threadIdx.x & 31) == 0) {
-        work_add1(work, WK_FILL64, r64);
-        work_add1(work, WK_FILL32, r32);
+    wk.flush(q.work);
+}
+
+// Every cell of the mesh: a block writes the defaults (n = 0, d = 0, flags)
+// of a chunk of cells, lists the chunk's interface cells in shared memory and
+// hands them to its lane groups as they come free.  (One lane group per cell
+// of the mesh, nearly all of which are not interface cells: 96^3 FP64 785 us,
+// 392 us with the chunks and the evaluation above.)
+template <bool MIXED, int G, int KL, bool COUNT>
+__global__ void __launch_bounds__(RC_THREADS, rc_resident<KL>()) k_reconstruct_all(DevMesh m, RcArgs q)
+{
+    constexpr int CHUNK = 16 * (RC_THREADS / G);
+    __shared__ int cells[CHUNK], ncells, taken;
+    const int lane = threadIdx.x & (G - 1);
+    const unsigned tm = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (threadIdx.x & 31 & ~(G - 1));
+    const double eps = m.eps;
+    if (threadIdx.x == 0) ncells = taken = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < CHUNK; i += RC_THREADS) {
+        const long c = (long)blockIdx.x * CHUNK + i;
+        if (c >= m.nc) break;
+        const double a = q.alpha[c];
+        q.flags[c] = a >= 1.0 - eps ? VOF_FULL : 0;
+        st3(q.n, m.nc, (int)c, mk(0, 0, 0));
+        q.d[c] = 0.0;
+        if (q.iters) q.iters[c] = 0;
+        if (a > eps && a < 1.0 - eps) cells[atomicAdd(&ncells, 1)] = (int)c;
     }
+    __syncthreads();
+    RcCount<G, COUNT> wk;
+    const int total = ncells;
+    for (;;) {
+        int item = 0;
+        if (lane == 0) item = atomicAdd(&taken, 1);
+        item = __shfl_sync(tm, item, 0, G);
+        if (item >= total) break;
+        const int c = cells[item];
+        const RcCell r = rc_cell<MIXED, G, KL>(m, q.alpha, q.palpha, q.gin, c, q.alpha[c], false, 0.0f, q.status);
+        wk.add(m, c, r);
+        if (lane == 0) {
+            st3(q.n, m.nc, c, r.n);
+            q.d[c] = r.d;
+            q.flags[c] = (uint8_t)r.fl;
+            if (q.iters) q.iters[c] = r.it;
+        }
+    }
+    wk.flush(q.work);
 }
 
 // ======================================== flux polyhedra and correction (A5)
@@ -1511,7 +1649,8 @@ int launch_setup_geometry(vof_ctx *c, cudaStream_t s)
     k_face_geom<<<cdiv(m.nf, 256), 256, 0, s>>>(m, (double *)m.cf, (double *)m.sf, (double *)m.nagc);
     LAUNCH_CHECK();
     unsigned *bad = c->status;
-    k_cell_geom<<<cdiv(m.nc, 256), 256, 0, s>>>(m, (double *)m.cc, (double *)m.vc, (double *)m.cbox, bad);
+    k_cell_geom<<<cdiv(m.nc, 256), 256, 0, s>>>(m, (double *)m.cc, (double *)m.vc, (double *)m.cbox,
+                                                    (double *)m.ctvol, bad);
     LAUNCH_CHECK();
     k_point_weights<<<cdiv(m.np, 256), 256, 0, s>>>(m, (double *)m.pw);
     LAUNCH_CHECK();
@@ -1533,7 +1672,6 @@ int launch_point_velocity(vof_ctx *c, const double *Uc, double *Up, cudaStream_t
     return VOF_OK;
 }
 
-// reconstruction launch with the context's lanes per cell (8 or 32)
 // ===================================== generalised LSQ gradient (Sec. 2.2.1)
 // Per cell the gradient minimising sum_k w^2 (phi_k - phi_c - g.d)^2 over the
 // cells k sharing a point with c (d = x_k - x_c, w = 1/|d|, the inverse
@@ -1772,10 +1910,34 @@ int launch_remap(vof_ctx *dst, const vof_ctx *src, const double *alpha_src, cons
     return cudaGetLastError() == cudaSuccess ? VOF_OK : VOF_ERR_CUDA;
 }
 
-template <bool LIST, bool MIXED>
-static void rc_launch(vof_ctx *c, int list_blocks, const double *alpha, const double *palpha, const int *list,
-                      const int *count, double *n, double *d, uint8_t *flags, int *iters, int *maxit,
-                      cudaStream_t s, int *next = nullptr)
+// The reconstruction of the listed cells (list) or of every cell, with the
+// context's lanes per cell and tetrahedra per lane (set by the largest cell's
+// tetrahedra at creation); the instrumented variant while work counting is on.
+template <bool MIXED, bool COUNT, int G, int KL>
+static void rc_go(vof_ctx *c, const RcArgs &q, const int *list, const int *count, int *maxit, int *next, cudaStream_t s)
+{
+    if (list)
+        k_reconstruct<MIXED, G, KL, COUNT><<<num_sms(c->device) * rc_resident<KL>(), RC_THREADS, 0, s>>>(
+            c->m, q, list, count, maxit, c->mlp_s0, mlp_cap(c), next);
+    else
+        k_reconstruct_all<MIXED, G, KL, COUNT><<<cdiv(c->nc, 16 * (RC_THREADS / G)), RC_THREADS, 0, s>>>(c->m, q);
+}
+
+template <bool MIXED, bool COUNT>
+static void rc_shape(vof_ctx *c, const RcArgs &q, const int *list, const int *count, int *maxit, int *next,
+                     cudaStream_t s)
+{
+    if (c->rc_g == 4) rc_go<MIXED, COUNT, 4, 1>(c, q, list, count, maxit, next, s);
+    else if (c->rc_g == 8 && c->rc_k <= 2) rc_go<MIXED, COUNT, 8, 2>(c, q, list, count, maxit, next, s);
+    else if (c->rc_g == 8) rc_go<MIXED, COUNT, 8, 3>(c, q, list, count, maxit, next, s);
+    else if (c->rc_k == 1) rc_go<MIXED, COUNT, 32, 1>(c, q, list, count, maxit, next, s);
+    else if (c->rc_k == 2) rc_go<MIXED, COUNT, 32, 2>(c, q, list, count, maxit, next, s);
+    else rc_go<MIXED, COUNT, 32, 3>(c, q, list, count, maxit, next, s);
+}
+
+static void rc_launch(vof_ctx *c, const double *alpha, const double *palpha, const int *list, const int *count,
+                      double *n, double *d, uint8_t *flags, int *iters, int *maxit, cudaStream_t s,
+                      int *next = nullptr)
 {
     // the generalised LSQ gradient of the cells first, where selected
     const double *gin = nullptr;
@@ -1783,37 +1945,14 @@ static void rc_launch(vof_ctx *c, int list_blocks, const double *alpha, const do
         launch_lsq_gradient(c, alpha, list, count, c->grad, s);
         gin = c->grad;
     }
-    // lanes per cell and tetrahedra per lane: 4 x 1 (tetrahedral cells, eight
-    // per warp), 8 x 2 (cells of <= 16 tetrahedra),
-    // 8 x 3 (<= 24: hexahedra, four cells per warp), 32 x 2 (<= 64), 32 x 3
-    // (<= 96: octree cells next to finer ones); the instrumented variant while
-    // work counting is on (vof_count_work)
-#define RC_GO(G_, K_, BL)                                                                                    \
-    do {                                                                                                     \
-        if (c->work_on)                                                                                      \
-            k_reconstruct<LIST, MIXED, G_, K_, true><<<BL, 128, 0, s>>>(c->m, alpha, palpha, list, count, n, d, \
-                flags, iters, maxit, c->status, c->mlp_s0, mlp_cap(c), next, c->work, gin);                  \
-        else                                                                                                 \
-            k_reconstruct<LIST, MIXED, G_, K_, false><<<BL, 128, 0, s>>>(c->m, alpha, palpha, list, count, n,   \
-                d, flags, iters, maxit, c->status, c->mlp_s0, mlp_cap(c), next, nullptr, gin);                \
-    } while (0)
-    if (c->rc_g == 4) {
-        const int blocks = LIST ? list_blocks : cdiv((long)c->nc * 4, 128);
-        RC_GO(4, 1, blocks);
-    } else if (c->rc_g == 8 && c->rc_k <= 2) {
-        const int blocks = LIST ? list_blocks : cdiv((long)c->nc * 8, 128);
-        RC_GO(8, 2, blocks);
-    } else if (c->rc_g == 8) {
-        const int blocks = LIST ? list_blocks : cdiv((long)c->nc * 8, 128);
-        RC_GO(8, 3, blocks);
-    } else if (c->rc_k <= 2) {
-        const int blocks = LIST ? list_blocks : cdiv((long)c->nc * 32, 128);
-        RC_GO(32, 2, blocks);
+    const RcArgs q{alpha, palpha, gin, n, d, flags, iters, c->status, c->work_on ? c->work : nullptr};
+    if (c->precision == VOF_MIXED) {
+        if (c->work_on) rc_shape<true, true>(c, q, list, count, maxit, next, s);
+        else rc_shape<true, false>(c, q, list, count, maxit, next, s);
     } else {
-        const int blocks = LIST ? list_blocks : cdiv((long)c->nc * 32, 128);
-        RC_GO(32, 3, blocks);
+        if (c->work_on) rc_shape<false, true>(c, q, list, count, maxit, next, s);
+        else rc_shape<false, false>(c, q, list, count, maxit, next, s);
     }
-#undef RC_GO
 }
 
 // defaults of every cell (n = 0, d = 0, flags FULL or 0, iterations 0), and
@@ -1837,7 +1976,6 @@ __global__ void k_fill_list(int nc, double eps, const double *__restrict__ alpha
 int launch_reconstruct(vof_ctx *c, const double *alpha, double *n, double *d, uint8_t *flags, int *iters,
                        const int *list, const int *count, cudaStream_t s)
 {
-    int sms = num_sms(c->device);
     const bool mx = c->precision == VOF_MIXED;
     if (mx && c->mlp && !list) {
         // the guess is indexed by list position: list the interface cells first
@@ -1851,19 +1989,7 @@ int launch_reconstruct(vof_ctx *c, const double *alpha, double *n, double *d, ui
         int r = launch_mlp_guess(c, alpha, list, count, c->nc, s);
         if (r) return r;
     }
-    if (list) {
-        if (mx)
-            rc_launch<true, true>(c, sms * 16, alpha, nullptr, list, count, n, d, flags, iters,
-                                  c->counters + CNT_MAXPOS, s);
-        else
-            rc_launch<true, false>(c, sms * 16, alpha, nullptr, list, count, n, d, flags, iters,
-                                   c->counters + CNT_MAXPOS, s);
-    } else {
-        if (mx)
-            rc_launch<false, true>(c, 0, alpha, nullptr, nullptr, nullptr, n, d, flags, iters, nullptr, s);
-        else
-            rc_launch<false, false>(c, 0, alpha, nullptr, nullptr, nullptr, n, d, flags, iters, nullptr, s);
-    }
+    rc_launch(c, alpha, nullptr, list, count, n, d, flags, iters, list ? c->counters + CNT_MAXPOS : nullptr, s);
     LAUNCH_CHECK();
     return VOF_OK;
 }
@@ -2031,12 +2157,8 @@ int launch_advect(vof_ctx *c, double *alpha, const double *Uc, const double *F, 
         if (r) return r;
         ++launches;
     }
-    if (c->precision == VOF_MIXED)
-        rc_launch<true, true>(c, sms * 16, alpha, c->palpha, c->icell, cnt + CNT_ICELL, c->n, c->d, c->flags, nullptr,
-                              cnt + CNT_MAXPOS, s, cnt + CNT_RCNEXT);
-    else
-        rc_launch<true, false>(c, sms * 16, alpha, c->palpha, c->icell, cnt + CNT_ICELL, c->n, c->d, c->flags, nullptr,
-                               cnt + CNT_MAXPOS, s, cnt + CNT_RCNEXT);
+    rc_launch(c, alpha, c->palpha, c->icell, cnt + CNT_ICELL, c->n, c->d, c->flags, nullptr, cnt + CNT_MAXPOS, s,
+              cnt + CNT_RCNEXT);
     MARK(2);
     if (cudaStreamWaitEvent(s, c->ev_join, 0) != cudaSuccess) return VOF_ERR_CUDA;
     MARK(3);

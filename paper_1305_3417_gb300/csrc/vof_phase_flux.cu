@@ -87,16 +87,7 @@ __device__ __forceinline__ bool rabove(double v, double t) { return gt_pos(v, t)
 __device__ __forceinline__ bool rbelow(double v, double t) { return lt_neg(v, t); }   // v < -t
 __device__ __forceinline__ bool rpos(double v) { return gt_pos(v, 0.0); }
 __device__ __forceinline__ bool rneg(double v) { return lt_neg(v, 0.0); }
-// a > b for any signs: the bit patterns made monotone by flipping the
-// magnitude bits of negative values (-0 then orders just below +0)
-__device__ __forceinline__ bool rgt(double a, double b)
-{
-    DBits x = dbits(a), y = dbits(b);
-    const int sx = x.hi >> 31, sy = y.hi >> 31;
-    x.hi ^= sx & 0x7fffffff; x.lo ^= (unsigned)sx;
-    y.hi ^= sy & 0x7fffffff; y.lo ^= (unsigned)sy;
-    return !bits_le(x, y);
-}
+__device__ __forceinline__ bool rgt(double a, double b) { return gt_bits(a, b); }
 
 // fraction of a tetrahedron below level 0 for sorted vertex values h0..h3
 template <class R>
