@@ -547,6 +547,36 @@ int vof_create(const vof_mesh *mesh, const vof_options *opt, vof_ctx **out)
     c->bpflag = dev_alloc<uint8_t>(c, np, &err);
     c->upb = dev_alloc<double>(c, 3 * (size_t)np, &err);
     c->ktl = dev_alloc<unsigned char>(c, e4 * 6 * (size_t)ctptr[nc], &err);
+    if (!err) {
+        // The phase flux's queue: a band face has about 2.5 KB of clip jobs
+        // (twice that in FP64); 256 (512) bytes per mesh face hold a band of a
+        // tenth of the faces, and the floor any band of a small mesh.  Faces
+        // beyond it are fluxed in the slower one-warp form, so where memory is
+        // short a smaller queue serves too.
+        const size_t unit = 16, per = c->precision == VOF_MIXED ? 256 : 512;
+        size_t bytes = std::max(per * (size_t)nf, per * (size_t)(1 << 17));
+        bytes = std::min(bytes, unit * ((size_t)1 << 31));
+        void *p = nullptr;
+        while (cudaMalloc(&p, bytes) != cudaSuccess && bytes > (1u << 20)) {
+            cudaGetLastError();
+            p = nullptr;
+            bytes /= 2;
+        }
+        if (!p || c->nbufs >= (int)(sizeof(c->bufs) / sizeof(c->bufs[0]))) err = VOF_ERR_CUDA;
+        else c->bufs[c->nbufs++] = p;
+        c->pf_arena = p;
+        c->pf_cap = (unsigned)(bytes / unit);
+        c->pf_bcap = (int)(bytes / unit / 14);  // the smallest batch
+        // units of work: a band face, or its parts where the band is small
+        const size_t units = std::max<size_t>(nf, 32 * (size_t)prop.multiProcessorCount);
+        c->pf_rec = dev_alloc<BandRec>(c, nf, &err);
+        c->pf_boff = dev_alloc<unsigned>(c, c->pf_bcap, &err);
+        c->pf_bnext = dev_alloc<int>(c, c->pf_bcap, &err);
+        c->pf_part = dev_alloc<double>(c, c->pf_bcap, &err);
+        c->pf_base = dev_alloc<double>(c, units, &err);
+        c->pf_head = dev_alloc<int2>(c, units, &err);
+        c->pf_ovf = dev_alloc<int>(c, units, &err);
+    }
     if (err) { vof_destroy(c); return err; }
     cudaMemset(c->work, 0, WK_LEN * sizeof(unsigned long long));
     cudaMemset(c->bscr, 0, sizeof(double) * 3 * nc);

@@ -229,5 +229,25 @@ __device__ __forceinline__ void face_tri(const DevMesh &m, int f, int t, bool fl
     if (flip) { V3 s = t1; t1 = t2; t2 = s; }
 }
 
+// Complement form: sum the void pieces and take V_alpha = F dt - void
+// (equal in exact arithmetic since the corrected polyhedron holds F dt
+// and the stencil covers it).  Full cells then need no clipping, where
+// the plain form clips them and skips empty ones; the form is chosen by
+// which of the two leaves fewer cells reaching the polyhedron's box
+// (stencils of one chunk: decide; ties, and longer stencils, by whether the
+// upwind cell is mostly phase).  A polyhedron inside full cells carries
+// exactly F dt, one inside empty cells exactly 0, and the rounding of
+// the clipping stays with mixed cells.  Not where the polyhedron can
+// leave the domain (the normal-sweep fallback at walls; a face touching
+// an open boundary), since the part outside is empty and the stencil
+// does not cover it.
+__device__ __forceinline__ void pf_form(const DevMesh &m, const double *F, const double *alpha, int f, double lam,
+                                        long long nstencil, bool &decide, bool &comp)
+{
+    const int up = F[f] > 0.0 ? __ldg(m.own + f) : (f < m.ni ? __ldg(m.nei + f) : __ldg(m.own + f));
+    const bool comp_ok = lam >= 0.0 && !__ldg(m.fopen + f);
+    decide = comp_ok && nstencil <= 32;  // warp-uniform
+    comp = comp_ok && ge_pos(alpha[up], 0.5);
+}
 
 }  // namespace vofd

@@ -54,7 +54,8 @@ struct DevMesh {
 // the context's counter buffer: per-step counters (the first CNT_LEN ints),
 // then the two words of the grid barrier, each on its own 128-byte line
 enum { CNT_BAND = 0, CNT_ICELL, CNT_MAXPOS, CNT_MAXCORR, CNT_FALLBACK, CNT_VIOL0, CNT_VIOL1, CNT_PEND, CNT_PFNEXT,
-       CNT_RCNEXT, CNT_BPASS, CNT_BACT0, CNT_BACT1, CNT_LEN = 16 };
+       CNT_RCNEXT, CNT_BPASS, CNT_BACT0, CNT_BACT1, CNT_PFOVF, CNT_PFQ = 14 /* two words, 8-byte aligned */,
+       CNT_CLNEXT = 16, CNT_OVNEXT, CNT_LEN = 24 };
 enum { CNT_BAR = 32, CNT_BARGEN = 64, CNT_ALLOC = 96 };
 // algorithmic work counted by the step kernels (vof_work_counts): the phase
 // flux's primitives (FP32 in the mixed form, FP64 in the plain one) -- signed
@@ -65,6 +66,17 @@ enum { CNT_BAR = 32, CNT_BARGEN = 64, CNT_ALLOC = 96 };
 // coefficient triangles and cubic evaluations (FP64)
 enum { WK_PRISM = 0, WK_TEST, WK_EDGE, WK_VOL, WK_FRAC, WK_SHIFT, WK_N, WK_FACES = WK_N, WK_FILL64, WK_FILL32,
        WK_CTRI, WK_CEVAL, WK_LEN = 12 };
+
+// What the phase flux's pair stage starts a band face from, by band slot
+// (written by the correction): face centre, stencil range, face-point range,
+// and the form (bit 0: complement, bit 1: chosen later by cell counts).
+struct __align__(16) BandRec {
+    double ox, oy, oz;
+    long long s0;
+    int f, b, n, ns;
+    unsigned form, pad[3];
+};
+static_assert(sizeof(BandRec) == 64, "four 16-byte loads");
 
 struct vof_ctx {
     int device;
@@ -123,6 +135,17 @@ struct vof_ctx {
     // mixed phase-flux launch configuration (0: defaults): warps per block 1-3,
     // grid multiplier over the resident blocks
     int pf_warps, pf_mult;
+    // queue between the phase flux's pair and clip stages: batches of clip jobs
+    // (arena of 16-byte units, per batch its first unit, predecessor and sum),
+    // per unit of work its own sum and last batch, and the band slots without room
+    BandRec *pf_rec;
+    void *pf_arena;
+    unsigned pf_cap;
+    int pf_bcap;
+    unsigned *pf_boff;
+    int *pf_bnext, *pf_ovf;
+    double *pf_part, *pf_base;
+    int2 *pf_head;
     int pf_stack;                // clip-piece stack per warp: 0 = 92 pieces, 1 = 56 (more resident warps)
     int rc_g;                    // reconstruction lanes per cell (4, 8 or 32; by form and cell size)
     int rc_k;                    // tetrahedra per lane (1, 2 or 3)

@@ -848,7 +848,8 @@ __device__ __forceinline__ void correct_face(const DevMesh &m, int f, int b, int
 template <bool LIST>
 __global__ void k_correct(DevMesh m, const double *__restrict__ U, const double *__restrict__ F,
                           double dt, const int *list, const int *count, double *lam_out,
-                          int *it_out, double *disp_out, int *maxit, int *nfallback, unsigned long long *work)
+                          int *it_out, double *disp_out, int *maxit, int *nfallback, unsigned long long *work,
+                          const double *__restrict__ alpha, BandRec *rec)
 {
     const int total = LIST ? *count : m.nf;
     unsigned ntri = 0, nev = 0;  // FP64 work: cubic coefficient triangles, cubic evaluations
@@ -862,6 +863,14 @@ __global__ void k_correct(DevMesh m, const double *__restrict__ U, const double 
         else
             correct_face<VOF_MAXFP>(m, f, b, n, U, F, dt, item, lam_out, it_out, disp_out, maxit, nfallback, ntri,
                                     nev);
+        if (LIST) {
+            const long long s0 = __ldg(m.sptr + f);
+            const int ns = (int)(__ldg(m.sptr + f + 1) - s0);
+            const V3 o = ld3(m.cf, m.nf, f);
+            bool decide, comp;
+            pf_form(m, F, alpha, f, lam_out[item], ns, decide, comp);
+            rec[item] = BandRec{o.x, o.y, o.z, s0, f, b, n, ns, (comp ? 1u : 0u) | (decide ? 2u : 0u), {0u, 0u, 0u}};
+        }
     }
     ntri = __reduce_add_sync(0xffffffffu, ntri);
     nev = __reduce_add_sync(0xffffffffu, nev);
@@ -2006,7 +2015,8 @@ int launch_correct_all(vof_ctx *c, const double *Up, const double *F, double dt,
                        cudaStream_t s)
 {
     k_correct<false><<<cdiv(c->nf, 128), 128, 0, s>>>(c->m, Up, F, dt, nullptr, nullptr, lambda, iters,
-                                                             nullptr, nullptr, nullptr, c->work_on ? c->work : nullptr);
+                                                             nullptr, nullptr, nullptr, c->work_on ? c->work : nullptr,
+                                                             nullptr, nullptr);
     LAUNCH_CHECK();
     return VOF_OK;
 }
@@ -2149,7 +2159,7 @@ int launch_advect(vof_ctx *c, double *alpha, const double *Uc, const double *F, 
     k_band_point_velocity<<<cdiv(m.np, 256), 256, 0, c->s_aux>>>(m, Uc, c->bpflag, c->upb);
     k_correct<true><<<sms * 8, 128, 0, c->s_aux>>>(m, c->upb, F, dt, c->band, cnt + CNT_BAND, c->lam_b, c->it_b,
                                                    c->disp_b, cnt + CNT_MAXCORR, cnt + CNT_FALLBACK,
-                                                   c->work_on ? c->work : nullptr);
+                                                   c->work_on ? c->work : nullptr, alpha, c->pf_rec);
     LAUNCH_CHECK();
     if (cudaEventRecord(c->ev_join, c->s_aux) != cudaSuccess) return VOF_ERR_CUDA;
     if (c->precision == VOF_MIXED && c->mlp) {

@@ -51,6 +51,8 @@ __device__ __forceinline__ double rmax(double a, double b) { return fmax(a, b); 
 __device__ __forceinline__ float rabs(float a) { return fabsf(a); }
 __device__ __forceinline__ float rfma(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double rfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float rmuladd(float a, float b, float c) { return __fadd_rn(__fmul_rn(a, b), c); }
+__device__ __forceinline__ double rmuladd(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float rnext(float a, float b) { return nextafterf(a, b); }
 __device__ __forceinline__ double rnext(double a, double b) { return nextafter(a, b); }
 __device__ __forceinline__ double rabs(double a) { return fabs(a); }
@@ -115,7 +117,9 @@ template <class R>
 __device__ __forceinline__ void rsort4(R &a, R &b, R &c, R &d)
 {
     R t;
-#define CS(p, q) if (rgt(p, q)) { t = p; p = q; q = t; }
+#define CS(p, q)                                                              \
+    if constexpr (sizeof(R) == 4) { t = rmin(p, q); q = rmax(p, q); p = t; }  \
+    else if (rgt(p, q)) { t = p; p = q; q = t; }
     CS(a, b) CS(c, d) CS(a, c) CS(b, d) CS(b, c)
 #undef CS
 }
@@ -153,6 +157,7 @@ struct MXArgs {
     const void *fpl, *cbl, *ktl;  // the context's tables (R4 of the form's type)
     const int *ctptr;
     int *next;                // list form: next band slot to take (zero before the launch), or null
+    const int *items;         // list form: the band slots to take (null: 0 .. count - 1)
 };
 
 constexpr int MX_CAND = 32;    // candidate cell tetrahedra buffered per warp: one per lane
@@ -162,32 +167,50 @@ constexpr int MX_QUEUE = MX_MAXT * MX_CAND;  // clip jobs: one per (T, K) pair a
 // for more resident warps)
 constexpr int MX_STACK_WIDE = 92, MX_STACK_SLIM = 56;
 
-// per warp; in FP32 the 48-byte tetrahedra are moved as three float4
-// (conflict-free across a warp)
-template <class R, int MX_STACK>
-struct __align__(16) MXShared {
-    RTet<R> S[MX_STACK];     // pieces
-    RTet<R> T[MX_MAXT];      // flux-polyhedron tetrahedra
-    R4<R> Kp[MX_CAND][5];    // outward unit-normal planes of the candidate cell tetrahedra, then
-                             // the cell's phase (or void) half-space; 80-byte rows (FP32): a warp's
-                             // float4 reads of different rows are conflict-free
-    R4<R> P6[VOF_MAXFP][5];  // per prism (face triangle swept): a0 a1 a2 b0 b1 b2, 18 values in 20
+// Shared memory of a warp, by stage.
+// the flux polyhedron: its prisms (one per face triangle swept) and tetrahedra
+template <class R>
+struct __align__(16) PolyShared {
+    R4<R> P6[VOF_MAXFP][5];  // per prism: a0 a1 a2 b0 b1 b2, 18 values in 20
     R Pb[VOF_MAXFP][6];      // prism box
-    R Kb[MX_CAND][6];
+    R4<R> Pc[VOF_MAXFP][2];  // its centre and half extents
     R Tv6[MX_MAXT];          // |6 vol(T)|
     R Tsg[MX_MAXT];          // sign of T in the flux polyhedron
-    R Kw[MX_CAND];           // weight: 1, or alpha (1-alpha) of an unoriented cell
-    // stencil cells of the current chunk that reach the polyhedron's box
+};
+// stencil cells of the current chunk that reach the polyhedron's box
+template <class R>
+struct __align__(16) CellShared {
     R4<R> CH[32];            // phase (or void) half-space
     R Cdc[32][3];            // cell centre - face centre
     R Cw[32];
     int Ct0[32];             // first tetrahedron
     int Cend[32];            // running count of tetrahedra, inclusive
-    unsigned short Sm[MX_STACK];  // piece: t | k << 5 | planes still to clip << 10
-    unsigned short Q[MX_QUEUE];   // clip job: t | k << 5 | plane mask << 10
+    unsigned char CuseH[32];
+};
+// buffered candidate cell tetrahedra, their pairs with the prisms and the clip jobs
+template <class R>
+struct __align__(16) CandShared {
+    R4<R> Kp[MX_CAND][5];    // outward unit-normal planes of the candidate cell tetrahedra, then
+                             // the cell's phase (or void) half-space; 80-byte rows (FP32): a warp's
+                             // float4 reads of different rows are conflict-free
+    R Kw[MX_CAND];           // weight: 1, or alpha (1-alpha) of an unoriented cell
+    unsigned short Q[MX_QUEUE];              // clip job: t | k << 5 | plane mask << 10
     unsigned short PQ[VOF_MAXFP * MX_CAND];  // (prism, candidate) pairs with overlapping boxes
     unsigned char KuseH[MX_CAND];
-    unsigned char CuseH[32];
+};
+// the clip queue's pieces; in FP32 the 48-byte tetrahedra are moved as three
+// float4 (conflict-free across a warp)
+template <class R, int MX_STACK>
+struct __align__(16) StackShared {
+    RTet<R> S[MX_STACK];     // pieces
+    RTet<R> T[MX_MAXT];      // flux-polyhedron tetrahedra
+    unsigned short Sm[MX_STACK];  // piece: t | k << 5 | planes still to clip << 10
+};
+// the whole flux of a face in one warp
+template <class R, int MX_STACK_>
+struct __align__(16) MXShared : PolyShared<R>, CellShared<R>, CandShared<R>, StackShared<R, MX_STACK_> {
+    static constexpr int MX_STACK = MX_STACK_;
+    R Kb[MX_CAND][6];
 };
 
 __device__ __forceinline__ RTet<float> ldT(const RTet<float> &t)
@@ -207,6 +230,9 @@ __device__ __forceinline__ void stT(RTet<float> &t, const RTet<float> &v)
 }
 __device__ __forceinline__ void stT(RTet<double> &t, const RTet<double> &v) { t = v; }
 
+template <class R>
+__device__ __forceinline__ R pdist(R4<R> p, R3<R> v) { return p.x * v.x + p.y * v.y + p.z * v.z - p.w; }
+
 // signed distances of the vertices to plane p, those within tol taken as 0;
 // nin / nup count the vertices strictly below / above
 template <class R>
@@ -216,7 +242,7 @@ __device__ __forceinline__ void fdist(const RTet<R> &t, R4<R> p, R tol, R s[4], 
     nup = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        R v = p.x * t.v[i].x + p.y * t.v[i].y + p.z * t.v[i].z - p.w;
+        R v = pdist<R>(p, t.v[i]);
         if constexpr (std::is_same<R, double>::value) {  // integer tests
             const bool up = rabove(v, tol), dn = rbelow(v, tol);
             s[i] = (up || dn) ? v : R(0);
@@ -231,12 +257,15 @@ __device__ __forceinline__ void fdist(const RTet<R> &t, R4<R> p, R tol, R s[4], 
     }
 }
 
-// the part of t below the plane (distances s, 1 <= nin <= 3 vertices strictly
-// below, at least one strictly above) as one tetrahedron (nin == 1) or three,
-// each handed to put(tet, i); vertices are ordered below-first by a
-// compare-exchange network so that every index stays static
-template <class R, class Put>
-__device__ __forceinline__ void fsplit(const RTet<R> &t, const R s[4], int nin, Put put)
+// The part of t below the plane (distances s, 1 <= nin <= 3 vertices strictly
+// below, at least one strictly above) as the tetrahedra (a0, a1, a2, b2) and,
+// for nin > 1, (a0, a1, b2, b1) and (a0, b0, b1, b2) of the points c[0..5] = a0 a1 a2
+// b0 b1 b2.  Vertices are ordered below-first by a compare-exchange network so
+// that every index stays static; the three cases (one, two or three below) run
+// as one with selected ends of the cut edges, not as three branches that the
+// lanes of a warp take one after another.
+template <class R>
+__device__ __forceinline__ void fsplit(const RTet<R> &t, const R s[4], int nin, R3<R> c[6])
 {
     using V = R3<R>;
     V P0 = t.v[0], P1 = t.v[1], P2 = t.v[2], P3 = t.v[3];
@@ -248,32 +277,33 @@ __device__ __forceinline__ void fsplit(const RTet<R> &t, const R s[4], int nin, 
     }
     MX_CX(0, 1) MX_CX(2, 3) MX_CX(0, 2) MX_CX(1, 3) MX_CX(1, 2)
 #undef MX_CX
-    // the three or four edge parameters sa / (sa - sb) from one division
-    // (the reciprocal of the denominators' product, then products): the
-    // divisions hold the FP64 pipe longest, and FP32 saves issue slots
-    auto ept = [](V a, V b, R t) { return a + (b - a) * t; };
-    if (nin == 1) {
-        const R d1 = S0 - S1, d2 = S0 - S2, d3 = S0 - S3, p12 = d1 * d2, q = rdiv(R(1), p12 * d3);
-        const R r3 = q * p12, q3 = q * d3, r1 = q3 * d2, r2 = q3 * d1;
-        put(RTet<R>{{P0, ept(P0, P1, S0 * r1), ept(P0, P2, S0 * r2), ept(P0, P3, S0 * r3)}}, 0);
-        return;
-    }
-    V a0, a1, a2, b0, b1, b2;
-    if (nin == 2) {
-        const R d1 = S0 - S2, d2 = S0 - S3, d3 = S1 - S2, d4 = S1 - S3;
-        const R p12 = d1 * d2, p123 = p12 * d3, q = rdiv(R(1), p123 * d4);
-        const R r4 = q * p123, q3 = q * d4, r3 = q3 * p12, q2 = q3 * d3, r1 = q2 * d2, r2 = q2 * d1;
-        a0 = P0; a1 = ept(P0, P2, S0 * r1); a2 = ept(P0, P3, S0 * r2);
-        b0 = P1; b1 = ept(P1, P2, S1 * r3); b2 = ept(P1, P3, S1 * r4);
-    } else {
-        const R d1 = S0 - S3, d2 = S1 - S3, d3 = S2 - S3, p12 = d1 * d2, q = rdiv(R(1), p12 * d3);
-        const R r3 = q * p12, q3 = q * d3, r1 = q3 * d2, r2 = q3 * d1;
-        a0 = P0; a1 = P1; a2 = P2;
-        b0 = ept(P0, P3, S0 * r1); b1 = ept(P1, P3, S1 * r2); b2 = ept(P2, P3, S2 * r3);
-    }
-    put(RTet<R>{{a0, a1, a2, b2}}, 0);
-    put(RTet<R>{{a0, a1, b2, b1}}, 1);
-    put(RTet<R>{{a0, b0, b1, b2}}, 2);
+    // cut edges from f (below) to g: (0,1) (0,2) (0,3) | (0,2) (0,3) (1,2) (1,3) | (0,3) (1,3) (2,3)
+    const bool n1 = nin == 1, n2 = nin == 2, n3 = nin == 3;
+    auto sel = [](bool p, V x, V y) { return V{p ? x.x : y.x, p ? x.y : y.y, p ? x.z : y.z}; };
+    const V g0 = sel(n1, P1, sel(n2, P2, P3)), f1 = sel(n3, P1, P0), g1 = sel(n1, P2, P3);
+    const V f2 = sel(n1, P0, sel(n2, P1, P2)), g2 = sel(n2, P2, P3);
+    const R sg0 = n1 ? S1 : n2 ? S2 : S3, sf1 = n3 ? S1 : S0, sg1 = n1 ? S2 : S3;
+    const R sf2 = n1 ? S0 : n2 ? S1 : S2, sg2 = n2 ? S2 : S3;
+    // the edge parameters sf / (sf - sg) from one division (the reciprocal of
+    // the denominators' product, then products): the divisions hold the FP64
+    // pipe longest, and FP32 saves issue slots
+    const R d1 = S0 - sg0, d2 = sf1 - sg1, d3 = sf2 - sg2, d4 = n2 ? S1 - S3 : R(1);
+    const R p12 = d1 * d2, p123 = p12 * d3, q = rdiv(R(1), p123 * d4);
+    const R r4 = q * p123, q3 = q * d4, r3 = q3 * p12, q2 = q3 * d3, r1 = q2 * d2, r2 = q2 * d1;
+    // (fused explicitly: the selects below let the compiler take the sums apart)
+    auto ept = [](V a, V b, R t) { return V{rfma(b.x - a.x, t, a.x), rfma(b.y - a.y, t, a.y), rfma(b.z - a.z, t, a.z)}; };
+    const V e0 = ept(P0, g0, S0 * r1), e1 = ept(f1, g1, sf1 * r2), e2 = ept(f2, g2, sf2 * r3);
+    const V e3 = ept(P1, P3, S1 * r4);
+    c[0] = P0;
+    c[1] = sel(n3, P1, e0);
+    c[2] = sel(n3, P2, e1);
+    c[3] = sel(n3, e0, P1);
+    // (the fourth point's product is rounded before the sum in FP32: so it always
+    // was, its two cases' sums having been one after their branches)
+    const V dd = sel(n3, g1 - f1, g2 - f2);
+    const R tt = n3 ? sf1 * r2 : sf2 * r3;
+    c[4] = V{rmuladd(dd.x, tt, P1.x), rmuladd(dd.y, tt, P1.y), rmuladd(dd.z, tt, P1.z)};
+    c[5] = sel(n2, e3, e2);
 }
 
 // The queued clip jobs, worked through by the whole warp, one piece per lane
@@ -285,16 +315,20 @@ __device__ __forceinline__ void fsplit(const RTet<R> &t, const R s[4], int nin, 
 //  - split step: a piece from the other stack (else a new job) is cut by its
 //    next plane and the parts below are pushed, to the leaves if one plane is
 //    left; a new job with one plane goes to the leaves whole (no leaf work in
-//    a split step: a step's lanes never mix the two kinds of work).
+//    a split step: a step's lanes never mix the two kinds of work).  FP32: a
+//    part none of whose points is below the plane after is dropped at once (the
+//    parts share six points, so this takes six distances, not a push, a pop
+//    and a step's share each).
 // A split step commits the longest prefix of lanes that leaves the two stacks
 // at most MX_STACK - 6 full; if none does, the top piece alone when it fits,
 // else a leaf step runs first (leaves need no room).  Every part of a split
 // piece has at most 4 planes to go, so the split pieces keep i + 1 + 2 (r - 1)
 // <= MX_STACK for depth i and r planes to go: the top one alone always fits
 // once the leaves are gone, and the stacks cannot overflow.
-template <class R, int MX_STACK, class Wk>
-__device__ __forceinline__ void mx_clip(MXShared<R, MX_STACK> &sh, int nq, R tol, Acc<R> &acc, Wk &wk)
+template <class R, class Sh, class Wk>
+__device__ __forceinline__ void mx_clip(Sh &sh, const unsigned short *Q, int nq, R tol, Acc<R> &acc, Wk &wk)
 {
+    constexpr int MX_STACK = Sh::MX_STACK;
     const int lane = threadIdx.x & 31;
     const unsigned le = ((1u << lane) << 1) - 1u;
     __syncwarp();
@@ -337,34 +371,59 @@ __device__ __forceinline__ void mx_clip(MXShared<R, MX_STACK> &sh, int nq, R tol
         const bool act = lane < p + r;
         RTet<R> t;
         unsigned meta = 0;
-        if (lane < p) {
-            t = ldT(sh.S[MX_STACK - nn + lane]);
-            meta = sh.Sm[MX_STACK - nn + lane];
-        } else if (act) {
-            meta = sh.Q[qn + lane - p];
-            t = ldT(sh.T[meta & 31]);
+        if (act) {
+            const RTet<R> *src;
+            if (lane < p) {
+                meta = sh.Sm[MX_STACK - nn + lane];
+                src = &sh.S[MX_STACK - nn + lane];
+            } else {
+                meta = Q[qn + lane - p];
+                src = &sh.T[meta & 31];
+            }
+            t = ldT(*src);
         }
         __syncwarp();  // every piece read before the pushes reuse the slots
-        int nch = 0, nin = 0, nup = 0, ti = 0, k = 0;
-        unsigned rem = 0;
+        int nin = 0, nup = 0, ti = 0, k = 0;
+        unsigned rem = 0, keep = 0;  // keep: parts to push
         R sd[4];
         bool cut = false, single = false;
+        R3<R> c[6];
+        int ndrop = 0;
         if (act) {
             ti = meta & 31;
             k = (meta >> 5) & 31;
             rem = meta >> 10;
             single = (rem & (rem - 1)) == 0;
-            if (single) nch = 1;  // a job with one plane goes to the leaves whole
+            if (single) keep = 1;  // a job with one plane goes to the leaves whole
             else {
                 const int j = __ffs(rem) - 1;
                 rem &= rem - 1;
                 fdist(t, sh.Kp[k][j], tol, sd, nin, nup);
                 if (nin > 0) {
-                    if (nup > 0) cut = true;
-                    nch = nup == 0 || nin == 1 ? 1 : 3;
+                    cut = nup > 0;
+                    keep = cut && nin > 1 ? 7 : 1;
+                }
+            }
+            c[0] = t.v[0]; c[1] = t.v[1]; c[2] = t.v[2]; c[5] = t.v[3];
+            if (cut) fsplit(t, sd, nin, c);
+            if constexpr (std::is_same<R, float>::value) {
+                if (keep && !single) {
+                    const R4<R> pn = sh.Kp[k][__ffs(rem) - 1];
+                    auto below = [&](int i) { return pdist<R>(pn, c[i]) < -tol; };
+                    const bool z0 = below(0), z1 = below(1), z2 = below(2), z5 = below(5);
+                    ndrop = __popc(keep);
+                    unsigned kept = z0 || z1 || z2 || z5 ? 1u : 0u;
+                    if (keep & 2u) {
+                        const bool z3 = below(3), z4 = below(4);
+                        kept |= z0 || z1 || z5 || z4 ? 2u : 0u;
+                        kept |= z0 || z3 || z4 || z5 ? 4u : 0u;
+                    }
+                    keep = kept;
+                    ndrop -= __popc(kept);
                 }
             }
         }
+        const int nch = __popc(keep);
         const bool toleaf = single || (rem & (rem - 1)) == 0;  // one plane left after this one
         const unsigned b0 = __ballot_sync(0xffffffffu, nch & 1), b1 = __ballot_sync(0xffffffffu, nch & 2);
         const unsigned bl = __ballot_sync(0xffffffffu, toleaf);
@@ -380,21 +439,25 @@ __device__ __forceinline__ void mx_clip(MXShared<R, MX_STACK> &sh, int nq, R tol
         const unsigned lm = L >= 32 ? 0xffffffffu : (1u << L) - 1u;
         const int top = MX_STACK - nn + min(L, p);  // the split stack's top after the pops
         if (lane < L) {
-            // work of the committed lanes (the others redo theirs later)
-            wk.add(WK_TEST, !single);
-            if (cut && nch > 0) wk.add(WK_EDGE, nin == 2 ? 4 : 3);
+            // work of the committed lanes (the others redo theirs later); a
+            // dropped part counts as tested
+            wk.add(WK_TEST, !single + ndrop);
+            if (cut) wk.add(WK_EDGE, nin == 2 ? 4 : 3);
             if (nch > 0) {
                 const unsigned cm = (unsigned)ti | ((unsigned)k << 5) | (rem << 10);
                 // parts of the lanes before this one that go the same way
                 const unsigned same = (toleaf ? bl : ~bl) & ((1u << lane) - 1u);
                 const int before = __popc(b0 & same) + 2 * __popc(b1 & same);
-                auto put = [&](const RTet<R> &c, int i) {
-                    const int at = toleaf ? nl + before + i : top - 1 - before - i;
-                    stT(sh.S[at], c);
+                int at = toleaf ? nl + before : top - 1 - before;
+                const int step = toleaf ? 1 : -1;
+                auto put = [&](const RTet<R> &x) {
+                    stT(sh.S[at], x);
                     sh.Sm[at] = (unsigned short)cm;
+                    at += step;
                 };
-                if (nup == 0) put(t, 0);
-                else fsplit(t, sd, nin, put);
+                if (keep & 1u) put(RTet<R>{{c[0], c[1], c[2], c[5]}});
+                if (keep & 2u) put(RTet<R>{{c[0], c[1], c[5], c[4]}});
+                if (keep & 4u) put(RTet<R>{{c[0], c[3], c[4], c[5]}});
             }
         }
         nl += __popc(b0 & bl & lm) + 2 * __popc(b1 & bl & lm);
@@ -404,31 +467,65 @@ __device__ __forceinline__ void mx_clip(MXShared<R, MX_STACK> &sh, int nq, R tol
     }
 }
 
+// rounding allowance of the box tests: coordinates within the polyhedron's box pb
+// (and the planes' offsets, of that size) carry a few roundings each, well
+// below a quarter of the on-plane band
+template <class R>
+__device__ __forceinline__ R box_slack(const R pb[6])
+{
+    R v = R(0);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) v = rmax(v, rabs(pb[i]));
+    return v * (sizeof(R) == 4 ? R(5e-7) : R(1e-15));
+}
+
+// a box (centre, half extents) lies wholly outside a plane, by slack
+template <class R>
+__device__ __forceinline__ bool beyond(R4<R> p, R4<R> ce, R4<R> he, R slack)
+{
+    const R s = rfma(p.x, ce.x, rfma(p.y, ce.y, rfma(p.z, ce.z, -p.w)));
+    const R r = rfma(rabs(p.x), he.x, rfma(rabs(p.y), he.y, rfma(rabs(p.z), he.z, slack)));
+    return s >= r;
+}
+
 // All (T, K) pairs of the buffered candidates, taken a prism (the three
 // tetrahedra of one swept face triangle) at a time.  First lane k tests
 // candidate k's box against each prism's box and the overlapping (prism, K)
 // pairs are listed; then each listed pair, one per lane, gets the signed
 // distances of the prism's six points to K's planes, from which each of its
 // three tetrahedra is classified: outside a plane, inside every plane (adds
-// |T| at once), or a clip job.
-template <class R, int MX_STACK, class Wk>
-__device__ __forceinline__ void mx_flush(MXShared<R, MX_STACK> &sh, int nt, int ncand, R tol, Acc<R> &acc,
-                                         Wk &wk)
+// |T| at once), or a clip job.  kb: the box of candidate 'lane'.  Returns the
+// number of jobs; used gets the candidates that have any.
+// FP32: a prism whose box lies wholly beyond a plane of the candidate (by slack,
+// which covers the roundings: its points then all classify as outside) is not
+// paired; a box against a plane takes 7 instructions, a pair about 60 a plane.
+template <class R, class Sh, class Wk>
+__device__ __forceinline__ int mx_pairs(Sh &sh, int nt, int ncand, const R kb[6], R tol, R slack, Acc<R> &acc,
+                                        unsigned &used, Wk &wk)
 {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const int nprism = nt / 3;
     int total = 0;
     {
-        R kb[6];
+        constexpr bool CULL = std::is_same<R, float>::value;
+        R4<R> pl[5];
+        if constexpr (CULL) {
 #pragma unroll
-        for (int q = 0; q < 6; ++q) kb[q] = lane < ncand ? sh.Kb[lane][q] : R(0);
+            for (int q = 0; q < 5; ++q) pl[q] = sh.Kp[lane][q];
+            if (lane >= ncand || !sh.KuseH[lane]) pl[4] = mk4<R>(R(0), R(0), R(0), R(1));
+        }
         for (int pr = 0; pr < nprism; ++pr) {
             const R *tb = sh.Pb[pr];
             const bool live = sh.Tsg[3 * pr] != R(0) || sh.Tsg[3 * pr + 1] != R(0) || sh.Tsg[3 * pr + 2] != R(0);
-            const bool ov = lane < ncand && live &&
-                            !(rgt(kb[0], tb[3]) || rgt(tb[0], kb[3]) || rgt(kb[1], tb[4]) || rgt(tb[1], kb[4]) ||
-                              rgt(kb[2], tb[5]) || rgt(tb[2], kb[5]));
+            bool ov = lane < ncand && live &&
+                      !(rgt(kb[0], tb[3]) || rgt(tb[0], kb[3]) || rgt(kb[1], tb[4]) || rgt(tb[1], kb[4]) ||
+                        rgt(kb[2], tb[5]) || rgt(tb[2], kb[5]));
+            if constexpr (CULL) {
+                const R4<R> ce = sh.Pc[pr][0], he = sh.Pc[pr][1];
+#pragma unroll
+                for (int q = 0; q < 5; ++q) ov = ov && !beyond<R>(pl[q], ce, he, slack);
+            }
             const unsigned bm = __ballot_sync(0xffffffffu, ov);
             if (ov) sh.PQ[total + __popc(bm & lt)] = (unsigned short)(pr | lane << 3);
             total += __popc(bm);
@@ -436,6 +533,7 @@ __device__ __forceinline__ void mx_flush(MXShared<R, MX_STACK> &sh, int nt, int 
     }
     __syncwarp();
     int nq = 0;
+    used = 0u;
     for (int pb = 0; pb < total; pb += 32) {
         const int pi = pb + lane;
         unsigned code[3] = {0u, 0u, 0u};
@@ -513,26 +611,233 @@ __device__ __forceinline__ void mx_flush(MXShared<R, MX_STACK> &sh, int nt, int 
             if (job[j]) sh.Q[nq + __popc(bm & lt)] = (unsigned short)code[j];
             nq += __popc(bm);
         }
+        used |= __reduce_or_sync(0xffffffffu, (job[0] ? 1u << (code[0] >> 5 & 31) : 0u) |
+                                                  (job[1] ? 1u << (code[1] >> 5 & 31) : 0u) |
+                                                  (job[2] ? 1u << (code[2] >> 5 & 31) : 0u));
     }
-    if (nq > 0) mx_clip(sh, nq, tol, acc, wk);
+    return nq;
+}
+
+// the pairs of the buffered candidates and the clipping of their jobs
+template <class R, class Sh, class Wk>
+__device__ __forceinline__ void mx_flush(Sh &sh, int nt, int ncand, R tol, R slack, Acc<R> &acc, Wk &wk)
+{
+    const int lane = threadIdx.x & 31;
+    R kb[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) kb[q] = lane < ncand ? sh.Kb[lane][q] : R(0);
+    unsigned used;
+    const int nq = mx_pairs(sh, nt, ncand, kb, tol, slack, acc, used, wk);
+    if (nq > 0) mx_clip(sh, sh.Q, nq, tol, acc, wk);
     __syncwarp();
 }
 
-// W warps (faces) per block; blocks per SM as shared memory allows (the FP64
-// form's per-warp buffers are twice as large)
-template <class R> constexpr int mx_resident(int w, int st)
-{
-    return st == MX_STACK_WIDE ? (w == 1 ? 15 : w == 2 ? 8 : 5) : (w == 1 ? 18 : w == 2 ? 9 : 6);
-}
-template <> constexpr int mx_resident<double>(int w, int) { return w == 1 ? 8 : 4; }
-
 template <class R> __device__ __forceinline__ R rconv(double v) { return (R)v; }
+
+// The flux polyhedron of face f (band slot item of a LIST form; points b .. b +
+// n - 1 of the face-point arrays) in the frame of the face centre: prisms with
+// their boxes, tetrahedra (a lane each) with signs and volumes in shared
+// memory (their vertices with KEEP_T), and the box pb of the whole.
+template <class R, bool LIST, bool KEEP_T, class Sh>
+__device__ __forceinline__ void mx_poly(const DevMesh &m, const MXArgs &a, Sh &sh, int item, int f, int b, int n, int nt,
+                                        R pb[6])
+{
+    using V = R3<R>;
+    const R4<R> *fpl = static_cast<const R4<R> *>(a.fpl);
+    const int lane = threadIdx.x & 31;
+    // ---- flux polyhedron tetrahedra in the face frame
+    R bx[6] = {R(3e38), R(3e38), R(3e38), R(-3e38), R(-3e38), R(-3e38)};
+    if (lane < nt) {
+        int pr = lane / 3, j = lane % 3;
+        auto disp = [&](int i) -> V {  // i < 0: face centre
+            V3 w;
+            if (LIST) {
+                const double *q = a.disp + (size_t)item * DISP_STRIDE + (i < 0 ? 0 : 3 + 3 * i);
+                w = mk(q[0], q[1], q[2]);
+            } else {
+                double lam = a.lambda[f];
+                if (lam < 0.0) {
+                    V3 S = ld3(m.sf, m.nf, f);
+                    w = S * (-lam * a.F[f] * a.dt / dot(S, S));
+                } else if (i >= 0) {
+                    w = ld3(a.Up, m.np, __ldg(m.fpts + b + i)) * (a.dt * lam);
+                } else {
+                    w = mk(0, 0, 0);
+                    for (int q = 0; q < n; ++q) w = w + ld3(a.Up, m.np, __ldg(m.fpts + b + q)) * (a.dt * lam);
+                    w = w * (1.0 / n);
+                }
+            }
+            return r3(rconv<R>(w.x), rconv<R>(w.y), rconv<R>(w.z));
+        };
+        V a0, a1, a2, w0, w1, w2;
+        long k0, k1, k2;
+        if (n == 3) {
+            k0 = __ldg(m.fkey + b); k1 = __ldg(m.fkey + b + 1); k2 = __ldg(m.fkey + b + 2);
+            a0 = ld43<R>(fpl, b); a1 = ld43<R>(fpl, b + 1); a2 = ld43<R>(fpl, b + 2);
+            w0 = disp(0); w1 = disp(1); w2 = disp(2);
+        } else {
+            int u = pr + 1 == n ? 0 : pr + 1;
+            k0 = -1; k1 = __ldg(m.fkey + b + pr); k2 = __ldg(m.fkey + b + u);
+            a0 = r3(R(0), R(0), R(0)); a1 = ld43<R>(fpl, b + pr); a2 = ld43<R>(fpl, b + u);
+            w0 = disp(-1); w1 = disp(pr); w2 = disp(u);
+        }
+        int par = 1;
+        if (k1 < k0) { V t = a0; a0 = a1; a1 = t; t = w0; w0 = w1; w1 = t; long q = k0; k0 = k1; k1 = q; par = -par; }
+        if (k2 < k1) { V t = a1; a1 = a2; a2 = t; t = w1; w1 = w2; w2 = t; long q = k1; k1 = k2; k2 = q; par = -par; }
+        if (k1 < k0) { V t = a0; a0 = a1; a1 = t; t = w0; w0 = w1; w1 = t; long q = k0; k0 = k1; k1 = q; par = -par; }
+        V b0 = a0 - w0, b1 = a1 - w1, b2 = a2 - w2;
+        RTet<R> T;
+        if (j == 0) T = RTet<R>{{a0, a1, a2, b2}};
+        else if (j == 1) T = RTet<R>{{a0, a1, b2, b1}};
+        else T = RTet<R>{{a0, b0, b1, b2}};
+        R v6 = rvol6(T.v[0], T.v[1], T.v[2], T.v[3]);
+        R sv = R(-par) * v6;
+        if constexpr (KEEP_T) stT(sh.T[lane], T);
+        sh.Tsg[lane] = sv > R(0) ? R(1) : (sv < R(0) ? R(-1) : R(0));
+        sh.Tv6[lane] = rabs(v6);
+        bx[0] = rmin(rmin(T.v[0].x, T.v[1].x), rmin(T.v[2].x, T.v[3].x));
+        bx[1] = rmin(rmin(T.v[0].y, T.v[1].y), rmin(T.v[2].y, T.v[3].y));
+        bx[2] = rmin(rmin(T.v[0].z, T.v[1].z), rmin(T.v[2].z, T.v[3].z));
+        bx[3] = rmax(rmax(T.v[0].x, T.v[1].x), rmax(T.v[2].x, T.v[3].x));
+        bx[4] = rmax(rmax(T.v[0].y, T.v[1].y), rmax(T.v[2].y, T.v[3].y));
+        bx[5] = rmax(rmax(T.v[0].z, T.v[1].z), rmax(T.v[2].z, T.v[3].z));
+        if (j == 0) {
+            R *q = reinterpret_cast<R *>(sh.P6[pr]);
+            const V pv[6] = {a0, a1, a2, b0, b1, b2};
+#pragma unroll
+            for (int i = 0; i < 6; ++i) { q[3 * i] = pv[i].x; q[3 * i + 1] = pv[i].y; q[3 * i + 2] = pv[i].z; }
+            R lo3[3] = {R(3e38), R(3e38), R(3e38)}, hi3[3] = {R(-3e38), R(-3e38), R(-3e38)};
+#pragma unroll
+            for (int i = 0; i < 6; ++i) {
+                lo3[0] = rmin(lo3[0], pv[i].x); lo3[1] = rmin(lo3[1], pv[i].y); lo3[2] = rmin(lo3[2], pv[i].z);
+                hi3[0] = rmax(hi3[0], pv[i].x); hi3[1] = rmax(hi3[1], pv[i].y); hi3[2] = rmax(hi3[2], pv[i].z);
+            }
+            for (int i = 0; i < 3; ++i) { sh.Pb[pr][i] = lo3[i]; sh.Pb[pr][3 + i] = hi3[i]; }
+            const R hf = R(0.5);
+            sh.Pc[pr][0] = mk4<R>(hf * (lo3[0] + hi3[0]), hf * (lo3[1] + hi3[1]), hf * (lo3[2] + hi3[2]), R(0));
+            sh.Pc[pr][1] = mk4<R>(hf * (hi3[0] - lo3[0]), hf * (hi3[1] - lo3[1]), hf * (hi3[2] - lo3[2]), R(0));
+        }
+    }
+    // bounding box of the whole polyhedron
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        R v = bx[i];
+#pragma unroll
+        for (int o2 = 16; o2 > 0; o2 >>= 1) {
+            R w = __shfl_xor_sync(0xffffffffu, v, o2);
+            v = i < 3 ? rmin(v, w) : rmax(v, w);
+        }
+        pb[i] = v;
+    }
+    __syncwarp();
+}
+
+// A chunk of 32 stencil cells of face f, a lane each, from entry sc: those that
+// reach the polyhedron's box pb and carry phase (void, where comp) go to shared
+// memory with their half-space, frame shift and tetrahedron range; ntot gets
+// the chunk's tetrahedra, ncell its cells.  decide: the stencil is this one
+// chunk, and comp is chosen here by which form leaves fewer cells.
+template <class R, class Sh>
+__device__ __forceinline__ void mx_chunk(const DevMesh &m, const MXArgs &a, Sh &sh, long long sc, long long s1,
+                                         const V3 &o, const R pb[6], bool decide, bool &comp, int &ntot, int &ncell)
+{
+    using V = R3<R>;
+    const R4<R> *cbl = static_cast<const R4<R> *>(a.cbl);
+    const int lane = threadIdx.x & 31;
+    const double eps = m.eps;
+    const long long s = sc + lane;
+    bool pass = false;
+    double al = 0.0, d = 0.0;
+    V dc = r3(R(0), R(0), R(0));
+    V3 hn = mk(0, 0, 0);
+    int t0 = 0, t1 = 0, fl = 0;
+    // the face centre in the cell's frame: on a periodic mesh
+    // the cell sits next to the face moved by its stencil
+    // translation t, and the cell, its tetrahedra and its
+    // plane are taken relative to o - t
+    V3 oc = o;
+    bool emp = false, ful = false;
+    if (s < s1) {
+        // everything about the cell in one round trip (its plane is read for
+        // nothing where the cell is dropped)
+        const int c = __ldg(m.scell + s);
+        al = a.alpha[c];
+        const V3 cc = ld3(m.cc, m.nc, c);
+        const R4<R> cb0 = ldg4(cbl, 2 * (long)c), cb1 = ldg4(cbl, 2 * (long)c + 1);
+        t0 = __ldg(a.ctptr + c);
+        t1 = __ldg(a.ctptr + c + 1);
+        fl = a.flags[c];
+        hn = mk(a.n[c], a.n[m.nc + c], a.n[2 * m.nc + c]);
+        d = a.d[c];
+        if (m.scode) oc = o - tshift(m, __ldg(m.scode + s));
+        // an empty cell carries no phase, a full cell no void
+        // thresholds on the integer pipe (bit-pattern order of doubles)
+        emp = le_pos(al, eps);
+        ful = ge_pos(al, 1.0 - eps);
+        if (decide || !(comp ? ful : emp)) {
+            dc = r3(rconv<R>(cc.x - oc.x), rconv<R>(cc.y - oc.y), rconv<R>(cc.z - oc.z));
+            pass = !(rgt(pb[0], cb1.x + dc.x) || rgt(cb0.x + dc.x, pb[3]) || rgt(pb[1], cb1.y + dc.y) ||
+                     rgt(cb0.y + dc.y, pb[4]) || rgt(pb[2], cb1.z + dc.z) || rgt(cb0.z + dc.z, pb[5]));
+        }
+    }
+    if (decide) {  // the whole stencil is this chunk
+        const int nful = __popc(__ballot_sync(0xffffffffu, pass && ful));
+        const int nemp = __popc(__ballot_sync(0xffffffffu, pass && emp));
+        if (nful != nemp) comp = nful > nemp;
+    }
+    pass = pass && !(comp ? ful : emp);
+    const int nkt = pass ? t1 - t0 : 0;
+    R wgt = R(1);
+    bool useH = false;
+    R4<R> H = mk4<R>(R(0), R(0), R(0), R(0));
+    if (pass && !emp && !ful) {
+        if (fl & VOF_ORIENTED) {
+            const double hd = d - dot(hn, oc);
+            // phase side n.x <= d; the void side is -n.x <= -d
+            R sg = comp ? R(-1) : R(1);
+            H = mk4<R>(sg * rconv<R>(hn.x), sg * rconv<R>(hn.y), sg * rconv<R>(hn.z),
+                       sg * rconv<R>(hd));
+            useH = true;
+        } else wgt = comp ? rconv<R>(1.0 - al) : rconv<R>(al);
+    }
+    int inc = nkt;
+#pragma unroll
+    for (int o2 = 1; o2 < 32; o2 <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, inc, o2);
+        if (lane >= o2) inc += v;
+    }
+    const unsigned pm = __ballot_sync(0xffffffffu, pass);
+    if (pass) {
+        const int r = __popc(pm & ((1u << lane) - 1u));
+        sh.CH[r] = H;
+        sh.Cdc[r][0] = dc.x; sh.Cdc[r][1] = dc.y; sh.Cdc[r][2] = dc.z;
+        sh.Cw[r] = wgt;
+        sh.CuseH[r] = useH;
+        sh.Ct0[r] = t0;
+        sh.Cend[r] = inc;
+    }
+    ntot = __shfl_sync(0xffffffffu, inc, 31);
+    ncell = __popc(pm);
+    __syncwarp();
+}
+
+// lane sums (and their compensations) merged across the warp
+template <class R>
+__device__ __forceinline__ void mx_merge(Acc<R> &acc)
+{
+#pragma unroll
+    for (int o2 = 16; o2 > 0; o2 >>= 1) {
+        const R xs = __shfl_xor_sync(0xffffffffu, acc.s, o2), xc = __shfl_xor_sync(0xffffffffu, acc.c, o2);
+        acc_add(acc, xs);
+        acc.c += xc;
+    }
+}
 
 template <class R, int MX_STACK, bool LIST, class Wk>
 __device__ __forceinline__ void phase_flux_body(const DevMesh &m, const MXArgs &a, MXShared<R, MX_STACK> &sh)
 {
     using V = R3<R>;
-    const R4<R> *fpl = static_cast<const R4<R> *>(a.fpl), *cbl = static_cast<const R4<R> *>(a.cbl);
+    const R4<R> *fpl = static_cast<const R4<R> *>(a.fpl);
     const R4<R> *ktl = static_cast<const R4<R> *>(a.ktl);
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -551,7 +856,8 @@ __device__ __forceinline__ void phase_flux_body(const DevMesh &m, const MXArgs &
         return __shfl_sync(0xffffffffu, v, 0);
     };
     Wk wk;
-    for (int item = dyn ? take() : warp; item < total; item = dyn ? take() : item + nwarps) {
+    for (int it = dyn ? take() : warp; it < total; it = dyn ? take() : it + nwarps) {
+        const int item = LIST && a.items ? a.items[it] : it;
         const int f = LIST ? a.list[item] : item;
         const long long s0 = __ldg(m.sptr + f), s1 = __ldg(m.sptr + f + 1);
         if (!LIST) {
@@ -578,113 +884,16 @@ __device__ __forceinline__ void phase_flux_body(const DevMesh &m, const MXArgs &
         }
         const V3 o = ld3(m.cf, m.nf, f);
         const int b = __ldg(m.fptr + f), n = __ldg(m.fptr + f + 1) - b;
-        // Complement form: sum the void pieces and take V_alpha = F dt - void
-        // (equal in exact arithmetic since the corrected polyhedron holds F dt
-        // and the stencil covers it).  Full cells then need no clipping, where
-        // the plain form clips them and skips empty ones; the form is chosen by
-        // which of the two leaves fewer cells reaching the polyhedron's box
-        // (stencils of one chunk; ties, and longer stencils, by whether the
-        // upwind cell is mostly phase).  A polyhedron inside full cells carries
-        // exactly F dt, one inside empty cells exactly 0, and the rounding of
-        // the clipping stays with mixed cells.  Not where the polyhedron can
-        // leave the domain (the normal-sweep fallback at walls; a face touching
-        // an open boundary), since the part outside is empty and the stencil
-        // does not cover it.
-        const double Ff = a.F[f];
-        const int up = Ff > 0.0 ? __ldg(m.own + f) : (f < m.ni ? __ldg(m.nei + f) : __ldg(m.own + f));
-        const double lamf = LIST ? a.lam_b[item] : a.lambda[f];
-        const bool comp_ok = lamf >= 0.0 && !__ldg(m.fopen + f);
-        const bool decide = comp_ok && s1 - s0 <= 32;  // warp-uniform
-        bool comp = comp_ok && ge_pos(a.alpha[up], 0.5);
+        bool decide, comp;
+        pf_form(m, a.F, a.alpha, f, LIST ? a.lam_b[item] : a.lambda[f], s1 - s0, decide, comp);
         const int nt = n == 3 ? 3 : 3 * n;
         // signed distances (to unit-normal planes) within the on-plane band of
         // the face (FP32: 2e-6 of the face size, FP64: 1e-14) are taken as zero:
         // points shared by the polyhedron and the cell tetrahedra come out of
         // different roundings and would otherwise look like cuts
         const R tol = ldg4(fpl, b).w;
-        // ---- flux polyhedron tetrahedra in the face frame
-        R bx[6] = {R(3e38), R(3e38), R(3e38), R(-3e38), R(-3e38), R(-3e38)};
-        if (lane < nt) {
-            int pr = lane / 3, j = lane % 3;
-            auto disp = [&](int i) -> V {  // i < 0: face centre
-                V3 w;
-                if (LIST) {
-                    const double *q = a.disp + (size_t)item * DISP_STRIDE + (i < 0 ? 0 : 3 + 3 * i);
-                    w = mk(q[0], q[1], q[2]);
-                } else {
-                    double lam = a.lambda[f];
-                    if (lam < 0.0) {
-                        V3 S = ld3(m.sf, m.nf, f);
-                        w = S * (-lam * a.F[f] * a.dt / dot(S, S));
-                    } else if (i >= 0) {
-                        w = ld3(a.Up, m.np, __ldg(m.fpts + b + i)) * (a.dt * lam);
-                    } else {
-                        w = mk(0, 0, 0);
-                        for (int q = 0; q < n; ++q) w = w + ld3(a.Up, m.np, __ldg(m.fpts + b + q)) * (a.dt * lam);
-                        w = w * (1.0 / n);
-                    }
-                }
-                return r3(rconv<R>(w.x), rconv<R>(w.y), rconv<R>(w.z));
-            };
-            V a0, a1, a2, w0, w1, w2;
-            long k0, k1, k2;
-            if (n == 3) {
-                k0 = __ldg(m.fkey + b); k1 = __ldg(m.fkey + b + 1); k2 = __ldg(m.fkey + b + 2);
-                a0 = ld43<R>(fpl, b); a1 = ld43<R>(fpl, b + 1); a2 = ld43<R>(fpl, b + 2);
-                w0 = disp(0); w1 = disp(1); w2 = disp(2);
-            } else {
-                int u = pr + 1 == n ? 0 : pr + 1;
-                k0 = -1; k1 = __ldg(m.fkey + b + pr); k2 = __ldg(m.fkey + b + u);
-                a0 = r3(R(0), R(0), R(0)); a1 = ld43<R>(fpl, b + pr); a2 = ld43<R>(fpl, b + u);
-                w0 = disp(-1); w1 = disp(pr); w2 = disp(u);
-            }
-            int par = 1;
-            if (k1 < k0) { V t = a0; a0 = a1; a1 = t; t = w0; w0 = w1; w1 = t; long q = k0; k0 = k1; k1 = q; par = -par; }
-            if (k2 < k1) { V t = a1; a1 = a2; a2 = t; t = w1; w1 = w2; w2 = t; long q = k1; k1 = k2; k2 = q; par = -par; }
-            if (k1 < k0) { V t = a0; a0 = a1; a1 = t; t = w0; w0 = w1; w1 = t; long q = k0; k0 = k1; k1 = q; par = -par; }
-            V b0 = a0 - w0, b1 = a1 - w1, b2 = a2 - w2;
-            RTet<R> T;
-            if (j == 0) T = RTet<R>{{a0, a1, a2, b2}};
-            else if (j == 1) T = RTet<R>{{a0, a1, b2, b1}};
-            else T = RTet<R>{{a0, b0, b1, b2}};
-            R v6 = rvol6(T.v[0], T.v[1], T.v[2], T.v[3]);
-            R sv = R(-par) * v6;
-            stT(sh.T[lane], T);
-            sh.Tsg[lane] = sv > R(0) ? R(1) : (sv < R(0) ? R(-1) : R(0));
-            sh.Tv6[lane] = rabs(v6);
-            bx[0] = rmin(rmin(T.v[0].x, T.v[1].x), rmin(T.v[2].x, T.v[3].x));
-            bx[1] = rmin(rmin(T.v[0].y, T.v[1].y), rmin(T.v[2].y, T.v[3].y));
-            bx[2] = rmin(rmin(T.v[0].z, T.v[1].z), rmin(T.v[2].z, T.v[3].z));
-            bx[3] = rmax(rmax(T.v[0].x, T.v[1].x), rmax(T.v[2].x, T.v[3].x));
-            bx[4] = rmax(rmax(T.v[0].y, T.v[1].y), rmax(T.v[2].y, T.v[3].y));
-            bx[5] = rmax(rmax(T.v[0].z, T.v[1].z), rmax(T.v[2].z, T.v[3].z));
-            if (j == 0) {
-                R *q = reinterpret_cast<R *>(sh.P6[pr]);
-                const V pv[6] = {a0, a1, a2, b0, b1, b2};
-#pragma unroll
-                for (int i = 0; i < 6; ++i) { q[3 * i] = pv[i].x; q[3 * i + 1] = pv[i].y; q[3 * i + 2] = pv[i].z; }
-                R lo3[3] = {R(3e38), R(3e38), R(3e38)}, hi3[3] = {R(-3e38), R(-3e38), R(-3e38)};
-#pragma unroll
-                for (int i = 0; i < 6; ++i) {
-                    lo3[0] = rmin(lo3[0], pv[i].x); lo3[1] = rmin(lo3[1], pv[i].y); lo3[2] = rmin(lo3[2], pv[i].z);
-                    hi3[0] = rmax(hi3[0], pv[i].x); hi3[1] = rmax(hi3[1], pv[i].y); hi3[2] = rmax(hi3[2], pv[i].z);
-                }
-                for (int i = 0; i < 3; ++i) { sh.Pb[pr][i] = lo3[i]; sh.Pb[pr][3 + i] = hi3[i]; }
-            }
-        }
-        // bounding box of the whole polyhedron
         R pb[6];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) {
-            R v = bx[i];
-#pragma unroll
-            for (int o2 = 16; o2 > 0; o2 >>= 1) {
-                R w = __shfl_xor_sync(0xffffffffu, v, o2);
-                v = i < 3 ? rmin(v, w) : rmax(v, w);
-            }
-            pb[i] = v;
-        }
-        __syncwarp();
+        mx_poly<R, LIST, true>(m, a, sh, item, f, b, n, nt, pb);
         Acc<R> acc;
         wk.add(WK_VOL, lane < nt);  // the flux polyhedron's tetrahedra
         wk.face();
@@ -703,77 +912,7 @@ __device__ __forceinline__ void phase_flux_body(const DevMesh &m, const MXArgs &
                 tb = 0;
                 ntot = 0;
                 if (sc < s1) {
-                    const long long s = sc + lane;
-                    bool pass = false;
-                    int c = 0;
-                    double al = 0.0;
-                    V dc = r3(R(0), R(0), R(0));
-                    // the face centre in the cell's frame: on a periodic mesh
-                    // the cell sits next to the face moved by its stencil
-                    // translation t, and the cell, its tetrahedra and its
-                    // plane are taken relative to o - t
-                    V3 oc = o;
-                    bool emp = false, ful = false;
-                    if (s < s1) {
-                        c = __ldg(m.scell + s);
-                        al = a.alpha[c];
-                        if (m.scode) oc = o - tshift(m, __ldg(m.scode + s));
-                        // an empty cell carries no phase, a full cell no void
-                        // thresholds on the integer pipe (bit-pattern order of doubles)
-                        emp = le_pos(al, eps);
-                        ful = ge_pos(al, 1.0 - eps);
-                        if (decide || !(comp ? ful : emp)) {
-                            const V3 cc = ld3(m.cc, m.nc, c);
-                            dc = r3(rconv<R>(cc.x - oc.x), rconv<R>(cc.y - oc.y), rconv<R>(cc.z - oc.z));
-                            const R4<R> cb0 = ldg4(cbl, 2 * (long)c), cb1 = ldg4(cbl, 2 * (long)c + 1);
-                            pass = !(rgt(pb[0], cb1.x + dc.x) || rgt(cb0.x + dc.x, pb[3]) || rgt(pb[1], cb1.y + dc.y) ||
-                                     rgt(cb0.y + dc.y, pb[4]) || rgt(pb[2], cb1.z + dc.z) || rgt(cb0.z + dc.z, pb[5]));
-                        }
-                    }
-                    if (decide) {  // the whole stencil is this chunk
-                        const int nful = __popc(__ballot_sync(0xffffffffu, pass && ful));
-                        const int nemp = __popc(__ballot_sync(0xffffffffu, pass && emp));
-                        if (nful != nemp) comp = nful > nemp;
-                    }
-                    pass = pass && !(comp ? ful : emp);
-                    int nkt = 0, t0 = 0;
-                    R wgt = R(1);
-                    bool useH = false;
-                    R4<R> H = mk4<R>(R(0), R(0), R(0), R(0));
-                    if (pass) {
-                        t0 = __ldg(a.ctptr + c);
-                        nkt = __ldg(a.ctptr + c + 1) - t0;
-                        if (gt_pos(al, eps) && lt_pos(al, 1.0 - eps)) {
-                            if (a.flags[c] & VOF_ORIENTED) {
-                                V3 hn = ld3(a.n, m.nc, c);
-                                double hd = a.d[c] - dot(hn, oc);
-                                // phase side n.x <= d; the void side is -n.x <= -d
-                                R sg = comp ? R(-1) : R(1);
-                                H = mk4<R>(sg * rconv<R>(hn.x), sg * rconv<R>(hn.y), sg * rconv<R>(hn.z),
-                                           sg * rconv<R>(hd));
-                                useH = true;
-                            } else wgt = comp ? rconv<R>(1.0 - al) : rconv<R>(al);
-                        }
-                    }
-                    int inc = nkt;
-#pragma unroll
-                    for (int o2 = 1; o2 < 32; o2 <<= 1) {
-                        const int v = __shfl_up_sync(0xffffffffu, inc, o2);
-                        if (lane >= o2) inc += v;
-                    }
-                    const unsigned pm = __ballot_sync(0xffffffffu, pass);
-                    if (pass) {
-                        const int r = __popc(pm & ((1u << lane) - 1u));
-                        sh.CH[r] = H;
-                        sh.Cdc[r][0] = dc.x; sh.Cdc[r][1] = dc.y; sh.Cdc[r][2] = dc.z;
-                        sh.Cw[r] = wgt;
-                        sh.CuseH[r] = useH;
-                        sh.Ct0[r] = t0;
-                        sh.Cend[r] = inc;
-                    }
-                    ntot = __shfl_sync(0xffffffffu, inc, 31);
-                    ncell = __popc(pm);
-                    __syncwarp();
+                    mx_chunk(m, a, sh, sc, s1, o, pb, decide, comp, ntot, ncell);
                     continue;
                 }
             }
@@ -817,7 +956,7 @@ __device__ __forceinline__ void phase_flux_body(const DevMesh &m, const MXArgs &
             }
             const unsigned cmask = __ballot_sync(0xffffffffu, cand);
             if (fin ? ncand > 0 : ncand + __popc(cmask) > MX_CAND) {
-                mx_flush(sh, nt, ncand, tol, acc, wk);
+                mx_flush(sh, nt, ncand, tol, box_slack<R>(pb), acc, wk);
                 ncand = 0;
                 continue;  // the batch again (or the end)
             }
@@ -834,34 +973,428 @@ __device__ __forceinline__ void phase_flux_body(const DevMesh &m, const MXArgs &
             tb += 32;
             __syncwarp();
         }
-        // lane sums (and their compensations) merged across the warp, then the
-        // 1/6 of the volumes in FP64
-#pragma unroll
-        for (int o2 = 16; o2 > 0; o2 >>= 1) {
-            const R xs = __shfl_xor_sync(0xffffffffu, acc.s, o2), xc = __shfl_xor_sync(0xffffffffu, acc.c, o2);
-            acc_add(acc, xs);
-            acc.c += xc;
-        }
+        mx_merge(acc);  // then the 1/6 of the volumes in FP64
         double va = ((double)acc.s + (double)acc.c) * (1.0 / 6.0);
-        if (comp) va = Ff * a.dt - va;
+        if (comp) va = a.F[f] * a.dt - va;
         if (lane == 0) a.Va[f] = va;
         __syncwarp();
     }
     wk.flush(a.work, lane);
 }
 
-template <bool LIST, int W, int ST, class Wk>
-__global__ void __launch_bounds__(W * 32, mx_resident<float>(W, ST)) k_phase_flux_mixed(DevMesh m, MXArgs a)
+// every face of the mesh (the standalone call): a warp per face does it all
+template <class R, int W, class Wk>
+__global__ void __launch_bounds__(W * 32, 8) k_phase_flux(DevMesh m, MXArgs a)
 {
-    __shared__ MXShared<float, ST> shm[W];
-    phase_flux_body<float, ST, LIST, Wk>(m, a, shm[threadIdx.x >> 5]);
+    extern __shared__ __align__(16) unsigned char pf_smem[];
+    phase_flux_body<R, MX_STACK_WIDE, false, Wk>(m, a,
+                                                 reinterpret_cast<MXShared<R, MX_STACK_WIDE> *>(pf_smem)[threadIdx.x >> 5]);
 }
 
-template <bool LIST, int W, class Wk>
-__global__ void __launch_bounds__(W * 32, mx_resident<double>(W, MX_STACK_WIDE)) k_phase_flux(DevMesh m, MXArgs a)
+
+// ================================================ the step's three launches
+// The fluxes of a step's band faces: pairs, clips, sums.
+//  - pairs (k_pf_pairs): a warp per band face, or per part of one where there
+//    are few, builds the flux polyhedron, finds the candidate cell tetrahedra
+//    and classifies the (prism, K) pairs; the clip jobs of up to 32 candidates
+//    go to the context's queue as one batch with what their clipping reads
+//    (planes, prism points), the tetrahedra inside every plane are summed here;
+//  - clips (k_pf_clip): a warp per batch works the jobs' pieces off;
+//  - sums (k_pf_finish): a thread per band face adds its batches and writes
+//    V_alpha; faces whose batches found no room in the queue are fluxed whole
+//    there, a warp each.
+// One launch that did all of it per face kept 16 warps on an SM (128 registers,
+// 13.6 KB of shared memory a warp) at 54 % of the issue slots, and took as long
+// as its slowest face where there are fewer faces than warps; the stages by
+// themselves keep 24, the clip work of a face spreads over several warps, and a
+// face's candidates too where the chip would be idle.  The pieces, their order
+// and their arithmetic are those of the one-launch form (the sums differ in
+// the order of compensated additions).
+struct PfQueue {
+    const uint4 *rec;             // per band slot: its face's record (BandRec)
+    uint4 *arena;                 // batches, in units of 16 bytes
+    unsigned cap;                 // units
+    unsigned long long *ctr;      // units taken (low word), batches (high word)
+    unsigned *boff;               // per batch: first unit, or PF_NONE
+    int *bnext;                   // per batch: the unit's previous batch, -1
+    double *part;                 // per batch: 6 x its volume
+    int bcap;
+    double *base;                 // per unit of work: 6 x the volume summed by the pair stage
+    int2 *head;                   // per unit: last batch (-1 none, PF_FAIL), complement form
+    int *ovf, *novf;              // band slots without room
+    int *next_pair, *next_clip, *next_ovf;
+    int pair_warps;               // warps of the pair launch
+};
+constexpr unsigned PF_NONE = 0xffffffffu;
+constexpr int PF_FAIL = -2;
+constexpr int PF_SPLIT = 3;       // a face in up to 2^3 parts
+
+// log2 of the parts a face is dealt into: as many as leave no part waiting for
+// a warp (parts repeat the polyhedron's set-up and the stencil pass, 15 % of a
+// face's work, so they pay only where warps would be idle)
+__device__ __forceinline__ int pf_split(int total, int warps)
 {
-    __shared__ MXShared<double, MX_STACK_WIDE> shm[W];
-    phase_flux_body<double, MX_STACK_WIDE, LIST, Wk>(m, a, shm[threadIdx.x >> 5]);
+    int ls = 0;
+    while (ls < PF_SPLIT && ((long long)total << (ls + 1)) <= warps) ++ls;
+    return ls;
+}
+
+// layout of a batch in 16-byte units: header (2), prism points, planes (five a
+// candidate), weights, job codes
+template <class R>
+struct PfLayout {
+    static constexpr unsigned RW = sizeof(R4<R>) / 16;
+    unsigned P, K, W, Q, end;
+    __device__ __forceinline__ PfLayout(unsigned nprism, unsigned nk, unsigned nq)
+    {
+        P = 2;
+        K = P + nprism * 5 * RW;
+        W = K + nk * 5 * RW;
+        Q = W + (nk * (unsigned)sizeof(R) + 15) / 16;
+        end = Q + (nq * 2 + 15) / 16;
+    }
+};
+
+constexpr int PF_RING = 64;       // cell tetrahedra between the box test and their planes
+constexpr int PF_FLUSH = 24;      // candidates from which the pairs are taken (at most MX_CAND)
+template <class R>
+struct __align__(16) PairShared : PolyShared<R>, CellShared<R>, CandShared<R> {
+    R Kb[MX_CAND][6];
+    R4<R> X[4];                   // the polyhedron's box: low (w: slack), high (w: tol), centre, half extents
+    double o[3];                  // face centre
+    int Cj[PF_RING];              // cell tetrahedron
+    unsigned char Cc[PF_RING];    // its cell in the chunk
+    unsigned char Kmap[MX_CAND];
+};
+
+template <class R, class Wk>
+__device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a, const PfQueue &q, PairShared<R> &sh)
+{
+    using V = R3<R>;
+    const R4<R> *fpl = static_cast<const R4<R> *>(a.fpl);
+    const R4<R> *ktl = static_cast<const R4<R> *>(a.ktl);
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const int total = *a.count, ls = pf_split(total, q.pair_warps), units = total << ls, msk = (1 << ls) - 1;
+    // the next unit is taken, and its record read (16 bytes by each of four
+    // lanes), while the current one is worked on
+    auto take = [&]() { return lane == 0 ? atomicAdd(q.next_pair, 1) : 0; };
+    auto record = [&](int u) {
+        return lane < 4 && u < units ? q.rec[4 * (size_t)(u >> ls) + lane] : make_uint4(0u, 0u, 0u, 0u);
+    };
+    Wk wk;
+    bool full = false;
+    int unit = __shfl_sync(0xffffffffu, take(), 0);
+    uint4 rec = record(unit);
+    while (unit < units) {
+        const int item = unit >> ls, part = unit & msk;
+        auto word = [&](unsigned v, int l) { return __shfl_sync(0xffffffffu, v, l); };
+        // (what only some stages need waits in shared memory, not in registers;
+        // lane 0 of the record holds ox and oy, lane 1 oz)
+        if (lane < 2) {
+            sh.o[2 * lane] = __hiloint2double((int)rec.y, (int)rec.x);
+            if (lane == 0) sh.o[1] = __hiloint2double((int)rec.w, (int)rec.z);
+        }
+        const long long s0 = (long long)((unsigned long long)word(rec.w, 1) << 32 | word(rec.z, 1));
+        const int f = (int)word(rec.x, 2), b = (int)word(rec.y, 2), n = (int)word(rec.z, 2);
+        const long long s1 = s0 + (int)word(rec.w, 2);
+        const unsigned form = word(rec.x, 3);
+        const bool decide = form & 2u;
+        bool comp = form & 1u;
+        const int taken = take();
+        const int nt = n == 3 ? 3 : 3 * n, nprism = nt / 3;
+        {
+            const R tol = ldg4(fpl, b).w;
+            R pb[6];
+            mx_poly<R, true, false>(m, a, sh, item, f, b, n, nt, pb);
+            if (lane == 0) {
+                const R hf = R(0.5);
+                sh.X[0] = mk4<R>(pb[0], pb[1], pb[2], box_slack<R>(pb));
+                sh.X[1] = mk4<R>(pb[3], pb[4], pb[5], tol);
+                sh.X[2] = mk4<R>(hf * (pb[0] + pb[3]), hf * (pb[1] + pb[4]), hf * (pb[2] + pb[5]), R(0));
+                sh.X[3] = mk4<R>(hf * (pb[3] - pb[0]), hf * (pb[4] - pb[1]), hf * (pb[5] - pb[2]), R(0));
+            }
+        }
+        const int next = __shfl_sync(0xffffffffu, taken, 0);
+        rec = record(next);
+        __syncwarp();
+        Acc<R> acc;
+        if (part == 0) {
+            wk.add(WK_VOL, lane < nt);  // the flux polyhedron's tetrahedra
+            wk.face();
+        }
+        int head = -1;
+        // The stencil is taken 32 cells at a time, one per lane, then the
+        // tetrahedra of those that reach the polyhedron, 32 at a time (a part
+        // takes every 2^ls-th such batch): those whose boxes reach it go to a
+        // ring; from the ring, 32 lanes wide, a tetrahedron gets its planes, is
+        // dropped where the polyhedron's box lies beyond one, and else becomes a
+        // candidate; from PF_FLUSH candidates on the pairs are classified.
+        long long sc = s0 - 32;
+        int tb = 0, ntot = 0, ncell = 0, bt = 0;
+        int base = 0, cnt = 0, nk = 0;  // ring: first entry, entries; candidates
+        for (;;) {
+            const bool cdone = tb >= ntot;
+            if (cnt >= 32 || (cdone && cnt > 0)) {
+                // ---- planes of the ring's first tetrahedra
+                const int nr = min(cnt, MX_CAND - nk);
+                bool keep = false;
+                R4<R> kp[4], H;
+                R kbx[6];
+                int ci = 0;
+                if (lane < nr) {
+                    const int e = (base + lane) & (PF_RING - 1);
+                    ci = sh.Cc[e];
+                    const R4<R> *kt = ktl + 6 * (size_t)sh.Cj[e];
+                    const V dc = r3(sh.Cdc[ci][0], sh.Cdc[ci][1], sh.Cdc[ci][2]);
+                    H = sh.CH[ci];
+                    const bool useH = sh.CuseH[ci];
+                    const R4<R> b0 = ldg4(kt, 4), b1 = ldg4(kt, 5);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) kp[i] = ldg4(kt, i);
+                    kbx[0] = b0.x + dc.x; kbx[1] = b0.y + dc.y; kbx[2] = b0.z + dc.z;
+                    kbx[3] = b1.x + dc.x; kbx[4] = b1.y + dc.y; kbx[5] = b1.z + dc.z;
+                    wk.add(WK_SHIFT, 4);
+                    keep = true;
+                    const R4<R> pce = sh.X[2], phe = sh.X[3];
+                    const R slack = sh.X[0].w;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const R4<R> pl = kp[i];
+                        kp[i] = mk4<R>(pl.x, pl.y, pl.z, pl.w + (pl.x * dc.x + pl.y * dc.y + pl.z * dc.z));
+                        if constexpr (sizeof(R) == 4) keep = keep && !beyond<R>(kp[i], pce, phe, slack);
+                    }
+                    if constexpr (sizeof(R) == 4) keep = keep && !(useH && beyond<R>(H, pce, phe, slack));
+                }
+                const unsigned km = __ballot_sync(0xffffffffu, keep);
+                if (keep) {
+                    const int r = nk + __popc(km & lt);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) sh.Kp[r][i] = kp[i];
+                    sh.Kp[r][4] = H;
+#pragma unroll
+                    for (int i = 0; i < 6; ++i) sh.Kb[r][i] = kbx[i];
+                    sh.Kw[r] = sh.Cw[ci];
+                    sh.KuseH[r] = sh.CuseH[ci];
+                }
+                nk += __popc(km);
+                base = (base + nr) & (PF_RING - 1);
+                cnt -= nr;
+                __syncwarp();
+                if (nk < PF_FLUSH) continue;
+            } else if (!cdone) {
+                // ---- boxes of the chunk's next 32 tetrahedra
+                if ((bt++ & msk) != part) { tb += 32; continue; }
+                // the cell of tetrahedron tb + lane: the cells that end at or
+                // before tb, plus one for each cell that ends inside the batch at
+                // or before this lane (cell 'lane' ends rel tetrahedra after tb)
+                const int rel = lane < ncell ? sh.Cend[lane] - tb : 0x7fffffff;
+                const unsigned ends = __reduce_or_sync(0xffffffffu, rel > 0 && rel < 32 ? 1u << rel : 0u);
+                const int ci = __popc(__ballot_sync(0xffffffffu, rel <= 0)) + __popc(ends & (((1u << lane) << 1) - 1u));
+                bool cand = false;
+                int j = 0;
+                if (tb + lane < ntot) {
+                    j = sh.Ct0[ci] + tb + lane - (ci ? sh.Cend[ci - 1] : 0);
+                    const V dc = r3(sh.Cdc[ci][0], sh.Cdc[ci][1], sh.Cdc[ci][2]);
+                    const R4<R> *kt = ktl + 6 * (size_t)j;
+                    const R4<R> b0 = ldg4(kt, 4), b1 = ldg4(kt, 5);
+                    const R4<R> lo = sh.X[0], hi = sh.X[1];
+                    cand = !(rgt(lo.x, b1.x + dc.x) || rgt(b0.x + dc.x, hi.x) || rgt(lo.y, b1.y + dc.y) ||
+                             rgt(b0.y + dc.y, hi.y) || rgt(lo.z, b1.z + dc.z) || rgt(b0.z + dc.z, hi.z));
+                }
+                const unsigned cmask = __ballot_sync(0xffffffffu, cand);
+                if (cand) {
+                    const int e = (base + cnt + __popc(cmask & lt)) & (PF_RING - 1);
+                    sh.Cj[e] = j;
+                    sh.Cc[e] = (unsigned char)ci;
+                }
+                cnt += __popc(cmask);
+                tb += 32;
+                __syncwarp();
+                continue;
+            } else {
+                // ---- next chunk
+                sc += 32;
+                tb = ntot = 0;
+                if (sc < s1) {
+                    const R4<R> lo = sh.X[0], hi = sh.X[1];
+                    const R pb[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
+                    mx_chunk(m, a, sh, sc, s1, mk(sh.o[0], sh.o[1], sh.o[2]), pb, decide, comp, ntot, ncell);
+                    continue;
+                }
+            }
+            // ---- pairs and clip jobs of the candidates
+            if (nk > 0) {
+                R kb[6];
+#pragma unroll
+                for (int i = 0; i < 6; ++i) kb[i] = lane < nk ? sh.Kb[lane][i] : R(0);
+                unsigned used;
+                const R tol = sh.X[1].w;
+                const int nq = mx_pairs(sh, nt, nk, kb, tol, sh.X[0].w, acc, used, wk);
+                if (nq > 0 && head != PF_FAIL) {
+                    // the jobs, as a batch of the queue (a warp that found no
+                    // room once adds nothing more: the counter stays near the
+                    // capacity, far from overflowing its halves)
+                    const int nu = __popc(used);
+                    const PfLayout<R> L(nprism, nu, nq);
+                    unsigned off = PF_NONE;
+                    int bi = -1;
+                    if (lane == 0 && !full) {
+                        const unsigned long long old = atomicAdd(q.ctr, (1ull << 32) | L.end);
+                        off = (unsigned)old;
+                        bi = (int)(old >> 32);
+                        if (bi >= q.bcap) bi = -1;
+                        else if (off > q.cap || L.end > q.cap - off) { q.boff[bi] = PF_NONE; bi = -1; }
+                        else { q.boff[bi] = off; q.bnext[bi] = head; }
+                    }
+                    if (used >> lane & 1u) sh.Kmap[__popc(used & lt)] = (unsigned char)lane;
+                    const R sg = lane < nt ? sh.Tsg[lane] : R(0);
+                    const unsigned pos = __ballot_sync(0xffffffffu, sg > R(0)), neg = __ballot_sync(0xffffffffu, sg < R(0));
+                    off = __shfl_sync(0xffffffffu, off, 0);
+                    bi = __shfl_sync(0xffffffffu, bi, 0);
+                    head = bi < 0 ? PF_FAIL : bi;
+                    full = bi < 0;
+                    if (bi >= 0) {
+                        uint4 *ob = q.arena + off;
+                        if (lane == 0) {
+                            const DBits t = dbits((double)tol);
+                            ob[0] = make_uint4((unsigned)nq | (unsigned)nu << 16 | (unsigned)nprism << 24, pos, neg, 0u);
+                            ob[1] = make_uint4(t.lo, (unsigned)t.hi, 0u, 0u);
+                        }
+                        const uint4 *ps = reinterpret_cast<const uint4 *>(sh.P6);
+                        for (unsigned i = lane; i < nprism * 5 * L.RW; i += 32) ob[L.P + i] = ps[i];
+                        for (unsigned i = lane; i < nu * 5 * L.RW; i += 32)
+                            ob[L.K + i] = reinterpret_cast<const uint4 *>(sh.Kp[sh.Kmap[i / (5 * L.RW)]])[i % (5 * L.RW)];
+                        if (lane < nu) reinterpret_cast<R *>(ob + L.W)[lane] = sh.Kw[sh.Kmap[lane]];
+                        auto code = [&](int i) -> unsigned {  // candidates renumbered among those used
+                            if (i >= nq) return 0u;
+                            const unsigned v = sh.Q[i], k = v >> 5 & 31;
+                            return (v & ~(31u << 5)) | (unsigned)__popc(used & ((1u << k) - 1u)) << 5;
+                        };
+                        unsigned *oq = reinterpret_cast<unsigned *>(ob + L.Q);
+                        for (int i = lane; 2 * i < nq; i += 32) oq[i] = code(2 * i) | code(2 * i + 1) << 16;
+                    }
+                }
+                nk = 0;
+                __syncwarp();
+            }
+            if (cdone && cnt == 0 && sc >= s1) break;
+        }
+        mx_merge(acc);
+        if (lane == 0) {
+            q.base[unit] = (double)acc.s + (double)acc.c;
+            q.head[unit] = make_int2(head, comp);
+            if (head == PF_FAIL) q.ovf[atomicAdd(q.novf, 1)] = item;
+        }
+        __syncwarp();
+        unit = next;
+    }
+    wk.flush(a.work, lane);
+}
+
+template <class R, int MX_STACK_>
+struct __align__(16) ClipShared : StackShared<R, MX_STACK_> {
+    static constexpr int MX_STACK = MX_STACK_;
+    R4<R> Kp[MX_CAND][5];
+    R Tsg[MX_MAXT];
+    R Kw[MX_CAND];
+};
+
+template <class R, int ST, class Wk>
+__device__ __forceinline__ void pf_clip_body(const MXArgs &a, const PfQueue &q, ClipShared<R, ST> &sh)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned long long ctr = *q.ctr;
+    const int nb = min((int)(ctr >> 32), q.bcap);
+    auto take = [&]() {
+        int v = 0;
+        if (lane == 0) v = atomicAdd(q.next_clip, 1);
+        return __shfl_sync(0xffffffffu, v, 0);
+    };
+    Wk wk;
+    for (int bi = take(); bi < nb; bi = take()) {
+        const unsigned off = q.boff[bi];
+        if (off == PF_NONE) continue;
+        const uint4 *ob = q.arena + off;
+        const uint4 h0 = ob[0], h1 = ob[1];
+        const int nq = h0.x & 0xffff, nu = h0.x >> 16 & 0xff, nprism = h0.x >> 24;
+        const PfLayout<R> L(nprism, nu, nq);
+        const R tol = (R)__hiloint2double((int)h1.y, (int)h1.x);
+        uint4 *kd = reinterpret_cast<uint4 *>(sh.Kp);
+        for (unsigned i = lane; i < nu * 5 * L.RW; i += 32) kd[i] = ob[L.K + i];
+        if (lane < nu) sh.Kw[lane] = reinterpret_cast<const R *>(ob + L.W)[lane];
+        if (lane < 3 * nprism) {
+            // T0 = a0 a1 a2 b2, T1 = a0 a1 b2 b1, T2 = a0 b0 b1 b2
+            const int j = lane % 3;
+            const R *p = reinterpret_cast<const R *>(ob + L.P) + 20 * (lane / 3);
+            auto at = [&](int i) { return r3(p[i], p[i + 1], p[i + 2]); };
+            stT(sh.T[lane], RTet<R>{{at(0), at(j == 2 ? 9 : 3), at(j == 0 ? 6 : j == 1 ? 15 : 12), at(j == 1 ? 12 : 15)}});
+            sh.Tsg[lane] = h0.y >> lane & 1u ? R(1) : h0.z >> lane & 1u ? R(-1) : R(0);
+        }
+        __syncwarp();
+        Acc<R> acc;
+        mx_clip(sh, reinterpret_cast<const unsigned short *>(ob + L.Q), nq, tol, acc, wk);
+        mx_merge(acc);
+        if (lane == 0) q.part[bi] = (double)acc.s + (double)acc.c;
+        __syncwarp();
+    }
+    wk.flush(a.work, lane);
+}
+
+// V_alpha of the band faces from their parts, in a fixed order
+__device__ __forceinline__ void pf_sums(const MXArgs &a, const PfQueue &q)
+{
+    const int total = *a.count, ls = pf_split(total, q.pair_warps);
+    for (int item = blockIdx.x * blockDim.x + threadIdx.x; item < total; item += gridDim.x * blockDim.x) {
+        double v = 0.0;
+        bool comp = false, fail = false;
+        for (int u = item << ls; u < (item + 1) << ls; ++u) {
+            const int2 h = q.head[u];
+            comp = h.y != 0;
+            fail |= h.x == PF_FAIL;
+            v += q.base[u];
+            for (int bi = h.x; bi >= 0; bi = q.bnext[bi]) v += q.part[bi];
+        }
+        if (fail) continue;
+        const int f = a.list[item];
+        v *= 1.0 / 6.0;
+        a.Va[f] = comp ? a.F[f] * a.dt - v : v;
+    }
+}
+
+constexpr int PP_W = 4;  // warps per block of the pair launch
+template <class R> constexpr int pp_resident() { return sizeof(R) == 4 ? 5 : 3; }
+template <class R, class Wk>
+__global__ void __launch_bounds__(PP_W * 32, pp_resident<R>()) k_pf_pairs(DevMesh m, MXArgs a, PfQueue q)
+{
+    extern __shared__ __align__(16) unsigned char pf_smem[];
+    pf_pairs_body<R, Wk>(m, a, q, reinterpret_cast<PairShared<R> *>(pf_smem)[threadIdx.x >> 5]);
+}
+
+template <class R> constexpr int pc_resident(int w, int st)
+{
+    return sizeof(R) == 8 ? 12 / w : st == MX_STACK_WIDE ? 24 / w : 28 / w;
+}
+template <class R, int W, int ST, class Wk>
+__global__ void __launch_bounds__(W * 32, pc_resident<R>(W, ST)) k_pf_clip(MXArgs a, PfQueue q)
+{
+    extern __shared__ __align__(16) unsigned char pf_smem[];
+    pf_clip_body<R, ST, Wk>(a, q, reinterpret_cast<ClipShared<R, ST> *>(pf_smem)[threadIdx.x >> 5]);
+}
+
+// (a.items, a.next and a.count describe the faces without room)
+template <class R, class Wk>
+__global__ void __launch_bounds__(64, sizeof(R) == 4 ? 8 : 4) k_pf_finish(DevMesh m, MXArgs a, PfQueue q, const int *count)
+{
+    extern __shared__ __align__(16) unsigned char pf_smem[];
+    {
+        MXArgs s = a;
+        s.count = count;
+        pf_sums(s, q);
+    }
+    if (*a.count > 0)
+        phase_flux_body<R, MX_STACK_WIDE, true, Wk>(
+            m, a, reinterpret_cast<MXShared<R, MX_STACK_WIDE> *>(pf_smem)[threadIdx.x >> 5]);
 }
 
 // geometry of every cell relative to its centre (context creation): face
@@ -976,66 +1509,113 @@ size_t phase_flux_table_entry_bytes(int precision)
     return precision == VOF_MIXED ? sizeof(float4) : sizeof(D4);
 }
 
-int launch_setup_mixed(vof_ctx *c, cudaStream_t s)
-{
-    return c->precision == VOF_MIXED ? setup_tables<float>(c, s) : setup_tables<double>(c, s);
-}
-
 static MXArgs mx_args(vof_ctx *c, const double *alpha, const double *n, const double *d, const uint8_t *flags,
                       const double *Up, const double *F, const double *lambda, double dt, double *Va,
                       const int *list, const int *count, const double *disp, unsigned long long *work)
 {
     return MXArgs{alpha, n, d, flags, Up, F, lambda, dt, Va, list, count, disp, c->lam_b, c->status, work,
-                  c->fpl, c->cbl, c->ktl, c->m.ctptr, nullptr};
+                  c->fpl, c->cbl, c->ktl, c->m.ctptr, nullptr, nullptr};
 }
 
-int launch_pf_all(vof_ctx *c, const double *alpha, const double *n, const double *d,
-                                const uint8_t *flags, const double *Up, const double *F, const double *lambda,
-                                double dt, double *Va, cudaStream_t s)
+// the band slots' work queue and counters (zeroed with the step's counters)
+static PfQueue pf_queue(vof_ctx *c, int pair_warps)
 {
-    MXArgs a = mx_args(c, alpha, n, d, flags, Up, F, lambda, dt, Va, nullptr, nullptr, nullptr,
-                       c->work_on ? c->work : nullptr);
-    if (c->precision == VOF_MIXED) {
-        if (c->work_on) k_phase_flux_mixed<false, 2, MX_STACK_WIDE, WkOn><<<cdiv((long)c->nf * 32, 64), 64, 0, s>>>(c->m, a);
-        else k_phase_flux_mixed<false, 2, MX_STACK_WIDE, WkOff><<<cdiv((long)c->nf * 32, 64), 64, 0, s>>>(c->m, a);
-    } else {
-        if (c->work_on) k_phase_flux<false, 1, WkOn><<<cdiv((long)c->nf * 32, 32), 32, 0, s>>>(c->m, a);
-        else k_phase_flux<false, 1, WkOff><<<cdiv((long)c->nf * 32, 32), 32, 0, s>>>(c->m, a);
-    }
-    return cudaGetLastError() == cudaSuccess ? VOF_OK : VOF_ERR_CUDA;
+    int *cnt = c->counters;
+    return PfQueue{reinterpret_cast<const uint4 *>(c->pf_rec), static_cast<uint4 *>(c->pf_arena), c->pf_cap, reinterpret_cast<unsigned long long *>(cnt + CNT_PFQ),
+                   c->pf_boff, c->pf_bnext, c->pf_part, c->pf_bcap, c->pf_base, c->pf_head, c->pf_ovf, cnt + CNT_PFOVF,
+                   cnt + CNT_PFNEXT, cnt + CNT_CLNEXT, cnt + CNT_OVNEXT, pair_warps};
 }
 
-int launch_pf_list(vof_ctx *c, const double *alpha, const double *F, double dt, int sms,
-                                 cudaStream_t s)
+// the kernels' shared memory (above the default limit), on the current device
+template <class K>
+static bool pf_smem(K kernel, size_t bytes)
 {
-    MXArgs a = mx_args(c, alpha, c->n, c->d, c->flags, nullptr, F, nullptr, dt, c->Va, c->band,
-                       c->counters + CNT_BAND, c->disp_b, c->work_on ? c->work : nullptr);
-    a.next = c->counters + CNT_PFNEXT;  // zeroed with the step's counters
-    if (c->precision != VOF_MIXED) {
-        // the FP64 form: one warp per block, as many blocks as shared memory allows
-        if (c->work_on) k_phase_flux<true, 1, WkOn><<<sms * mx_resident<double>(1, MX_STACK_WIDE), 32, 0, s>>>(c->m, a);
-        else k_phase_flux<true, 1, WkOff><<<sms * mx_resident<double>(1, MX_STACK_WIDE), 32, 0, s>>>(c->m, a);
-        return cudaGetLastError() == cudaSuccess ? VOF_OK : VOF_ERR_CUDA;
-    }
-    // launch configuration (vof_batch_tune): warps per block, stack depth, and
-    // grid = SMs x resident blocks x multiplier
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+}
+template <class R, int W, class Wk>
+static bool pf_smem_form()
+{
+    bool ok = pf_smem(k_phase_flux<R, W, Wk>, W * sizeof(MXShared<R, MX_STACK_WIDE>)) &&
+              pf_smem(k_pf_pairs<R, Wk>, PP_W * sizeof(PairShared<R>)) &&
+              pf_smem(k_pf_finish<R, Wk>, 2 * sizeof(MXShared<R, MX_STACK_WIDE>)) &&
+              pf_smem(k_pf_clip<R, 1, MX_STACK_WIDE, Wk>, sizeof(ClipShared<R, MX_STACK_WIDE>));
+    if constexpr (sizeof(R) == 4)
+        ok = ok && pf_smem(k_pf_clip<R, 2, MX_STACK_WIDE, Wk>, 2 * sizeof(ClipShared<R, MX_STACK_WIDE>)) &&
+             pf_smem(k_pf_clip<R, 3, MX_STACK_WIDE, Wk>, 3 * sizeof(ClipShared<R, MX_STACK_WIDE>)) &&
+             pf_smem(k_pf_clip<R, 1, MX_STACK_SLIM, Wk>, sizeof(ClipShared<R, MX_STACK_SLIM>)) &&
+             pf_smem(k_pf_clip<R, 2, MX_STACK_SLIM, Wk>, 2 * sizeof(ClipShared<R, MX_STACK_SLIM>)) &&
+             pf_smem(k_pf_clip<R, 3, MX_STACK_SLIM, Wk>, 3 * sizeof(ClipShared<R, MX_STACK_SLIM>));
+    return ok;
+}
+
+template <class R, int W, int ST, class Wk>
+static int go_clip(const MXArgs &a, const PfQueue &q, int sms, int mult, cudaStream_t s)
+{
+    constexpr size_t bytes = W * sizeof(ClipShared<R, ST>);
+    k_pf_clip<R, W, ST, Wk><<<sms * pc_resident<R>(W, ST) * mult, 32 * W, bytes, s>>>(a, q);
+    return VOF_OK;
+}
+
+template <class R, class Wk>
+static int go_list(vof_ctx *c, const MXArgs &a, int sms, cudaStream_t s)
+{
+    const int pblocks = sms * pp_resident<R>();
+    const PfQueue q = pf_queue(c, pblocks * PP_W);
+    constexpr size_t pbytes = PP_W * sizeof(PairShared<R>), fbytes = 2 * sizeof(MXShared<R, MX_STACK_WIDE>);
+    k_pf_pairs<R, Wk><<<pblocks, 32 * PP_W, pbytes, s>>>(c->m, a, q);
+    // launch configuration of the clips (vof_tune): warps per block, stack
+    // depth, and grid = SMs x resident blocks x multiplier
     const int w = c->pf_warps >= 1 && c->pf_warps <= 3 ? c->pf_warps : 2;
     const int mult = c->pf_mult >= 1 ? c->pf_mult : 1;
-    const bool slim = c->pf_stack == 1;
-#define PF_GO(W_, ST_, WK_)                                                                                  \
-    k_phase_flux_mixed<true, W_, ST_, WK_><<<sms * mx_resident<float>(W_, ST_) * mult, 32 * W_, 0, s>>>(c->m, a)
-    if (c->work_on) {  // instrumented variant (vof_count_work), two warps per block
-        if (slim) PF_GO(2, MX_STACK_SLIM, WkOn);
-        else PF_GO(2, MX_STACK_WIDE, WkOn);
-    } else if (slim) {
-        if (w == 1) PF_GO(1, MX_STACK_SLIM, WkOff);
-        else if (w == 2) PF_GO(2, MX_STACK_SLIM, WkOff);
-        else PF_GO(3, MX_STACK_SLIM, WkOff);
-    } else {
-        if (w == 1) PF_GO(1, MX_STACK_WIDE, WkOff);
-        else if (w == 2) PF_GO(2, MX_STACK_WIDE, WkOff);
-        else PF_GO(3, MX_STACK_WIDE, WkOff);
-    }
-#undef PF_GO
+    int r;
+    if constexpr (sizeof(R) == 4) {
+        if (c->pf_stack == 1)
+            r = w == 1 ? go_clip<R, 1, MX_STACK_SLIM, Wk>(a, q, sms, mult, s)
+                       : w == 2 ? go_clip<R, 2, MX_STACK_SLIM, Wk>(a, q, sms, mult, s)
+                                : go_clip<R, 3, MX_STACK_SLIM, Wk>(a, q, sms, mult, s);
+        else
+            r = w == 1 ? go_clip<R, 1, MX_STACK_WIDE, Wk>(a, q, sms, mult, s)
+                       : w == 2 ? go_clip<R, 2, MX_STACK_WIDE, Wk>(a, q, sms, mult, s)
+                                : go_clip<R, 3, MX_STACK_WIDE, Wk>(a, q, sms, mult, s);
+    } else r = go_clip<R, 1, MX_STACK_WIDE, Wk>(a, q, sms, 1, s);
+    if (r) return r;
+    MXArgs o = a;
+    o.items = q.ovf;
+    o.count = q.novf;
+    o.next = q.next_ovf;
+    k_pf_finish<R, Wk><<<sms * 4, 64, fbytes, s>>>(c->m, o, q, a.count);
     return cudaGetLastError() == cudaSuccess ? VOF_OK : VOF_ERR_CUDA;
+}
+
+template <class R, int W, class Wk>
+static int go_all(vof_ctx *c, const MXArgs &a, cudaStream_t s)
+{
+    constexpr size_t bytes = W * sizeof(MXShared<R, MX_STACK_WIDE>);
+    k_phase_flux<R, W, Wk><<<cdiv(c->nf, W), 32 * W, bytes, s>>>(c->m, a);
+    return cudaGetLastError() == cudaSuccess ? VOF_OK : VOF_ERR_CUDA;
+}
+
+int launch_pf_all(vof_ctx *c, const double *alpha, const double *n, const double *d, const uint8_t *flags,
+                  const double *Up, const double *F, const double *lambda, double dt, double *Va, cudaStream_t s)
+{
+    const MXArgs a = mx_args(c, alpha, n, d, flags, Up, F, lambda, dt, Va, nullptr, nullptr, nullptr,
+                             c->work_on ? c->work : nullptr);
+    if (c->precision == VOF_MIXED) return c->work_on ? go_all<float, 2, WkOn>(c, a, s) : go_all<float, 2, WkOff>(c, a, s);
+    return c->work_on ? go_all<double, 1, WkOn>(c, a, s) : go_all<double, 1, WkOff>(c, a, s);
+}
+
+int launch_pf_list(vof_ctx *c, const double *alpha, const double *F, double dt, int sms, cudaStream_t s)
+{
+    const MXArgs a = mx_args(c, alpha, c->n, c->d, c->flags, nullptr, F, nullptr, dt, c->Va, c->band,
+                             c->counters + CNT_BAND, c->disp_b, c->work_on ? c->work : nullptr);
+    if (c->precision == VOF_MIXED) return c->work_on ? go_list<float, WkOn>(c, a, sms, s) : go_list<float, WkOff>(c, a, sms, s);
+    return c->work_on ? go_list<double, WkOn>(c, a, sms, s) : go_list<double, WkOff>(c, a, sms, s);
+}
+
+int launch_setup_mixed(vof_ctx *c, cudaStream_t s)
+{
+    const bool ok = c->precision == VOF_MIXED ? pf_smem_form<float, 2, WkOff>() && pf_smem_form<float, 2, WkOn>()
+                                              : pf_smem_form<double, 1, WkOff>() && pf_smem_form<double, 1, WkOn>();
+    if (!ok) return VOF_ERR_CUDA;
+    return c->precision == VOF_MIXED ? setup_tables<float>(c, s) : setup_tables<double>(c, s);
 }
