@@ -568,7 +568,7 @@ int vof_create(const vof_mesh *mesh, const vof_options *opt, vof_ctx **out)
         c->pf_cap = (unsigned)(bytes / unit);
         c->pf_bcap = (int)(bytes / unit / 14);  // the smallest batch
         // units of work: a band face, or its parts where the band is small
-        const size_t units = std::max<size_t>(nf, 32 * (size_t)prop.multiProcessorCount);
+        const size_t units = std::max<size_t>(nf, 128 * (size_t)prop.multiProcessorCount);
         c->pf_rec = dev_alloc<BandRec>(c, nf, &err);
         c->pf_boff = dev_alloc<unsigned>(c, c->pf_bcap, &err);
         c->pf_bnext = dev_alloc<int>(c, c->pf_bcap, &err);

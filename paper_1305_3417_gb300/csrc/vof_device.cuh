@@ -135,6 +135,15 @@ __device__ __forceinline__ bool gt_bits(double a, double b)
     y.hi ^= sy & 0x7fffffff; y.lo ^= (unsigned)sy;
     return !bits_le(x, y);
 }
+// x truncated to FP32 on the integer pipe (the FP64 pipe's conversion costs as
+// much as an FMA there): relative error below 2^-23; magnitudes below 2^-126
+// become 0, above the FP32 range a large finite number
+__device__ __forceinline__ float tf(double x)
+{
+    const DBits b = dbits(x);
+    const int h = min(max((b.hi & 0x7fffffff) - 0x38000000, 0), 0x0fefffff);
+    return __uint_as_float(__funnelshift_l(b.lo, (unsigned)h, 3) | ((unsigned)b.hi & 0x80000000u));
+}
 // a is +0 or -0
 __device__ __forceinline__ bool is_zero(double a)
 {

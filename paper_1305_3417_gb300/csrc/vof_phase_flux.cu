@@ -169,11 +169,11 @@ constexpr int MX_STACK_WIDE = 92, MX_STACK_SLIM = 56;
 
 // Shared memory of a warp, by stage.
 // the flux polyhedron: its prisms (one per face triangle swept) and tetrahedra
-template <class R>
+template <class R, class B = R>
 struct __align__(16) PolyShared {
     R4<R> P6[VOF_MAXFP][5];  // per prism: a0 a1 a2 b0 b1 b2, 18 values in 20
-    R Pb[VOF_MAXFP][6];      // prism box
-    R4<R> Pc[VOF_MAXFP][2];  // its centre and half extents
+    B Pb[VOF_MAXFP][6];      // prism box
+    R4<B> Pc[VOF_MAXFP][2];  // its centre and half extents
     R Tv6[MX_MAXT];          // |6 vol(T)|
     R Tsg[MX_MAXT];          // sign of T in the flux polyhedron
 };
@@ -229,6 +229,9 @@ __device__ __forceinline__ void stT(RTet<float> &t, const RTet<float> &v)
     p[2] = make_float4(v.v[2].z, v.v[3].x, v.v[3].y, v.v[3].z);
 }
 __device__ __forceinline__ void stT(RTet<double> &t, const RTet<double> &v) { t = v; }
+
+__device__ __forceinline__ float tof(float x) { return x; }
+__device__ __forceinline__ float tof(double x) { return tf(x); }
 
 template <class R>
 __device__ __forceinline__ R pdist(R4<R> p, R3<R> v) { return p.x * v.x + p.y * v.y + p.z * v.z - p.w; }
@@ -315,7 +318,7 @@ __device__ __forceinline__ void fsplit(const RTet<R> &t, const R s[4], int nin, 
 //  - split step: a piece from the other stack (else a new job) is cut by its
 //    next plane and the parts below are pushed, to the leaves if one plane is
 //    left; a new job with one plane goes to the leaves whole (no leaf work in
-//    a split step: a step's lanes never mix the two kinds of work).  FP32: a
+//    a split step: a step's lanes never mix the two kinds of work).  A
 //    part none of whose points is below the plane after is dropped at once (the
 //    parts share six points, so this takes six distances, not a push, a pop
 //    and a step's share each).
@@ -406,21 +409,26 @@ __device__ __forceinline__ void mx_clip(Sh &sh, const unsigned short *Q, int nq,
             }
             c[0] = t.v[0]; c[1] = t.v[1]; c[2] = t.v[2]; c[5] = t.v[3];
             if (cut) fsplit(t, sd, nin, c);
-            if constexpr (std::is_same<R, float>::value) {
-                if (keep && !single) {
-                    const R4<R> pn = sh.Kp[k][__ffs(rem) - 1];
-                    auto below = [&](int i) { return pdist<R>(pn, c[i]) < -tol; };
-                    const bool z0 = below(0), z1 = below(1), z2 = below(2), z5 = below(5);
-                    ndrop = __popc(keep);
-                    unsigned kept = z0 || z1 || z2 || z5 ? 1u : 0u;
-                    if (keep & 2u) {
-                        const bool z3 = below(3), z4 = below(4);
-                        kept |= z0 || z1 || z5 || z4 ? 2u : 0u;
-                        kept |= z0 || z3 || z4 || z5 ? 4u : 0u;
-                    }
-                    keep = kept;
-                    ndrop -= __popc(kept);
+            if (keep && !single) {
+                // the points below the plane after (FP64: those not clearly
+                // above it by an FP32 distance; a part kept for nothing is
+                // dropped when its own turn comes)
+                const R4<R> pn = sh.Kp[k][__ffs(rem) - 1];
+                const float4 pf = make_float4(tof(pn.x), tof(pn.y), tof(pn.z), tof(pn.w));
+                auto below = [&](int i) {
+                    if constexpr (std::is_same<R, float>::value) return pdist<R>(pn, c[i]) < -tol;
+                    else return pdist<float>(pf, r3(tof(c[i].x), tof(c[i].y), tof(c[i].z))) < (float)tol * 1.2e9f;
+                };
+                const bool z0 = below(0), z1 = below(1), z2 = below(2), z5 = below(5);
+                ndrop = __popc(keep);
+                unsigned kept = z0 || z1 || z2 || z5 ? 1u : 0u;
+                if (keep & 2u) {
+                    const bool z3 = below(3), z4 = below(4);
+                    kept |= z0 || z1 || z5 || z4 ? 2u : 0u;
+                    kept |= z0 || z3 || z4 || z5 ? 4u : 0u;
                 }
+                keep = kept;
+                ndrop -= __popc(kept);
             }
         }
         const int nch = __popc(keep);
@@ -638,15 +646,19 @@ template <class R> __device__ __forceinline__ R rconv(double v) { return (R)v; }
 // n - 1 of the face-point arrays) in the frame of the face centre: prisms with
 // their boxes, tetrahedra (a lane each) with signs and volumes in shared
 // memory (their vertices with KEEP_T), and the box pb of the whole.
-template <class R, bool LIST, bool KEEP_T, class Sh>
+// B = float in an FP64 form: prism points and boxes in FP32 too (for the pair
+// stage's FP32 tests), the boxes widened over the truncation.
+template <class R, bool LIST, bool KEEP_T, class B, class Sh>
 __device__ __forceinline__ void mx_poly(const DevMesh &m, const MXArgs &a, Sh &sh, int item, int f, int b, int n, int nt,
-                                        R pb[6])
+                                        B pb[6])
 {
     using V = R3<R>;
+    constexpr bool F32BOX = !std::is_same<R, B>::value;
+    auto box = [](R v) -> B { if constexpr (std::is_same<R, B>::value) return v; else return tf(v); };
     const R4<R> *fpl = static_cast<const R4<R> *>(a.fpl);
     const int lane = threadIdx.x & 31;
     // ---- flux polyhedron tetrahedra in the face frame
-    R bx[6] = {R(3e38), R(3e38), R(3e38), R(-3e38), R(-3e38), R(-3e38)};
+    B bx[6] = {B(3e38), B(3e38), B(3e38), B(-3e38), B(-3e38), B(-3e38)};
     if (lane < nt) {
         int pr = lane / 3, j = lane % 3;
         auto disp = [&](int i) -> V {  // i < 0: face centre
@@ -695,36 +707,48 @@ __device__ __forceinline__ void mx_poly(const DevMesh &m, const MXArgs &a, Sh &s
         if constexpr (KEEP_T) stT(sh.T[lane], T);
         sh.Tsg[lane] = sv > R(0) ? R(1) : (sv < R(0) ? R(-1) : R(0));
         sh.Tv6[lane] = rabs(v6);
-        bx[0] = rmin(rmin(T.v[0].x, T.v[1].x), rmin(T.v[2].x, T.v[3].x));
-        bx[1] = rmin(rmin(T.v[0].y, T.v[1].y), rmin(T.v[2].y, T.v[3].y));
-        bx[2] = rmin(rmin(T.v[0].z, T.v[1].z), rmin(T.v[2].z, T.v[3].z));
-        bx[3] = rmax(rmax(T.v[0].x, T.v[1].x), rmax(T.v[2].x, T.v[3].x));
-        bx[4] = rmax(rmax(T.v[0].y, T.v[1].y), rmax(T.v[2].y, T.v[3].y));
-        bx[5] = rmax(rmax(T.v[0].z, T.v[1].z), rmax(T.v[2].z, T.v[3].z));
         if (j == 0) {
+            // (the prism's points are its tetrahedra's: its box is theirs together)
             R *q = reinterpret_cast<R *>(sh.P6[pr]);
             const V pv[6] = {a0, a1, a2, b0, b1, b2};
-#pragma unroll
-            for (int i = 0; i < 6; ++i) { q[3 * i] = pv[i].x; q[3 * i + 1] = pv[i].y; q[3 * i + 2] = pv[i].z; }
-            R lo3[3] = {R(3e38), R(3e38), R(3e38)}, hi3[3] = {R(-3e38), R(-3e38), R(-3e38)};
+            B px[6], py[6], pz[6];
 #pragma unroll
             for (int i = 0; i < 6; ++i) {
-                lo3[0] = rmin(lo3[0], pv[i].x); lo3[1] = rmin(lo3[1], pv[i].y); lo3[2] = rmin(lo3[2], pv[i].z);
-                hi3[0] = rmax(hi3[0], pv[i].x); hi3[1] = rmax(hi3[1], pv[i].y); hi3[2] = rmax(hi3[2], pv[i].z);
+                q[3 * i] = pv[i].x; q[3 * i + 1] = pv[i].y; q[3 * i + 2] = pv[i].z;
+                px[i] = box(pv[i].x); py[i] = box(pv[i].y); pz[i] = box(pv[i].z);
             }
-            for (int i = 0; i < 3; ++i) { sh.Pb[pr][i] = lo3[i]; sh.Pb[pr][3 + i] = hi3[i]; }
-            const R hf = R(0.5);
-            sh.Pc[pr][0] = mk4<R>(hf * (lo3[0] + hi3[0]), hf * (lo3[1] + hi3[1]), hf * (lo3[2] + hi3[2]), R(0));
-            sh.Pc[pr][1] = mk4<R>(hf * (hi3[0] - lo3[0]), hf * (hi3[1] - lo3[1]), hf * (hi3[2] - lo3[2]), R(0));
+            if constexpr (F32BOX) {
+                float *qf = reinterpret_cast<float *>(sh.P6f[pr]);
+#pragma unroll
+                for (int i = 0; i < 6; ++i) { qf[3 * i] = px[i]; qf[3 * i + 1] = py[i]; qf[3 * i + 2] = pz[i]; }
+            }
+            bx[0] = bx[3] = px[0]; bx[1] = bx[4] = py[0]; bx[2] = bx[5] = pz[0];
+#pragma unroll
+            for (int i = 1; i < 6; ++i) {
+                bx[0] = rmin(bx[0], px[i]); bx[1] = rmin(bx[1], py[i]); bx[2] = rmin(bx[2], pz[i]);
+                bx[3] = rmax(bx[3], px[i]); bx[4] = rmax(bx[4], py[i]); bx[5] = rmax(bx[5], pz[i]);
+            }
+            if constexpr (F32BOX) {
+                B w = B(0);
+#pragma unroll
+                for (int i = 0; i < 6; ++i) w = rmax(w, rabs(bx[i]));
+                w *= B(2.5e-7);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) { bx[i] -= w; bx[3 + i] += w; }
+            }
+            for (int i = 0; i < 6; ++i) sh.Pb[pr][i] = bx[i];
+            const B hf = B(0.5);
+            sh.Pc[pr][0] = mk4<B>(hf * (bx[0] + bx[3]), hf * (bx[1] + bx[4]), hf * (bx[2] + bx[5]), B(0));
+            sh.Pc[pr][1] = mk4<B>(hf * (bx[3] - bx[0]), hf * (bx[4] - bx[1]), hf * (bx[5] - bx[2]), B(0));
         }
     }
     // bounding box of the whole polyhedron
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
-        R v = bx[i];
+        B v = bx[i];
 #pragma unroll
         for (int o2 = 16; o2 > 0; o2 >>= 1) {
-            R w = __shfl_xor_sync(0xffffffffu, v, o2);
+            B w = __shfl_xor_sync(0xffffffffu, v, o2);
             v = i < 3 ? rmin(v, w) : rmax(v, w);
         }
         pb[i] = v;
@@ -737,9 +761,10 @@ __device__ __forceinline__ void mx_poly(const DevMesh &m, const MXArgs &a, Sh &s
 // memory with their half-space, frame shift and tetrahedron range; ntot gets
 // the chunk's tetrahedra, ncell its cells.  decide: the stencil is this one
 // chunk, and comp is chosen here by which form leaves fewer cells.
-template <class R, class Sh>
+// B = float in an FP64 form: box tests in FP32, wide by its roundings.
+template <class R, class B, class Sh>
 __device__ __forceinline__ void mx_chunk(const DevMesh &m, const MXArgs &a, Sh &sh, long long sc, long long s1,
-                                         const V3 &o, const R pb[6], bool decide, bool &comp, int &ntot, int &ncell)
+                                         const V3 &o, const B pb[6], bool decide, bool &comp, int &ntot, int &ncell)
 {
     using V = R3<R>;
     const R4<R> *cbl = static_cast<const R4<R> *>(a.cbl);
@@ -776,8 +801,18 @@ __device__ __forceinline__ void mx_chunk(const DevMesh &m, const MXArgs &a, Sh &
         ful = ge_pos(al, 1.0 - eps);
         if (decide || !(comp ? ful : emp)) {
             dc = r3(rconv<R>(cc.x - oc.x), rconv<R>(cc.y - oc.y), rconv<R>(cc.z - oc.z));
-            pass = !(rgt(pb[0], cb1.x + dc.x) || rgt(cb0.x + dc.x, pb[3]) || rgt(pb[1], cb1.y + dc.y) ||
-                     rgt(cb0.y + dc.y, pb[4]) || rgt(pb[2], cb1.z + dc.z) || rgt(cb0.z + dc.z, pb[5]));
+            if constexpr (std::is_same<R, B>::value)
+                pass = !(rgt(pb[0], cb1.x + dc.x) || rgt(cb0.x + dc.x, pb[3]) || rgt(pb[1], cb1.y + dc.y) ||
+                         rgt(cb0.y + dc.y, pb[4]) || rgt(pb[2], cb1.z + dc.z) || rgt(cb0.z + dc.z, pb[5]));
+            else {
+                auto apart = [](float l, float h, double c0, double c1, double s) {
+                    const float d = tf(s), f0 = tf(c0), f1 = tf(c1);
+                    const float w = 5e-7f * (fabsf(d) + fabsf(f0) + fabsf(f1));
+                    return l > f1 + d + w || f0 + d - w > h;
+                };
+                pass = !(apart(pb[0], pb[3], cb0.x, cb1.x, dc.x) || apart(pb[1], pb[4], cb0.y, cb1.y, dc.y) ||
+                         apart(pb[2], pb[5], cb0.z, cb1.z, dc.z));
+            }
         }
     }
     if (decide) {  // the whole stencil is this chunk
@@ -893,7 +928,7 @@ __device__ __forceinline__ void phase_flux_body(const DevMesh &m, const MXArgs &
         // different roundings and would otherwise look like cuts
         const R tol = ldg4(fpl, b).w;
         R pb[6];
-        mx_poly<R, LIST, true>(m, a, sh, item, f, b, n, nt, pb);
+        mx_poly<R, LIST, true, R>(m, a, sh, item, f, b, n, nt, pb);
         Acc<R> acc;
         wk.add(WK_VOL, lane < nt);  // the flux polyhedron's tetrahedra
         wk.face();
@@ -912,7 +947,7 @@ __device__ __forceinline__ void phase_flux_body(const DevMesh &m, const MXArgs &
                 tb = 0;
                 ntot = 0;
                 if (sc < s1) {
-                    mx_chunk(m, a, sh, sc, s1, o, pb, decide, comp, ntot, ncell);
+                    mx_chunk<R, R>(m, a, sh, sc, s1, o, pb, decide, comp, ntot, ncell);
                     continue;
                 }
             }
@@ -1027,6 +1062,7 @@ struct PfQueue {
 };
 constexpr unsigned PF_NONE = 0xffffffffu;
 constexpr int PF_FAIL = -2;
+constexpr int PF_OVER = 2;        // parts per warp of the launch at most
 constexpr int PF_SPLIT = 3;       // a face in up to 2^3 parts
 
 // log2 of the parts a face is dealt into: as many as leave no part waiting for
@@ -1035,7 +1071,7 @@ constexpr int PF_SPLIT = 3;       // a face in up to 2^3 parts
 __device__ __forceinline__ int pf_split(int total, int warps)
 {
     int ls = 0;
-    while (ls < PF_SPLIT && ((long long)total << (ls + 1)) <= warps) ++ls;
+    while (ls < PF_SPLIT && ((long long)total << (ls + 1)) <= PF_OVER * (long long)warps) ++ls;
     return ls;
 }
 
@@ -1067,9 +1103,182 @@ struct __align__(16) PairShared : PolyShared<R>, CellShared<R>, CandShared<R> {
     unsigned char Kmap[MX_CAND];
 };
 
+// The FP64 form classifies in FP32 wherever that is clear of its roundings and
+// in FP64 only the planes that are not (the FP64 pipe issues one warp
+// instruction in about 64 cycles on its sub-partition): boxes, prism points and
+// shifted planes are held in FP32 as well, with each candidate's rounding
+// allowance; the FP64 planes stay in the cell's frame and are shifted where
+// they are used.  Every decision is the one FP64 throughout takes.
+template <>
+struct __align__(16) PairShared<double> : PolyShared<double, float>, CellShared<double> {
+    float4 P6f[VOF_MAXFP][5];
+    D4 Kp[MX_CAND][5];            // planes in the cell frame, then the half-space in the face frame
+    double Kdc[MX_CAND][3];       // cell centre - face centre
+    double Kw[MX_CAND];
+    float4 Kf[MX_CAND][5];        // planes and half-space in the face frame, FP32
+    float Kb[MX_CAND][6];
+    float Km[MX_CAND];            // rounding allowance of the FP32 distances
+    float4 X[4];
+    double o[3];
+    int Cj[PF_RING];
+    unsigned short Q[MX_QUEUE], PQ[VOF_MAXFP * MX_CAND];
+    unsigned char QA[MX_QUEUE];   // planes to decide in FP64
+    unsigned char Cc[PF_RING];
+    unsigned char KuseH[MX_CAND], Kmap[MX_CAND];
+};
+
+// all (T, K) pairs of the candidates, as mx_pairs
+template <class Wk>
+__device__ __forceinline__ int pf_pairs64(PairShared<double> &sh, int nt, int ncand, double tol, Acc<double> &acc,
+                                          unsigned &used, Wk &wk)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const int nprism = nt / 3;
+    int total = 0;
+    {
+        const bool live0 = lane < ncand;
+        float4 pl[5];
+        float kb[6], mg = 0.0f;
+        if (live0) {
+            mg = sh.Km[lane];
+#pragma unroll
+            for (int q = 0; q < 5; ++q) pl[q] = sh.Kf[lane][q];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) kb[q] = sh.Kb[lane][q];
+        }
+        for (int pr = 0; pr < nprism; ++pr) {
+            const float *tb = sh.Pb[pr];
+            const bool live = sh.Tsg[3 * pr] != 0.0 || sh.Tsg[3 * pr + 1] != 0.0 || sh.Tsg[3 * pr + 2] != 0.0;
+            bool ov = live0 && live;
+            if (ov) {
+                ov = !(kb[0] > tb[3] + mg || tb[0] > kb[3] + mg || kb[1] > tb[4] + mg || tb[1] > kb[4] + mg ||
+                       kb[2] > tb[5] + mg || tb[2] > kb[5] + mg);
+                const float4 ce = sh.Pc[pr][0], he = sh.Pc[pr][1];
+#pragma unroll
+                for (int q = 0; q < 5; ++q) ov = ov && !beyond<float>(pl[q], ce, he, mg);
+            }
+            const unsigned bm = __ballot_sync(0xffffffffu, ov);
+            if (ov) sh.PQ[total + __popc(bm & lt)] = (unsigned short)(pr | lane << 3);
+            total += __popc(bm);
+        }
+    }
+    __syncwarp();
+    // FP32 distances of a pair's six prism points to the planes: what is clearly
+    // outside ends here; the rest is listed with its clear cuts and the planes
+    // that need FP64 (a point within the allowance where it matters)
+    int ns = 0;
+    for (int pb = 0; pb < total; pb += 32) {
+        const int pi = pb + lane;
+        unsigned code[3] = {0u, 0u, 0u}, amb[3] = {0u, 0u, 0u};
+        bool live[3] = {false, false, false};
+        if (pi < total) {
+            const unsigned pc = sh.PQ[pi];
+            const int pr = pc & 7, k = pc >> 3;
+            float v[20];
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+                const float4 x = sh.P6f[pr][i];
+                v[4 * i] = x.x; v[4 * i + 1] = x.y; v[4 * i + 2] = x.z; v[4 * i + 3] = x.w;
+            }
+            const int npl = sh.KuseH[k] ? 5 : 4;
+            const float mg = sh.Km[k];
+            unsigned mask[3] = {0u, 0u, 0u};
+            bool outside[3] = {false, false, false};
+#pragma unroll
+            for (int q = 0; q < 5; ++q) {
+                const float4 pl = sh.Kf[k][q];
+                float d[6];
+#pragma unroll
+                for (int i = 0; i < 6; ++i)
+                    d[i] = fmaf(pl.x, v[3 * i], fmaf(pl.y, v[3 * i + 1], fmaf(pl.z, v[3 * i + 2], -pl.w)));
+                const float l01 = fminf(d[0], d[1]), h01 = fmaxf(d[0], d[1]);
+                const float lo[3] = {fminf(l01, fminf(d[2], d[5])), fminf(l01, fminf(d[5], d[4])),
+                                     fminf(fminf(d[0], d[3]), fminf(d[4], d[5]))};
+                const float hi[3] = {fmaxf(h01, fmaxf(d[2], d[5])), fmaxf(h01, fmaxf(d[5], d[4])),
+                                     fmaxf(fmaxf(d[0], d[3]), fmaxf(d[4], d[5]))};
+                if (q < npl) {
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) {
+                        outside[j] |= lo[j] > mg;
+                        if (hi[j] > mg) mask[j] |= 1u << q;
+                        if (fabsf(hi[j]) <= mg || fabsf(lo[j]) <= mg) amb[j] |= 1u << q;
+                    }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const int t = 3 * pr + j;
+                live[j] = sh.Tsg[t] != 0.0 && !outside[j];
+                code[j] = (unsigned)t | ((unsigned)k << 5) | (mask[j] << 10);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const unsigned bm = __ballot_sync(0xffffffffu, live[j]);
+            if (live[j]) {
+                const int at = ns + __popc(bm & lt);
+                sh.Q[at] = (unsigned short)code[j];
+                sh.QA[at] = (unsigned char)amb[j];
+            }
+            ns += __popc(bm);
+        }
+    }
+    __syncwarp();
+    // the listed (T, K), one per lane: the open planes in FP64, then outside,
+    // inside (summed) or a clip job (the list is compacted in place)
+    int nq = 0;
+    used = 0u;
+    for (int sb = 0; sb < ns; sb += 32) {
+        const bool act = sb + lane < ns;
+        unsigned meta = 0, amb = 0;
+        if (act) {
+            meta = sh.Q[sb + lane];
+            amb = sh.QA[sb + lane];
+        }
+        const int t = meta & 31, k = meta >> 5 & 31, j = t % 3;
+        unsigned mask = meta >> 10;
+        const double *p = reinterpret_cast<const double *>(sh.P6[t / 3]);
+        const int at[4] = {0, j == 2 ? 9 : 3, j == 0 ? 6 : j == 1 ? 15 : 12, j == 1 ? 12 : 15};
+        bool out = !act;
+        while (__any_sync(0xffffffffu, amb != 0u && !out)) {
+            if (amb != 0u && !out) {
+                const int q = __ffs(amb) - 1;
+                amb &= amb - 1;
+                D4 pl = sh.Kp[k][q];
+                if (q < 4) {
+                    const double *dc = sh.Kdc[k];
+                    pl.w = pl.w + (pl.x * dc[0] + pl.y * dc[1] + pl.z * dc[2]);
+                }
+                wk.add(WK_TEST, 1);
+                bool below = false, above = false;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const double *x = p + at[i];
+                    const double d = fma(pl.x, x[0], fma(pl.y, x[1], fma(pl.z, x[2], -pl.w)));
+                    below |= rbelow(d, tol);
+                    above |= rabove(d, tol);
+                }
+                if (!below) out = true;
+                mask = above ? mask | 1u << q : mask & ~(1u << q);
+            }
+        }
+        if (!out && mask == 0u) acc_add(acc, sh.Tsg[t] * sh.Kw[k] * sh.Tv6[t]);
+        const bool job = !out && mask != 0u;
+        const unsigned bm = __ballot_sync(0xffffffffu, job);
+        if (job) sh.Q[nq + __popc(bm & lt)] = (unsigned short)((meta & 0x3ffu) | mask << 10);
+        nq += __popc(bm);
+        used |= __reduce_or_sync(0xffffffffu, job ? 1u << k : 0u);
+        __syncwarp();
+    }
+    return nq;
+}
+
 template <class R, class Wk>
 __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a, const PfQueue &q, PairShared<R> &sh)
 {
+    constexpr bool F64 = std::is_same<R, double>::value;
+    using B = float;  // boxes
     using V = R3<R>;
     const R4<R> *fpl = static_cast<const R4<R> *>(a.fpl);
     const R4<R> *ktl = static_cast<const R4<R> *>(a.ktl);
@@ -1105,14 +1314,14 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
         const int nt = n == 3 ? 3 : 3 * n, nprism = nt / 3;
         {
             const R tol = ldg4(fpl, b).w;
-            R pb[6];
-            mx_poly<R, true, false>(m, a, sh, item, f, b, n, nt, pb);
+            B pb[6];
+            mx_poly<R, true, false, B>(m, a, sh, item, f, b, n, nt, pb);
             if (lane == 0) {
-                const R hf = R(0.5);
-                sh.X[0] = mk4<R>(pb[0], pb[1], pb[2], box_slack<R>(pb));
-                sh.X[1] = mk4<R>(pb[3], pb[4], pb[5], tol);
-                sh.X[2] = mk4<R>(hf * (pb[0] + pb[3]), hf * (pb[1] + pb[4]), hf * (pb[2] + pb[5]), R(0));
-                sh.X[3] = mk4<R>(hf * (pb[3] - pb[0]), hf * (pb[4] - pb[1]), hf * (pb[5] - pb[2]), R(0));
+                const B hf = B(0.5);
+                sh.X[0] = mk4<B>(pb[0], pb[1], pb[2], box_slack<B>(pb));
+                sh.X[1] = mk4<B>(pb[3], pb[4], pb[5], (B)tol);
+                sh.X[2] = mk4<B>(hf * (pb[0] + pb[3]), hf * (pb[1] + pb[4]), hf * (pb[2] + pb[5]), B(0));
+                sh.X[3] = mk4<B>(hf * (pb[3] - pb[0]), hf * (pb[4] - pb[1]), hf * (pb[5] - pb[2]), B(0));
             }
         }
         const int next = __shfl_sync(0xffffffffu, taken, 0);
@@ -1140,31 +1349,47 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
                 const int nr = min(cnt, MX_CAND - nk);
                 bool keep = false;
                 R4<R> kp[4], H;
-                R kbx[6];
+                B kbx[6];
+                float4 kf[4], hf4;
+                float mg = 0.0f;
                 int ci = 0;
                 if (lane < nr) {
                     const int e = (base + lane) & (PF_RING - 1);
                     ci = sh.Cc[e];
                     const R4<R> *kt = ktl + 6 * (size_t)sh.Cj[e];
                     const V dc = r3(sh.Cdc[ci][0], sh.Cdc[ci][1], sh.Cdc[ci][2]);
+                    const R3<float> df = r3(tof(dc.x), tof(dc.y), tof(dc.z));
                     H = sh.CH[ci];
                     const bool useH = sh.CuseH[ci];
                     const R4<R> b0 = ldg4(kt, 4), b1 = ldg4(kt, 5);
 #pragma unroll
                     for (int i = 0; i < 4; ++i) kp[i] = ldg4(kt, i);
-                    kbx[0] = b0.x + dc.x; kbx[1] = b0.y + dc.y; kbx[2] = b0.z + dc.z;
-                    kbx[3] = b1.x + dc.x; kbx[4] = b1.y + dc.y; kbx[5] = b1.z + dc.z;
-                    wk.add(WK_SHIFT, 4);
+                    kbx[0] = tof(b0.x) + df.x; kbx[1] = tof(b0.y) + df.y; kbx[2] = tof(b0.z) + df.z;
+                    kbx[3] = tof(b1.x) + df.x; kbx[4] = tof(b1.y) + df.y; kbx[5] = tof(b1.z) + df.z;
+                    const float4 pce = sh.X[2], phe = sh.X[3];
                     keep = true;
-                    const R4<R> pce = sh.X[2], phe = sh.X[3];
-                    const R slack = sh.X[0].w;
+                    if constexpr (F64) {
+                        // allowance: a few FP32 roundings of what enters a distance
+                        const float rs = sh.X[0].w * 2e6f + fmaxf(fabsf(df.x), fmaxf(fabsf(df.y), fabsf(df.z))) +
+                                         fmaxf(fabsf(tof(kp[3].w)), fabsf(tof(H.w)));
+                        mg = 2e-6f * rs;
+                    } else mg = sh.X[0].w;
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const R4<R> pl = kp[i];
-                        kp[i] = mk4<R>(pl.x, pl.y, pl.z, pl.w + (pl.x * dc.x + pl.y * dc.y + pl.z * dc.z));
-                        if constexpr (sizeof(R) == 4) keep = keep && !beyond<R>(kp[i], pce, phe, slack);
+                        if constexpr (F64) {
+                            kf[i] = make_float4(tof(pl.x), tof(pl.y), tof(pl.z), 0.0f);
+                            kf[i].w = tof(pl.w) + (kf[i].x * df.x + kf[i].y * df.y + kf[i].z * df.z);
+                            keep = keep && !beyond<float>(kf[i], pce, phe, mg);
+                        } else {
+                            wk.add(WK_SHIFT, 1);
+                            kp[i] = mk4<R>(pl.x, pl.y, pl.z, pl.w + (pl.x * dc.x + pl.y * dc.y + pl.z * dc.z));
+                            keep = keep && !beyond<R>(kp[i], pce, phe, mg);
+                        }
                     }
-                    if constexpr (sizeof(R) == 4) keep = keep && !(useH && beyond<R>(H, pce, phe, slack));
+                    hf4 = make_float4(tof(H.x), tof(H.y), tof(H.z), tof(H.w));
+                    keep = keep && !(useH && beyond<float>(hf4, pce, phe, mg));
+                    if (!useH) hf4 = make_float4(0.0f, 0.0f, 0.0f, 1.0f);  // (nothing is beyond it)
                 }
                 const unsigned km = __ballot_sync(0xffffffffu, keep);
                 if (keep) {
@@ -1174,6 +1399,13 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
                     sh.Kp[r][4] = H;
 #pragma unroll
                     for (int i = 0; i < 6; ++i) sh.Kb[r][i] = kbx[i];
+                    if constexpr (F64) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) sh.Kf[r][i] = kf[i];
+                        sh.Kf[r][4] = hf4;
+                        sh.Km[r] = mg;
+                        sh.Kdc[r][0] = sh.Cdc[ci][0]; sh.Kdc[r][1] = sh.Cdc[ci][1]; sh.Kdc[r][2] = sh.Cdc[ci][2];
+                    }
                     sh.Kw[r] = sh.Cw[ci];
                     sh.KuseH[r] = sh.CuseH[ci];
                 }
@@ -1198,9 +1430,18 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
                     const V dc = r3(sh.Cdc[ci][0], sh.Cdc[ci][1], sh.Cdc[ci][2]);
                     const R4<R> *kt = ktl + 6 * (size_t)j;
                     const R4<R> b0 = ldg4(kt, 4), b1 = ldg4(kt, 5);
-                    const R4<R> lo = sh.X[0], hi = sh.X[1];
-                    cand = !(rgt(lo.x, b1.x + dc.x) || rgt(b0.x + dc.x, hi.x) || rgt(lo.y, b1.y + dc.y) ||
-                             rgt(b0.y + dc.y, hi.y) || rgt(lo.z, b1.z + dc.z) || rgt(b0.z + dc.z, hi.z));
+                    const float4 lo = sh.X[0], hi = sh.X[1];
+                    if constexpr (F64) {
+                        auto apart = [](float l, float h, double c0, double c1, double s) {
+                            const float d = tf(s), f0 = tf(c0), f1 = tf(c1);
+                            const float w = 5e-7f * (fabsf(d) + fabsf(f0) + fabsf(f1));
+                            return l > f1 + d + w || f0 + d - w > h;
+                        };
+                        cand = !(apart(lo.x, hi.x, b0.x, b1.x, dc.x) || apart(lo.y, hi.y, b0.y, b1.y, dc.y) ||
+                                 apart(lo.z, hi.z, b0.z, b1.z, dc.z));
+                    } else
+                        cand = !(rgt(lo.x, b1.x + dc.x) || rgt(b0.x + dc.x, hi.x) || rgt(lo.y, b1.y + dc.y) ||
+                                 rgt(b0.y + dc.y, hi.y) || rgt(lo.z, b1.z + dc.z) || rgt(b0.z + dc.z, hi.z));
                 }
                 const unsigned cmask = __ballot_sync(0xffffffffu, cand);
                 if (cand) {
@@ -1217,20 +1458,26 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
                 sc += 32;
                 tb = ntot = 0;
                 if (sc < s1) {
-                    const R4<R> lo = sh.X[0], hi = sh.X[1];
-                    const R pb[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
-                    mx_chunk(m, a, sh, sc, s1, mk(sh.o[0], sh.o[1], sh.o[2]), pb, decide, comp, ntot, ncell);
+                    const float4 lo = sh.X[0], hi = sh.X[1];
+                    const B pb[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
+                    mx_chunk<R, B>(m, a, sh, sc, s1, mk(sh.o[0], sh.o[1], sh.o[2]), pb, decide, comp, ntot, ncell);
                     continue;
                 }
             }
             // ---- pairs and clip jobs of the candidates
             if (nk > 0) {
-                R kb[6];
-#pragma unroll
-                for (int i = 0; i < 6; ++i) kb[i] = lane < nk ? sh.Kb[lane][i] : R(0);
                 unsigned used;
-                const R tol = sh.X[1].w;
-                const int nq = mx_pairs(sh, nt, nk, kb, tol, sh.X[0].w, acc, used, wk);
+                int nq;
+                R tol;
+                if constexpr (F64) tol = ldg4(fpl, b).w;
+                else tol = sh.X[1].w;
+                if constexpr (F64) nq = pf_pairs64(sh, nt, nk, tol, acc, used, wk);
+                else {
+                    R kb[6];
+#pragma unroll
+                    for (int i = 0; i < 6; ++i) kb[i] = lane < nk ? sh.Kb[lane][i] : R(0);
+                    nq = mx_pairs(sh, nt, nk, kb, tol, sh.X[0].w, acc, used, wk);
+                }
                 if (nq > 0 && head != PF_FAIL) {
                     // the jobs, as a batch of the queue (a warp that found no
                     // room once adds nothing more: the counter stays near the
@@ -1263,8 +1510,19 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
                         }
                         const uint4 *ps = reinterpret_cast<const uint4 *>(sh.P6);
                         for (unsigned i = lane; i < nprism * 5 * L.RW; i += 32) ob[L.P + i] = ps[i];
-                        for (unsigned i = lane; i < nu * 5 * L.RW; i += 32)
-                            ob[L.K + i] = reinterpret_cast<const uint4 *>(sh.Kp[sh.Kmap[i / (5 * L.RW)]])[i % (5 * L.RW)];
+                        R4<R> *ok = reinterpret_cast<R4<R> *>(ob + L.K);
+                        for (int i = lane; i < nu * 5; i += 32) {
+                            const int k = sh.Kmap[i / 5], c = i % 5;
+                            R4<R> pl = sh.Kp[k][c];
+                            if constexpr (F64) {
+                                if (c < 4) {
+                                    const double *dc = sh.Kdc[k];
+                                    wk.add(WK_SHIFT, 1);
+                                    pl.w = pl.w + (pl.x * dc[0] + pl.y * dc[1] + pl.z * dc[2]);
+                                }
+                            }
+                            ok[i] = pl;
+                        }
                         if (lane < nu) reinterpret_cast<R *>(ob + L.W)[lane] = sh.Kw[sh.Kmap[lane]];
                         auto code = [&](int i) -> unsigned {  // candidates renumbered among those used
                             if (i >= nq) return 0u;
@@ -1362,10 +1620,11 @@ __device__ __forceinline__ void pf_sums(const MXArgs &a, const PfQueue &q)
     }
 }
 
-constexpr int PP_W = 4;  // warps per block of the pair launch
-template <class R> constexpr int pp_resident() { return sizeof(R) == 4 ? 5 : 3; }
+// warps per block of the pair launch, and blocks per SM
+template <class R> constexpr int pp_warps() { return sizeof(R) == 4 ? 4 : 2; }
+template <class R> constexpr int pp_resident() { return sizeof(R) == 4 ? 5 : 6; }
 template <class R, class Wk>
-__global__ void __launch_bounds__(PP_W * 32, pp_resident<R>()) k_pf_pairs(DevMesh m, MXArgs a, PfQueue q)
+__global__ void __launch_bounds__(pp_warps<R>() * 32, pp_resident<R>()) k_pf_pairs(DevMesh m, MXArgs a, PfQueue q)
 {
     extern __shared__ __align__(16) unsigned char pf_smem[];
     pf_pairs_body<R, Wk>(m, a, q, reinterpret_cast<PairShared<R> *>(pf_smem)[threadIdx.x >> 5]);
@@ -1536,7 +1795,7 @@ template <class R, int W, class Wk>
 static bool pf_smem_form()
 {
     bool ok = pf_smem(k_phase_flux<R, W, Wk>, W * sizeof(MXShared<R, MX_STACK_WIDE>)) &&
-              pf_smem(k_pf_pairs<R, Wk>, PP_W * sizeof(PairShared<R>)) &&
+              pf_smem(k_pf_pairs<R, Wk>, pp_warps<R>() * sizeof(PairShared<R>)) &&
               pf_smem(k_pf_finish<R, Wk>, 2 * sizeof(MXShared<R, MX_STACK_WIDE>)) &&
               pf_smem(k_pf_clip<R, 1, MX_STACK_WIDE, Wk>, sizeof(ClipShared<R, MX_STACK_WIDE>));
     if constexpr (sizeof(R) == 4)
@@ -1560,9 +1819,9 @@ template <class R, class Wk>
 static int go_list(vof_ctx *c, const MXArgs &a, int sms, cudaStream_t s)
 {
     const int pblocks = sms * pp_resident<R>();
-    const PfQueue q = pf_queue(c, pblocks * PP_W);
-    constexpr size_t pbytes = PP_W * sizeof(PairShared<R>), fbytes = 2 * sizeof(MXShared<R, MX_STACK_WIDE>);
-    k_pf_pairs<R, Wk><<<pblocks, 32 * PP_W, pbytes, s>>>(c->m, a, q);
+    const PfQueue q = pf_queue(c, pblocks * pp_warps<R>());
+    constexpr size_t pbytes = pp_warps<R>() * sizeof(PairShared<R>), fbytes = 2 * sizeof(MXShared<R, MX_STACK_WIDE>);
+    k_pf_pairs<R, Wk><<<pblocks, 32 * pp_warps<R>(), pbytes, s>>>(c->m, a, q);
     // launch configuration of the clips (vof_tune): warps per block, stack
     // depth, and grid = SMs x resident blocks x multiplier
     const int w = c->pf_warps >= 1 && c->pf_warps <= 3 ? c->pf_warps : 2;
