@@ -60,26 +60,38 @@ bool finite_pos(double x) { return std::isfinite(x) && x > 0.0; }
 
 }  // namespace
 
-// regions of the global bounding step, cut into segments of at most 4096
-// cells; replaces any earlier regions (buffers of earlier calls stay owned by
-// the context until vof_destroy)
+// regions of the global bounding step, cut into segments (a block's share of
+// the update): a cell a thread on small meshes, so that they spread over the
+// SMs, more where there are thousands of segments anyway; replaces any
+// earlier regions (buffers of earlier calls stay owned by the context until
+// vof_destroy)
 int set_bound_regions(vof_ctx *c, const int *reg_cell, int nreg)
 {
-    constexpr int SEG = 4096;
+    const int SEG = c->nc <= (1 << 18) ? SEG_STEP : c->nc <= (1 << 22) ? 4 * SEG_STEP : 16 * SEG_STEP;
     std::vector<int4> seg;
-    std::vector<int> rs(1, 0);
+    std::vector<int> rs(1, 0), at;
     for (int r = 0; r < nreg; ++r) {
-        for (int a = reg_cell[r]; a < reg_cell[r + 1]; a += SEG)
-            seg.push_back(make_int4(r, a, std::min(a + SEG, reg_cell[r + 1]), 0));
+        for (int a = reg_cell[r]; a < reg_cell[r + 1]; a += SEG) {
+            const int b = std::min(a + SEG, reg_cell[r + 1]);
+            // (regions cover the cells in order)
+            while ((long)at.size() * SEG_STEP < b) at.push_back((int)seg.size());
+            seg.push_back(make_int4(r, a, b, 0));
+        }
         rs.push_back((int)seg.size());
     }
     if (seg.empty()) seg.push_back(make_int4(0, 0, 0, 0));
+    if (at.empty()) at.push_back(0);
     int err = 0;
     c->seg = dev_copy(c, seg.data(), seg.size(), &err);
     c->reg_seg = dev_copy(c, rs.data(), rs.size(), &err);
-    c->gpartial = dev_alloc<double>(c, 4 * seg.size(), &err);
+    c->seg_at = dev_copy(c, at.data(), at.size(), &err);
+    c->sd = dev_alloc<double>(c, SEG_COLS * seg.size(), &err);
+    c->seg_mixed = dev_alloc<uint8_t>(c, seg.size(), &err);
+    c->segmark = dev_alloc<unsigned>(c, seg.size(), &err);
+    c->dl = dev_alloc<int>(c, seg.size(), &err);
     c->reg_tot = dev_alloc<double>(c, 6 * (size_t)nreg, &err);  // per region: Ep, Em, Sp, Sm, Ep/Sp, Em/Sm
     if (err) return err;
+    if (cudaMemset(c->segmark, 0, sizeof(unsigned) * seg.size()) != cudaSuccess) return VOF_ERR_CUDA;
     c->nseg = (int)seg.size();
     c->nreg = nreg;
     return VOF_OK;
@@ -515,8 +527,9 @@ int vof_create(const vof_mesh *mesh, const vof_options *opt, vof_ctx **out)
     c->band = dev_alloc<int>(c, nf, &err);
     c->icell = dev_alloc<int>(c, nc, &err);
     c->viol[0] = dev_alloc<int>(c, nc, &err);
-    c->pend_c = dev_alloc<int>(c, 8 * (size_t)nc, &err);
-    c->pend_a = dev_alloc<double>(c, 8 * (size_t)nc, &err);
+    c->rl = dev_alloc<int>(c, nc, &err);
+    c->ra = dev_alloc<double>(c, nc, &err);
+    c->cmark = dev_alloc<unsigned>(c, nc, &err);
     c->counters = dev_alloc<int>(c, CNT_ALLOC, &err);
     c->lam_b = dev_alloc<double>(c, nf, &err);
     c->disp_b = dev_alloc<double>(c, (size_t)nf * (VOF_MAXFP + 1) * 3, &err);
@@ -526,8 +539,7 @@ int vof_create(const vof_mesh *mesh, const vof_options *opt, vof_ctx **out)
     c->flags = dev_alloc<uint8_t>(c, nc, &err);
     c->pit = dev_alloc<int>(c, nc, &err);
     c->Va = dev_alloc<double>(c, nf, &err);
-    c->bscr = dev_alloc<double>(c, 3 * (size_t)nc, &err);
-    c->partial = dev_alloc<double>(c, 10 * 1024, &err);
+    c->bscr = dev_alloc<double>(c, 4 * (size_t)nc, &err);
     c->stats_dev = dev_alloc<double>(c, VOF_S_LEN, &err);
     c->status = dev_alloc<unsigned>(c, 1, &err);
     c->h_alpha = dev_alloc<double>(c, nc, &err);
@@ -579,7 +591,8 @@ int vof_create(const vof_mesh *mesh, const vof_options *opt, vof_ctx **out)
     }
     if (err) { vof_destroy(c); return err; }
     cudaMemset(c->work, 0, WK_LEN * sizeof(unsigned long long));
-    cudaMemset(c->bscr, 0, sizeof(double) * 3 * nc);
+    cudaMemset(c->bscr, 0, sizeof(double) * 4 * nc);
+    cudaMemset(c->cmark, 0, sizeof(unsigned) * nc);
     cudaMemset(c->counters, 0, sizeof(int) * CNT_ALLOC);
     cudaMemset(c->status, 0, sizeof(unsigned));
     cudaMemset(c->n, 0, sizeof(double) * 3 * nc);

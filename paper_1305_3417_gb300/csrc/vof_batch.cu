@@ -30,33 +30,11 @@ struct vof_batch {
 
 namespace {
 
-// Per case the sum of V_c alpha_c over its cells, in a fixed order, in two
-// launches over the segments (<= 4096 cells of one case) that the global
-// bounding step uses: a block sums a segment (thread-strided partial sums, then
-// a fixed tree), then a warp a case's segments.  Bound by reading 16 B per cell
-// once; (one block per case left all but the cases' SMs idle and
-// ran as long as its largest case took one SM: 32 cases of up to 83k cells,
-// 246 us of the step's 2262; now 2049).
-constexpr int CM_THREADS = 256;
-__global__ void __launch_bounds__(CM_THREADS) k_segment_mass(const double *__restrict__ alpha,
-                                                             const double *__restrict__ vc,
-                                                             const int4 *__restrict__ seg, double *part)
-{
-    const int4 sg = seg[blockIdx.x];
-    double v = 0.0;
-#pragma unroll 4
-    for (int c = sg.y + threadIdx.x; c < sg.z; c += CM_THREADS) v += vc[c] * alpha[c];
-    v = vofd::warp_sum(v);
-    __shared__ double sh[CM_THREADS / 32];
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double r = 0.0;
-        for (int k = 0; k < CM_THREADS / 32; ++k) r += sh[k];
-        part[blockIdx.x] = r;
-    }
-}
-
+// Per case the sum of V_c alpha_c over its cells, in a fixed order: a warp a
+// case adds the masses that the step left per segment of the case.  (One block
+// per case reading the case's cells again left all but the cases' SMs idle and
+// ran as long as its largest case took one SM: 246 us of a step of 2262 for 32
+// cases of up to 83k cells.)
 __global__ void k_case_mass(const double *__restrict__ part, const int *__restrict__ reg_seg, int ncases, double *out)
 {
     const int cs = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
@@ -82,11 +60,9 @@ int enqueue_step(vof_batch *b, double *alpha, const double *U, const double *F, 
     int r = launch_advect(b->ctx, alpha, U, F, 1.0, stats, s);
     if (r) return r;
     if (case_mass) {
-        // (the context's regions are the cases; gpartial is free again after
-        // the step's bounding)
-        const vof_ctx *c = b->ctx;
-        k_segment_mass<<<c->nseg, CM_THREADS, 0, s>>>(alpha, c->m.vc, c->seg, c->gpartial);
-        k_case_mass<<<(b->ncases + 3) / 4, 128, 0, s>>>(c->gpartial, c->reg_seg, b->ncases, case_mass);
+        const vof_ctx *c = b->ctx;  // (its regions are the cases)
+        k_case_mass<<<(b->ncases + 3) / 4, 128, 0, s>>>(c->sd + (size_t)SEG_COL_MASS * c->nseg, c->reg_seg, b->ncases,
+                                                        case_mass);
         if (cudaGetLastError() != cudaSuccess) return VOF_ERR_CUDA;
     }
     return VOF_OK;

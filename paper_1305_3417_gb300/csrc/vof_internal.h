@@ -53,9 +53,12 @@ struct DevMesh {
 
 // the context's counter buffer: per-step counters (the first CNT_LEN ints),
 // then the two words of the grid barrier, each on its own 128-byte line
-enum { CNT_BAND = 0, CNT_ICELL, CNT_MAXPOS, CNT_MAXCORR, CNT_FALLBACK, CNT_VIOL0, CNT_VIOL1, CNT_PEND, CNT_PFNEXT,
-       CNT_RCNEXT, CNT_BPASS, CNT_BACT0, CNT_BACT1, CNT_PFOVF, CNT_PFQ = 14 /* two words, 8-byte aligned */,
-       CNT_CLNEXT = 16, CNT_OVNEXT, CNT_LEN = 24 };
+enum { CNT_BAND = 0, CNT_ICELL, CNT_MAXPOS, CNT_MAXCORR, CNT_FALLBACK, CNT_PFNEXT, CNT_RCNEXT, CNT_PFOVF,
+       CNT_PFQ = 8 /* two words, 8-byte aligned */, CNT_CLNEXT = 10, CNT_OVNEXT,
+       // the update group's
+       CNT_UPD = 12, CNT_VIOL0 = CNT_UPD, CNT_VIOL1, CNT_BPASS, CNT_BACT0, CNT_BACT1, CNT_NRL0, CNT_NRL1, CNT_LEFT0,
+       CNT_LEFT1, CNT_NDL, CNT_UPD_N = CNT_NDL - CNT_UPD + 1, CNT_LEN = 24,
+       CNT_EPOCH = 28 /* kept from step to step */ };
 enum { CNT_BAR = 32, CNT_BARGEN = 64, CNT_ALLOC = 96 };
 // algorithmic work counted by the step kernels (vof_work_counts): the phase
 // flux's primitives (FP32 in the mixed form, FP64 in the plain one) -- signed
@@ -78,6 +81,10 @@ struct __align__(16) BandRec {
 };
 static_assert(sizeof(BandRec) == 64, "four 16-byte loads");
 
+// columns of the per-segment table; the one with the masses after the step
+constexpr int SEG_COLS = 11, SEG_COL_MASS = 4;
+constexpr int SEG_STEP = 256;  // the smallest segment size (seg_at's step)
+
 struct vof_ctx {
     int device;
     int np, nf, ni, nc;
@@ -89,8 +96,7 @@ struct vof_ctx {
     int nbufs;
     // per-step scratch
     uint8_t *pstate;
-    int *band, *icell, *viol[2], *pend_c;
-    double *pend_a;
+    int *band, *icell, *viol[2];
     int *counters;               // CNT_ALLOC ints, laid out as CNT_* above
     double *lam_b, *disp_b;      // per band slot
     int *it_b;
@@ -98,16 +104,21 @@ struct vof_ctx {
     uint8_t *flags;
     int *pit;
     double *Va;
-    double *bscr;                // redistribution scratch, 3 doubles per cell
-    double *gpartial;            // global bounding partial sums, 4 per segment
+    // redistribution: 4 doubles per cell, receivers of a pass and their new
+    // values, marks per cell and per segment, changed segments
+    double *bscr, *ra;
+    int *rl, *dl;
+    unsigned *cmark, *segmark;
+    double *sd;                  // per-segment table (masses, extrema, mesh-wide sums)
     // regions of the global bounding step (whole mesh, or the cases of a
     // batch): segments {region, first cell, end cell, -} and, per region, its
     // segment range and totals
     int nseg, nreg;
     int4 *seg;
     int *reg_seg;
+    int *seg_at;                 // per SEG_STEP cells: the segment of the first
+    uint8_t *seg_mixed;          // per segment: cells beyond [0, 1] or strictly inside
     double *reg_tot;
-    double *partial;             // reduction partials
     double *stats_dev;           // internal stats buffer
     unsigned *status;
     double *h_alpha;               // device staging for vof_advect_host; U and F double-buffered

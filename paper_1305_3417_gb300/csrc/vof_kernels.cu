@@ -972,132 +972,247 @@ __device__ double clip_tet(const Tet &T, const V3 *pn, const double *pd, int np,
 }
 
 // ============================================================ update (A7)
+// The cells are taken in segments (contiguous, at most a thousand or a few
+// thousand cells of one region: set_bound_regions).  The update leaves, per
+// segment, the step's masses and extrema and the sums that the redistribution's
+// mesh-wide part needs; the redistribution then only recomputes the segments it
+// changes, instead of sweeping every cell twice more.
 constexpr int UPD_THREADS = 256;
-constexpr int UPD_BLOCKS = 1024;
-// partial layout per block: [mass_before, mass_after, min, max, boundary_out]
 
-__device__ __forceinline__ void block_reduce5(double v[5], double *out)
+// Columns of the per-segment table (SD_N columns of nseg values): before the
+// redistribution: masses before and after the update, extrema, boundary outflow;
+// after it (as before, until changed): mass, extrema; and, filled only where the
+// mesh-wide fallback runs, excess and deficit volume, free and phase volume of
+// the strictly mixed cells.
+enum { SD_MB = 0, SD_MINP, SD_MAXP, SD_OUT, SD_M, SD_MIN, SD_MAX, SD_EP, SD_EM, SD_SP, SD_SM, SD_N };
+constexpr int SD_UPD = SD_EP;  // the columns that the update fills
+static_assert(SD_N == SEG_COLS && SD_M == SEG_COL_MASS, "the table as its other users see it");
+
+// order of doubles on the integer pipe
+__device__ __forceinline__ double min_bits(double a, double b) { return gt_bits(a, b) ? b : a; }
+__device__ __forceinline__ double max_bits(double a, double b) { return gt_bits(a, b) ? a : b; }
+__device__ __forceinline__ bool is_exc(double a) { return gt_pos(a, 1.0 + BOUND_TOL); }
+__device__ __forceinline__ bool is_def(double a) { return lt_neg(a, BOUND_TOL); }
+__device__ __forceinline__ bool is_mixed(double a) { return gt_pos(a, BOUND_TOL) && lt_pos(a, 1.0 - BOUND_TOL); }
+
+// a warp's sum of v in a fixed order, skipped where every lane has zero (an
+// FP64 add occupies its pipe for many cycles; most segments are empty)
+__device__ __forceinline__ double warp_sum_nz(double v)
 {
-    __shared__ double sh[5][UPD_THREADS / 32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    return __any_sync(0xffffffffu, !is_zero(v)) ? warp_sum(v) : 0.0;
+}
+__device__ __forceinline__ double warp_min_bits(double v)
+{
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
-        v[1] += __shfl_xor_sync(0xffffffffu, v[1], o);
-        v[2] = fmin(v[2], __shfl_xor_sync(0xffffffffu, v[2], o));
-        v[3] = fmax(v[3], __shfl_xor_sync(0xffffffffu, v[3], o));
-        v[4] += __shfl_xor_sync(0xffffffffu, v[4], o);
-    }
-    if (lane == 0) for (int i = 0; i < 5; ++i) sh[i][w] = v[i];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double r[5] = {0.0, 0.0, 1e300, -1e300, 0.0};
-        for (int k = 0; k < UPD_THREADS / 32; ++k) {
-            r[0] += sh[0][k]; r[1] += sh[1][k];
-            r[2] = fmin(r[2], sh[2][k]); r[3] = fmax(r[3], sh[3][k]);
-            r[4] += sh[4][k];
-        }
-        for (int i = 0; i < 5; ++i) out[i] = r[i];
-    }
-    __syncthreads();
+    for (int o = 16; o > 0; o >>= 1) v = min_bits(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+__device__ __forceinline__ double warp_max_bits(double v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = max_bits(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
 }
 
+// A block per segment, a thread per cell.  Bound by HBM (28 B of cell CSR, 16 of
+// alpha, 8 of V a cell, each face's flux once) and, on small meshes, by the chain
+// of dependent loads.  An empty cell without flux costs no FP64 instruction and
+// a full one without flux no division (the FP64 pipe runs at 1/62 of FP32).
 __global__ void __launch_bounds__(UPD_THREADS) k_update(DevMesh m, double *alpha, const double *__restrict__ Va,
-                                                        double *partial, int *viol, int *nviol, int cap,
-                                                        unsigned *status)
+                                                        const int4 *__restrict__ seg, int nseg, double *sd,
+                                                        uint8_t *seg_mixed, int *viol, int *nviol, unsigned *status)
 {
-    double v[5] = {0.0, 0.0, 1e300, -1e300, 0.0};
-    bool zero = false;
+    __shared__ double sh[UPD_THREADS / 32][SD_UPD];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int nb = m.nf - m.ni;
-    const int stride = gridDim.x * blockDim.x;
-    const int lim = m.nc > nb ? m.nc : nb;
-    for (int i0 = blockIdx.x * blockDim.x; i0 < lim; i0 += stride) {
-        int c = i0 + threadIdx.x;
-        bool bad = false;
-        if (c < m.nc) {
-            // A cell whose face fluxes are all zero (the bulk of either phase
-            // away from the band) has s = +0; the FP64 sum runs only where some
-            // flux is not zero, so warps of such cells issue no FP64 adds.
-            const int k0 = m.cptr[c], k1 = m.cptr[c + 1];
-            unsigned nz = 0;
-            // (cflux: the cell's faces, a periodic copy read as its face seen
-            // from the neighbour; the cell's own faces on other meshes)
+    for (int sgi = blockIdx.x; sgi < nseg; sgi += gridDim.x) {
+        const int4 sg = seg[sgi];
+        double mb = 0.0, ma = 0.0, out = 0.0, lo = 1e300, hi = -1e300;
+        bool special = false;  // some cell beyond [0, 1] or strictly inside
+        for (int i0 = sg.y; i0 < sg.z; i0 += UPD_THREADS) {
+            const int c = i0 + threadIdx.x;
+            bool bad = false;
+            if (c < sg.z) {
+                // A cell whose face fluxes are all zero (the bulk of either phase
+                // away from the band) has s = +0; the FP64 sum runs only where some
+                // flux is not zero, so warps of such cells issue no FP64 adds.
+                const int k0 = m.cptr[c], k1 = m.cptr[c + 1];
+                const double a0 = alpha[c];
+                unsigned nz = 0;
+                // (cflux: the cell's faces, a periodic copy read as its face seen
+                // from the neighbour; the cell's own faces on other meshes)
 #pragma unroll 4
-            for (int k = k0; k < k1; ++k) {
-                DBits b = dbits(Va[m.cflux[k] >> 1]);
-                nz |= (unsigned)(b.hi & 0x7fffffff) | b.lo;
-            }
-            double s = 0.0;
-            if (nz)
                 for (int k = k0; k < k1; ++k) {
-                    int code = m.cflux[k];
-                    double x = Va[code >> 1];
-                    s += (code & 1) ? -x : x;
+                    DBits b = dbits(Va[m.cflux[k] >> 1]);
+                    nz |= (unsigned)(b.hi & 0x7fffffff) | b.lo;
                 }
-            double a0 = alpha[c];
-            if (is_zero(s) && is_pzero(a0)) {
-                zero = true;  // an empty cell with no flux: alpha stays +0
-            } else {
-                double V = m.vc[c];
-                double a1 = a0 - s / V;
-                alpha[c] = a1;
-                v[0] += V * a0;
-                v[1] += V * a1;
-                v[2] = fmin(v[2], a1);
-                v[3] = fmax(v[3], a1);
-                bad = gt_pos(a1, 1.0 + BOUND_TOL) || lt_neg(a1, BOUND_TOL);
+                double s = 0.0;
+                if (nz)
+                    for (int k = k0; k < k1; ++k) {
+                        int code = m.cflux[k];
+                        double x = Va[code >> 1];
+                        s += (code & 1) ? -x : x;
+                    }
+                double a1 = a0;
+                if (!is_zero(s) || !is_pzero(a0)) {  // (an empty cell with no flux: alpha stays +0)
+                    const double V = m.vc[c];
+                    if (!is_zero(s)) {
+                        a1 = a0 - s / V;
+                        alpha[c] = a1;
+                    }
+                    mb = fma(V, a0, mb);
+                    ma = fma(V, a1, ma);
+                    bad = is_exc(a1) || is_def(a1);
+                    special |= bad || is_mixed(a1);
+                }
+                lo = min_bits(lo, a1);
+                hi = max_bits(hi, a1);
             }
+            if (viol) warp_append(bad, c, viol, nviol, m.nc, status);
         }
-        if (c < nb) v[4] += Va[m.ni + c];
-        if (viol) warp_append(bad, c, viol, nviol, cap, status);
-    }
-    if (zero) {
-        v[2] = fmin(v[2], 0.0);
-        v[3] = fmax(v[3], 0.0);
-    }
-    block_reduce5(v, partial + 5 * blockIdx.x);
-}
-
-// final reduction of the per-block partials into stats: one block, each thread
-// folds a fixed strided subset, then a fixed tree (deterministic)
-constexpr int ST_THREADS = 256;
-
-__device__ __forceinline__ void fold5(double *r, const double *p)
-{
-    r[0] += p[0]; r[1] += p[1]; r[2] = fmin(r[2], p[2]); r[3] = fmax(r[3], p[3]); r[4] += p[4];
-}
-
-// called by every thread of a block of ST_THREADS threads
-__device__ void stats_block(const double *partial, int nblk, const int *counters, double *stats, int post,
-                            const double *bound_partial, int nblk_post)
-{
-    __shared__ double sh[2][5][ST_THREADS];
-    double r[5] = {0.0, 0.0, 1e300, -1e300, 0.0}, q[5] = {0.0, 0.0, 1e300, -1e300, 0.0};
-    for (int k = threadIdx.x; k < nblk; k += ST_THREADS) fold5(r, partial + 5 * k);
-    if (post)
-        for (int k = threadIdx.x; k < nblk_post; k += ST_THREADS) fold5(q, bound_partial + 5 * k);
-    for (int i = 0; i < 5; ++i) { sh[0][i][threadIdx.x] = r[i]; sh[1][i][threadIdx.x] = q[i]; }
-    __syncthreads();
-    for (int w = ST_THREADS / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-            for (int t = 0; t < 2; ++t) {
-                double a[5], b2[5];
-                for (int i = 0; i < 5; ++i) { a[i] = sh[t][i][threadIdx.x]; b2[i] = sh[t][i][threadIdx.x + w]; }
-                fold5(a, b2);
-                for (int i = 0; i < 5; ++i) sh[t][i][threadIdx.x] = a[i];
+        // boundary faces: a chunk of them goes with each segment
+        for (int f = sgi * UPD_THREADS + threadIdx.x; f < nb; f += nseg * UPD_THREADS) {
+            const double v = Va[m.ni + f];
+            if (!is_zero(v)) out += v;
+        }
+        double v[SD_UPD];
+        v[SD_MB] = warp_sum_nz(mb);
+        v[SD_OUT] = warp_sum_nz(out);
+        v[SD_M] = warp_sum_nz(ma);
+        v[SD_MIN] = v[SD_MINP] = warp_min_bits(lo);
+        v[SD_MAX] = v[SD_MAXP] = warp_max_bits(hi);
+        if (lane == 0)
+#pragma unroll
+            for (int i = 0; i < SD_UPD; ++i) sh[w][i] = v[i];
+        const int any = __syncthreads_or(special);
+        if (threadIdx.x == 0) seg_mixed[sgi] = any != 0;
+        if (threadIdx.x < SD_UPD) {
+            const int i = threadIdx.x;
+            double r = sh[0][i];
+            for (int k = 1; k < UPD_THREADS / 32; ++k) {
+                const double x = sh[k][i];
+                if (i == SD_MIN || i == SD_MINP) r = min_bits(r, x);
+                else if (i == SD_MAX || i == SD_MAXP) r = max_bits(r, x);
+                else if (!is_zero(x)) r += x;
             }
+            sd[(size_t)i * nseg + sgi] = r;
         }
         __syncthreads();
     }
-    if (threadIdx.x != 0) return;
-    stats[VOF_S_MASS_BEFORE] = sh[0][0][0];
-    stats[VOF_S_MIN_PRE] = sh[0][2][0];
-    stats[VOF_S_MAX_PRE] = sh[0][3][0];
-    stats[VOF_S_BOUNDARY_OUT] = sh[0][4][0];
-    const int t = post ? 1 : 0;
-    stats[VOF_S_MASS_AFTER] = sh[t][1][0];
-    stats[VOF_S_MIN_POST] = sh[t][2][0];
-    stats[VOF_S_MAX_POST] = sh[t][3][0];
+}
+
+// A segment by a whole warp: fn(c, a) for every cell in order (lane-strided), then
+// gn(c) for the cells for which fn returned true, 32 at a time in order: the
+// few cells that take FP64 arithmetic are gathered first, since an FP64
+// instruction costs the warp the same for one lane as for all.
+constexpr int SEG_CHUNK = 256;
+template <class Fn, class Gn>
+__device__ __forceinline__ void seg_cells(const double *alpha, int4 sg, unsigned short *list, Fn fn, Gn gn)
+{
+    const int lane = threadIdx.x & 31;
+    for (int c0 = sg.y; c0 < sg.z; c0 += SEG_CHUNK) {
+        const int c1 = min(c0 + SEG_CHUNK, sg.z);
+        int cnt = 0;
+        double a[SEG_CHUNK / 32];
+#pragma unroll
+        for (int u = 0; u < SEG_CHUNK / 32; ++u) {
+            const int c = c0 + 32 * u + lane;
+            a[u] = c < c1 ? alpha[c] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < SEG_CHUNK / 32; ++u) {
+            const int c = c0 + 32 * u + lane;
+            const bool hit = c < c1 && fn(c, a[u]);
+            const unsigned hm = __ballot_sync(0xffffffffu, hit);
+            if (hit) list[cnt + __popc(hm & ((1u << lane) - 1u))] = (unsigned short)(c - c0);
+            cnt += __popc(hm);
+        }
+        __syncwarp();
+        for (int i = lane; i < cnt; i += 32) gn(c0 + list[i]);
+        __syncwarp();
+    }
+}
+
+// columns SD_M, SD_MIN, SD_MAX again after cells of the segment changed
+__device__ __forceinline__ void seg_mass(const DevMesh &m, const double *alpha, int4 sg, int sgi, int nseg, double *sd,
+                                         unsigned short *list)
+{
+    double ma = 0.0, lo = 1e300, hi = -1e300;
+    seg_cells(alpha, sg, list,
+              [&](int, double a) {
+                  lo = min_bits(lo, a);
+                  hi = max_bits(hi, a);
+                  return !is_pzero(a);
+              },
+              [&](int c) { ma = fma(m.vc[c], alpha[c], ma); });
+    ma = warp_sum_nz(ma);
+    lo = warp_min_bits(lo);
+    hi = warp_max_bits(hi);
+    if ((threadIdx.x & 31) == 0) {
+        sd[(size_t)SD_M * nseg + sgi] = ma;
+        sd[(size_t)SD_MIN * nseg + sgi] = lo;
+        sd[(size_t)SD_MAX * nseg + sgi] = hi;
+    }
+}
+
+// columns SD_EP .. SD_SM: what the mesh-wide fallback spreads and who takes it
+__device__ __forceinline__ void seg_room(const DevMesh &m, const double *alpha, int4 sg, int sgi, int nseg, double *sd,
+                                         unsigned short *list)
+{
+    double ep = 0.0, em = 0.0, sp = 0.0, sm = 0.0;
+    seg_cells(alpha, sg, list, [&](int, double a) { return is_exc(a) || is_def(a) || is_mixed(a); },
+              [&](int c) {
+                  const double a = alpha[c], V = m.vc[c];
+                  if (is_exc(a)) ep += (a - 1.0) * V;
+                  else if (is_def(a)) em += -a * V;
+                  else {
+                      sp += (1.0 - a) * V;
+                      sm += a * V;
+                  }
+              });
+    const double v[4] = {warp_sum_nz(ep), warp_sum_nz(em), warp_sum_nz(sp), warp_sum_nz(sm)};
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sd[(size_t)(SD_EP + i) * nseg + sgi] = v[i];
+}
+
+// The step's statistics from the segment table (a block of any number of full
+// warps, at most 32): a fixed tree.
+__device__ void stats_block(const double *sd, int nseg, const int *counters, double *stats, unsigned *status)
+{
+    __shared__ double sh[32][7];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    constexpr int COL[7] = {SD_MB, SD_OUT, SD_M, SD_MINP, SD_MIN, SD_MAXP, SD_MAX};
+    double v[7] = {0.0, 0.0, 0.0, 1e300, 1e300, -1e300, -1e300};
+    for (int k = threadIdx.x; k < nseg; k += blockDim.x)
+#pragma unroll
+        for (int i = 0; i < 7; ++i) {
+            const double x = sd[(size_t)COL[i] * nseg + k];
+            if (i < 3) { if (!is_zero(x)) v[i] += x; }
+            else v[i] = i < 5 ? min_bits(v[i], x) : max_bits(v[i], x);
+        }
+    auto warp = [&]() {
+#pragma unroll
+        for (int i = 0; i < 7; ++i) v[i] = i < 3 ? warp_sum_nz(v[i]) : i < 5 ? warp_min_bits(v[i]) : warp_max_bits(v[i]);
+    };
+    warp();
+    if (lane == 0)
+#pragma unroll
+        for (int i = 0; i < 7; ++i) sh[w][i] = v[i];
+    __syncthreads();
+    if (w != 0) return;
+#pragma unroll
+    for (int i = 0; i < 7; ++i) v[i] = lane < nw ? sh[lane][i] : i < 3 ? 0.0 : i < 5 ? 1e300 : -1e300;
+    warp();
+    if (lane != 0) return;
+    stats[VOF_S_MASS_BEFORE] = v[0];
+    stats[VOF_S_BOUNDARY_OUT] = v[1];
+    stats[VOF_S_MASS_AFTER] = v[2];
+    stats[VOF_S_MIN_PRE] = v[3];
+    stats[VOF_S_MIN_POST] = v[4];
+    stats[VOF_S_MAX_PRE] = v[5];
+    stats[VOF_S_MAX_POST] = v[6];
+    if (status && (gt_pos(v[6], 1.0 + BOUND_FLAG) || lt_neg(v[4], BOUND_FLAG))) atomicOr(status, VOF_ST_BOUND_RESIDUAL);
     if (counters) {
         stats[VOF_S_N_INTERFACE] = counters[CNT_ICELL];
         stats[VOF_S_N_BAND] = counters[CNT_BAND];
@@ -1107,14 +1222,13 @@ __device__ void stats_block(const double *partial, int nblk, const int *counters
         stats[VOF_S_N_BOUND_SOURCES] = counters[CNT_VIOL0];
         stats[VOF_S_N_BOUND_LEFT] = counters[CNT_VIOL1];
     }
-    if (!post) stats[VOF_S_BOUND_PASSES] = stats[VOF_S_BOUND_GLOBAL] = 0.0;
 }
 
-__global__ void __launch_bounds__(ST_THREADS) k_stats(const double *partial, int nblk, const int *counters,
-                                                      double *stats, int post, const double *bound_partial,
-                                                      int nblk_post)
+constexpr int ST_THREADS = 512;
+__global__ void __launch_bounds__(ST_THREADS) k_stats(const double *sd, int nseg, const int *counters, double *stats)
 {
-    stats_block(partial, nblk, counters, stats, post, bound_partial, nblk_post);
+    stats_block(sd, nseg, counters, stats, nullptr);
+    if (threadIdx.x == 0) stats[VOF_S_BOUND_PASSES] = stats[VOF_S_BOUND_GLOBAL] = 0.0;
 }
 
 // ------------------------------------------ redistribution passes (reading R10)
@@ -1129,273 +1243,29 @@ __global__ void __launch_bounds__(ST_THREADS) k_stats(const double *partial, int
 // next pass.  Passes run while some source has both something left and a
 // receiver with room.  Every touched cell's new value is a gather over its
 // face neighbours in face order.
-// Face neighbours of x in face order, handed to fn(s, k) (s the neighbour, k
-// its cface slot).  The indices of a chunk of up to BP_CHUNK neighbours are
-// loaded together, and fn's own loads across the unrolled chunk can issue
-// together too: a few dependent load rounds per chunk instead of a chain per
-// neighbour.
-constexpr int BP_CHUNK = 8;
+// A cell is worked on by BP_LANES lanes, each taking every BP_LANES-th of its
+// faces: one short chain of loads an item, and little code -- each phase runs
+// once, so its instructions come from L2 as it goes (unrolled over a cell's
+// faces, a phase took 10 us on 21 sources).
+constexpr int BP_LANES = 8;
 template <class Fn>
 __device__ __forceinline__ void for_nbrs(const DevMesh &m, int x, Fn fn)
 {
-    const int k0 = m.cptr[x], k1 = m.cptr[x + 1];
-    for (int kb = k0; kb < k1; kb += BP_CHUNK) {
-        int nb[BP_CHUNK];
+#pragma unroll 1
+    for (int k = m.cptr[x] + (int)(threadIdx.x & (BP_LANES - 1)), k1 = m.cptr[x + 1]; k < k1; k += BP_LANES) {
+        const int nb = m.cnb[k];
+        if (nb >= 0) fn(nb);
+    }
+}
+// sum over a cell's lanes, in a fixed order
+__device__ __forceinline__ double lanes_sum(double v)
+{
+    const unsigned gm = ((1u << BP_LANES) - 1u) << (threadIdx.x & 31 & ~(BP_LANES - 1));
 #pragma unroll
-        for (int j = 0; j < BP_CHUNK; ++j) nb[j] = kb + j < k1 ? m.cnb[kb + j] : -1;
-#pragma unroll
-        for (int j = 0; j < BP_CHUNK; ++j)
-            if (nb[j] >= 0) fn(nb[j], kb + j);
-    }
+    for (int o = BP_LANES / 2; o > 0; o >>= 1) v += __shfl_xor_sync(gm, v, o);
+    return v;
 }
-__device__ __forceinline__ bool is_exc(double a) { return a > 1.0 + BOUND_TOL; }
-__device__ __forceinline__ bool is_def(double a) { return a < -BOUND_TOL; }
-__device__ __forceinline__ double recv_w(double a, double V)
-{
-    return (a > BOUND_TOL && a < 1.0 - BOUND_TOL) ? a * (1.0 - a) * V : 0.0;
-}
-
-// scratch per cell: [1/W (0 where the source has no receiver), receiver
-// scales sp, sm]
-enum { BS_RW = 0, BS_SP, BS_SM, BS_N = 3 };
-
-struct BoundBufs {
-    int *la;             // source list (from the update kernel), capacity nc
-    const int *n0;       // its count
-    int *pc;             // pending cells, capacity cap_pend
-    double *pa;          // pending values
-    double *bs;          // BS_N doubles per cell
-    int *npass;          // out: passes that moved something
-    int *act;            // two counters of active sources (pass parity)
-    int cap, cap_pend;
-};
-
-
-// lowest-index source among x's face neighbours (and x itself if self)
-__device__ __forceinline__ int first_source(const DevMesh &m, const double *alpha, int x, bool self)
-{
-    int first = 0x7fffffff;
-    if (self) {
-        double ax = alpha[x];
-        if (is_exc(ax) || is_def(ax)) first = x;
-    }
-    for_nbrs(m, x, [&](int s, int) {
-        double as = alpha[s];
-        if ((is_exc(as) || is_def(as)) && s < first) first = s;
-    });
-    return first;
-}
-
-// One pass as three phases over the source list (count on the device): the
-// receiver weight around each source, receiver scales, new values (a source's
-// own placement summed where its new value is formed), then apply; t0 / nt:
-// this thread's index and the thread count of the grid.
-// A source with something left and a receiver is counted in *act.
-__device__ __forceinline__ void bp_room(const DevMesh &m, const double *alpha, const BoundBufs &b, int *act, long t0, long nt)
-{
-    const int n = min(*b.n0, b.cap);
-    int active = 0;
-    for (long i = t0; i < n; i += nt) {
-        int c = b.la[i];
-        const double a = alpha[c];
-        double W = 0.0;
-        if (is_exc(a) || is_def(a))
-            for_nbrs(m, c, [&](int nb, int) { W += recv_w(alpha[nb], m.vc[nb]); });
-        b.bs[BS_N * (size_t)c + BS_RW] = W > 0.0 ? 1.0 / W : 0.0;
-        active += W > 0.0;
-    }
-    if (active) atomicAdd(act, active);
-}
-
-// one thread per (source, face slot): slot j takes the faces j, j + BP_SLOTS, ...
-constexpr int BP_SLOTS = 8;
-
-__device__ __forceinline__ void bp_scale(const DevMesh &m, const double *alpha, const BoundBufs &b, long t0, long nt)
-{
-    const long n = min(*b.n0, b.cap);
-    double *bs = b.bs;
-    for (long t = t0; t < n * BP_SLOTS; t += nt) {
-        int c = b.la[t / BP_SLOTS];
-        for (int k = m.cptr[c] + (int)(t % BP_SLOTS); k < m.cptr[c + 1]; k += BP_SLOTS) {
-            int r = m.cnb[k];
-            if (r < 0 || first_source(m, alpha, r, false) != c) continue;
-            const double ar = alpha[r], Vr = m.vc[r], wr = recv_w(ar, Vr);
-            const double Rp = wr > 0.0 ? (1.0 - ar) * Vr : 0.0, Rm = wr > 0.0 ? ar * Vr : 0.0;
-            double Qp = 0.0, Qm = 0.0;
-            if (wr > 0.0)
-                for_nbrs(m, r, [&](int s, int) {
-                    const double as = alpha[s], rW = bs[BS_N * (size_t)s + BS_RW];
-                    if (rW > 0.0) {
-                        if (is_exc(as)) Qp += (as - 1.0) * m.vc[s] * (wr * rW);
-                        else if (is_def(as)) Qm += -as * m.vc[s] * (wr * rW);
-                    }
-                });
-            bs[BS_N * (size_t)r + BS_SP] = Qp > Rp ? Rp / Qp : 1.0;
-            bs[BS_N * (size_t)r + BS_SM] = Qm > Rm ? Rm / Qm : 1.0;
-        }
-    }
-}
-
-// new values of the sources and their neighbours, each cell once: by the
-// lowest-index source in its closed face neighbourhood
-__device__ __forceinline__ void bp_new(const DevMesh &m, const double *alpha, const BoundBufs &b, int *npend, unsigned *status,
-                       long t0, long nt)
-{
-    const long n = min(*b.n0, b.cap);
-    const double *bs = b.bs;
-    for (long t = t0; t < n * BP_SLOTS; t += nt) {
-        int c = b.la[t / BP_SLOTS];
-        // slot 0 takes the source itself (k = cptr[c] - 1)
-        for (int k = m.cptr[c] - 1 + (int)(t % BP_SLOTS); k < m.cptr[c + 1]; k += BP_SLOTS) {
-            int x = k < m.cptr[c] ? c : m.cnb[k];
-            if (x < 0 || first_source(m, alpha, x, true) != c) continue;
-            const double ax = alpha[x], V = m.vc[x], wx = recv_w(ax, V);
-            double dV = 0.0;
-            const bool xe = is_exc(ax);
-            if (xe || is_def(ax)) {
-                // a source: what it places in its receivers (each scaled to fit)
-                const double rWx = bs[BS_N * (size_t)x + BS_RW];
-                if (rWx > 0.0) {
-                    const double e = xe ? (ax - 1.0) * V : -ax * V;
-                    double g = 0.0;
-                    for_nbrs(m, x, [&](int nb, int) {
-                        const double w = recv_w(alpha[nb], m.vc[nb]);
-                        if (w > 0.0) g += e * (w * rWx) * bs[BS_N * (size_t)nb + (xe ? BS_SP : BS_SM)];
-                    });
-                    dV += xe ? -g : g;
-                }
-            } else if (wx > 0.0) {
-                // a receiver: what its source neighbours place in it
-                const double SPx = bs[BS_N * (size_t)x + BS_SP], SMx = bs[BS_N * (size_t)x + BS_SM];
-                for_nbrs(m, x, [&](int s, int) {
-                    const double as = alpha[s], rW = bs[BS_N * (size_t)s + BS_RW];
-                    if (rW > 0.0) {
-                        if (is_exc(as)) dV += (as - 1.0) * m.vc[s] * (wx * rW) * SPx;
-                        else if (is_def(as)) dV -= -as * m.vc[s] * (wx * rW) * SMx;
-                    }
-                });
-            }
-            if (dV != 0.0) {
-                int pos = atomicAdd(npend, 1);
-                if (pos < b.cap_pend) { b.pc[pos] = x; b.pa[pos] = (ax * V + dV) / V; }
-                else atomicOr(status, VOF_ST_CAPACITY);
-            }
-        }
-    }
-}
-
-__device__ __forceinline__ void bp_apply(double *alpha, const int *pc, const double *pa, const int *npend, int cap, long t0, long nt)
-{
-    const int n = min(*npend, cap);
-    for (long i = t0; i < n; i += nt) alpha[pc[i]] = pa[i];
-}
-
-// Global fallback for what the local passes leave (a source none of whose face
-// neighbours is an interface cell with room): the total excess (deficit) of a
-// region (the whole mesh, or one case of a batch) goes to every cell of that
-// region strictly inside (tol, 1-tol) in proportion to its free (phase)
-// volume; sources are set to 1 (0).  A region's cells are contiguous and cut
-// into segments; one block sums a segment, then one warp per region sums its
-// segments in order (deterministic).
-constexpr int GB_THREADS = 256;
-
-// one segment, by a whole block of GB_THREADS threads
-// A thread takes the cells c, c + blockDim.x, ... of the segment in order; the
-// loads of SEG_UNROLL consecutive ones of its cells are issued together.
-constexpr int SEG_UNROLL = 4;
-__device__ void seg_reduce(const DevMesh &m, const double *alpha, int4 sg, double *spartial, int *nleft)
-{
-    double v[4] = {0.0, 0.0, 0.0, 0.0};  // Ep, Em, Sp, Sm
-    int left = 0;
-    auto cell = [&](int c, double a) {
-        if (gt_pos(a, 1.0 + BOUND_TOL)) { v[0] += (a - 1.0) * m.vc[c]; ++left; }
-        else if (lt_neg(a, BOUND_TOL)) { v[1] += -a * m.vc[c]; ++left; }
-        else if (gt_pos(a, BOUND_TOL) && lt_pos(a, 1.0 - BOUND_TOL)) {
-            double V = m.vc[c];
-            v[2] += (1.0 - a) * V;
-            v[3] += a * V;
-        }
-    };
-    const int step = blockDim.x;
-    int c = sg.y + threadIdx.x;
-    for (; c + (SEG_UNROLL - 1) * step < sg.z; c += SEG_UNROLL * step) {
-        double a[SEG_UNROLL];
-#pragma unroll
-        for (int u = 0; u < SEG_UNROLL; ++u) a[u] = alpha[c + u * step];
-#pragma unroll
-        for (int u = 0; u < SEG_UNROLL; ++u) cell(c + u * step, a[u]);
-    }
-    for (; c < sg.z; c += step) cell(c, alpha[c]);
-    left = __reduce_add_sync(0xffffffffu, left);
-    if ((threadIdx.x & 31) == 0 && left) atomicAdd(nleft, left);
-    __shared__ double sh[4][GB_THREADS / 32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int i = 0; i < 4; ++i) {
-        double x = warp_sum(v[i]);
-        if (lane == 0) sh[i][w] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int i = 0; i < 4; ++i) {
-            double r = 0.0;
-            for (int k = 0; k < GB_THREADS / 32; ++k) r += sh[i][k];
-            spartial[i] = r;
-        }
-    __syncthreads();
-}
-
-// region r, by a whole warp: totals[REG_TOT * r + 0..3] = Ep, Em, Sp, Sm and
-// [4], [5] the shares Ep / Sp, Em / Sm of the global step (0 where none)
-constexpr int REG_TOT = 6;
-__device__ void region_totals(const int *reg_seg, int r, const double *spartial, double *totals)
-{
-    const int lane = threadIdx.x & 31;
-    double t[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int k = reg_seg[r] + lane; k < reg_seg[r + 1]; k += 32)
-        for (int i = 0; i < 4; ++i) t[i] += spartial[4 * k + i];
-    for (int i = 0; i < 4; ++i) t[i] = warp_sum(t[i]);
-    if (lane == 0) {
-        double *o = totals + REG_TOT * (size_t)r;
-        for (int i = 0; i < 4; ++i) o[i] = t[i];
-        o[4] = t[0] > 0.0 && t[2] > 0.0 ? t[0] / t[2] : 0.0;
-        o[5] = t[1] > 0.0 && t[3] > 0.0 ? t[1] / t[3] : 0.0;
-    }
-}
-
-// one segment, by a whole block: the global step where its region needs one,
-// then the segment's share of the post-bounding mass and extrema (v as in the
-// update partials; +0 cells add nothing to the mass and set 'zero')
-__device__ void seg_apply(const DevMesh &m, double *alpha, int4 sg, const double *totals, double v[5], bool &zero,
-                          bool &bad)
-{
-    const double *tt = totals + REG_TOT * (size_t)sg.x;
-    const double Ep = tt[0], Em = tt[1], Sp = tt[2], Sm = tt[3], sp = tt[4], sm = tt[5];
-    const bool apply = !((Ep == 0.0 && Em == 0.0) || Ep > Sp || Em > Sm);
-    auto cell = [&](int c, double a) {
-        if (apply) {
-            // a cell strictly inside takes Ep (1 - a) V / Sp and gives Em a V / Sm:
-            // a + (Ep / Sp)(1 - a) - (Em / Sm) a, no division per cell
-            if (gt_pos(a, 1.0 + BOUND_TOL)) alpha[c] = a = 1.0;
-            else if (lt_neg(a, BOUND_TOL)) alpha[c] = a = 0.0;
-            else if (gt_pos(a, BOUND_TOL) && lt_pos(a, 1.0 - BOUND_TOL)) alpha[c] = a = a + sp * (1.0 - a) - sm * a;
-        }
-        if (is_pzero(a)) { zero = true; return; }
-        v[1] += m.vc[c] * a;
-        v[2] = fmin(v[2], a);
-        v[3] = fmax(v[3], a);
-        bad |= gt_pos(a, 1.0 + BOUND_FLAG) || lt_neg(a, BOUND_FLAG);
-    };
-    const int step = blockDim.x;
-    int c = sg.y + threadIdx.x;
-    for (; c + (SEG_UNROLL - 1) * step < sg.z; c += SEG_UNROLL * step) {
-        double a[SEG_UNROLL];
-#pragma unroll
-        for (int u = 0; u < SEG_UNROLL; ++u) a[u] = alpha[c + u * step];
-#pragma unroll
-        for (int u = 0; u < SEG_UNROLL; ++u) cell(c + u * step, a[u]);
-    }
-    for (; c < sg.z; c += step) cell(c, alpha[c]);
-}
+__device__ __forceinline__ double recv_w(double a, double V) { return is_mixed(a) ? a * (1.0 - a) * V : 0.0; }
 
 // Grid-wide barrier of a cooperative launch (every block resident): a block
 // arrives on the count; the last to arrive resets it and advances the generation
@@ -1420,13 +1290,14 @@ __device__ bool grid_sync(unsigned *count, unsigned *generation, unsigned *statu
             atomicAdd(generation, 1u);
         } else {
             long it = 0;
-            unsigned pause = 32;
+            unsigned pause = 16;
             while (*gen == g) {
                 if (++it > limit) {
                     atomicOr(status, VOF_ST_TIMEOUT);
                     gave_up = 1;
                     break;
                 }
+                if (it <= 16) continue;  // (a barrier usually completes within a few polls)
                 __nanosleep(pause);
                 if (pause < 1024) pause <<= 1;
             }
@@ -1437,91 +1308,261 @@ __device__ bool grid_sync(unsigned *count, unsigned *generation, unsigned *statu
     return !gave_up;
 }
 
-// The whole redistribution, the post-bounding mass and the step statistics in
-// one cooperative launch, a grid barrier between the phases: passes of the
-// local redistribution (weights, scales, new values, apply) while
-// some source has something left and a receiver, segment sums, region totals,
-// global fallback with the mass partials, statistics (block 0).
+// The redistribution of a step: passes over the sources and their receivers,
+// the mesh-wide fallback for what no local pass can place (a source none of
+// whose face neighbours is an interface cell with room): the total excess
+// (deficit) of a region (the whole mesh, or one case of a batch) goes to every
+// cell of that region strictly inside (tol, 1-tol) in proportion to its free
+// (phase) volume, and sources are set to 1 (0); then the step's statistics.
+//
+// A pass has three phases with a barrier after each: sources weigh their
+// receivers and list them, each once (marked with the pass's own number, so the
+// marks need no clearing); receivers gather their requests, scale them and
+// form their new value; sources take off what was placed while the receivers'
+// values are written.  The phases are chains of a few dependent loads over
+// hundreds of items: barriers, first-time instruction fetches and, where many
+// cells are strictly inside, FP64 work on few SMs are the cost.  On meshes up to
+// BOUND_CLUSTER_CELLS the kernel is one cluster of eight blocks with the
+// hardware's cluster barrier, beyond that one block per SM of a cooperative
+// launch (the update and this, 24^3: 38 us; 32^3-based octree 69 in one cluster,
+// 62 over all SMs; 64^3 film 76 / 63; 48^3 tetrahedra, with a fallback, 230 /
+// 143; 128^3 114 / 95).  With four barriers a pass over 608 blocks and two
+// sweeps over every cell in each step they took 60 us on the 32^2 disc without a
+// source (now 19), 94 at 24^3, 135 on the octree, 117 on the film, 153 at 128^3.
 struct BoundStep {
     double *alpha;
-    BoundBufs b;
-    int *npend;
+    int *src;                    // sources (from the update)
+    int *nsrc;                   // their count
+    int *rl, *nrl;               // receivers of a pass, counts by pass parity
+    double *ra;                  // their new values
+    double *bs;                  // BS_N doubles per cell
+    unsigned *mark;              // per cell: the pass that listed it
+    unsigned *segmark;           // per segment: the launch that changed it
+    int *dl, *ndl;               // changed segments
+    unsigned *epoch;             // numbers used so far
+    int *npass, *act, *left;     // passes that moved something; sources with a receiver, sources left, by pass parity
+    int *nleft;                  // out: sources left to the fallback
     const int4 *seg;
+    const int *seg_at;           // per SEG_STEP cells: the segment of the first
     int nseg;
-    double *gpartial;            // 4 per segment
-    int *nleft;
+    const uint8_t *seg_mixed;    // per segment: cells beyond [0, 1] or strictly inside
+    double *sd;
     const int *reg_seg;
     int nreg;
-    double *reg_tot;
-    double *mpartial;            // 5 per block: post-bounding mass, extrema
-    const double *upartial;      // the update kernel's partials
-    int nupd;
+    double *reg_tot;             // REG_TOT per region
     const int *counters;         // or null: no counter statistics
     double *stats;
     unsigned *bar_count;         // grid barrier: arrivals (zero before the launch)
     unsigned *bar_gen;           // and generation (any value)
     unsigned *status;
 };
+// scratch per cell: source: 1/W (0 where it has no receiver); receiver:
+// weight, scales for excess and deficit
+enum { BS_RW = 0, BS_W, BS_SP, BS_SM, BS_N = 4 };
+// per region: Ep, Em, Sp, Sm and the shares Ep / Sp, Em / Sm of the mesh-wide
+// step (0 where none)
+constexpr int REG_TOT = 6;
+constexpr int BA_THREADS = 1024;
+constexpr int BA_CLUSTER = 8;
+constexpr int BOUND_CLUSTER_CELLS = 1 << 15;
 
-constexpr int BA_THREADS = 256;
-static_assert(BA_THREADS == GB_THREADS && BA_THREADS == UPD_THREADS && BA_THREADS == ST_THREADS,
-              "the phases share one block shape");
-
-__global__ void __launch_bounds__(BA_THREADS, 4) k_bound_step(DevMesh m, BoundStep a)
+// region r, by a whole warp
+__device__ void region_totals(const int *reg_seg, int r, const double *sd, const uint8_t *seg_mixed, int nseg,
+                              double *totals)
 {
-    const long t0 = blockIdx.x * (long)blockDim.x + threadIdx.x, nt = (long)gridDim.x * blockDim.x;
-    // the passes have few items (sources x slots): item i goes to block
-    // i mod gridDim.x, so that they spread over every SM rather than fill the
-    // first few blocks (the FP64 divisions of a phase run on all SMs' units)
-    const long tl = threadIdx.x * (long)gridDim.x + blockIdx.x;
+    const int lane = threadIdx.x & 31;
+    double t[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int k = reg_seg[r] + lane; k < reg_seg[r + 1]; k += 32)
+        if (seg_mixed[k])
+            for (int i = 0; i < 4; ++i) t[i] += sd[(size_t)(SD_EP + i) * nseg + k];
+    for (int i = 0; i < 4; ++i) t[i] = warp_sum(t[i]);
+    if (lane == 0) {
+        double *o = totals + REG_TOT * (size_t)r;
+        for (int i = 0; i < 4; ++i) o[i] = t[i];
+        o[4] = t[0] > 0.0 && t[2] > 0.0 ? t[0] / t[2] : 0.0;
+        o[5] = t[1] > 0.0 && t[3] > 0.0 ? t[1] / t[3] : 0.0;
+    }
+}
+__device__ __forceinline__ bool region_applies(const double *tt)
+{
+    return !((tt[0] == 0.0 && tt[1] == 0.0) || tt[0] > tt[2] || tt[1] > tt[3]);
+}
+
+template <bool CLUSTER>
+__global__ void __launch_bounds__(BA_THREADS, 1) k_bound_step(DevMesh m, BoundStep a)
+{
+    // item i goes to block i mod gridDim.x: the few items of a phase spread over
+    // every SM of the launch
+    const int tl = threadIdx.x * gridDim.x + blockIdx.x, nt = gridDim.x * blockDim.x;
+    const int wl = (threadIdx.x >> 5) * gridDim.x + blockIdx.x, nw = nt >> 5;
+    const int gl = (threadIdx.x / BP_LANES) * gridDim.x + blockIdx.x, ng = nt / BP_LANES;
+    const bool first = (threadIdx.x & (BP_LANES - 1)) == 0;
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
-    // act[p & 1] counts pass p's active sources; it was zeroed by the pass
-    // before (act[0] before the launch), after every block had read it
+    auto sync = [&]() -> bool {
+        if constexpr (CLUSTER) {
+            __syncthreads();
+            if (threadIdx.x == 0) __threadfence();
+            asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
+            if (threadIdx.x == 0) __threadfence();
+            __syncthreads();
+            return true;
+        } else return grid_sync(a.bar_count, a.bar_gen, a.status);
+    };
+    auto volat = [](const int *p) { return *(const volatile int *)p; };
+    __shared__ unsigned short lists[BA_THREADS / 32][SEG_CHUNK];
+    unsigned short *list = lists[threadIdx.x >> 5];
+    const int n = min(*a.nsrc, m.nc);
+    const unsigned e0 = *a.epoch;
+    int npass = 0, nleft = n;
+    if (n > 0) {
+        auto touch = [&](int c) {  // c's segment has changed
+            int k = a.seg_at[c / SEG_STEP];
+            if (a.nreg > 1)
+                while (c >= a.seg[k].z) ++k;
+            if (atomicExch(a.segmark + k, e0 + 1) != e0 + 1) a.dl[atomicAdd(a.ndl, 1)] = k;
+        };
 #pragma unroll 1
-    for (int p = 0; p < BOUND_PASSES_MAX; ++p) {
-        int *act = a.b.act + (p & 1);
-        if (lead) {
-            a.b.act[(p + 1) & 1] = 0;
-            *a.npend = 0;  // the previous pass's apply phase is behind a barrier
+        for (int p = 0; p < BOUND_PASSES_MAX; ++p) {
+            const unsigned ep = e0 + 1 + p;
+            int *act = a.act + (p & 1), *nrl = a.nrl + (p & 1), *left = a.left + (p & 1);
+            if (lead) {  // the next pass's counters (last read before the previous pass's last barrier)
+                a.act[(p + 1) & 1] = 0;
+                a.nrl[(p + 1) & 1] = 0;
+            }
+            // ---- sources: weight of the receivers around, which are listed
+            for (int i = gl; i < n; i += ng) {
+                const int c = a.src[i];
+                const double as = a.alpha[c];
+                double W = 0.0;
+                if (is_exc(as) || is_def(as))
+                    for_nbrs(m, c, [&](int nb) {
+                        const double w = recv_w(a.alpha[nb], m.vc[nb]);
+                        if (is_zero(w)) return;
+                        W += w;
+                        if (atomicExch(a.mark + nb, ep) != ep) a.rl[atomicAdd(nrl, 1)] = nb;
+                    });
+                W = lanes_sum(W);
+                if (first) {
+                    a.bs[BS_N * (size_t)c + BS_RW] = W > 0.0 ? 1.0 / W : 0.0;
+                    if (W > 0.0) atomicAdd(act, 1);
+                }
+            }
+            if (!sync()) return;
+            // (the previous pass's count of sources left was read after its last
+            // barrier: it may be cleared only behind this one)
+            if (lead) a.left[(p + 1) & 1] = 0;
+            if (volat(act) == 0) break;
+            npass = p + 1;
+            // ---- receivers: requests, scales, new value
+            const int nr = volat(nrl);
+            for (int i = gl; i < nr; i += ng) {
+                const int r = a.rl[i];
+                const double ar = a.alpha[r], V = m.vc[r], wr = recv_w(ar, V);
+                double Qp = 0.0, Qm = 0.0;
+                for_nbrs(m, r, [&](int s) {
+                    const double as = a.alpha[s];
+                    const bool xe = is_exc(as);
+                    if (!xe && !is_def(as)) return;
+                    const double q = m.vc[s] * (wr * a.bs[BS_N * (size_t)s + BS_RW]);
+                    if (xe) Qp += (as - 1.0) * q;
+                    else Qm += -as * q;
+                });
+                Qp = lanes_sum(Qp);
+                Qm = lanes_sum(Qm);
+                if (first) {
+                    const double Rp = (1.0 - ar) * V, Rm = ar * V;
+                    const double sp = Qp > Rp ? Rp / Qp : 1.0, sm = Qm > Rm ? Rm / Qm : 1.0;
+                    double *b = a.bs + BS_N * (size_t)r;
+                    b[BS_W] = wr;
+                    b[BS_SP] = sp;
+                    b[BS_SM] = sm;
+                    const double dV = Qp * sp - Qm * sm;
+                    a.ra[i] = dV != 0.0 ? (ar * V + dV) / V : ar;
+                }
+            }
+            if (!sync()) return;
+            // ---- sources take off what was placed; receivers' values
+            for (int i = gl; i < n; i += ng) {
+                const int c = a.src[i];
+                const double as = a.alpha[c];
+                const bool xe = is_exc(as);
+                if (!xe && !is_def(as)) continue;
+                const double rW = a.bs[BS_N * (size_t)c + BS_RW], V = m.vc[c];
+                double g = 0.0;
+                if (rW > 0.0) {
+                    const double e = (xe ? (as - 1.0) * V : -as * V) * rW;
+                    for_nbrs(m, c, [&](int nb) {
+                        const double *b = a.bs + BS_N * (size_t)nb;
+                        if (a.mark[nb] == ep) g += e * b[BS_W] * b[xe ? BS_SP : BS_SM];
+                    });
+                }
+                g = lanes_sum(g);
+                if (first) {
+                    double an = as;
+                    if (g != 0.0) {
+                        an = (as * V + (xe ? -g : g)) / V;
+                        a.alpha[c] = an;
+                        touch(c);
+                    }
+                    if (is_exc(an) || is_def(an)) atomicAdd(left, 1);
+                }
+            }
+            for (int i = tl; i < nr; i += nt) {
+                const int r = a.rl[i];
+                a.alpha[r] = a.ra[i];
+                touch(r);
+            }
+            if (!sync()) return;
+            nleft = volat(left);
+            if (nleft == 0) break;
         }
-        bp_room(m, a.alpha, a.b, act, tl, nt);
-        if (!grid_sync(a.bar_count, a.bar_gen, a.status)) return;
-        if (*(volatile int *)act == 0) break;
-        if (lead) *a.b.npass = p + 1;
-        bp_scale(m, a.alpha, a.b, tl, nt);
-        if (!grid_sync(a.bar_count, a.bar_gen, a.status)) return;
-        bp_new(m, a.alpha, a.b, a.npend, a.status, tl, nt);
-        if (!grid_sync(a.bar_count, a.bar_gen, a.status)) return;
-        bp_apply(a.alpha, a.b.pc, a.b.pa, a.npend, a.b.cap_pend, tl, nt);
-        if (!grid_sync(a.bar_count, a.bar_gen, a.status)) return;
+        if (nleft > 0) {
+            for (int k = wl; k < a.nseg; k += nw)
+                if (a.seg_mixed[k]) seg_room(m, a.alpha, a.seg[k], k, a.nseg, a.sd, list);
+            if (!sync()) return;
+            for (int r = wl; r < a.nreg; r += nw)
+                region_totals(a.reg_seg, r, a.sd, a.seg_mixed, a.nseg, a.reg_tot);
+            if (!sync()) return;
+            // a cell strictly inside takes Ep (1 - a) V / Sp and gives Em a V / Sm:
+            // a + (Ep / Sp)(1 - a) - (Em / Sm) a, no division per cell
+            for (int k = wl; k < a.nseg; k += nw) {
+                if (!a.seg_mixed[k]) continue;
+                const int4 sg = a.seg[k];
+                const double *tt = a.reg_tot + REG_TOT * (size_t)sg.x;
+                if (!region_applies(tt)) continue;
+                const double sp = tt[4], sm = tt[5];
+                seg_cells(a.alpha, sg, list, [&](int, double x) { return is_exc(x) || is_def(x) || is_mixed(x); },
+                          [&](int c) {
+                              const double x = a.alpha[c];
+                              a.alpha[c] = is_exc(x) ? 1.0 : is_def(x) ? 0.0 : x + sp * (1.0 - x) - sm * x;
+                          });
+                seg_mass(m, a.alpha, sg, k, a.nseg, a.sd, list);
+            }
+        }
+        if (npass > 0) {
+            // (a segment changed by a pass and by the fallback is summed twice,
+            // by whichever warps: the same sums)
+            const int nd = volat(a.ndl);
+            if (nleft > 0 && !sync()) return;
+            for (int i = wl; i < nd; i += nw) seg_mass(m, a.alpha, a.seg[a.dl[i]], a.dl[i], a.nseg, a.sd, list);
+        }
+        if (!sync()) return;
     }
-    for (int sgi = blockIdx.x; sgi < a.nseg; sgi += gridDim.x)
-        seg_reduce(m, a.alpha, a.seg[sgi], a.gpartial + 4 * (size_t)sgi, a.nleft);
-    if (!grid_sync(a.bar_count, a.bar_gen, a.status)) return;
-    for (int r = (int)(t0 >> 5); r < a.nreg; r += (int)(nt >> 5)) region_totals(a.reg_seg, r, a.gpartial, a.reg_tot);
-    if (!grid_sync(a.bar_count, a.bar_gen, a.status)) return;
-    double v[5] = {0.0, 0.0, 1e300, -1e300, 0.0};
-    bool zero = false, bad = false;
-    for (int sgi = blockIdx.x; sgi < a.nseg; sgi += gridDim.x) seg_apply(m, a.alpha, a.seg[sgi], a.reg_tot, v, zero, bad);
-    if (zero) {
-        v[2] = fmin(v[2], 0.0);
-        v[3] = fmax(v[3], 0.0);
-    }
-    if (bad) atomicOr(a.status, VOF_ST_BOUND_RESIDUAL);
-    block_reduce5(v, a.mpartial + 5 * blockIdx.x);
-    if (!grid_sync(a.bar_count, a.bar_gen, a.status)) return;
-    if (blockIdx.x == 0) {
-        stats_block(a.upartial, a.nupd, a.counters, a.stats, 1, a.mpartial, gridDim.x);
-        if (threadIdx.x == 0) {
-            // volume the global fallback moved (regions where it applied)
-            double gv = 0.0;
+    if (blockIdx.x != 0) return;
+    if (lead) *a.nleft = nleft;
+    __syncthreads();
+    stats_block(a.sd, a.nseg, a.counters, a.stats, a.status);
+    if (lead) {
+        *a.npass = npass;
+        *a.epoch = e0 + (unsigned)npass + 2;
+        double gv = 0.0;  // volume the fallback moved (regions where it applied)
+        if (nleft > 0)
             for (int r = 0; r < a.nreg; ++r) {
                 const double *tt = a.reg_tot + REG_TOT * (size_t)r;
-                if (!((tt[0] == 0.0 && tt[1] == 0.0) || tt[0] > tt[2] || tt[1] > tt[3])) gv += tt[0] + tt[1];
+                if (region_applies(tt)) gv += tt[0] + tt[1];
             }
-            a.stats[VOF_S_BOUND_PASSES] = *(volatile int *)a.b.npass;
-            a.stats[VOF_S_BOUND_GLOBAL] = gv;
-        }
+        a.stats[VOF_S_BOUND_PASSES] = npass;
+        a.stats[VOF_S_BOUND_GLOBAL] = gv;
     }
 }
 
@@ -1543,25 +1584,24 @@ __global__ void k_zero_int(int *p, int n)
     if (i < n) p[i] = 0;
 }
 
-// the update group's counters: violations before / after the local passes,
-// pending cells, passes, the first pass's active sources, and the grid
-// barrier's arrival count
+// the update group's counters (standalone update; a step zeroes them with the rest)
 __global__ void k_zero_update(int *cnt)
 {
     const int i = threadIdx.x;
-    if (i < 3) cnt[CNT_VIOL0 + i] = 0;
-    if (i == 3) cnt[CNT_BAR] = 0;
-    if (i == 4) cnt[CNT_BPASS] = 0;
-    if (i == 5) cnt[CNT_BACT0] = 0;
+    if (i < CNT_UPD_N) cnt[CNT_UPD + i] = 0;
+    if (i == CNT_UPD_N) cnt[CNT_BAR] = 0;
 }
 
 // ============================================== band classification (A2, R9)
 // per point: all cells empty (bit 0) / all full (bit 1); for the other points
 // (every point of an interface cell is one) the IDW point value of Eq.
 // idwpointphi, in the order the reconstruction would sum it
-__global__ void k_point_state(DevMesh m, const double *__restrict__ alpha, uint8_t *state, double *palpha)
+// (and the step's counters, which only later kernels use)
+__global__ void k_point_state(DevMesh m, const double *__restrict__ alpha, uint8_t *state, double *palpha, int *cnt)
 {
     int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < CNT_LEN) cnt[p] = 0;
+    if (p == CNT_LEN) cnt[CNT_BAR] = 0;
     if (p >= m.np) return;
     bool all_e = true, all_f = true;
     const double full = 1.0 - m.eps;
@@ -1616,16 +1656,6 @@ __global__ void k_classify(DevMesh m, const double *__restrict__ alpha, const do
 
 inline int cdiv(long a, long b) { return (int)((a + b - 1) / b); }
 
-// Grid of the update kernel: the blocks resident at once (at most
-// UPD_BLOCKS), so that no block of the grid-stride loop waits for a second wave.
-template <class K>
-int resident_blocks(K kernel, int sms)
-{
-    int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, UPD_THREADS, 0) != cudaSuccess || occ < 1) occ = 1;
-    return sms * occ < UPD_BLOCKS ? sms * occ : UPD_BLOCKS;
-}
-
 }  // namespace
 
 // ================================================================ launchers
@@ -1645,13 +1675,6 @@ static int num_sms(int dev)
     }
     return g_sms;
 }
-static int g_upd_blocks = 0;
-static int upd_blocks(int dev)
-{
-    if (g_upd_blocks == 0) g_upd_blocks = resident_blocks(k_update, num_sms(dev));
-    return g_upd_blocks;
-}
-
 int launch_setup_geometry(vof_ctx *c, cudaStream_t s)
 {
     DevMesh &m = c->m;
@@ -2027,38 +2050,44 @@ int launch_phase_flux_all(vof_ctx *c, const double *alpha, const double *n, cons
     return launch_pf_all(c, alpha, n, d, flags, Up, F, lambda, dt, Va, s);
 }
 
-// The bounding pass, post-bounding mass and statistics: one cooperative
-// launch of k_bound_step, as many blocks as are resident at once (at most
-// UPD_BLOCKS: the mass partials' room).
-static int g_bound_blocks = 0;
-static int launch_bound_step(vof_ctx *c, double *alpha, int nupd, const int *counters, double *stats,
-                             cudaStream_t s)
+// The update, then the redistribution with the statistics (or the statistics
+// alone); counters: the step's, or null.
+static int launch_update_group(vof_ctx *c, double *alpha, const double *Va, const int *counters, double *stats,
+                               cudaStream_t s)
 {
-    if (g_bound_blocks == 0) {
-        int occ = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_bound_step, BA_THREADS, 0) != cudaSuccess || occ < 1)
-            return VOF_ERR_CUDA;
-        g_bound_blocks = std::min(num_sms(c->device) * occ, UPD_BLOCKS);
-    }
     int *cnt = c->counters;
-    BoundStep a{alpha,
-                BoundBufs{c->viol[0], cnt + CNT_VIOL0, c->pend_c, c->pend_a, c->bscr, cnt + CNT_BPASS,
-                          cnt + CNT_BACT0, c->nc, 8 * c->nc},
-                cnt + CNT_PEND, c->seg, c->nseg, c->gpartial, cnt + CNT_VIOL1, c->reg_seg, c->nreg, c->reg_tot,
-                c->partial + 5 * UPD_BLOCKS, c->partial, nupd, counters, stats,
-                reinterpret_cast<unsigned *>(cnt + CNT_BAR), reinterpret_cast<unsigned *>(cnt + CNT_BARGEN), c->status};
+    k_update<<<std::min(c->nseg, num_sms(c->device) * 8), UPD_THREADS, 0, s>>>(
+        c->m, alpha, Va, c->seg, c->nseg, c->sd, c->seg_mixed, c->bound ? c->viol[0] : nullptr, cnt + CNT_VIOL0,
+        c->status);
+    LAUNCH_CHECK();
+    if (!c->bound) {
+        k_stats<<<1, ST_THREADS, 0, s>>>(c->sd, c->nseg, counters, stats);
+        LAUNCH_CHECK();
+        return VOF_OK;
+    }
+    const BoundStep a{alpha, c->viol[0], cnt + CNT_VIOL0, c->rl, cnt + CNT_NRL0, c->ra, c->bscr, c->cmark, c->segmark,
+                      c->dl, cnt + CNT_NDL, reinterpret_cast<unsigned *>(cnt + CNT_EPOCH), cnt + CNT_BPASS,
+                      cnt + CNT_BACT0, cnt + CNT_LEFT0, cnt + CNT_VIOL1, c->seg, c->seg_at, c->nseg, c->seg_mixed, c->sd, c->reg_seg,
+                      c->nreg, c->reg_tot, counters, stats, reinterpret_cast<unsigned *>(cnt + CNT_BAR),
+                      reinterpret_cast<unsigned *>(cnt + CNT_BARGEN), c->status};
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(g_bound_blocks);
     cfg.blockDim = dim3(BA_THREADS);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, k_bound_step, c->m, a) != cudaSuccess) return VOF_ERR_CUDA;
-    return VOF_OK;
+    if (c->nc <= BOUND_CLUSTER_CELLS) {
+        cfg.gridDim = dim3(BA_CLUSTER);
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = BA_CLUSTER;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        return cudaLaunchKernelEx(&cfg, k_bound_step<true>, c->m, a) == cudaSuccess ? VOF_OK : VOF_ERR_CUDA;
+    }
+    cfg.gridDim = dim3(num_sms(c->device));
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    return cudaLaunchKernelEx(&cfg, k_bound_step<false>, c->m, a) == cudaSuccess ? VOF_OK : VOF_ERR_CUDA;
 }
 
 int launch_barrier_probe(vof_ctx *c, int skip, cudaStream_t s)
@@ -2110,23 +2139,10 @@ int launch_courant(vof_ctx *c, const double *F, double dt, double *co, cudaStrea
 
 int launch_update(vof_ctx *c, double *alpha, const double *Va, double *stats, cudaStream_t s)
 {
-    int *cnt = c->counters;
-    int launches = 0;
-    k_zero_update<<<1, 32, 0, s>>>(cnt);
-    const int nu = upd_blocks(c->device);
-    k_update<<<nu, UPD_THREADS, 0, s>>>(c->m, alpha, Va, c->partial, c->bound ? c->viol[0] : nullptr,
-                                        cnt + CNT_VIOL0, c->nc, c->status);
+    k_zero_update<<<1, 32, 0, s>>>(c->counters);
     LAUNCH_CHECK();
-    launches += 3;
-    if (c->bound) {
-        int r = launch_bound_step(c, alpha, nu, nullptr, stats ? stats : c->stats_dev, s);
-        if (r) return r;
-    } else {
-        k_stats<<<1, ST_THREADS, 0, s>>>(c->partial, nu, nullptr, stats ? stats : c->stats_dev, 0, nullptr, 0);
-        LAUNCH_CHECK();
-    }
-    c->launches = launches;
-    return VOF_OK;
+    c->launches = 3;
+    return launch_update_group(c, alpha, Va, nullptr, stats ? stats : c->stats_dev, s);
 }
 
 int launch_advect(vof_ctx *c, double *alpha, const double *Uc, const double *F, double dt, double *stats,
@@ -2140,11 +2156,10 @@ int launch_advect(vof_ctx *c, double *alpha, const double *Uc, const double *F, 
     if (c->prof_ev && c->prof_steps < c->prof_max) ev = c->prof_ev + (size_t)c->prof_steps++ * (VOF_PROF_GROUPS + 1);
 #define MARK(i) do { if (ev) cudaEventRecord(ev[i], s); } while (0)
     MARK(0);
-    k_zero_int<<<1, 32, 0, s>>>(cnt, CNT_LEN);
-    k_point_state<<<cdiv(m.np, 256), 256, 0, s>>>(m, alpha, c->pstate, c->palpha);
+    k_point_state<<<cdiv(m.np, 256), 256, 0, s>>>(m, alpha, c->pstate, c->palpha, cnt);
     k_classify<<<sms * 16, 256, 0, s>>>(m, alpha, F, dt, c->pstate, c->Va, c->band, cnt + CNT_BAND, c->icell,
                                         cnt + CNT_ICELL, c->bpflag, c->status);
-    launches += 3;
+    launches += 2;
     LAUNCH_CHECK();
     MARK(1);
     // The correction (band point velocities, then lambda per band face) needs
@@ -2176,23 +2191,15 @@ int launch_advect(vof_ctx *c, double *alpha, const double *Uc, const double *F, 
         int r = launch_pf_list(c, alpha, F, dt, sms, s);
         if (r) return r;
     }
-    launches += 4;  // reconstruct, band point velocities, correct, phase flux
+    launches += 6;  // reconstruct, band point velocities, correct, phase flux (pairs, clips, sums)
     LAUNCH_CHECK();
     MARK(4);
     // update + bounding + stats
-    k_zero_update<<<1, 32, 0, s>>>(cnt);
-    const int nu = upd_blocks(c->device);
-    k_update<<<nu, UPD_THREADS, 0, s>>>(m, alpha, c->Va, c->partial, c->bound ? c->viol[0] : nullptr,
-                                        cnt + CNT_VIOL0, c->nc, c->status);
-    launches += 3;
-    LAUNCH_CHECK();
-    if (c->bound) {
-        int r = launch_bound_step(c, alpha, nu, cnt, stats ? stats : c->stats_dev, s);
+    {
+        int r = launch_update_group(c, alpha, c->Va, cnt, stats ? stats : c->stats_dev, s);
         if (r) return r;
-    } else {
-        k_stats<<<1, ST_THREADS, 0, s>>>(c->partial, nu, cnt, stats ? stats : c->stats_dev, 0, nullptr, 0);
-        LAUNCH_CHECK();
     }
+    launches += 2;
     MARK(5);
 #undef MARK
     c->launches = launches;
