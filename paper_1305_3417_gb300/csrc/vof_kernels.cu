@@ -271,8 +271,8 @@ struct RcCell {
 //
 // MIXED: the offset is measured from the end of the cell's extent that is
 // nearer in volume (target t = a from below, or 1 - a from above), so that
-// cells near 0 and 1 keep their relative precision: safeguarded Newton steps on
-// the fill in FP32 until its residual is within 1e-5 t (ten times its
+// cells near 0 and 1 keep their relative precision: safeguarded Newton steps (on
+// logarithms) in FP32 until the fill's residual is within 1e-5 t (ten times its
 // rounding) and one more, then one FP64 evaluation with derivatives, on whose
 // cubic the offset is finished when the step stays short of the next vertex
 // projection (nearly always: the FP32 offset is good to about 1e-6); else
@@ -398,7 +398,10 @@ __device__ __forceinline__ RcCell rc_cell(const DevMesh &m, const double *__rest
             if (sure) {
                 if (gf < 0.0f) A = x; else B = x;
             }
-            float xn = x - __fdividef(gf, dpart);
+            // Newton on log f against log x: near an end the fill is a power of
+            // the distance (cube, square or first), where this lands at once
+            // and plain steps crawl
+            float xn = x * __expf(__fdividef(part * __logf(__fdividef(tf, part)), x * dpart));
             if (!(xn > A && xn < B)) xn = 0.5f * (A + B);
             if (!(xn > A && xn < B)) break;  // bracket at FP32 resolution
             x = xn;
@@ -520,14 +523,12 @@ struct RcCount {
 // The listed cells; with a counter a lane group takes its next cell as it
 // finishes one (cells differ in positioning iterations), else static striding.
 template <bool MIXED, int G, int KL, bool COUNT>
-__global__ void __launch_bounds__(RC_THREADS, rc_resident<KL>())
-k_reconstruct(DevMesh m, RcArgs q, const int *list, const int *count, int *maxit, const float *__restrict__ s0,
-              int s0cap, int *next)
+__device__ __forceinline__ void rc_list(const DevMesh &m, const RcArgs &q, const int *list, int total, int *maxit,
+                                        const float *__restrict__ s0, int s0cap, int *next)
 {
     const int lane = threadIdx.x & (G - 1);
     const unsigned tm = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (threadIdx.x & 31 & ~(G - 1));
     const int group = (blockIdx.x * blockDim.x + threadIdx.x) / G, ngroups = (gridDim.x * blockDim.x) / G;
-    const int total = *count;
     const double eps = m.eps;
     RcCount<G, COUNT> wk;
     auto take = [&]() {
@@ -555,6 +556,30 @@ k_reconstruct(DevMesh m, RcArgs q, const int *list, const int *count, int *maxit
     wk.flush(q.work);
 }
 
+// With no more cells than the launch has warps (in a step), narrow groups would leave most
+// warps without one while each cell's chain is as many instructions longer as
+// it has tetrahedra per lane: a warp takes a cell then (24^3, 252 cells: the
+// reconstruction's share of the step 57 -> 32 us, with the logarithmic steps).
+template <bool MIXED, int G, int KL, bool COUNT>
+__global__ void __launch_bounds__(RC_THREADS, rc_resident<KL>())
+k_reconstruct(DevMesh m, RcArgs q, const int *list, const int *count, int *maxit, const float *__restrict__ s0,
+              int s0cap, int *next)
+{
+    const int total = *count;
+    if constexpr (G < 32) {
+        if (next && total <= (int)(gridDim.x * blockDim.x) / 32) {
+            rc_list<MIXED, 32, (G * KL + 31) / 32, COUNT>(m, q, list, total, maxit, s0, s0cap, next);
+            return;
+        }
+    }
+    rc_list<MIXED, G, KL, COUNT>(m, q, list, total, maxit, s0, s0cap, next);
+}
+
+// cells per block of k_reconstruct_all: two per lane group, since interface cells come
+// in clumps and a block works its own off (mixed 90^3 film: 212 us with 16 a
+// group, 99 with 4, 82 with 2)
+template <int G> constexpr int rc_chunk() { return 2 * (RC_THREADS / G); }
+
 // Every cell of the mesh: a block writes the defaults (n = 0, d = 0, flags)
 // of a chunk of cells, lists the chunk's interface cells in shared memory and
 // hands them to its lane groups as they come free.  (One lane group per cell
@@ -563,7 +588,7 @@ k_reconstruct(DevMesh m, RcArgs q, const int *list, const int *count, int *maxit
 template <bool MIXED, int G, int KL, bool COUNT>
 __global__ void __launch_bounds__(RC_THREADS, rc_resident<KL>()) k_reconstruct_all(DevMesh m, RcArgs q)
 {
-    constexpr int CHUNK = 16 * (RC_THREADS / G);
+    constexpr int CHUNK = rc_chunk<G>();
     __shared__ int cells[CHUNK], ncells, taken;
     const int lane = threadIdx.x & (G - 1);
     const unsigned tm = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (threadIdx.x & 31 & ~(G - 1));
@@ -619,11 +644,12 @@ __device__ __forceinline__ void prism_cubic(V3 a0, V3 a1, V3 a2, V3 w0, V3 w1, V
     if (k1 < k0) { V3 t = a0; a0 = a1; a1 = t; t = w0; w0 = w1; w1 = t; long u = k0; k0 = k1; k1 = u; par = -par; }
     if (k2 < k1) { V3 t = a1; a1 = a2; a2 = t; t = w1; w1 = w2; w2 = t; long u = k1; k1 = k2; k2 = u; par = -par; }
     if (k1 < k0) { V3 t = a0; a0 = a1; a1 = t; t = w0; w0 = w1; w1 = t; long u = k0; k0 = k1; k1 = u; par = -par; }
-    V3 E1 = a1 - a0, E2 = a2 - a0;
+    // (with det(a,b,c) = a.(b x c): k2 = E1.(w2 x (w0+w1)) + E2.(w0 x w1), k3 = -w2.(w0 x w1))
+    const V3 E1 = a1 - a0, E2 = a2 - a0, w01 = w0 + w1, c01 = cross(w0, w1);
     const double f = par > 0 ? -1.0 / 6.0 : 1.0 / 6.0;
-    double t1 = -det3(E1, E2, w0 + w1 + w2) * f;
-    double t2 = (det3(E1, w2, w1) + det3(w0, w1, E2) + det3(w0, E1, w2)) * f;
-    double t3 = -det3(w0, w1, w2) * f;
+    const double t1 = -dot(cross(E1, E2), w01 + w2) * f;
+    const double t2 = (dot(E1, cross(w2, w01)) + dot(E2, c01)) * f;
+    const double t3 = -dot(w2, c01) * f;
     q.c1 += t1; q.c2 += t2; q.c3 += t3;
     q.s1 += fabs(t1); q.s2 += fabs(t2); q.s3 += fabs(t3);
 }
@@ -1952,7 +1978,7 @@ static void rc_go(vof_ctx *c, const RcArgs &q, const int *list, const int *count
         k_reconstruct<MIXED, G, KL, COUNT><<<num_sms(c->device) * rc_resident<KL>(), RC_THREADS, 0, s>>>(
             c->m, q, list, count, maxit, c->mlp_s0, mlp_cap(c), next);
     else
-        k_reconstruct_all<MIXED, G, KL, COUNT><<<cdiv(c->nc, 16 * (RC_THREADS / G)), RC_THREADS, 0, s>>>(c->m, q);
+        k_reconstruct_all<MIXED, G, KL, COUNT><<<cdiv(c->nc, rc_chunk<G>()), RC_THREADS, 0, s>>>(c->m, q);
 }
 
 template <bool MIXED, bool COUNT>
