@@ -474,6 +474,12 @@ int vof_create(const vof_mesh *mesh, const vof_options *opt, vof_ctx **out)
     int err = 0;
     DevMesh &m = c->m;
     m.np = np; m.nf = nf; m.ni = ni; m.nc = nc; m.eps = c->eps;
+    m.fuse = fptr[1] - fptr[0];
+    for (int f = 0; f < nf && m.fuse; ++f)
+        if (fptr[f + 1] - fptr[f] != m.fuse) m.fuse = 0;
+    m.cuse = cptr[1] - cptr[0];
+    for (int x = 0; x < nc && m.cuse; ++x)
+        if (cptr[x + 1] - cptr[x] != m.cuse) m.cuse = 0;
     m.px = dev_copy(c, mesh->px, np, &err);
     m.py = dev_copy(c, mesh->py, np, &err);
     m.pz = dev_copy(c, mesh->pz, np, &err);

@@ -14,6 +14,7 @@
 // pointers are device pointers owned by the context.
 struct DevMesh {
     int np, nf, ni, nc;
+    int fuse, cuse;              // points of every face, faces of every cell (0: not all the same)
     double eps;
     const double *px, *py, *pz;
     const int *fptr, *fpts, *own, *nei;

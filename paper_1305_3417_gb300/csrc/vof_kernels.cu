@@ -1062,7 +1062,8 @@ __global__ void __launch_bounds__(UPD_THREADS) k_update(DevMesh m, double *alpha
                 // A cell whose face fluxes are all zero (the bulk of either phase
                 // away from the band) has s = +0; the FP64 sum runs only where some
                 // flux is not zero, so warps of such cells issue no FP64 adds.
-                const int k0 = m.cptr[c], k1 = m.cptr[c + 1];
+                // (six faces everywhere: no offsets to read)
+                const int k0 = m.cuse == 6 ? 6 * c : m.cptr[c], k1 = m.cuse == 6 ? k0 + 6 : m.cptr[c + 1];
                 const double a0 = alpha[c];
                 unsigned nz = 0;
                 // (cflux: the cell's faces, a periodic copy read as its face seen
@@ -1655,18 +1656,34 @@ __global__ void k_classify(DevMesh m, const double *__restrict__ alpha, const do
         const int i = i0 + threadIdx.x;
         bool isband = false, isint = false;
         if (i < m.nf) {
-            double Ff = F[i];
-            double v = 0.0;
-            // (a periodic face's copy carries no flux)
-            if (!is_zero(Ff) && !(i >= m.ni && (dbits(Ff).hi < 0 || (m.fimg && m.fimg[i - m.ni] >= 0)))) {
-                unsigned st = 3u;
+            // the face's points: four at once on a mesh of quadrilaterals (16 of
+            // the 24 bytes a face that the mesh costs otherwise, and one load
+            // less in the chain); the flux only where some point has phase
+            // (128^3: 54 -> 35 us)
+            unsigned st = 3u;
+            int4 q = make_int4(0, 0, 0, 0);
+            int k0 = 0, k1 = 0;
+            if (m.fuse == 4) {
+                q = __ldg(reinterpret_cast<const int4 *>(m.fpts) + i);
+                st = state[q.x] & state[q.y] & state[q.z] & state[q.w];
+            } else {
+                k0 = m.fptr[i];
+                k1 = m.fptr[i + 1];
 #pragma unroll 4
-                for (int k = m.fptr[i]; k < m.fptr[i + 1]; ++k) st &= state[m.fpts[k]];
-                if (st & 1u) v = 0.0;
-                else if (st & 2u) v = Ff * dt;
-                else {
-                    isband = true;
-                    for (int k = m.fptr[i]; k < m.fptr[i + 1]; ++k) bpflag[m.fpts[k]] = 1;
+                for (int k = k0; k < k1; ++k) st &= state[m.fpts[k]];
+            }
+            double v = 0.0;
+            if (!(st & 1u)) {
+                const double Ff = F[i];
+                // (a periodic face's copy carries no flux)
+                if (!is_zero(Ff) && !(i >= m.ni && (dbits(Ff).hi < 0 || (m.fimg && m.fimg[i - m.ni] >= 0)))) {
+                    if (st & 2u) v = Ff * dt;
+                    else {
+                        isband = true;
+                        if (m.fuse == 4) bpflag[q.x] = bpflag[q.y] = bpflag[q.z] = bpflag[q.w] = 1;
+                        else
+                            for (int k = k0; k < k1; ++k) bpflag[m.fpts[k]] = 1;
+                    }
                 }
             }
             Va[i] = v;
