@@ -144,6 +144,12 @@ __device__ __forceinline__ float tf(double x)
     const int h = min(max((b.hi & 0x7fffffff) - 0x38000000, 0), 0x0fefffff);
     return __uint_as_float(__funnelshift_l(b.lo, (unsigned)h, 3) | ((unsigned)b.hi & 0x80000000u));
 }
+// a normal FP32 number as a double, on the integer pipe
+__device__ __forceinline__ double fd(float x)
+{
+    const unsigned b = __float_as_uint(x);
+    return __hiloint2double((int)(((b & 0x7fffffffu) >> 3) + 0x38000000u | (b & 0x80000000u)), (int)(b << 29));
+}
 // a is +0 or -0
 __device__ __forceinline__ bool is_zero(double a)
 {

@@ -52,14 +52,22 @@ __device__ __forceinline__ float rabs(float a) { return fabsf(a); }
 __device__ __forceinline__ float rfma(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double rfma(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float rmuladd(float a, float b, float c) { return __fadd_rn(__fmul_rn(a, b), c); }
-__device__ __forceinline__ double rmuladd(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float rnext(float a, float b) { return nextafterf(a, b); }
 __device__ __forceinline__ double rnext(double a, double b) { return nextafter(a, b); }
 __device__ __forceinline__ double rabs(double a) { return fabs(a); }
 // divisions of the clip: the fast FP32 reciprocal-multiply (2 ulp, far inside
-// the mixed form's rounding) or a correctly rounded FP64 division
+// the mixed form's rounding), or FP64 by the FP32 reciprocal of the truncated
+// divisor refined twice (error squared each time: to the last place or so),
+// four FP64 instructions; the full division where the divisor leaves the FP32 range
 __device__ __forceinline__ float rdiv(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double rdiv(double a, double b) { return a / b; }
+__device__ __noinline__ double full_div(double a, double b) { return a / b; }
+__device__ __forceinline__ double rdiv(double a, double b)
+{
+    const float f = tf(b), r0 = __fdividef(1.0f, f);
+    if (!(fabsf(f) > 1e-30f && fabsf(f) < 1e30f)) return full_div(a, b);
+    const double r1 = fd(r0), r2 = fma(r1, fma(-b, r1, 1.0), r1), q = a * r2;
+    return fma(r2, fma(-b, q, a), q);
+}
 
 template <class R> __device__ __forceinline__ R4<R> mk4(R x, R y, R z, R w);
 template <> __device__ __forceinline__ float4 mk4<float>(float x, float y, float z, float w) { return make_float4(x, y, z, w); }
@@ -98,6 +106,16 @@ __device__ __forceinline__ R rfrac_below(R h0, R h1, R h2, R h3)
     if (!rneg(h0)) return R(0);
     if (!rpos(h3)) return R(1);
     // one division per case
+    if constexpr (std::is_same<R, double>::value) {
+        // one vertex below or one above: the same cut seen from either end
+        const bool low = !rneg(h1);
+        if (low || !rpos(h2)) {
+            const R x = low ? -h0 : h3, d30 = h3 - h0;
+            const R e1 = low ? h1 - h0 : h3 - h1, e2 = low ? h2 - h0 : h3 - h2;
+            const R q = rdiv(x * x * x, d30 * e1 * e2);
+            return low ? q : R(1) - q;
+        }
+    }
     if (!rneg(h1)) {
         const R x = -h0;
         return rdiv(x * x * x, (h1 - h0) * (h2 - h0) * (h3 - h0));
@@ -233,8 +251,10 @@ __device__ __forceinline__ void stT(RTet<double> &t, const RTet<double> &v) { t 
 __device__ __forceinline__ float tof(float x) { return x; }
 __device__ __forceinline__ float tof(double x) { return tf(x); }
 
-template <class R>
-__device__ __forceinline__ R pdist(R4<R> p, R3<R> v) { return p.x * v.x + p.y * v.y + p.z * v.z - p.w; }
+// signed distance to plane p (FP64: three instructions, not four, of a pipe that
+// issues one in many cycles)
+__device__ __forceinline__ float pdist(float4 p, R3<float> v) { return p.x * v.x + p.y * v.y + p.z * v.z - p.w; }
+__device__ __forceinline__ double pdist(D4 p, R3<double> v) { return fma(p.x, v.x, fma(p.y, v.y, fma(p.z, v.z, -p.w))); }
 
 // signed distances of the vertices to plane p, those within tol taken as 0;
 // nin / nup count the vertices strictly below / above
@@ -245,7 +265,7 @@ __device__ __forceinline__ void fdist(const RTet<R> &t, R4<R> p, R tol, R s[4], 
     nup = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        R v = pdist<R>(p, t.v[i]);
+        R v = pdist(p, t.v[i]);
         if constexpr (std::is_same<R, double>::value) {  // integer tests
             const bool up = rabove(v, tol), dn = rbelow(v, tol);
             s[i] = (up || dn) ? v : R(0);
@@ -301,11 +321,14 @@ __device__ __forceinline__ void fsplit(const RTet<R> &t, const R s[4], int nin, 
     c[1] = sel(n3, P1, e0);
     c[2] = sel(n3, P2, e1);
     c[3] = sel(n3, e0, P1);
-    // (the fourth point's product is rounded before the sum in FP32: so it always
-    // was, its two cases' sums having been one after their branches)
-    const V dd = sel(n3, g1 - f1, g2 - f2);
-    const R tt = n3 ? sf1 * r2 : sf2 * r3;
-    c[4] = V{rmuladd(dd.x, tt, P1.x), rmuladd(dd.y, tt, P1.y), rmuladd(dd.z, tt, P1.z)};
+    if constexpr (std::is_same<R, double>::value) c[4] = sel(n3, e1, e2);
+    else {
+        // (this point's product is rounded before the sum: so it always was in
+        // the mixed form, its two cases' sums having been one after their branches)
+        const V dd = sel(n3, g1 - f1, g2 - f2);
+        const R tt = n3 ? sf1 * r2 : sf2 * r3;
+        c[4] = V{rmuladd(dd.x, tt, P1.x), rmuladd(dd.y, tt, P1.y), rmuladd(dd.z, tt, P1.z)};
+    }
     c[5] = sel(n2, e3, e2);
 }
 
@@ -416,8 +439,8 @@ __device__ __forceinline__ void mx_clip(Sh &sh, const unsigned short *Q, int nq,
                 const R4<R> pn = sh.Kp[k][__ffs(rem) - 1];
                 const float4 pf = make_float4(tof(pn.x), tof(pn.y), tof(pn.z), tof(pn.w));
                 auto below = [&](int i) {
-                    if constexpr (std::is_same<R, float>::value) return pdist<R>(pn, c[i]) < -tol;
-                    else return pdist<float>(pf, r3(tof(c[i].x), tof(c[i].y), tof(c[i].z))) < (float)tol * 1.2e9f;
+                    if constexpr (std::is_same<R, float>::value) return pdist(pn, c[i]) < -tol;
+                    else return pdist(pf, r3(tof(c[i].x), tof(c[i].y), tof(c[i].z))) < (float)tol * 1.2e9f;
                 };
                 const bool z0 = below(0), z1 = below(1), z2 = below(2), z5 = below(5);
                 ndrop = __popc(keep);
@@ -1063,7 +1086,7 @@ struct PfQueue {
 constexpr unsigned PF_NONE = 0xffffffffu;
 constexpr int PF_FAIL = -2;
 constexpr int PF_OVER = 2;        // parts per warp of the launch at most
-constexpr int PF_SPLIT = 3;       // a face in up to 2^3 parts
+constexpr int PF_SPLIT = 4;       // a face in up to 2^4 parts
 
 // log2 of the parts a face is dealt into: as many as leave no part waiting for
 // a warp (parts repeat the polyhedron's set-up and the stencil pass, 15 % of a
@@ -1622,7 +1645,7 @@ __device__ __forceinline__ void pf_sums(const MXArgs &a, const PfQueue &q)
 
 // warps per block of the pair launch, and blocks per SM
 template <class R> constexpr int pp_warps() { return sizeof(R) == 4 ? 4 : 2; }
-template <class R> constexpr int pp_resident() { return sizeof(R) == 4 ? 5 : 6; }
+template <class R> constexpr int pp_resident() { return sizeof(R) == 4 ? 4 : 6; }
 template <class R, class Wk>
 __global__ void __launch_bounds__(pp_warps<R>() * 32, pp_resident<R>()) k_pf_pairs(DevMesh m, MXArgs a, PfQueue q)
 {
