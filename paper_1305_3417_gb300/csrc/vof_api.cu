@@ -567,11 +567,11 @@ int vof_create(const vof_mesh *mesh, const vof_options *opt, vof_ctx **out)
     c->ktl = dev_alloc<unsigned char>(c, e4 * 6 * (size_t)ctptr[nc], &err);
     if (!err) {
         // The phase flux's queue: a band face has about 2.5 KB of clip jobs
-        // (twice that in FP64); 256 (512) bytes per mesh face hold a band of a
-        // tenth of the faces, and the floor any band of a small mesh.  Faces
+        // (twice that in FP64); 512 (1024) bytes per mesh face hold a band of a
+        // fifth of the faces, and the floor any band of a small mesh.  Faces
         // beyond it are fluxed in the slower one-warp form, so where memory is
         // short a smaller queue serves too.
-        const size_t unit = 16, per = c->precision == VOF_MIXED ? 256 : 512;
+        const size_t unit = 16, per = c->precision == VOF_MIXED ? 512 : 1024;
         size_t bytes = std::max(per * (size_t)nf, per * (size_t)(1 << 17));
         bytes = std::min(bytes, unit * ((size_t)1 << 31));
         void *p = nullptr;
