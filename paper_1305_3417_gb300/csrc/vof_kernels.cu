@@ -804,7 +804,7 @@ __global__ void k_flux_polyhedra(DevMesh m, const double *__restrict__ Up, const
 template <int N>
 __device__ __forceinline__ void correct_face(const DevMesh &m, int f, int b, int n, const double *__restrict__ U,
                                              const double *__restrict__ F, double dt, int item, double *lam_out,
-                                             int *it_out, double *disp_out, int *maxit, int *nfallback,
+                                             int *it_out, void *disp_out, bool disp32, int *maxit, int *nfallback,
                                              unsigned &ntri, unsigned &nev)
 {
     constexpr bool FIXED = N <= 4;
@@ -851,7 +851,6 @@ __device__ __forceinline__ void correct_face(const DevMesh &m, int f, int b, int
     if (maxit && its > 0) atomicMax(maxit, its);
     if (lam < 0.0 && nfallback) atomicAdd(nfallback, 1);
     if (disp_out) {
-        double *o = disp_out + (size_t)item * DISP_STRIDE;
         V3 wc = mk(0, 0, 0);
         if (lam < 0.0) {
             wc = S * (-lam * F[f] * dt / dot(S, S));
@@ -863,10 +862,21 @@ __device__ __forceinline__ void correct_face(const DevMesh &m, int f, int b, int
                 if (i < nn) { W[i] = W[i] * lam; wc = wc + W[i]; }
             wc = wc * inv_n(nn);
         }
-        o[0] = wc.x; o[1] = wc.y; o[2] = wc.z;
+        // (in the type of the phase flux: converted once here, not by each of
+        // its warps' lanes)
+        auto put = [&](int i, const V3 &w) {
+            if (disp32) {
+                float *o = static_cast<float *>(disp_out) + (size_t)item * DISP_STRIDE + i;
+                o[0] = (float)w.x; o[1] = (float)w.y; o[2] = (float)w.z;
+            } else {
+                double *o = static_cast<double *>(disp_out) + (size_t)item * DISP_STRIDE + i;
+                o[0] = w.x; o[1] = w.y; o[2] = w.z;
+            }
+        };
+        put(0, wc);
 #pragma unroll
         for (int i = 0; i < N; ++i)
-            if (i < nn) { o[3 + 3 * i] = W[i].x; o[4 + 3 * i] = W[i].y; o[5 + 3 * i] = W[i].z; }
+            if (i < nn) put(3 + 3 * i, W[i]);
     }
 }
 
@@ -874,7 +884,7 @@ __device__ __forceinline__ void correct_face(const DevMesh &m, int f, int b, int
 template <bool LIST>
 __global__ void k_correct(DevMesh m, const double *__restrict__ U, const double *__restrict__ F,
                           double dt, const int *list, const int *count, double *lam_out,
-                          int *it_out, double *disp_out, int *maxit, int *nfallback, unsigned long long *work,
+                          int *it_out, void *disp_out, bool disp32, int *maxit, int *nfallback, unsigned long long *work,
                           const double *__restrict__ alpha, BandRec *rec)
 {
     const int total = LIST ? *count : m.nf;
@@ -883,11 +893,11 @@ __global__ void k_correct(DevMesh m, const double *__restrict__ U, const double 
         const int f = LIST ? list[item] : item;
         const int b = __ldg(m.fptr + f), n = __ldg(m.fptr + f + 1) - b;
         if (n == 4)
-            correct_face<4>(m, f, b, n, U, F, dt, item, lam_out, it_out, disp_out, maxit, nfallback, ntri, nev);
+            correct_face<4>(m, f, b, n, U, F, dt, item, lam_out, it_out, disp_out, disp32, maxit, nfallback, ntri, nev);
         else if (n == 3)
-            correct_face<3>(m, f, b, n, U, F, dt, item, lam_out, it_out, disp_out, maxit, nfallback, ntri, nev);
+            correct_face<3>(m, f, b, n, U, F, dt, item, lam_out, it_out, disp_out, disp32, maxit, nfallback, ntri, nev);
         else
-            correct_face<VOF_MAXFP>(m, f, b, n, U, F, dt, item, lam_out, it_out, disp_out, maxit, nfallback, ntri,
+            correct_face<VOF_MAXFP>(m, f, b, n, U, F, dt, item, lam_out, it_out, disp_out, disp32, maxit, nfallback, ntri,
                                     nev);
         if (LIST) {
             const long long s0 = __ldg(m.sptr + f);
@@ -2081,7 +2091,7 @@ int launch_correct_all(vof_ctx *c, const double *Up, const double *F, double dt,
                        cudaStream_t s)
 {
     k_correct<false><<<cdiv(c->nf, 128), 128, 0, s>>>(c->m, Up, F, dt, nullptr, nullptr, lambda, iters,
-                                                             nullptr, nullptr, nullptr, c->work_on ? c->work : nullptr,
+                                                             nullptr, false, nullptr, nullptr, c->work_on ? c->work : nullptr,
                                                              nullptr, nullptr);
     LAUNCH_CHECK();
     return VOF_OK;
@@ -2216,7 +2226,7 @@ int launch_advect(vof_ctx *c, double *alpha, const double *Uc, const double *F, 
         return VOF_ERR_CUDA;
     k_band_point_velocity<<<cdiv(m.np, 256), 256, 0, c->s_aux>>>(m, Uc, c->bpflag, c->upb);
     k_correct<true><<<sms * 8, 128, 0, c->s_aux>>>(m, c->upb, F, dt, c->band, cnt + CNT_BAND, c->lam_b, c->it_b,
-                                                   c->disp_b, cnt + CNT_MAXCORR, cnt + CNT_FALLBACK,
+                                                   c->disp_b, c->precision == VOF_MIXED, cnt + CNT_MAXCORR, cnt + CNT_FALLBACK,
                                                    c->work_on ? c->work : nullptr, alpha, c->pf_rec);
     LAUNCH_CHECK();
     if (cudaEventRecord(c->ev_join, c->s_aux) != cudaSuccess) return VOF_ERR_CUDA;

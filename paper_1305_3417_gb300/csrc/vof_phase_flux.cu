@@ -169,7 +169,8 @@ struct MXArgs {
     double dt;
     double *Va;
     const int *list, *count;
-    const double *disp, *lam_b;
+    const void *disp;         // list form: displacements of a face's centre and points, in the form's type
+    const double *lam_b;
     unsigned *status;
     unsigned long long *work;
     const void *fpl, *cbl, *ktl;  // the context's tables (R4 of the form's type)
@@ -199,9 +200,9 @@ struct __align__(16) PolyShared {
 template <class R>
 struct __align__(16) CellShared {
     R4<R> CH[32];            // phase (or void) half-space
-    R Cdc[32][3];            // cell centre - face centre
+    R4<R> Cd[32];            // cell centre - face centre; w (as bits): first tetrahedron less the
+                             // chunk's tetrahedra before it
     R Cw[32];
-    int Ct0[32];             // first tetrahedron
     int Cend[32];            // running count of tetrahedra, inclusive
     unsigned char CuseH[32];
 };
@@ -247,6 +248,15 @@ __device__ __forceinline__ void stT(RTet<float> &t, const RTet<float> &v)
     p[2] = make_float4(v.v[2].z, v.v[3].x, v.v[3].y, v.v[3].z);
 }
 __device__ __forceinline__ void stT(RTet<double> &t, const RTet<double> &v) { t = v; }
+
+// an int kept in the unused component of a vector
+template <class R> __device__ __forceinline__ R int_bits(int i)
+{
+    if constexpr (std::is_same<R, float>::value) return __int_as_float(i);
+    else return __hiloint2double(0x3ff00000, i);
+}
+__device__ __forceinline__ int bits_int(float x) { return __float_as_int(x); }
+__device__ __forceinline__ int bits_int(double x) { return __double2loint(x); }
 
 __device__ __forceinline__ float tof(float x) { return x; }
 __device__ __forceinline__ float tof(double x) { return tf(x); }
@@ -687,8 +697,8 @@ __device__ __forceinline__ void mx_poly(const DevMesh &m, const MXArgs &a, Sh &s
         auto disp = [&](int i) -> V {  // i < 0: face centre
             V3 w;
             if (LIST) {
-                const double *q = a.disp + (size_t)item * DISP_STRIDE + (i < 0 ? 0 : 3 + 3 * i);
-                w = mk(q[0], q[1], q[2]);
+                const R *q = static_cast<const R *>(a.disp) + (size_t)item * DISP_STRIDE + (i < 0 ? 0 : 3 + 3 * i);
+                return r3(q[0], q[1], q[2]);
             } else {
                 double lam = a.lambda[f];
                 if (lam < 0.0) {
@@ -868,10 +878,9 @@ __device__ __forceinline__ void mx_chunk(const DevMesh &m, const MXArgs &a, Sh &
     if (pass) {
         const int r = __popc(pm & ((1u << lane) - 1u));
         sh.CH[r] = H;
-        sh.Cdc[r][0] = dc.x; sh.Cdc[r][1] = dc.y; sh.Cdc[r][2] = dc.z;
+        sh.Cd[r] = mk4<R>(dc.x, dc.y, dc.z, int_bits<R>(t0 - (inc - nkt)));
         sh.Cw[r] = wgt;
         sh.CuseH[r] = useH;
-        sh.Ct0[r] = t0;
         sh.Cend[r] = inc;
     }
     ntot = __shfl_sync(0xffffffffu, inc, 31);
@@ -990,15 +999,13 @@ __device__ __forceinline__ void phase_flux_body(const DevMesh &m, const MXArgs &
             if (!fin && tb + lane < ntot) {
                 // this lane's tetrahedron: planes and box move from the cell frame
                 // to the face frame by the shift dc
-                const int g = tb + lane;
-                const int j = sh.Ct0[ci] + g - (ci ? sh.Cend[ci - 1] : 0);
-                const V dc = r3(sh.Cdc[ci][0], sh.Cdc[ci][1], sh.Cdc[ci][2]);
-                const R4<R> *q = ktl + 6 * (size_t)j;
+                const R4<R> dc = sh.Cd[ci];
+                const size_t j = bits_int(dc.w) + tb + lane;
                 // box and planes in one round trip to L2 (the planes of the
                 // tetrahedra the box test drops are read for nothing)
-                const R4<R> b0 = ldg4(q, 4), b1 = ldg4(q, 5);
+                const R4<R> b0 = ldg4(ktl, 6 * j + 4), b1 = ldg4(ktl, 6 * j + 5);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) kp[i] = ldg4(q, i);
+                for (int i = 0; i < 4; ++i) kp[i] = ldg4(ktl, 6 * j + i);
                 kbx[0] = b0.x + dc.x; kbx[1] = b0.y + dc.y; kbx[2] = b0.z + dc.z;
                 kbx[3] = b1.x + dc.x; kbx[4] = b1.y + dc.y; kbx[5] = b1.z + dc.z;
                 cand = !(rgt(pb[0], kbx[3]) || rgt(kbx[0], pb[3]) || rgt(pb[1], kbx[4]) || rgt(kbx[1], pb[4]) ||
@@ -1115,6 +1122,7 @@ struct PfLayout {
 };
 
 constexpr int PF_RING = 64;       // cell tetrahedra between the box test and their planes
+constexpr int PO_LANE = 8;        // open (plane, point) of a pair decided at a time
 constexpr int PF_FLUSH = 24;      // candidates from which the pairs are taken (at most MX_CAND)
 template <class R>
 struct __align__(16) PairShared : PolyShared<R>, CellShared<R>, CandShared<R> {
@@ -1130,12 +1138,12 @@ struct __align__(16) PairShared : PolyShared<R>, CellShared<R>, CandShared<R> {
 // in FP64 only the planes that are not (the FP64 pipe issues one warp
 // instruction in about 64 cycles on its sub-partition): boxes, prism points and
 // shifted planes are held in FP32 as well, with each candidate's rounding
-// allowance; the FP64 planes stay in the cell's frame and are shifted where
-// they are used.  Every decision is the one FP64 throughout takes.
+// allowance; the FP64 planes stay in the cell's frame until then.  Every
+// decision is the one FP64 throughout takes.
 template <>
 struct __align__(16) PairShared<double> : PolyShared<double, float>, CellShared<double> {
     float4 P6f[VOF_MAXFP][5];
-    D4 Kp[MX_CAND][5];            // planes in the cell frame, then the half-space in the face frame
+    D4 Kp[MX_CAND][5];            // planes (in the cell frame until the pairs are taken) and the half-space
     double Kdc[MX_CAND][3];       // cell centre - face centre
     double Kw[MX_CAND];
     float4 Kf[MX_CAND][5];        // planes and half-space in the face frame, FP32
@@ -1145,7 +1153,8 @@ struct __align__(16) PairShared<double> : PolyShared<double, float>, CellShared<
     double o[3];
     int Cj[PF_RING];
     unsigned short Q[MX_QUEUE], PQ[VOF_MAXFP * MX_CAND];
-    unsigned char QA[MX_QUEUE];   // planes to decide in FP64
+    unsigned short O[32 * PO_LANE];  // open (plane, point) of the pairs at hand: 6 plane + point | pair << 5
+    unsigned Oin[32], Oout[32];   // (plane, point) bits of the pairs at hand
     unsigned char Cc[PF_RING];
     unsigned char KuseH[MX_CAND], Kmap[MX_CAND];
 };
@@ -1187,16 +1196,35 @@ __device__ __forceinline__ int pf_pairs64(PairShared<double> &sh, int nt, int nc
         }
     }
     __syncwarp();
-    // FP32 distances of a pair's six prism points to the planes: what is clearly
-    // outside ends here; the rest is listed with its clear cuts and the planes
-    // that need FP64 (a point within the allowance where it matters)
-    int ns = 0;
+    // The planes into the face frame, in FP64 (12 instructions of its pipe).
+    if (lane < ncand) {
+        const double *dc = sh.Kdc[lane];
+        wk.add(WK_SHIFT, 4);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            D4 &pl = sh.Kp[lane][q];
+            pl.w = pl.w + (pl.x * dc[0] + pl.y * dc[1] + pl.z * dc[2]);
+        }
+    }
+    __syncwarp();
+    // A pair a lane: FP32 distances of the prism's six points to the planes give
+    // for each (plane, point) clearly inside (bit 6 q + i of in), clearly outside
+    // (out) or open; of the open ones those that can change what becomes of one
+    // of the prism's tetrahedra are listed, dense over the warp, and decided in
+    // FP64, a (plane, point) a lane.  (A tetrahedron's open planes decided by
+    // its own lane, four points at a time, took ten times the FP64 instructions:
+    // the planes shared by a face's cells and polyhedron are open everywhere,
+    // most others nowhere; pairs of 64^3 hexahedra 402 -> 370 us, and 317
+    // with the loops over the planes rolled: the launch waited for instructions.)
+    constexpr unsigned M[3] = {0x27u, 0x33u, 0x39u};  // T0 = a0 a1 a2 b2, T1 = a0 a1 b2 b1, T2 = a0 b0 b1 b2
+    int nq = 0;
+    used = 0u;
     for (int pb = 0; pb < total; pb += 32) {
         const int pi = pb + lane;
-        unsigned code[3] = {0u, 0u, 0u}, amb[3] = {0u, 0u, 0u};
-        bool live[3] = {false, false, false};
+        unsigned in = 0u, out = 0u, open = 0u, live = 0u, pc = 0u;
+        int npl = 0;
         if (pi < total) {
-            const unsigned pc = sh.PQ[pi];
+            pc = sh.PQ[pi];
             const int pr = pc & 7, k = pc >> 3;
             float v[20];
 #pragma unroll
@@ -1204,97 +1232,107 @@ __device__ __forceinline__ int pf_pairs64(PairShared<double> &sh, int nt, int nc
                 const float4 x = sh.P6f[pr][i];
                 v[4 * i] = x.x; v[4 * i + 1] = x.y; v[4 * i + 2] = x.z; v[4 * i + 3] = x.w;
             }
-            const int npl = sh.KuseH[k] ? 5 : 4;
+            npl = sh.KuseH[k] ? 5 : 4;
             const float mg = sh.Km[k];
-            unsigned mask[3] = {0u, 0u, 0u};
-            bool outside[3] = {false, false, false};
+#pragma unroll
+            for (int j = 0; j < 3; ++j) live |= (unsigned)(sh.Tsg[3 * pr + j] != 0.0) << j;
+#pragma unroll 1
+            for (int q = 0; q < npl; ++q) {
+                const float4 pl = sh.Kf[k][q];
+                unsigned lo = 0u, hi = 0u;
+#pragma unroll
+                for (int i = 0; i < 6; ++i) {
+                    const float d = fmaf(pl.x, v[3 * i], fmaf(pl.y, v[3 * i + 1], fmaf(pl.z, v[3 * i + 2], -pl.w)));
+                    lo |= (unsigned)(d < -mg) << i;
+                    hi |= (unsigned)(d > mg) << i;
+                }
+                in |= lo << 6 * q;
+                out |= hi << 6 * q;
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+                    if ((hi & M[j]) == M[j]) live &= ~(1u << j);
+            }
+#pragma unroll 1
+            for (int q = 0; q < npl; ++q) {
+                const unsigned lo = in >> 6 * q & 63u, hi = out >> 6 * q & 63u;
+                unsigned need = 0u;
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+                    if ((live >> j & 1u) && (!(lo & M[j]) || !(hi & M[j]))) need |= M[j];
+                open |= (need & ~(lo | hi)) << 6 * q;
+            }
+        }
+        while (__any_sync(0xffffffffu, open != 0u)) {
+            // up to PO_LANE of each lane's
+            const int c = min(__popc(open), PO_LANE);
+            int at = c;
+#pragma unroll
+            for (int o2 = 1; o2 < 32; o2 <<= 1) {
+                const int w = __shfl_up_sync(0xffffffffu, at, o2);
+                if (lane >= o2) at += w;
+            }
+            const int n = __shfl_sync(0xffffffffu, at, 31);
+            at -= c;
+            for (int i = 0; i < c; ++i) {
+                sh.O[at + i] = (unsigned short)((__ffs(open) - 1) | lane << 5);
+                open &= open - 1;
+            }
+            sh.Oin[lane] = in;
+            sh.Oout[lane] = out;
+            __syncwarp();
+            for (int i = lane; i < n; i += 32) {
+                const unsigned w = sh.O[i], bit = w & 31, l = w >> 5, pk = sh.PQ[pb + l], q = bit / 6, x = bit % 6;
+                const D4 pl = sh.Kp[pk >> 3][q];
+                const double *p = reinterpret_cast<const double *>(sh.P6[pk & 7]) + 3 * x;
+                wk.add(WK_TEST, !(i & 3));  // (four distances make a test)
+                const double d = fma(pl.x, p[0], fma(pl.y, p[1], fma(pl.z, p[2], -pl.w)));
+                if (rbelow(d, tol)) atomicOr(&sh.Oin[l], 1u << bit);
+                if (rabove(d, tol)) atomicOr(&sh.Oout[l], 1u << bit);
+            }
+            __syncwarp();
+            in = sh.Oin[lane];
+            out = sh.Oout[lane];
+        }
+        // outside (no point inside some plane), inside every plane (summed) or a
+        // clip job
+        const int pr = pc & 7, k = pc >> 3;
+#pragma unroll 1
+        for (int j = 0; j < 3; ++j) {
+            const unsigned mj = 0x393327u >> 8 * j & 63u;
+            unsigned mask = 0u;
+            bool outside = !(live >> j & 1u);
 #pragma unroll
             for (int q = 0; q < 5; ++q) {
-                const float4 pl = sh.Kf[k][q];
-                float d[6];
-#pragma unroll
-                for (int i = 0; i < 6; ++i)
-                    d[i] = fmaf(pl.x, v[3 * i], fmaf(pl.y, v[3 * i + 1], fmaf(pl.z, v[3 * i + 2], -pl.w)));
-                const float l01 = fminf(d[0], d[1]), h01 = fmaxf(d[0], d[1]);
-                const float lo[3] = {fminf(l01, fminf(d[2], d[5])), fminf(l01, fminf(d[5], d[4])),
-                                     fminf(fminf(d[0], d[3]), fminf(d[4], d[5]))};
-                const float hi[3] = {fmaxf(h01, fmaxf(d[2], d[5])), fmaxf(h01, fmaxf(d[5], d[4])),
-                                     fmaxf(fmaxf(d[0], d[3]), fmaxf(d[4], d[5]))};
                 if (q < npl) {
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) {
-                        outside[j] |= lo[j] > mg;
-                        if (hi[j] > mg) mask[j] |= 1u << q;
-                        if (fabsf(hi[j]) <= mg || fabsf(lo[j]) <= mg) amb[j] |= 1u << q;
-                    }
+                    if (!(in >> 6 * q & mj)) outside = true;
+                    if (out >> 6 * q & mj) mask |= 1u << q;
                 }
             }
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                const int t = 3 * pr + j;
-                live[j] = sh.Tsg[t] != 0.0 && !outside[j];
-                code[j] = (unsigned)t | ((unsigned)k << 5) | (mask[j] << 10);
-            }
+            const int t = 3 * pr + j;
+            if (!outside && mask == 0u) acc_add(acc, sh.Tsg[t] * sh.Kw[k] * sh.Tv6[t]);
+            const bool job = !outside && mask != 0u;
+            const unsigned bm = __ballot_sync(0xffffffffu, job);
+            if (job) sh.Q[nq + __popc(bm & lt)] = (unsigned short)((unsigned)t | (unsigned)k << 5 | mask << 10);
+            nq += __popc(bm);
+            used |= __reduce_or_sync(0xffffffffu, job ? 1u << k : 0u);
         }
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const unsigned bm = __ballot_sync(0xffffffffu, live[j]);
-            if (live[j]) {
-                const int at = ns + __popc(bm & lt);
-                sh.Q[at] = (unsigned short)code[j];
-                sh.QA[at] = (unsigned char)amb[j];
-            }
-            ns += __popc(bm);
-        }
-    }
-    __syncwarp();
-    // the listed (T, K), one per lane: the open planes in FP64, then outside,
-    // inside (summed) or a clip job (the list is compacted in place)
-    int nq = 0;
-    used = 0u;
-    for (int sb = 0; sb < ns; sb += 32) {
-        const bool act = sb + lane < ns;
-        unsigned meta = 0, amb = 0;
-        if (act) {
-            meta = sh.Q[sb + lane];
-            amb = sh.QA[sb + lane];
-        }
-        const int t = meta & 31, k = meta >> 5 & 31, j = t % 3;
-        unsigned mask = meta >> 10;
-        const double *p = reinterpret_cast<const double *>(sh.P6[t / 3]);
-        const int at[4] = {0, j == 2 ? 9 : 3, j == 0 ? 6 : j == 1 ? 15 : 12, j == 1 ? 12 : 15};
-        bool out = !act;
-        while (__any_sync(0xffffffffu, amb != 0u && !out)) {
-            if (amb != 0u && !out) {
-                const int q = __ffs(amb) - 1;
-                amb &= amb - 1;
-                D4 pl = sh.Kp[k][q];
-                if (q < 4) {
-                    const double *dc = sh.Kdc[k];
-                    pl.w = pl.w + (pl.x * dc[0] + pl.y * dc[1] + pl.z * dc[2]);
-                }
-                wk.add(WK_TEST, 1);
-                bool below = false, above = false;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const double *x = p + at[i];
-                    const double d = fma(pl.x, x[0], fma(pl.y, x[1], fma(pl.z, x[2], -pl.w)));
-                    below |= rbelow(d, tol);
-                    above |= rabove(d, tol);
-                }
-                if (!below) out = true;
-                mask = above ? mask | 1u << q : mask & ~(1u << q);
-            }
-        }
-        if (!out && mask == 0u) acc_add(acc, sh.Tsg[t] * sh.Kw[k] * sh.Tv6[t]);
-        const bool job = !out && mask != 0u;
-        const unsigned bm = __ballot_sync(0xffffffffu, job);
-        if (job) sh.Q[nq + __popc(bm & lt)] = (unsigned short)((meta & 0x3ffu) | mask << 10);
-        nq += __popc(bm);
-        used |= __reduce_or_sync(0xffffffffu, job ? 1u << k : 0u);
-        __syncwarp();
     }
     return nq;
+}
+
+// a sum and its compensation in 8 bytes: in FP32 side by side, added in FP64
+// where they are read (a thread per face there, one lane of 32 here)
+__device__ __forceinline__ void put_sum(double *a, int i, const Acc<float> &v)
+{
+    reinterpret_cast<float2 *>(a)[i] = make_float2(v.s, v.c);
+}
+__device__ __forceinline__ void put_sum(double *a, int i, const Acc<double> &v) { a[i] = v.s + v.c; }
+template <class R> __device__ __forceinline__ double get_sum(const double *a, int i)
+{
+    if constexpr (std::is_same<R, float>::value) {
+        const float2 v = reinterpret_cast<const float2 *>(a)[i];
+        return (double)v.x + (double)v.y;
+    } else return a[i];
 }
 
 template <class R, class Wk>
@@ -1379,14 +1417,14 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
                 if (lane < nr) {
                     const int e = (base + lane) & (PF_RING - 1);
                     ci = sh.Cc[e];
-                    const R4<R> *kt = ktl + 6 * (size_t)sh.Cj[e];
-                    const V dc = r3(sh.Cdc[ci][0], sh.Cdc[ci][1], sh.Cdc[ci][2]);
+                    const size_t j = sh.Cj[e];
+                    const R4<R> dc = sh.Cd[ci];
                     const R3<float> df = r3(tof(dc.x), tof(dc.y), tof(dc.z));
                     H = sh.CH[ci];
                     const bool useH = sh.CuseH[ci];
-                    const R4<R> b0 = ldg4(kt, 4), b1 = ldg4(kt, 5);
+                    const R4<R> b0 = ldg4(ktl, 6 * j + 4), b1 = ldg4(ktl, 6 * j + 5);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) kp[i] = ldg4(kt, i);
+                    for (int i = 0; i < 4; ++i) kp[i] = ldg4(ktl, 6 * j + i);
                     kbx[0] = tof(b0.x) + df.x; kbx[1] = tof(b0.y) + df.y; kbx[2] = tof(b0.z) + df.z;
                     kbx[3] = tof(b1.x) + df.x; kbx[4] = tof(b1.y) + df.y; kbx[5] = tof(b1.z) + df.z;
                     const float4 pce = sh.X[2], phe = sh.X[3];
@@ -1427,7 +1465,8 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
                         for (int i = 0; i < 4; ++i) sh.Kf[r][i] = kf[i];
                         sh.Kf[r][4] = hf4;
                         sh.Km[r] = mg;
-                        sh.Kdc[r][0] = sh.Cdc[ci][0]; sh.Kdc[r][1] = sh.Cdc[ci][1]; sh.Kdc[r][2] = sh.Cdc[ci][2];
+                        const D4 dc = sh.Cd[ci];
+                        sh.Kdc[r][0] = dc.x; sh.Kdc[r][1] = dc.y; sh.Kdc[r][2] = dc.z;
                     }
                     sh.Kw[r] = sh.Cw[ci];
                     sh.KuseH[r] = sh.CuseH[ci];
@@ -1438,8 +1477,7 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
                 __syncwarp();
                 if (nk < PF_FLUSH) continue;
             } else if (!cdone) {
-                // ---- boxes of the chunk's next 32 tetrahedra
-                if ((bt++ & msk) != part) { tb += 32; continue; }
+                // ---- boxes of the part's next batch of 32 tetrahedra
                 // the cell of tetrahedron tb + lane: the cells that end at or
                 // before tb, plus one for each cell that ends inside the batch at
                 // or before this lane (cell 'lane' ends rel tetrahedra after tb)
@@ -1449,10 +1487,9 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
                 bool cand = false;
                 int j = 0;
                 if (tb + lane < ntot) {
-                    j = sh.Ct0[ci] + tb + lane - (ci ? sh.Cend[ci - 1] : 0);
-                    const V dc = r3(sh.Cdc[ci][0], sh.Cdc[ci][1], sh.Cdc[ci][2]);
-                    const R4<R> *kt = ktl + 6 * (size_t)j;
-                    const R4<R> b0 = ldg4(kt, 4), b1 = ldg4(kt, 5);
+                    const R4<R> dc = sh.Cd[ci];
+                    j = bits_int(dc.w) + tb + lane;
+                    const R4<R> b0 = ldg4(ktl, 6 * (size_t)j + 4), b1 = ldg4(ktl, 6 * (size_t)j + 5);
                     const float4 lo = sh.X[0], hi = sh.X[1];
                     if constexpr (F64) {
                         auto apart = [](float l, float h, double c0, double c1, double s) {
@@ -1473,13 +1510,15 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
                     sh.Cc[e] = (unsigned char)ci;
                 }
                 cnt += __popc(cmask);
-                tb += 32;
+                tb += 32 << ls;
                 __syncwarp();
                 continue;
             } else {
                 // ---- next chunk
                 sc += 32;
-                tb = ntot = 0;
+                bt += (ntot + 31) >> 5;
+                tb = ((part - bt) & msk) << 5;
+                ntot = 0;
                 if (sc < s1) {
                     const float4 lo = sh.X[0], hi = sh.X[1];
                     const B pb[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
@@ -1527,24 +1566,18 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
                     if (bi >= 0) {
                         uint4 *ob = q.arena + off;
                         if (lane == 0) {
-                            const DBits t = dbits((double)tol);
                             ob[0] = make_uint4((unsigned)nq | (unsigned)nu << 16 | (unsigned)nprism << 24, pos, neg, 0u);
-                            ob[1] = make_uint4(t.lo, (unsigned)t.hi, 0u, 0u);
+                            if constexpr (F64) {
+                                const DBits t = dbits(tol);
+                                ob[1] = make_uint4(t.lo, (unsigned)t.hi, 0u, 0u);
+                            } else ob[1] = make_uint4(__float_as_uint(tol), 0u, 0u, 0u);
                         }
                         const uint4 *ps = reinterpret_cast<const uint4 *>(sh.P6);
                         for (unsigned i = lane; i < nprism * 5 * L.RW; i += 32) ob[L.P + i] = ps[i];
                         R4<R> *ok = reinterpret_cast<R4<R> *>(ob + L.K);
                         for (int i = lane; i < nu * 5; i += 32) {
                             const int k = sh.Kmap[i / 5], c = i % 5;
-                            R4<R> pl = sh.Kp[k][c];
-                            if constexpr (F64) {
-                                if (c < 4) {
-                                    const double *dc = sh.Kdc[k];
-                                    wk.add(WK_SHIFT, 1);
-                                    pl.w = pl.w + (pl.x * dc[0] + pl.y * dc[1] + pl.z * dc[2]);
-                                }
-                            }
-                            ok[i] = pl;
+                            ok[i] = sh.Kp[k][c];
                         }
                         if (lane < nu) reinterpret_cast<R *>(ob + L.W)[lane] = sh.Kw[sh.Kmap[lane]];
                         auto code = [&](int i) -> unsigned {  // candidates renumbered among those used
@@ -1563,7 +1596,7 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
         }
         mx_merge(acc);
         if (lane == 0) {
-            q.base[unit] = (double)acc.s + (double)acc.c;
+            put_sum(q.base, unit, acc);
             q.head[unit] = make_int2(head, comp);
             if (head == PF_FAIL) q.ovf[atomicAdd(q.novf, 1)] = item;
         }
@@ -1600,7 +1633,9 @@ __device__ __forceinline__ void pf_clip_body(const MXArgs &a, const PfQueue &q, 
         const uint4 h0 = ob[0], h1 = ob[1];
         const int nq = h0.x & 0xffff, nu = h0.x >> 16 & 0xff, nprism = h0.x >> 24;
         const PfLayout<R> L(nprism, nu, nq);
-        const R tol = (R)__hiloint2double((int)h1.y, (int)h1.x);
+        R tol;
+        if constexpr (std::is_same<R, double>::value) tol = __hiloint2double((int)h1.y, (int)h1.x);
+        else tol = __uint_as_float(h1.x);
         uint4 *kd = reinterpret_cast<uint4 *>(sh.Kp);
         for (unsigned i = lane; i < nu * 5 * L.RW; i += 32) kd[i] = ob[L.K + i];
         if (lane < nu) sh.Kw[lane] = reinterpret_cast<const R *>(ob + L.W)[lane];
@@ -1616,13 +1651,14 @@ __device__ __forceinline__ void pf_clip_body(const MXArgs &a, const PfQueue &q, 
         Acc<R> acc;
         mx_clip(sh, reinterpret_cast<const unsigned short *>(ob + L.Q), nq, tol, acc, wk);
         mx_merge(acc);
-        if (lane == 0) q.part[bi] = (double)acc.s + (double)acc.c;
+        if (lane == 0) put_sum(q.part, bi, acc);
         __syncwarp();
     }
     wk.flush(a.work, lane);
 }
 
 // V_alpha of the band faces from their parts, in a fixed order
+template <class R>
 __device__ __forceinline__ void pf_sums(const MXArgs &a, const PfQueue &q)
 {
     const int total = *a.count, ls = pf_split(total, q.pair_warps);
@@ -1633,8 +1669,8 @@ __device__ __forceinline__ void pf_sums(const MXArgs &a, const PfQueue &q)
             const int2 h = q.head[u];
             comp = h.y != 0;
             fail |= h.x == PF_FAIL;
-            v += q.base[u];
-            for (int bi = h.x; bi >= 0; bi = q.bnext[bi]) v += q.part[bi];
+            v += get_sum<R>(q.base, u);
+            for (int bi = h.x; bi >= 0; bi = q.bnext[bi]) v += get_sum<R>(q.part, bi);
         }
         if (fail) continue;
         const int f = a.list[item];
@@ -1643,7 +1679,10 @@ __device__ __forceinline__ void pf_sums(const MXArgs &a, const PfQueue &q)
     }
 }
 
-// warps per block of the pair launch, and blocks per SM
+// warps per block of the pair launch, and blocks per SM: FP32 3 / 4 / 5 / 6
+// blocks take 434 / 364 / 380 / 410 us at 128^3 hexahedra (fewer leave the issue
+// slots idle, more leave the L1 less room and spill); FP64 is held by its shared
+// memory
 template <class R> constexpr int pp_warps() { return sizeof(R) == 4 ? 4 : 2; }
 template <class R> constexpr int pp_resident() { return sizeof(R) == 4 ? 4 : 6; }
 template <class R, class Wk>
@@ -1672,7 +1711,7 @@ __global__ void __launch_bounds__(64, sizeof(R) == 4 ? 8 : 4) k_pf_finish(DevMes
     {
         MXArgs s = a;
         s.count = count;
-        pf_sums(s, q);
+        pf_sums<R>(s, q);
     }
     if (*a.count > 0)
         phase_flux_body<R, MX_STACK_WIDE, true, Wk>(
@@ -1793,7 +1832,7 @@ size_t phase_flux_table_entry_bytes(int precision)
 
 static MXArgs mx_args(vof_ctx *c, const double *alpha, const double *n, const double *d, const uint8_t *flags,
                       const double *Up, const double *F, const double *lambda, double dt, double *Va,
-                      const int *list, const int *count, const double *disp, unsigned long long *work)
+                      const int *list, const int *count, const void *disp, unsigned long long *work)
 {
     return MXArgs{alpha, n, d, flags, Up, F, lambda, dt, Va, list, count, disp, c->lam_b, c->status, work,
                   c->fpl, c->cbl, c->ktl, c->m.ctptr, nullptr, nullptr};
