@@ -572,7 +572,7 @@ int vof_create(const vof_mesh *mesh, const vof_options *opt, vof_ctx **out)
         // beyond it are fluxed in the slower one-warp form, so where memory is
         // short a smaller queue serves too.
         const size_t unit = 16, per = c->precision == VOF_MIXED ? 512 : 1024;
-        size_t bytes = std::max(per * (size_t)nf, per * (size_t)(1 << 17));
+        size_t bytes = std::max(per * (size_t)nf, per * (size_t)(1 << 16));
         bytes = std::min(bytes, unit * ((size_t)1 << 31));
         void *p = nullptr;
         while (cudaMalloc(&p, bytes) != cudaSuccess && bytes > (1u << 20)) {

@@ -135,6 +135,14 @@ __device__ __forceinline__ bool gt_bits(double a, double b)
     y.hi ^= sy & 0x7fffffff; y.lo ^= (unsigned)sy;
     return !bits_le(x, y);
 }
+// Dependent launches (launch_after): a kernel begins while the one before it on
+// the stream ends, and waits here, before it reads or writes anything, until
+// that one has completed and its results are visible (at once where it was
+// launched in the ordinary way) ...
+__device__ __forceinline__ void previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// ... and the one before it says from where on it may begin: at its start where
+// all its blocks are resident or it is short, else as its warps run out of work
+__device__ __forceinline__ void next_kernel() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // x truncated to FP32 on the integer pipe (the FP64 pipe's conversion costs as
 // much as an FMA there): relative error below 2^-23; magnitudes below 2^-126
 // become 0, above the FP32 range a large finite number

@@ -802,7 +802,7 @@ __global__ void k_flux_polyhedra(DevMesh m, const double *__restrict__ Up, const
 // the face has exactly N points and every array index is static after
 // unrolling (registers); N = VOF_MAXFP: any n (local arrays).
 template <int N>
-__device__ __forceinline__ void correct_face(const DevMesh &m, int f, int b, int n, const double *__restrict__ U,
+__device__ __forceinline__ void correct_face(const DevMesh &m, int f, int b, int n, const double *U,
                                              const double *__restrict__ F, double dt, int item, double *lam_out,
                                              int *it_out, void *disp_out, bool disp32, int *maxit, int *nfallback,
                                              unsigned &ntri, unsigned &nev)
@@ -817,7 +817,7 @@ __device__ __forceinline__ void correct_face(const DevMesh &m, int f, int b, int
             int p = __ldg(m.fpts + b + i);
             id[i] = __ldg(m.fkey + b + i);  // the point's index (its master's on a periodic mesh)
             A[i] = ldP(m, p);
-            W[i] = ld3(U, m.np, p) * dt;
+            W[i] = mk(U[p], U[m.np + p], U[2 * m.np + p]) * dt;
         }
     }
     const double tau = F[f] * dt;
@@ -882,11 +882,12 @@ __device__ __forceinline__ void correct_face(const DevMesh &m, int f, int b, int
 
 // One thread per face (LIST: per band slot).  U holds the point velocities.
 template <bool LIST>
-__global__ void k_correct(DevMesh m, const double *__restrict__ U, const double *__restrict__ F,
+__global__ void k_correct(DevMesh m, const double *U, const double *__restrict__ F,
                           double dt, const int *list, const int *count, double *lam_out,
                           int *it_out, void *disp_out, bool disp32, int *maxit, int *nfallback, unsigned long long *work,
                           const double *__restrict__ alpha, BandRec *rec)
 {
+    previous_kernel();
     const int total = LIST ? *count : m.nf;
     unsigned ntri = 0, nev = 0;  // FP64 work: cubic coefficient triangles, cubic evaluations
     for (int item = blockIdx.x * blockDim.x + threadIdx.x; item < total; item += gridDim.x * blockDim.x) {
@@ -921,6 +922,7 @@ __global__ void k_correct(DevMesh m, const double *__restrict__ U, const double 
 // flag cleared for the next step.
 __global__ void k_band_point_velocity(DevMesh m, const double *__restrict__ Uc, uint8_t *flag, double *Up)
 {
+    next_kernel();
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < m.np; p += gridDim.x * blockDim.x) {
         if (!flag[p]) continue;
         flag[p] = 0;
@@ -1054,10 +1056,12 @@ __device__ __forceinline__ double warp_max_bits(double v)
 // alpha, 8 of V a cell, each face's flux once) and, on small meshes, by the chain
 // of dependent loads.  An empty cell without flux costs no FP64 instruction and
 // a full one without flux no division (the FP64 pipe runs at 1/62 of FP32).
-__global__ void __launch_bounds__(UPD_THREADS) k_update(DevMesh m, double *alpha, const double *__restrict__ Va,
+__global__ void __launch_bounds__(UPD_THREADS) k_update(DevMesh m, double *alpha, const double *Va,
                                                         const int4 *__restrict__ seg, int nseg, double *sd,
                                                         uint8_t *seg_mixed, int *viol, int *nviol, unsigned *status)
 {
+    next_kernel();
+    previous_kernel();
     __shared__ double sh[UPD_THREADS / 32][SD_UPD];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int nb = m.nf - m.ni;
@@ -1264,6 +1268,7 @@ __device__ void stats_block(const double *sd, int nseg, const int *counters, dou
 constexpr int ST_THREADS = 512;
 __global__ void __launch_bounds__(ST_THREADS) k_stats(const double *sd, int nseg, const int *counters, double *stats)
 {
+    previous_kernel();
     stats_block(sd, nseg, counters, stats, nullptr);
     if (threadIdx.x == 0) stats[VOF_S_BOUND_PASSES] = stats[VOF_S_BOUND_GLOBAL] = 0.0;
 }
@@ -1428,6 +1433,7 @@ __device__ __forceinline__ bool region_applies(const double *tt)
 template <bool CLUSTER>
 __global__ void __launch_bounds__(BA_THREADS, 1) k_bound_step(DevMesh m, BoundStep a)
 {
+    previous_kernel();
     // item i goes to block i mod gridDim.x: the few items of a phase spread over
     // every SM of the launch
     const int tl = threadIdx.x * gridDim.x + blockIdx.x, nt = gridDim.x * blockDim.x;
@@ -1636,6 +1642,7 @@ __global__ void k_zero_update(int *cnt)
 // (and the step's counters, which only later kernels use)
 __global__ void k_point_state(DevMesh m, const double *__restrict__ alpha, uint8_t *state, double *palpha, int *cnt)
 {
+    next_kernel();
     int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p < CNT_LEN) cnt[p] = 0;
     if (p == CNT_LEN) cnt[CNT_BAR] = 0;
@@ -1657,10 +1664,13 @@ __global__ void k_point_state(DevMesh m, const double *__restrict__ alpha, uint8
     }
 }
 
+// (what the previous kernel wrote is not declared __restrict__: this one may have
+// begun before, see previous_kernel)
 __global__ void k_classify(DevMesh m, const double *__restrict__ alpha, const double *__restrict__ F,
-                           double dt, const uint8_t *__restrict__ state, double *Va, int *band, int *nband,
+                           double dt, const uint8_t *state, double *Va, int *band, int *nband,
                            int *icell, int *nicell, uint8_t *bpflag, unsigned *status)
 {
+    previous_kernel();
     const int lim = m.nf > m.nc ? m.nf : m.nc;
     for (int i0 = blockIdx.x * blockDim.x; i0 < lim; i0 += gridDim.x * blockDim.x) {
         const int i = i0 + threadIdx.x;
@@ -2109,14 +2119,12 @@ static int launch_update_group(vof_ctx *c, double *alpha, const double *Va, cons
                                cudaStream_t s)
 {
     int *cnt = c->counters;
-    k_update<<<std::min(c->nseg, num_sms(c->device) * 8), UPD_THREADS, 0, s>>>(
-        c->m, alpha, Va, c->seg, c->nseg, c->sd, c->seg_mixed, c->bound ? c->viol[0] : nullptr, cnt + CNT_VIOL0,
-        c->status);
+    if (launch_after(k_update, std::min(c->nseg, num_sms(c->device) * 8), UPD_THREADS, 0, s, c->m, alpha, Va, c->seg,
+                     c->nseg, c->sd, c->seg_mixed, c->bound ? c->viol[0] : nullptr, cnt + CNT_VIOL0, c->status))
+        return VOF_ERR_CUDA;
     LAUNCH_CHECK();
     if (!c->bound) {
-        k_stats<<<1, ST_THREADS, 0, s>>>(c->sd, c->nseg, counters, stats);
-        LAUNCH_CHECK();
-        return VOF_OK;
+        return launch_after(k_stats, 1, ST_THREADS, 0, s, c->sd, c->nseg, counters, stats);
     }
     const BoundStep a{alpha, c->viol[0], cnt + CNT_VIOL0, c->rl, cnt + CNT_NRL0, c->ra, c->bscr, c->cmark, c->segmark,
                       c->dl, cnt + CNT_NDL, reinterpret_cast<unsigned *>(cnt + CNT_EPOCH), cnt + CNT_BPASS,
@@ -2127,10 +2135,13 @@ static int launch_update_group(vof_ctx *c, double *alpha, const double *Va, cons
     cfg.blockDim = dim3(BA_THREADS);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     cfg.attrs = at;
     cfg.numAttrs = 1;
     if (c->nc <= BOUND_CLUSTER_CELLS) {
+        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.numAttrs = 2;
         cfg.gridDim = dim3(BA_CLUSTER);
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = BA_CLUSTER;
@@ -2210,8 +2221,9 @@ int launch_advect(vof_ctx *c, double *alpha, const double *Uc, const double *F, 
 #define MARK(i) do { if (ev) cudaEventRecord(ev[i], s); } while (0)
     MARK(0);
     k_point_state<<<cdiv(m.np, 256), 256, 0, s>>>(m, alpha, c->pstate, c->palpha, cnt);
-    k_classify<<<sms * 16, 256, 0, s>>>(m, alpha, F, dt, c->pstate, c->Va, c->band, cnt + CNT_BAND, c->icell,
-                                        cnt + CNT_ICELL, c->bpflag, c->status);
+    if (launch_after(k_classify, sms * 16, 256, 0, s, m, alpha, F, dt, c->pstate, c->Va, c->band, cnt + CNT_BAND,
+                     c->icell, cnt + CNT_ICELL, c->bpflag, c->status))
+        return VOF_ERR_CUDA;
     launches += 2;
     LAUNCH_CHECK();
     MARK(1);
@@ -2225,9 +2237,10 @@ int launch_advect(vof_ctx *c, double *alpha, const double *Uc, const double *F, 
     if (wait_before_correct && cudaStreamWaitEvent(c->s_aux, wait_before_correct, 0) != cudaSuccess)
         return VOF_ERR_CUDA;
     k_band_point_velocity<<<cdiv(m.np, 256), 256, 0, c->s_aux>>>(m, Uc, c->bpflag, c->upb);
-    k_correct<true><<<sms * 8, 128, 0, c->s_aux>>>(m, c->upb, F, dt, c->band, cnt + CNT_BAND, c->lam_b, c->it_b,
-                                                   c->disp_b, c->precision == VOF_MIXED, cnt + CNT_MAXCORR, cnt + CNT_FALLBACK,
-                                                   c->work_on ? c->work : nullptr, alpha, c->pf_rec);
+    if (launch_after(k_correct<true>, sms * 8, 128, 0, c->s_aux, m, c->upb, F, dt, c->band, cnt + CNT_BAND, c->lam_b,
+                     c->it_b, c->disp_b, c->precision == VOF_MIXED, cnt + CNT_MAXCORR, cnt + CNT_FALLBACK,
+                     c->work_on ? c->work : nullptr, alpha, c->pf_rec))
+        return VOF_ERR_CUDA;
     LAUNCH_CHECK();
     if (cudaEventRecord(c->ev_join, c->s_aux) != cudaSuccess) return VOF_ERR_CUDA;
     if (c->precision == VOF_MIXED && c->mlp) {

@@ -141,6 +141,7 @@ __global__ void __launch_bounds__(GT) k_mlp_pass(MlpWeights w, const float *__re
                                                  const float *__restrict__ target, int n, float *out, float *part,
                                                  double *lpart)
 {
+    vofd::next_kernel();
     extern __shared__ __align__(16) unsigned char mlp_smem[];
     MlpShared &sh = *reinterpret_cast<MlpShared *>(mlp_smem);
     const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5, g = lane >> 2, t = lane & 3;
@@ -357,9 +358,10 @@ __global__ void __launch_bounds__(GT) k_mlp_pass(MlpWeights w, const float *__re
 // sums the blocks' partials in block order into the flat gradient (and the
 // caller's copy of it), and the squared errors into *loss (host memory)
 constexpr int RED_T = 64;
-__global__ void __launch_bounds__(RED_T) k_mlp_reduce(const float *__restrict__ part, const double *__restrict__ lpart,
-                                                      int nb, float *grad, float *copy, float *loss)
+__global__ void __launch_bounds__(RED_T) k_mlp_reduce(const float *part, const double *lpart, int nb, float *grad,
+                                                      float *copy, float *loss)
 {
+    vofd::previous_kernel();
     const int i = blockIdx.x * RED_T + threadIdx.x;
     if (i < NPARAM) {
         float s = 0.0f;
@@ -544,9 +546,9 @@ int mlp_gradient(vof_mlp *q, const float *feat, const float *target, int n, floa
 {
     const int nb = std::min(cdiv(n, TILE), q->nblk);
     k_mlp_pass<true><<<nb, GT, sizeof(MlpShared), s>>>(mlp_weights(q), feat, target, n, nullptr, q->part, q->lpart);
-    k_mlp_reduce<<<cdiv(NPARAM, RED_T), RED_T, 0, s>>>(q->part, q->lpart, nb, q->grad, copy,
-                                                       want_loss ? q->h_loss : nullptr);
-    return cudaGetLastError() == cudaSuccess ? VOF_OK : VOF_ERR_CUDA;
+    if (cudaGetLastError() != cudaSuccess) return VOF_ERR_CUDA;
+    return launch_after(k_mlp_reduce, cdiv(NPARAM, RED_T), RED_T, 0, s, q->part, q->lpart, nb, q->grad, copy,
+                        want_loss ? q->h_loss : nullptr);
 }
 
 int mlp_pack(vof_mlp *q, cudaStream_t s)

@@ -1611,6 +1611,7 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
         }
         unit = next;
     }
+    next_kernel();
     wk.flush(a.work, lane);
 }
 
@@ -1626,6 +1627,7 @@ template <class R, int ST, class Wk>
 __device__ __forceinline__ void pf_clip_body(const MXArgs &a, const PfQueue &q, ClipShared<R, ST> &sh)
 {
     const int lane = threadIdx.x & 31;
+    previous_kernel();
     const unsigned long long ctr = *q.ctr;
     const int nb = min((int)(ctr >> 32), q.bcap);
     auto take = [&]() {
@@ -1662,6 +1664,7 @@ __device__ __forceinline__ void pf_clip_body(const MXArgs &a, const PfQueue &q, 
         if (lane == 0) put_sum(q.part, bi, acc);
         __syncwarp();
     }
+    next_kernel();
     wk.flush(a.work, lane);
 }
 
@@ -1697,6 +1700,7 @@ template <class R, class Wk>
 __global__ void __launch_bounds__(pp_warps<R>() * 32, pp_resident<R>()) k_pf_pairs(DevMesh m, MXArgs a, PfQueue q)
 {
     extern __shared__ __align__(16) unsigned char pf_smem[];
+    previous_kernel();
     pf_pairs_body<R, Wk>(m, a, q, reinterpret_cast<PairShared<R> *>(pf_smem)[threadIdx.x >> 5]);
 }
 
@@ -1715,6 +1719,8 @@ __global__ void __launch_bounds__(W * 32, pc_resident<R>(W, ST)) k_pf_clip(MXArg
 template <class R, class Wk>
 __global__ void __launch_bounds__(64, sizeof(R) == 4 ? 8 : 4) k_pf_finish(DevMesh m, MXArgs a, PfQueue q, const int *count)
 {
+    next_kernel();
+    previous_kernel();
     extern __shared__ __align__(16) unsigned char pf_smem[];
     {
         MXArgs s = a;
@@ -1881,8 +1887,7 @@ template <class R, int W, int ST, class Wk>
 static int go_clip(const MXArgs &a, const PfQueue &q, int sms, int mult, cudaStream_t s)
 {
     constexpr size_t bytes = W * sizeof(ClipShared<R, ST>);
-    k_pf_clip<R, W, ST, Wk><<<sms * pc_resident<R>(W, ST) * mult, 32 * W, bytes, s>>>(a, q);
-    return VOF_OK;
+    return launch_after(k_pf_clip<R, W, ST, Wk>, sms * pc_resident<R>(W, ST) * mult, 32 * W, bytes, s, a, q);
 }
 
 template <class R, class Wk>
@@ -1912,7 +1917,8 @@ static int go_list(vof_ctx *c, const MXArgs &a, int sms, cudaStream_t s)
     o.items = q.ovf;
     o.count = q.novf;
     o.next = q.next_ovf;
-    k_pf_finish<R, Wk><<<sms * 4, 64, fbytes, s>>>(c->m, o, q, a.count);
+    r = launch_after(k_pf_finish<R, Wk>, sms * 4, 64, fbytes, s, c->m, o, q, a.count);
+    if (r) return r;
     return cudaGetLastError() == cudaSuccess ? VOF_OK : VOF_ERR_CUDA;
 }
 
