@@ -148,8 +148,8 @@ int vof_batch_advect(vof_batch *b, double *alpha, const double *U_dt, const doub
 
 // Times one step (vof_advect's launch sequence, from the state alpha copied
 // into the context's staging buffer: no allocation) for every launch
-// configuration of the mixed phase flux -- clip-piece stack depth 92 or 56,
-// 1, 2 or 3 warps (faces) per block, grid multipliers 1, 2, 4 over the
+// configuration of the mixed form's clips -- clip-piece stack depth 92 or 56,
+// 1, 2 or 3 warps (job batches) per block, grid multipliers 1, 2, 4 over the
 // resident blocks -- and keeps the fastest; an FP64 context keeps its launch
 static int tune_launch(vof_ctx *c, const double *alpha, const double *U, const double *F, double dt, cudaStream_t s,
                        int *best_out, float *ms_out)

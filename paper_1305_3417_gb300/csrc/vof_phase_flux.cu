@@ -1,10 +1,12 @@
 // Phase flux (A6, Eqs. S'_f, S''_f): the flux-polyhedron tetrahedra T of a
 // band face, the cell tetrahedra K of its stencil cells and their PLIC planes
-// are taken to a frame centred on the face centre and intersected there, one
-// warp per face.  One source for both forms:
+// are taken to a frame centred on the face centre and intersected there: in a
+// step by three launches over the band faces (pairs, clips, sums; below), in
+// the standalone call by a warp per face of the mesh.  One source for both forms:
 //  - mixed (R = float): FP32 clipping, pieces summed per lane with TwoSum
 //    compensation and finished in FP64 (reading R13 on the on-plane band);
-//  - plain (R = double): the same structure in FP64 throughout.
+//  - plain (R = double): the same structure in FP64 (what FP32 decides beyond
+//    its roundings, it decides).
 //
 // Only the frame shift of a stencil cell (its centre minus the face centre) and
 // of its plane offset are formed in FP64; the cell's own geometry comes from
@@ -675,6 +677,20 @@ __device__ __forceinline__ void mx_flush(Sh &sh, int nt, int ncand, R tol, R sla
 
 template <class R> __device__ __forceinline__ R rconv(double v) { return (R)v; }
 
+// over the warp in one instruction (ten for a shuffle tree; pair stage 1 % faster)
+__device__ __forceinline__ float warp_min(float v)
+{
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float warp_max(float v)
+{
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+
 // The flux polyhedron of face f (band slot item of a LIST form; points b .. b +
 // n - 1 of the face-point arrays) in the frame of the face centre: prisms with
 // their boxes, tetrahedra (a lane each) with signs and volumes in shared
@@ -778,13 +794,16 @@ __device__ __forceinline__ void mx_poly(const DevMesh &m, const MXArgs &a, Sh &s
     // bounding box of the whole polyhedron
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
-        B v = bx[i];
+        if constexpr (std::is_same<B, float>::value) pb[i] = i < 3 ? warp_min(bx[i]) : warp_max(bx[i]);
+        else {
+            B v = bx[i];
 #pragma unroll
-        for (int o2 = 16; o2 > 0; o2 >>= 1) {
-            B w = __shfl_xor_sync(0xffffffffu, v, o2);
-            v = i < 3 ? rmin(v, w) : rmax(v, w);
+            for (int o2 = 16; o2 > 0; o2 >>= 1) {
+                B w = __shfl_xor_sync(0xffffffffu, v, o2);
+                v = i < 3 ? rmin(v, w) : rmax(v, w);
+            }
+            pb[i] = v;
         }
-        pb[i] = v;
     }
     __syncwarp();
 }
