@@ -1408,15 +1408,27 @@ constexpr int BA_THREADS = 1024;
 constexpr int BA_CLUSTER = 8;
 constexpr int BOUND_CLUSTER_CELLS = 1 << 15;
 
-// region r, by a whole warp
+// region r, by a whole warp; eight segments' flags and sums are read at a time
+// (the sums of segments without mixed cells are not kept up and left out)
 __device__ void region_totals(const int *reg_seg, int r, const double *sd, const uint8_t *seg_mixed, int nseg,
                               double *totals)
 {
     const int lane = threadIdx.x & 31;
     double t[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int k = reg_seg[r] + lane; k < reg_seg[r + 1]; k += 32)
-        if (seg_mixed[k])
-            for (int i = 0; i < 4; ++i) t[i] += sd[(size_t)(SD_EP + i) * nseg + k];
+    const int k1 = reg_seg[r + 1];
+    for (int k = reg_seg[r] + lane; k < k1; k += 8 * 32) {
+        unsigned in = 0u;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) in |= (unsigned)(k + 32 * u < k1 && seg_mixed[k + 32 * u]) << u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            double v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = k + 32 * u < k1 ? sd[(size_t)(SD_EP + i) * nseg + k + 32 * u] : 0.0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) t[i] += in >> u & 1u ? v[u] : 0.0;
+        }
+    }
     for (int i = 0; i < 4; ++i) t[i] = warp_sum(t[i]);
     if (lane == 0) {
         double *o = totals + REG_TOT * (size_t)r;
