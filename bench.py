@@ -50,11 +50,14 @@ FILL_FLOPS = 30
 #    (E1, E2, the summed stream vector and four 3x3 determinants) 110, one cubic
 #    evaluation with its scale and Newton step 20
 CTRI_FLOPS, CEVAL_FLOPS = 110, 20
+# the launches of a step's phase flux (one timed group)
+PF_KERNELS = "k_pf_pairs + k_pf_clip + k_pf_finish"
 # algorithmic HBM bytes per internal face and step (flux 8, owner/neighbour 8,
 # face point indices 20, alpha r/w and volume 8, point data 28)
 BYTES_PER_FACE = 72.0
 
-# DRAM bytes per launch of the mixed phase-flux kernel: dram__bytes_read.sum +
+# DRAM bytes per launch of the mixed phase flux (here of its earlier form, one
+# launch a step; its sources have changed since): dram__bytes_read.sum +
 # dram__bytes_write.sum, mean of the two timed launches of one ncu capture of
 # the default launch shape (ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,
 # gpu__time_duration.sum -k regex:k_phase_flux_mixed -s 3 -c 3 python bench.py
@@ -520,7 +523,7 @@ def run_batch(args, world, rank, local):
     f32, f64, pf = work_flops(work, False)
     alu = vof.vof_probe_fma(local, vof.MIXED)
     achieved = pf / (per_launch["phase_flux"] * 1e-3) / 1e12
-    roof = {"kernel": "k_phase_flux_mixed", "bound": "alu", "achieved": achieved, "peak": alu / 1e12,
+    roof = {"kernel": PF_KERNELS, "bound": "alu", "achieved": achieved, "peak": alu / 1e12,
             "unit": "TFLOP/s", "frac": achieved * 1e12 / alu, "traffic": None,
             "peak_source": "measured FP32 FMA probe (vof_probe_fma)", "group_ms_per_step": per_launch,
             "work_per_launch": work, "flops_per_launch": pf}
@@ -825,7 +828,7 @@ def main():
         other = {"precision": "fp64" if oprec == vof.FP64 else "mixed", "value": m.n_internal / (oms * 1e-3) / 1e6,
                  "unit": UNIT, "ms_per_step": oms, "steps": ns,
                  "group_ms_per_step": {g: v / max(onprof, 1) for g, v in ogroup.items()},
-                 "roofline": {"kernel": "k_phase_flux" if oprec == vof.FP64 else "k_phase_flux_mixed", "bound": "alu",
+                 "roofline": {"kernel": PF_KERNELS, "bound": "alu",
                               "achieved": opf / (ot_pf * 1e-3) / 1e12, "peak": opk / 1e12, "unit": "TFLOP/s",
                               "frac": opf / (ot_pf * 1e-3) / opk,
                               "peak_source": f"measured {'FP64' if oprec == vof.FP64 else 'FP32'} FMA probe",
@@ -880,7 +883,7 @@ def main():
         achieved = pf / (per_launch[dom] * 1e-3) / 1e12
         traffic = captured_traffic(args.workload, m.shape[0], "fp64" if prec == vof.FP64 else "mixed") \
             if args.skip == 0 else None
-        roof = {"kernel": "k_phase_flux" if prec == vof.FP64 else "k_phase_flux_mixed", "bound": "alu",
+        roof = {"kernel": PF_KERNELS, "bound": "alu",
                 "achieved": achieved, "peak": alu / 1e12, "unit": "TFLOP/s", "frac": achieved * 1e12 / alu,
                 "traffic": traffic, "traffic_unit": "bytes per launch (ncu capture)",
                 "peak_source": f"measured {'FP64' if prec == vof.FP64 else 'FP32'} FMA probe (vof_probe_fma)",

@@ -15,7 +15,9 @@
  *   PyTorch tensors).  They must stay valid until `stream` reaches the call.
  *   Every per-step call is asynchronous on `stream` (a cudaStream_t; NULL is
  *   the legacy default stream) and allocates no memory: the context allocates
- *   all of its scratch in vof_create.
+ *   all of its scratch in vof_create (the largest: the cell tetrahedra's planes,
+ *   and the phase flux's queue of clip jobs, 512 bytes per face, 1024 in FP64;
+ *   band faces that find no room in it are fluxed more slowly).
  * - Vectors are structure-of-arrays: x block, then y block, then z block.
  * - Face f of the mesh has points face_pts[face_ptr[f] .. face_ptr[f+1]),
  *   ordered so that the right-hand area vector S_f points from owner[f] to
@@ -314,10 +316,11 @@ int vof_batch_advect(vof_batch *batch, double *alpha, const double *U_dt, const 
 
 /* Autotuner for the phase-flux launch of a mixed batch: times one step from
  * the state alpha (left unchanged: the steps run on a copy in the context's
- * staging buffer) for every launch configuration -- the per-warp staging of
- * clip pieces in shared memory (a stack of 92 pieces, or of 56 for more
- * resident warps), 1, 2 or 3 warps (faces) per block, and grid multipliers
- * 1, 2 and 4 over the resident blocks -- keeps the fastest for later steps,
+ * staging buffer) for every configuration of its clip launch -- the per-warp
+ * staging of clip pieces in shared memory (a stack of 92 pieces, or of 56 for
+ * more resident warps), 1, 2 or 3 warps (each on a face's job batch) per
+ * block, and grid multipliers 1, 2 and 4 over the resident blocks -- keeps the
+ * fastest for later steps,
  * and returns it as config = 256 * stack + 16 * warps + multiplier (stack 0:
  * 92 pieces, 1: 56) with its step time in ms (either pointer may be NULL).
  * An FP64 batch keeps its launch (config 0).  Synchronous on `stream`. */
@@ -409,7 +412,9 @@ int vof_profile_end(vof_ctx *ctx, double *group_ms, int *steps);
  *  [9] face triangles whose swept prism enters the correction's cubic,
  *  [10] cubic evaluations of the correction,
  *  [11] reserved (0).
- * [0]-[5] are FP32 work in a VOF_MIXED context and FP64 in a VOF_FP64 one;
+ * [0]-[5] are FP32 work in a VOF_MIXED context and FP64 in a VOF_FP64 one,
+ * where what a step decides in FP32 is not counted and four open distances of
+ * its pair stage count as one piece-plane test;
  * [7], [9], [10] are FP64.  Reading synchronises `stream`; reset zeroes the
  * counters. */
 enum { VOF_WORK_LEN = 12 };

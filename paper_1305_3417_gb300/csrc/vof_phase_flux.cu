@@ -1234,7 +1234,8 @@ __device__ __forceinline__ int pf_pairs64(PairShared<double> &sh, int nt, int nc
     // its own lane, four points at a time, took ten times the FP64 instructions:
     // the planes shared by a face's cells and polyhedron are open everywhere,
     // most others nowhere; pairs of 64^3 hexahedra 402 -> 370 us, and 317
-    // with the loops over the planes rolled: the launch waited for instructions.)
+    // with the loops over the planes rolled: the launch waited for instructions;
+    // 281 since.)
     constexpr unsigned M[3] = {0x27u, 0x33u, 0x39u};  // T0 = a0 a1 a2 b2, T1 = a0 a1 b2 b1, T2 = a0 b0 b1 b2
     int nq = 0;
     used = 0u;
