@@ -1581,6 +1581,7 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
                         else { q.boff[bi] = off; q.bnext[bi] = head; }
                     }
                     if (used >> lane & 1u) sh.Kmap[__popc(used & lt)] = (unsigned char)lane;
+                    __syncwarp();  // the map and the job codes are read by other lanes below
                     const R sg = lane < nt ? sh.Tsg[lane] : R(0);
                     const unsigned pos = __ballot_sync(0xffffffffu, sg > R(0)), neg = __ballot_sync(0xffffffffu, sg < R(0));
                     off = __shfl_sync(0xffffffffu, off, 0);
