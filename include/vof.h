@@ -306,8 +306,9 @@ vof_ctx *vof_batch_context(vof_batch *batch);
  * folded into its inputs: U_dt [3*n_cells] = U_c dt_case and F_dt [n_faces] =
  * F_f dt_case (the method uses the field only through these products), so the
  * step runs with dt = 1.  The step's kernels are captured into a CUDA graph at
- * the first call (again when an array pointer or the launch configuration
- * changes) and replayed as one graph launch on an internal stream that is
+ * the first call (again when an array pointer, the launch configuration or a
+ * setting of the batch's context changes: gradient, network, work counting) and
+ * replayed as one graph launch on an internal stream that is
  * ordered after, and before, `stream` by events.  stats (device, VOF_S_LEN)
  * and case_mass (device [ncases]: sum of V alpha per case after the step, in a
  * fixed order) may be NULL.  Errors: VOF_ERR_INVALID_ARG, VOF_ERR_CUDA. */

@@ -728,6 +728,7 @@ int vof_set_gradient(vof_ctx *c, int kind)
         int r = build_lsq(c);
         if (r) return r;
     }
+    if (c->grad_kind != kind) ++c->cfg_gen;
     c->grad_kind = kind;
     return VOF_OK;
 }
@@ -926,6 +927,7 @@ int vof_probe_barrier(vof_ctx *c, int skip_block, void *stream)
 int vof_count_work(vof_ctx *c, int on)
 {
     if (!c) return VOF_ERR_INVALID_ARG;
+    if (c->work_on != (on ? 1 : 0)) ++c->cfg_gen;
     c->work_on = on ? 1 : 0;
     return VOF_OK;
 }

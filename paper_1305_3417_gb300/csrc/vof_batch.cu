@@ -6,8 +6,9 @@
 // the per-warp load balancing of the narrow-band kernels and every launch cover
 // all cases at once.  The method uses a velocity field only through F dt and
 // U dt, so each case's own time step is folded into its F and U and the batch
-// steps with dt = 1.  A step is captured once into a CUDA graph (all its
-// kernels) and replayed as one graph launch; the phase-flux launch shape is
+// steps with dt = 1.  A step is captured into a CUDA graph (all its kernels),
+// again when an array, the launch shape or a setting of the context changes, and
+// replayed as one graph launch; the phase-flux launch shape is
 // chosen by timing the candidates on the batch itself.
 #include <cuda_runtime.h>
 
@@ -26,6 +27,7 @@ struct vof_batch {
     cudaGraphExec_t exec;
     const void *key[5];       // arrays baked into the graph
     int key_cfg;              // launch configuration baked into the graph
+    unsigned key_gen;         // and the context's settings (vof_ctx::cfg_gen)
 };
 
 namespace {
@@ -122,7 +124,9 @@ int vof_batch_advect(vof_batch *b, double *alpha, const double *U_dt, const doub
     if (cudaSetDevice(c->device) != cudaSuccess) return VOF_ERR_CUDA;
     if (!stats) stats = c->stats_dev;
     const void *key[5] = {alpha, U_dt, F_dt, stats, case_mass};
-    if (b->exec && (std::memcmp(key, b->key, sizeof(key)) != 0 || b->key_cfg != cfg_code(c))) drop_graph(b);
+    if (b->exec && (std::memcmp(key, b->key, sizeof(key)) != 0 || b->key_cfg != cfg_code(c) ||
+                    b->key_gen != c->cfg_gen))
+        drop_graph(b);
     if (!b->exec) {
         cudaGraph_t g = nullptr;
         if (cudaStreamBeginCapture(b->gs, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return VOF_ERR_CUDA;
@@ -137,6 +141,7 @@ int vof_batch_advect(vof_batch *b, double *alpha, const double *U_dt, const doub
         if (e != cudaSuccess) { b->exec = nullptr; return VOF_ERR_CUDA; }
         std::memcpy(b->key, key, sizeof(key));
         b->key_cfg = cfg_code(c);
+        b->key_gen = c->cfg_gen;
     }
     cudaStream_t s = (cudaStream_t)stream;
     if (cudaEventRecord(b->ev_in, s) != cudaSuccess || cudaStreamWaitEvent(b->gs, b->ev_in, 0) != cudaSuccess ||

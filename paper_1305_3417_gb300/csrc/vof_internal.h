@@ -175,6 +175,10 @@ struct vof_ctx {
     int mlp_feat_cap;
     int *mlp_nbr;                // per cell: 27 lattice-slot cell indices (-1: itself)
     float *mlp_geo;              // per cell: 6 shape numbers
+    // counts the changes of what a step's launches hold besides their arguments
+    // (gradient, network and its buffers, work counting): a captured step is
+    // good for one value
+    unsigned cfg_gen;
     // kernel-group timing (vof_profile_begin / _end)
     cudaEvent_t *prof_ev;
     int prof_max, prof_steps;

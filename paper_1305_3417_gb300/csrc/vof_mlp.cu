@@ -681,6 +681,7 @@ int vof_set_guess(vof_ctx *c, vof_mlp *q)
     if (!c) return VOF_ERR_INVALID_ARG;
     if (cudaSetDevice(c->device) != cudaSuccess) return VOF_ERR_CUDA;
     if (q && q->device != c->device) return VOF_ERR_INVALID_ARG;
+    ++c->cfg_gen;  // (also for the same network again: its weights or buffers may be new ones)
     if (q && !c->mlp_nbr) {
         if (cudaMalloc(&c->mlp_nbr, sizeof(int) * 27 * (size_t)c->nc) != cudaSuccess ||
             cudaMalloc(&c->mlp_geo, sizeof(float) * 6 * (size_t)c->nc) != cudaSuccess)
