@@ -344,6 +344,21 @@ __device__ __forceinline__ void fsplit(const RTet<R> &t, const R s[4], int nin, 
     c[5] = sel(n2, e3, e2);
 }
 
+// What an FP32 distance of a point of the flux polyhedron (box pb, M its largest
+// coordinate) to a unit-normal plane has to exceed for the point to lie above
+// the plane: truncated operands and four roundings err by 8.4e-7 M + 3.6e-7 |w|
+// at most, w the plane's offset, which is below 1.8 M where the plane can cut
+// the polyhedron; 2e-6 M is above that.  It goes with the polyhedron's extent, not
+// with the face's: along a needle cell the sweep is hundreds of face sizes long.
+template <class B>
+__device__ __forceinline__ float drop_slack(const B pb[6])
+{
+    float v = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) v = fmaxf(v, fabsf(tof(pb[i])));
+    return 2e-6f * v;
+}
+
 // The queued clip jobs, worked through by the whole warp, one piece per lane
 // and step.  Pieces with one plane left (leaves) stack up from the bottom of S,
 // the others down from its top, and a step works on one kind only, so that the
@@ -364,7 +379,7 @@ __device__ __forceinline__ void fsplit(const RTet<R> &t, const R s[4], int nin, 
 // <= MX_STACK for depth i and r planes to go: the top one alone always fits
 // once the leaves are gone, and the stacks cannot overflow.
 template <class R, class Sh, class Wk>
-__device__ __forceinline__ void mx_clip(Sh &sh, const unsigned short *Q, int nq, R tol, Acc<R> &acc, Wk &wk)
+__device__ __forceinline__ void mx_clip(Sh &sh, const unsigned short *Q, int nq, R tol, float drop, Acc<R> &acc, Wk &wk)
 {
     constexpr int MX_STACK = Sh::MX_STACK;
     const int lane = threadIdx.x & 31;
@@ -445,14 +460,14 @@ __device__ __forceinline__ void mx_clip(Sh &sh, const unsigned short *Q, int nq,
             c[0] = t.v[0]; c[1] = t.v[1]; c[2] = t.v[2]; c[5] = t.v[3];
             if (cut) fsplit(t, sd, nin, c);
             if (keep && !single) {
-                // the points below the plane after (FP64: those not clearly
-                // above it by an FP32 distance; a part kept for nothing is
-                // dropped when its own turn comes)
+                // the points below the plane after (FP64: those not above it
+                // by an FP32 distance beyond its roundings (drop_slack); a part
+                // kept for nothing is dropped when its own turn comes)
                 const R4<R> pn = sh.Kp[k][__ffs(rem) - 1];
                 const float4 pf = make_float4(tof(pn.x), tof(pn.y), tof(pn.z), tof(pn.w));
                 auto below = [&](int i) {
                     if constexpr (std::is_same<R, float>::value) return pdist(pn, c[i]) < -tol;
-                    else return pdist(pf, r3(tof(c[i].x), tof(c[i].y), tof(c[i].z))) < (float)tol * 1.2e9f;
+                    else return pdist(pf, r3(tof(c[i].x), tof(c[i].y), tof(c[i].z))) < drop;
                 };
                 const bool z0 = below(0), z1 = below(1), z2 = below(2), z5 = below(5);
                 ndrop = __popc(keep);
@@ -663,7 +678,7 @@ __device__ __forceinline__ int mx_pairs(Sh &sh, int nt, int ncand, const R kb[6]
 
 // the pairs of the buffered candidates and the clipping of their jobs
 template <class R, class Sh, class Wk>
-__device__ __forceinline__ void mx_flush(Sh &sh, int nt, int ncand, R tol, R slack, Acc<R> &acc, Wk &wk)
+__device__ __forceinline__ void mx_flush(Sh &sh, int nt, int ncand, R tol, R slack, float drop, Acc<R> &acc, Wk &wk)
 {
     const int lane = threadIdx.x & 31;
     R kb[6];
@@ -671,7 +686,7 @@ __device__ __forceinline__ void mx_flush(Sh &sh, int nt, int ncand, R tol, R sla
     for (int q = 0; q < 6; ++q) kb[q] = lane < ncand ? sh.Kb[lane][q] : R(0);
     unsigned used;
     const int nq = mx_pairs(sh, nt, ncand, kb, tol, slack, acc, used, wk);
-    if (nq > 0) mx_clip(sh, sh.Q, nq, tol, acc, wk);
+    if (nq > 0) mx_clip(sh, sh.Q, nq, tol, drop, acc, wk);
     __syncwarp();
 }
 
@@ -1040,7 +1055,7 @@ __device__ __forceinline__ void phase_flux_body(const DevMesh &m, const MXArgs &
             }
             const unsigned cmask = __ballot_sync(0xffffffffu, cand);
             if (fin ? ncand > 0 : ncand + __popc(cmask) > MX_CAND) {
-                mx_flush(sh, nt, ncand, tol, box_slack<R>(pb), acc, wk);
+                mx_flush(sh, nt, ncand, tol, box_slack<R>(pb), drop_slack(pb), acc, wk);
                 ncand = 0;
                 continue;  // the batch again (or the end)
             }
@@ -1594,7 +1609,9 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
                             ob[0] = make_uint4((unsigned)nq | (unsigned)nu << 16 | (unsigned)nprism << 24, pos, neg, 0u);
                             if constexpr (F64) {
                                 const DBits t = dbits(tol);
-                                ob[1] = make_uint4(t.lo, (unsigned)t.hi, 0u, 0u);
+                                const float4 lo = sh.X[0], hi = sh.X[1];
+                                const float box[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
+                                ob[1] = make_uint4(t.lo, (unsigned)t.hi, __float_as_uint(drop_slack(box)), 0u);
                             } else ob[1] = make_uint4(__float_as_uint(tol), 0u, 0u, 0u);
                         }
                         const uint4 *ps = reinterpret_cast<const uint4 *>(sh.P6);
@@ -1680,7 +1697,7 @@ __device__ __forceinline__ void pf_clip_body(const MXArgs &a, const PfQueue &q, 
         }
         __syncwarp();
         Acc<R> acc;
-        mx_clip(sh, reinterpret_cast<const unsigned short *>(ob + L.Q), nq, tol, acc, wk);
+        mx_clip(sh, reinterpret_cast<const unsigned short *>(ob + L.Q), nq, tol, __uint_as_float(h1.z), acc, wk);
         mx_merge(acc);
         if (lane == 0) put_sum(q.part, bi, acc);
         __syncwarp();

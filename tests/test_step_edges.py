@@ -1,5 +1,7 @@
 """What a step does at its edges: shared memory handed between the lanes of a
-warp, settings changed between batch steps.
+warp, settings changed between batch steps, cells of any aspect ratio.
+
+FP64 is held to the replay tolerance against the oracle (1e-11).
 """
 import os
 import re
@@ -94,3 +96,40 @@ def test_batch_follows_its_context(torch, what):
         step()
         assert seen[-1][1] == seen[1][1]
     B.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("aspect", [1, 30, 300, 1000, 3000])
+def test_sliver_along_needle_cells(torch, oracle_lib, aspect):
+    """A plane just inside the far end of a sweep along needle cells: the flux is
+    the sliver between the two (of phase, or of void), 3e-10 to 1e-6 cells thick,
+    in the step and in its stages called one by one."""
+    from paper_1305_3417_gb300 import vof
+    n = (6, 3, 3)
+    m = I.hex_mesh(n, (6.0, 3.0 / aspect, 3.0 / aspect), periodic="xyz")
+    om = oracle_lib.OracleMesh(m)
+    F = np.asarray(om.geometry()[3]).reshape(3, -1)[0]      # u = (1, 0, 0)
+    U = np.zeros((3, m.n_cells))
+    U[0] = 1.0
+    i = np.arange(m.n_cells) % n[0]
+    ctx = vof.VofContext(m, precision=0, bound=False)
+    tF, tU = T(torch, F), T(torch, U)
+    Up = ctx.point_velocity(tU)
+    for dt in (0.3, 0.5, 0.61, 0.97):
+        lam = ctx.correct_flux(Up, tF, dt)[0]
+        for thick in (3e-10, 1e-9, 3e-9, 1e-8, 3e-8, 5e-8, 1e-7, 1e-6):
+            for phase in (True, False):
+                a = np.where((i >= 1) & (i < 3), 1.0, 0.0)
+                if phase:
+                    a[i == 3] = 1.0 - dt + thick
+                else:
+                    a[i == 0] = dt - thick
+                want, _, st = om.advect(a.copy(), U, F, dt, bound=False)
+                assert st == 0
+                t, b = T(torch, a), T(torch, a)
+                ctx.advect(t, tU, tF, dt)
+                ctx.update(b, ctx.phase_flux(b, *ctx.reconstruct(b)[:3], Up, tF, lam, dt))
+                for got in (t, b):
+                    assert np.abs(got.cpu().numpy() - want).max() < 1e-11, (dt, thick, phase)
+    assert ctx.status() == 0
+    ctx.close()
