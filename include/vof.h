@@ -110,7 +110,10 @@ typedef struct {
     int device;     /* CUDA device ordinal */
 } vof_options;
 
-/* stats[] layout (doubles, device memory) written by vof_update / vof_advect */
+/* stats[] layout (doubles, device memory) written by vof_update / vof_advect.
+ * A NaN fraction shows in the masses and as MAX_PRE (MIN_PRE with its sign bit
+ * set); the redistribution passes leave it alone and the fallback sets it to 1
+ * (0 with its sign bit set). */
 enum {
     VOF_S_MASS_BEFORE = 0, VOF_S_MASS_AFTER, VOF_S_MIN_PRE, VOF_S_MAX_PRE, VOF_S_MIN_POST,
     VOF_S_MAX_POST, VOF_S_N_INTERFACE, VOF_S_N_BAND, VOF_S_MAX_POS_IT, VOF_S_MAX_CORR_IT,

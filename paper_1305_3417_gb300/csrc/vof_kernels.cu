@@ -1308,6 +1308,10 @@ __device__ __forceinline__ double lanes_sum(double v)
     return v;
 }
 __device__ __forceinline__ double recv_w(double a, double V) { return is_mixed(a) ? a * (1.0 - a) * V : 0.0; }
+// a source of a pass.  FP compares, not is_exc / is_def: a NaN fraction is no
+// source (it would make its neighbours NaN); it is left to the fallback.
+__device__ __forceinline__ bool src_exc(double a) { return a > 1.0 + BOUND_TOL; }
+__device__ __forceinline__ bool src_def(double a) { return a < -BOUND_TOL; }
 
 // Grid-wide barrier of a cooperative launch (every block resident): a block
 // arrives on the count; the last to arrive resets it and advances the generation
@@ -1489,7 +1493,7 @@ __global__ void __launch_bounds__(BA_THREADS, 1) k_bound_step(DevMesh m, BoundSt
                 const int c = a.src[i];
                 const double as = a.alpha[c];
                 double W = 0.0;
-                if (is_exc(as) || is_def(as))
+                if (src_exc(as) || src_def(as))
                     for_nbrs(m, c, [&](int nb) {
                         const double w = recv_w(a.alpha[nb], m.vc[nb]);
                         if (is_zero(w)) return;
@@ -1516,8 +1520,8 @@ __global__ void __launch_bounds__(BA_THREADS, 1) k_bound_step(DevMesh m, BoundSt
                 double Qp = 0.0, Qm = 0.0;
                 for_nbrs(m, r, [&](int s) {
                     const double as = a.alpha[s];
-                    const bool xe = is_exc(as);
-                    if (!xe && !is_def(as)) return;
+                    const bool xe = src_exc(as);
+                    if (!xe && !src_def(as)) return;
                     const double q = m.vc[s] * (wr * a.bs[BS_N * (size_t)s + BS_RW]);
                     if (xe) Qp += (as - 1.0) * q;
                     else Qm += -as * q;
@@ -1540,8 +1544,11 @@ __global__ void __launch_bounds__(BA_THREADS, 1) k_bound_step(DevMesh m, BoundSt
             for (int i = gl; i < n; i += ng) {
                 const int c = a.src[i];
                 const double as = a.alpha[c];
-                const bool xe = is_exc(as);
-                if (!xe && !is_def(as)) continue;
+                const bool xe = src_exc(as);
+                if (!xe && !src_def(as)) {
+                    if (first && as != as) atomicAdd(left, 1);
+                    continue;
+                }
                 const double rW = a.bs[BS_N * (size_t)c + BS_RW], V = m.vc[c];
                 double g = 0.0;
                 if (rW > 0.0) {
@@ -1559,7 +1566,7 @@ __global__ void __launch_bounds__(BA_THREADS, 1) k_bound_step(DevMesh m, BoundSt
                         a.alpha[c] = an;
                         touch(c);
                     }
-                    if (is_exc(an) || is_def(an)) atomicAdd(left, 1);
+                    if (src_exc(an) || src_def(an)) atomicAdd(left, 1);
                 }
             }
             for (int i = tl; i < nr; i += nt) {

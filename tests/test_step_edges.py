@@ -1,5 +1,6 @@
 """What a step does at its edges: shared memory handed between the lanes of a
-warp, settings changed between batch steps, cells of any aspect ratio.
+warp, settings changed between batch steps, cells of any aspect ratio,
+NaN fractions.
 
 FP64 is held to the replay tolerance against the oracle (1e-11).
 """
@@ -133,3 +134,33 @@ def test_sliver_along_needle_cells(torch, oracle_lib, aspect):
                     assert np.abs(got.cpu().numpy() - want).max() < 1e-11, (dt, thick, phase)
     assert ctx.status() == 0
     ctx.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nz", [32, 33])            # 2^15 cells: one cluster; above: every SM
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_nan_stays_out_of_the_redistribution(torch, nz, sign):
+    """A NaN fraction is neither source nor receiver of a local pass: every
+    other cell comes out as if that cell were full, bit for bit; the mesh-wide
+    fallback then sets it to 1 (0 with the sign bit set)."""
+    from paper_1305_3417_gb300 import vof
+    m = I.hex_mesh((32, 32, nz))
+    rng = np.random.default_rng(nz)
+    a = rng.uniform(0.2, 0.8, m.n_cells)
+    a[rng.uniform(size=m.n_cells) < 0.02] = 1.01    # excess with room all around
+    cells = [0, 32 * 32 * 16 + 500, m.n_cells - 1]
+    Va = T(torch, np.zeros(m.n_faces))
+    ctx = vof.VofContext(m)
+    out = []
+    for x in (1.0, np.copysign(np.nan, sign)):
+        b = a.copy()
+        b[cells] = x
+        t = T(torch, b)
+        st = ctx.update(t, Va).cpu().numpy()
+        out.append((t.cpu().numpy(), int(st[vof.S["bound_passes"]])))
+    ctx.close()
+    (full, p0), (got, p1) = out
+    assert p0 == p1 > 0 and full.max() <= 1.0 + 1e-13
+    assert np.all(got[cells] == (1.0 if sign > 0 else 0.0))
+    rest = np.setdiff1d(np.arange(m.n_cells), cells)
+    assert np.array_equal(got[rest], full[rest])
