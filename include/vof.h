@@ -17,7 +17,7 @@
  *   the legacy default stream) and allocates no memory: the context allocates
  *   all of its scratch in vof_create (the largest: the cell tetrahedra's planes,
  *   and the phase flux's queue of clip jobs, 512 bytes per face, 1024 in FP64;
- *   band faces that find no room in it are fluxed more slowly).
+ *   band faces that find no room in it are fluxed more slowly, to the same bits).
  * - Vectors are structure-of-arrays: x block, then y block, then z block.
  * - Face f of the mesh has points face_pts[face_ptr[f] .. face_ptr[f+1]),
  *   ordered so that the right-hand area vector S_f points from owner[f] to
@@ -415,7 +415,7 @@ int vof_profile_end(vof_ctx *ctx, double *group_ms, int *steps);
  *  [8] FP32 fill evaluations of the positioning, per cell tetrahedron,
  *  [9] face triangles whose swept prism enters the correction's cubic,
  *  [10] cubic evaluations of the correction,
- *  [11] reserved (0).
+ *  [11] band faces that found no room in the phase flux's queue of clip jobs.
  * [0]-[5] are FP32 work in a VOF_MIXED context and FP64 in a VOF_FP64 one,
  * where what a step decides in FP32 is not counted and four open distances of
  * its pair stage count as one piece-plane test;

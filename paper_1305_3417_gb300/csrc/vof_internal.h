@@ -67,9 +67,10 @@ enum { CNT_BAR = 32, CNT_BARGEN = 64, CNT_ALLOC = 96 };
 // plane, edge intersections, tetrahedron volumes, closed-form cut fractions,
 // plane shifts to the face frame -- and band faces; the reconstruction's fill
 // evaluations per cell tetrahedron (FP64, FP32); the correction's cubic
-// coefficient triangles and cubic evaluations (FP64)
+// coefficient triangles and cubic evaluations (FP64); the band faces that found
+// no room in the queue of clip jobs
 enum { WK_PRISM = 0, WK_TEST, WK_EDGE, WK_VOL, WK_FRAC, WK_SHIFT, WK_N, WK_FACES = WK_N, WK_FILL64, WK_FILL32,
-       WK_CTRI, WK_CEVAL, WK_LEN = 12 };
+       WK_CTRI, WK_CEVAL, WK_NOROOM, WK_LEN = 12 };
 
 // What the phase flux's pair stage starts a band face from, by band slot
 // (written by the correction): face centre, stencil range, face-point range,
@@ -148,8 +149,8 @@ struct vof_ctx {
     // grid multiplier over the resident blocks
     int pf_warps, pf_mult;
     // queue between the phase flux's pair and clip stages: batches of clip jobs
-    // (arena of 16-byte units, per batch its first unit, predecessor and sum),
-    // per unit of work its own sum and last batch, and the band slots without room
+    // (arena of 16-byte units, per batch its first unit, successor and sum),
+    // per unit of work its own sum and first batch, and the units without room
     BandRec *pf_rec;
     void *pf_arena;
     unsigned pf_cap;

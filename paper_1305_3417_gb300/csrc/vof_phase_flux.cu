@@ -172,13 +172,10 @@ struct MXArgs {
     double *Va;
     const int *list, *count;
     const void *disp;         // list form: displacements of a face's centre and points, in the form's type
-    const double *lam_b;
     unsigned *status;
     unsigned long long *work;
     const void *fpl, *cbl, *ktl;  // the context's tables (R4 of the form's type)
     const int *ctptr;
-    int *next;                // list form: next band slot to take (zero before the launch), or null
-    const int *items;         // list form: the band slots to take (null: 0 .. count - 1)
 };
 
 constexpr int MX_CAND = 32;    // candidate cell tetrahedra buffered per warp: one per lane
@@ -934,7 +931,7 @@ __device__ __forceinline__ void mx_merge(Acc<R> &acc)
     }
 }
 
-template <class R, int MX_STACK, bool LIST, class Wk>
+template <class R, int MX_STACK, class Wk>
 __device__ __forceinline__ void phase_flux_body(const DevMesh &m, const MXArgs &a, MXShared<R, MX_STACK> &sh)
 {
     using V = R3<R>;
@@ -943,25 +940,11 @@ __device__ __forceinline__ void phase_flux_body(const DevMesh &m, const MXArgs &
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int total = LIST ? *a.count : m.nf;
     const double eps = m.eps;
-    // Band faces differ in cost by an order of magnitude (a face whose
-    // polyhedron cuts interface cells clips, one among uniform cells hardly
-    // does): in the list form a warp takes its next face from a counter as it
-    // finishes one, so that no warp ends long after the others; a face's flux
-    // is one warp's work either way.
-    const bool dyn = LIST && a.next != nullptr;
-    auto take = [&]() {
-        int v = 0;
-        if (lane == 0) v = atomicAdd(a.next, 1);
-        return __shfl_sync(0xffffffffu, v, 0);
-    };
     Wk wk;
-    for (int it = dyn ? take() : warp; it < total; it = dyn ? take() : it + nwarps) {
-        const int item = LIST && a.items ? a.items[it] : it;
-        const int f = LIST ? a.list[item] : item;
+    for (int f = warp; f < m.nf; f += nwarps) {
         const long long s0 = __ldg(m.sptr + f), s1 = __ldg(m.sptr + f + 1);
-        if (!LIST) {
+        {
             double Ff = a.F[f];
             bool all_e = true, all_f = true;
             for (long long s = s0 + lane; s < s1; s += 32) {
@@ -986,7 +969,7 @@ __device__ __forceinline__ void phase_flux_body(const DevMesh &m, const MXArgs &
         const V3 o = ld3(m.cf, m.nf, f);
         const int b = __ldg(m.fptr + f), n = __ldg(m.fptr + f + 1) - b;
         bool decide, comp;
-        pf_form(m, a.F, a.alpha, f, LIST ? a.lam_b[item] : a.lambda[f], s1 - s0, decide, comp);
+        pf_form(m, a.F, a.alpha, f, a.lambda[f], s1 - s0, decide, comp);
         const int nt = n == 3 ? 3 : 3 * n;
         // signed distances (to unit-normal planes) within the on-plane band of
         // the face (FP32: 2e-6 of the face size, FP64: 1e-14) are taken as zero:
@@ -994,7 +977,7 @@ __device__ __forceinline__ void phase_flux_body(const DevMesh &m, const MXArgs &
         // different roundings and would otherwise look like cuts
         const R tol = ldg4(fpl, b).w;
         R pb[6];
-        mx_poly<R, LIST, true, R>(m, a, sh, item, f, b, n, nt, pb);
+        mx_poly<R, false, true, R>(m, a, sh, 0, f, b, n, nt, pb);
         Acc<R> acc;
         wk.add(WK_VOL, lane < nt);  // the flux polyhedron's tetrahedra
         wk.face();
@@ -1086,8 +1069,7 @@ template <class R, int W, class Wk>
 __global__ void __launch_bounds__(W * 32, 8) k_phase_flux(DevMesh m, MXArgs a)
 {
     extern __shared__ __align__(16) unsigned char pf_smem[];
-    phase_flux_body<R, MX_STACK_WIDE, false, Wk>(m, a,
-                                                 reinterpret_cast<MXShared<R, MX_STACK_WIDE> *>(pf_smem)[threadIdx.x >> 5]);
+    phase_flux_body<R, MX_STACK_WIDE, Wk>(m, a, reinterpret_cast<MXShared<R, MX_STACK_WIDE> *>(pf_smem)[threadIdx.x >> 5]);
 }
 
 
@@ -1099,9 +1081,10 @@ __global__ void __launch_bounds__(W * 32, 8) k_phase_flux(DevMesh m, MXArgs a)
 //    go to the context's queue as one batch with what their clipping reads
 //    (planes, prism points), the tetrahedra inside every plane are summed here;
 //  - clips (k_pf_clip): a warp per batch works the jobs' pieces off;
-//  - sums (k_pf_finish): a thread per band face adds its batches and writes
-//    V_alpha; faces whose batches found no room in the queue are fluxed whole
-//    there, a warp each.
+//  - sums (k_pf_finish): a lane per unit of work adds its batches, the units of a
+//    face make its V_alpha; faces whose batches found no room in the queue go through the pair
+//    stage again there, a warp each, which clips every batch at once: the same
+//    batches, pieces and sums, so which faces found room changes no bit.
 // One launch that did all of it per face kept 16 warps on an SM (128 registers,
 // 13.6 KB of shared memory a warp) at 54 % of the issue slots, and took as long
 // as its slowest face where there are fewer faces than warps; the stages by
@@ -1115,12 +1098,12 @@ struct PfQueue {
     unsigned cap;                 // units
     unsigned long long *ctr;      // units taken (low word), batches (high word)
     unsigned *boff;               // per batch: first unit, or PF_NONE
-    int *bnext;                   // per batch: the unit's previous batch, -1
+    int *bnext;                   // per batch: the unit's next batch, -1
     double *part;                 // per batch: 6 x its volume
     int bcap;
     double *base;                 // per unit of work: 6 x the volume summed by the pair stage
-    int2 *head;                   // per unit: last batch (-1 none, PF_FAIL), complement form
-    int *ovf, *novf;              // band slots without room
+    int2 *head;                   // per unit: first batch (-1 none, PF_FAIL), complement form
+    int *ovf, *novf;              // units without room
     int *next_pair, *next_clip, *next_ovf;
     int pair_warps;               // warps of the pair launch
 };
@@ -1370,17 +1353,237 @@ template <class R> __device__ __forceinline__ double get_sum(const double *a, in
     } else return a[i];
 }
 
+// a band face's record, a quarter in each of the first four lanes
+struct PfFace {
+    int f, b, n, nt;
+    long long s0, s1;
+    bool decide, comp;
+};
+// (what only some stages need waits in shared memory, not in registers; lane 0
+// of the record holds ox and oy, lane 1 oz)
+template <class R>
+__device__ __forceinline__ PfFace pf_face(const uint4 &rec, PairShared<R> &sh)
+{
+    const int lane = threadIdx.x & 31;
+    auto word = [&](unsigned v, int l) { return __shfl_sync(0xffffffffu, v, l); };
+    if (lane < 2) {
+        sh.o[2 * lane] = __hiloint2double((int)rec.y, (int)rec.x);
+        if (lane == 0) sh.o[1] = __hiloint2double((int)rec.w, (int)rec.z);
+    }
+    PfFace p;
+    p.s0 = (long long)((unsigned long long)word(rec.w, 1) << 32 | word(rec.z, 1));
+    p.f = (int)word(rec.x, 2);
+    p.b = (int)word(rec.y, 2);
+    p.n = (int)word(rec.z, 2);
+    p.s1 = p.s0 + (int)word(rec.w, 2);
+    const unsigned form = word(rec.x, 3);
+    p.decide = form & 2u;
+    p.comp = form & 1u;
+    p.nt = p.n == 3 ? 3 : 3 * p.n;
+    return p;
+}
+
+// its flux polyhedron, and the box's numbers
+template <class R>
+__device__ __forceinline__ void pf_poly(const DevMesh &m, const MXArgs &a, PairShared<R> &sh, int item, const PfFace &p)
+{
+    using B = float;
+    const R tol = ldg4(static_cast<const R4<R> *>(a.fpl), p.b).w;
+    B pb[6];
+    mx_poly<R, true, false, B>(m, a, sh, item, p.f, p.b, p.n, p.nt, pb);
+    if ((threadIdx.x & 31) == 0) {
+        const B hf = B(0.5);
+        sh.X[0] = mk4<B>(pb[0], pb[1], pb[2], box_slack<B>(pb));
+        sh.X[1] = mk4<B>(pb[3], pb[4], pb[5], (B)tol);
+        sh.X[2] = mk4<B>(hf * (pb[0] + pb[3]), hf * (pb[1] + pb[4]), hf * (pb[2] + pb[5]), B(0));
+        sh.X[3] = mk4<B>(hf * (pb[3] - pb[0]), hf * (pb[4] - pb[1]), hf * (pb[5] - pb[2]), B(0));
+    }
+}
+template <class R>
+__device__ __forceinline__ float pf_drop(const PairShared<R> &sh)
+{
+    const float4 lo = sh.X[0], hi = sh.X[1];
+    const float box[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
+    return drop_slack(box);
+}
+
+// The pairs of part 'part' of 2^ls of a face: volumes inside every plane go to
+// acc, and sink(nq, used, tol) gets the clip jobs of up to 32 candidates at a time
+// (sh.Q, nq of them; used: the candidates that have any; sh.Kp, sh.Kw).
+template <class R, class Wk, class Sink>
+__device__ __forceinline__ void pf_stencil(const DevMesh &m, const MXArgs &a, PairShared<R> &sh, const PfFace &p, int part,
+                                           int ls, bool &comp, Acc<R> &acc, Wk &wk, Sink sink)
+{
+    constexpr bool F64 = std::is_same<R, double>::value;
+    using B = float;  // boxes
+    const R4<R> *fpl = static_cast<const R4<R> *>(a.fpl);
+    const R4<R> *ktl = static_cast<const R4<R> *>(a.ktl);
+    const int lane = threadIdx.x & 31, msk = (1 << ls) - 1;
+    const unsigned lt = (1u << lane) - 1u;
+    const long long s0 = p.s0, s1 = p.s1;
+    const int b = p.b, nt = p.nt;
+    const bool decide = p.decide;
+    // The stencil is taken 32 cells at a time, one per lane, then the
+    // tetrahedra of those that reach the polyhedron, 32 at a time (a part
+    // takes every 2^ls-th such batch): those whose boxes reach it go to a
+    // ring; from the ring, 32 lanes wide, a tetrahedron gets its planes, is
+    // dropped where the polyhedron's box lies beyond one, and else becomes a
+    // candidate; from PF_FLUSH candidates on the pairs are classified.
+    long long sc = s0 - 32;
+    int tb = 0, ntot = 0, ncell = 0, bt = 0;
+    int base = 0, cnt = 0, nk = 0;  // ring: first entry, entries; candidates
+    for (;;) {
+        const bool cdone = tb >= ntot;
+        if (cnt >= 32 || (cdone && cnt > 0)) {
+            // ---- planes of the ring's first tetrahedra
+            const int nr = min(cnt, MX_CAND - nk);
+            bool keep = false;
+            R4<R> kp[4], H;
+            B kbx[6];
+            float4 kf[4], hf4;
+            float mg = 0.0f;
+            int ci = 0;
+            if (lane < nr) {
+                const int e = (base + lane) & (PF_RING - 1);
+                ci = sh.Cc[e];
+                const size_t j = sh.Cj[e];
+                const R4<R> dc = sh.Cd[ci];
+                const R3<float> df = r3(tof(dc.x), tof(dc.y), tof(dc.z));
+                H = sh.CH[ci];
+                const bool useH = sh.CuseH[ci];
+                const R4<R> b0 = ldg4(ktl, 6 * j + 4), b1 = ldg4(ktl, 6 * j + 5);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) kp[i] = ldg4(ktl, 6 * j + i);
+                kbx[0] = tof(b0.x) + df.x; kbx[1] = tof(b0.y) + df.y; kbx[2] = tof(b0.z) + df.z;
+                kbx[3] = tof(b1.x) + df.x; kbx[4] = tof(b1.y) + df.y; kbx[5] = tof(b1.z) + df.z;
+                const float4 pce = sh.X[2], phe = sh.X[3];
+                keep = true;
+                if constexpr (F64) {
+                    // allowance: a few FP32 roundings of what enters a distance
+                    const float rs = sh.X[0].w * 2e6f + fmaxf(fabsf(df.x), fmaxf(fabsf(df.y), fabsf(df.z))) +
+                                     fmaxf(fabsf(tof(kp[3].w)), fabsf(tof(H.w)));
+                    mg = 2e-6f * rs;
+                } else mg = sh.X[0].w;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const R4<R> pl = kp[i];
+                    if constexpr (F64) {
+                        kf[i] = make_float4(tof(pl.x), tof(pl.y), tof(pl.z), 0.0f);
+                        kf[i].w = tof(pl.w) + (kf[i].x * df.x + kf[i].y * df.y + kf[i].z * df.z);
+                        keep = keep && !beyond<float>(kf[i], pce, phe, mg);
+                    } else {
+                        wk.add(WK_SHIFT, 1);
+                        kp[i] = mk4<R>(pl.x, pl.y, pl.z, pl.w + (pl.x * dc.x + pl.y * dc.y + pl.z * dc.z));
+                        keep = keep && !beyond<R>(kp[i], pce, phe, mg);
+                    }
+                }
+                hf4 = make_float4(tof(H.x), tof(H.y), tof(H.z), tof(H.w));
+                keep = keep && !(useH && beyond<float>(hf4, pce, phe, mg));
+                if (!useH) hf4 = make_float4(0.0f, 0.0f, 0.0f, 1.0f);  // (nothing is beyond it)
+            }
+            const unsigned km = __ballot_sync(0xffffffffu, keep);
+            if (keep) {
+                const int r = nk + __popc(km & lt);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) sh.Kp[r][i] = kp[i];
+                sh.Kp[r][4] = H;
+#pragma unroll
+                for (int i = 0; i < 6; ++i) sh.Kb[r][i] = kbx[i];
+                if constexpr (F64) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) sh.Kf[r][i] = kf[i];
+                    sh.Kf[r][4] = hf4;
+                    sh.Km[r] = mg;
+                    const D4 dc = sh.Cd[ci];
+                    sh.Kdc[r][0] = dc.x; sh.Kdc[r][1] = dc.y; sh.Kdc[r][2] = dc.z;
+                }
+                sh.Kw[r] = sh.Cw[ci];
+                sh.KuseH[r] = sh.CuseH[ci];
+            }
+            nk += __popc(km);
+            base = (base + nr) & (PF_RING - 1);
+            cnt -= nr;
+            __syncwarp();
+            if (nk < PF_FLUSH) continue;
+        } else if (!cdone) {
+            // ---- boxes of the part's next batch of 32 tetrahedra
+            // the cell of tetrahedron tb + lane: the cells that end at or
+            // before tb, plus one for each cell that ends inside the batch at
+            // or before this lane (cell 'lane' ends rel tetrahedra after tb)
+            const int rel = lane < ncell ? sh.Cend[lane] - tb : 0x7fffffff;
+            const unsigned ends = __reduce_or_sync(0xffffffffu, rel > 0 && rel < 32 ? 1u << rel : 0u);
+            const int ci = __popc(__ballot_sync(0xffffffffu, rel <= 0)) + __popc(ends & (((1u << lane) << 1) - 1u));
+            bool cand = false;
+            int j = 0;
+            if (tb + lane < ntot) {
+                const R4<R> dc = sh.Cd[ci];
+                j = bits_int(dc.w) + tb + lane;
+                const R4<R> b0 = ldg4(ktl, 6 * (size_t)j + 4), b1 = ldg4(ktl, 6 * (size_t)j + 5);
+                const float4 lo = sh.X[0], hi = sh.X[1];
+                if constexpr (F64) {
+                    auto apart = [](float l, float h, double c0, double c1, double s) {
+                        const float d = tf(s), f0 = tf(c0), f1 = tf(c1);
+                        const float w = 5e-7f * (fabsf(d) + fabsf(f0) + fabsf(f1));
+                        return l > f1 + d + w || f0 + d - w > h;
+                    };
+                    cand = !(apart(lo.x, hi.x, b0.x, b1.x, dc.x) || apart(lo.y, hi.y, b0.y, b1.y, dc.y) ||
+                             apart(lo.z, hi.z, b0.z, b1.z, dc.z));
+                } else
+                    cand = !(rgt(lo.x, b1.x + dc.x) || rgt(b0.x + dc.x, hi.x) || rgt(lo.y, b1.y + dc.y) ||
+                             rgt(b0.y + dc.y, hi.y) || rgt(lo.z, b1.z + dc.z) || rgt(b0.z + dc.z, hi.z));
+            }
+            const unsigned cmask = __ballot_sync(0xffffffffu, cand);
+            if (cand) {
+                const int e = (base + cnt + __popc(cmask & lt)) & (PF_RING - 1);
+                sh.Cj[e] = j;
+                sh.Cc[e] = (unsigned char)ci;
+            }
+            cnt += __popc(cmask);
+            tb += 32 << ls;
+            __syncwarp();
+            continue;
+        } else {
+            // ---- next chunk
+            sc += 32;
+            bt += (ntot + 31) >> 5;
+            tb = ((part - bt) & msk) << 5;
+            ntot = 0;
+            if (sc < s1) {
+                const float4 lo = sh.X[0], hi = sh.X[1];
+                const B pb[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
+                mx_chunk<R, B>(m, a, sh, sc, s1, mk(sh.o[0], sh.o[1], sh.o[2]), pb, decide, comp, ntot, ncell);
+                continue;
+            }
+        }
+        // ---- pairs and clip jobs of the candidates
+        if (nk > 0) {
+            unsigned used;
+            int nq;
+            R tol;
+            if constexpr (F64) tol = ldg4(fpl, b).w;
+            else tol = sh.X[1].w;
+            if constexpr (F64) nq = pf_pairs64(sh, nt, nk, tol, acc, used, wk);
+            else {
+                R kb[6];
+#pragma unroll
+                for (int i = 0; i < 6; ++i) kb[i] = lane < nk ? sh.Kb[lane][i] : R(0);
+                nq = mx_pairs(sh, nt, nk, kb, tol, sh.X[0].w, acc, used, wk);
+            }
+            if (nq > 0) sink(nq, used, tol);
+            nk = 0;
+            __syncwarp();
+        }
+        if (cdone && cnt == 0 && sc >= s1) break;
+    }
+}
+
 template <class R, class Wk>
 __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a, const PfQueue &q, PairShared<R> &sh)
 {
     constexpr bool F64 = std::is_same<R, double>::value;
-    using B = float;  // boxes
-    using V = R3<R>;
-    const R4<R> *fpl = static_cast<const R4<R> *>(a.fpl);
-    const R4<R> *ktl = static_cast<const R4<R> *>(a.ktl);
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
-    const int total = *a.count, ls = pf_split(total, q.pair_warps), units = total << ls, msk = (1 << ls) - 1;
+    const int total = *a.count, ls = pf_split(total, q.pair_warps), units = total << ls;
     // the next unit is taken, and its record read (16 bytes by each of four
     // lanes), while the current one is worked on; with few units a warp takes it
     // when it is done, not ahead of a warp that is free (24^3 hexahedra, 1.6
@@ -1396,251 +1599,83 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
     int unit = __shfl_sync(0xffffffffu, take(), 0);
     uint4 rec = record(unit);
     while (unit < units) {
-        const int item = unit >> ls, part = unit & msk;
-        auto word = [&](unsigned v, int l) { return __shfl_sync(0xffffffffu, v, l); };
-        // (what only some stages need waits in shared memory, not in registers;
-        // lane 0 of the record holds ox and oy, lane 1 oz)
-        if (lane < 2) {
-            sh.o[2 * lane] = __hiloint2double((int)rec.y, (int)rec.x);
-            if (lane == 0) sh.o[1] = __hiloint2double((int)rec.w, (int)rec.z);
-        }
-        const long long s0 = (long long)((unsigned long long)word(rec.w, 1) << 32 | word(rec.z, 1));
-        const int f = (int)word(rec.x, 2), b = (int)word(rec.y, 2), n = (int)word(rec.z, 2);
-        const long long s1 = s0 + (int)word(rec.w, 2);
-        const unsigned form = word(rec.x, 3);
-        const bool decide = form & 2u;
-        bool comp = form & 1u;
+        const int item = unit >> ls, part = unit & ((1 << ls) - 1);
+        const PfFace p = pf_face(rec, sh);
         const int taken = ahead ? take() : 0;
-        const int nt = n == 3 ? 3 : 3 * n, nprism = nt / 3;
-        {
-            const R tol = ldg4(fpl, b).w;
-            B pb[6];
-            mx_poly<R, true, false, B>(m, a, sh, item, f, b, n, nt, pb);
-            if (lane == 0) {
-                const B hf = B(0.5);
-                sh.X[0] = mk4<B>(pb[0], pb[1], pb[2], box_slack<B>(pb));
-                sh.X[1] = mk4<B>(pb[3], pb[4], pb[5], (B)tol);
-                sh.X[2] = mk4<B>(hf * (pb[0] + pb[3]), hf * (pb[1] + pb[4]), hf * (pb[2] + pb[5]), B(0));
-                sh.X[3] = mk4<B>(hf * (pb[3] - pb[0]), hf * (pb[4] - pb[1]), hf * (pb[5] - pb[2]), B(0));
-            }
-        }
+        pf_poly(m, a, sh, item, p);
         int next = __shfl_sync(0xffffffffu, taken, 0);
         if (ahead) rec = record(next);
         __syncwarp();
         Acc<R> acc;
         if (part == 0) {
-            wk.add(WK_VOL, lane < nt);  // the flux polyhedron's tetrahedra
+            wk.add(WK_VOL, lane < p.nt);  // the flux polyhedron's tetrahedra
             wk.face();
         }
-        int head = -1;
-        // The stencil is taken 32 cells at a time, one per lane, then the
-        // tetrahedra of those that reach the polyhedron, 32 at a time (a part
-        // takes every 2^ls-th such batch): those whose boxes reach it go to a
-        // ring; from the ring, 32 lanes wide, a tetrahedron gets its planes, is
-        // dropped where the polyhedron's box lies beyond one, and else becomes a
-        // candidate; from PF_FLUSH candidates on the pairs are classified.
-        long long sc = s0 - 32;
-        int tb = 0, ntot = 0, ncell = 0, bt = 0;
-        int base = 0, cnt = 0, nk = 0;  // ring: first entry, entries; candidates
-        for (;;) {
-            const bool cdone = tb >= ntot;
-            if (cnt >= 32 || (cdone && cnt > 0)) {
-                // ---- planes of the ring's first tetrahedra
-                const int nr = min(cnt, MX_CAND - nk);
-                bool keep = false;
-                R4<R> kp[4], H;
-                B kbx[6];
-                float4 kf[4], hf4;
-                float mg = 0.0f;
-                int ci = 0;
-                if (lane < nr) {
-                    const int e = (base + lane) & (PF_RING - 1);
-                    ci = sh.Cc[e];
-                    const size_t j = sh.Cj[e];
-                    const R4<R> dc = sh.Cd[ci];
-                    const R3<float> df = r3(tof(dc.x), tof(dc.y), tof(dc.z));
-                    H = sh.CH[ci];
-                    const bool useH = sh.CuseH[ci];
-                    const R4<R> b0 = ldg4(ktl, 6 * j + 4), b1 = ldg4(ktl, 6 * j + 5);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) kp[i] = ldg4(ktl, 6 * j + i);
-                    kbx[0] = tof(b0.x) + df.x; kbx[1] = tof(b0.y) + df.y; kbx[2] = tof(b0.z) + df.z;
-                    kbx[3] = tof(b1.x) + df.x; kbx[4] = tof(b1.y) + df.y; kbx[5] = tof(b1.z) + df.z;
-                    const float4 pce = sh.X[2], phe = sh.X[3];
-                    keep = true;
-                    if constexpr (F64) {
-                        // allowance: a few FP32 roundings of what enters a distance
-                        const float rs = sh.X[0].w * 2e6f + fmaxf(fabsf(df.x), fmaxf(fabsf(df.y), fabsf(df.z))) +
-                                         fmaxf(fabsf(tof(kp[3].w)), fabsf(tof(H.w)));
-                        mg = 2e-6f * rs;
-                    } else mg = sh.X[0].w;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const R4<R> pl = kp[i];
-                        if constexpr (F64) {
-                            kf[i] = make_float4(tof(pl.x), tof(pl.y), tof(pl.z), 0.0f);
-                            kf[i].w = tof(pl.w) + (kf[i].x * df.x + kf[i].y * df.y + kf[i].z * df.z);
-                            keep = keep && !beyond<float>(kf[i], pce, phe, mg);
-                        } else {
-                            wk.add(WK_SHIFT, 1);
-                            kp[i] = mk4<R>(pl.x, pl.y, pl.z, pl.w + (pl.x * dc.x + pl.y * dc.y + pl.z * dc.z));
-                            keep = keep && !beyond<R>(kp[i], pce, phe, mg);
-                        }
-                    }
-                    hf4 = make_float4(tof(H.x), tof(H.y), tof(H.z), tof(H.w));
-                    keep = keep && !(useH && beyond<float>(hf4, pce, phe, mg));
-                    if (!useH) hf4 = make_float4(0.0f, 0.0f, 0.0f, 1.0f);  // (nothing is beyond it)
-                }
-                const unsigned km = __ballot_sync(0xffffffffu, keep);
-                if (keep) {
-                    const int r = nk + __popc(km & lt);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) sh.Kp[r][i] = kp[i];
-                    sh.Kp[r][4] = H;
-#pragma unroll
-                    for (int i = 0; i < 6; ++i) sh.Kb[r][i] = kbx[i];
-                    if constexpr (F64) {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) sh.Kf[r][i] = kf[i];
-                        sh.Kf[r][4] = hf4;
-                        sh.Km[r] = mg;
-                        const D4 dc = sh.Cd[ci];
-                        sh.Kdc[r][0] = dc.x; sh.Kdc[r][1] = dc.y; sh.Kdc[r][2] = dc.z;
-                    }
-                    sh.Kw[r] = sh.Cw[ci];
-                    sh.KuseH[r] = sh.CuseH[ci];
-                }
-                nk += __popc(km);
-                base = (base + nr) & (PF_RING - 1);
-                cnt -= nr;
-                __syncwarp();
-                if (nk < PF_FLUSH) continue;
-            } else if (!cdone) {
-                // ---- boxes of the part's next batch of 32 tetrahedra
-                // the cell of tetrahedron tb + lane: the cells that end at or
-                // before tb, plus one for each cell that ends inside the batch at
-                // or before this lane (cell 'lane' ends rel tetrahedra after tb)
-                const int rel = lane < ncell ? sh.Cend[lane] - tb : 0x7fffffff;
-                const unsigned ends = __reduce_or_sync(0xffffffffu, rel > 0 && rel < 32 ? 1u << rel : 0u);
-                const int ci = __popc(__ballot_sync(0xffffffffu, rel <= 0)) + __popc(ends & (((1u << lane) << 1) - 1u));
-                bool cand = false;
-                int j = 0;
-                if (tb + lane < ntot) {
-                    const R4<R> dc = sh.Cd[ci];
-                    j = bits_int(dc.w) + tb + lane;
-                    const R4<R> b0 = ldg4(ktl, 6 * (size_t)j + 4), b1 = ldg4(ktl, 6 * (size_t)j + 5);
-                    const float4 lo = sh.X[0], hi = sh.X[1];
-                    if constexpr (F64) {
-                        auto apart = [](float l, float h, double c0, double c1, double s) {
-                            const float d = tf(s), f0 = tf(c0), f1 = tf(c1);
-                            const float w = 5e-7f * (fabsf(d) + fabsf(f0) + fabsf(f1));
-                            return l > f1 + d + w || f0 + d - w > h;
-                        };
-                        cand = !(apart(lo.x, hi.x, b0.x, b1.x, dc.x) || apart(lo.y, hi.y, b0.y, b1.y, dc.y) ||
-                                 apart(lo.z, hi.z, b0.z, b1.z, dc.z));
-                    } else
-                        cand = !(rgt(lo.x, b1.x + dc.x) || rgt(b0.x + dc.x, hi.x) || rgt(lo.y, b1.y + dc.y) ||
-                                 rgt(b0.y + dc.y, hi.y) || rgt(lo.z, b1.z + dc.z) || rgt(b0.z + dc.z, hi.z));
-                }
-                const unsigned cmask = __ballot_sync(0xffffffffu, cand);
-                if (cand) {
-                    const int e = (base + cnt + __popc(cmask & lt)) & (PF_RING - 1);
-                    sh.Cj[e] = j;
-                    sh.Cc[e] = (unsigned char)ci;
-                }
-                cnt += __popc(cmask);
-                tb += 32 << ls;
-                __syncwarp();
-                continue;
-            } else {
-                // ---- next chunk
-                sc += 32;
-                bt += (ntot + 31) >> 5;
-                tb = ((part - bt) & msk) << 5;
-                ntot = 0;
-                if (sc < s1) {
-                    const float4 lo = sh.X[0], hi = sh.X[1];
-                    const B pb[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
-                    mx_chunk<R, B>(m, a, sh, sc, s1, mk(sh.o[0], sh.o[1], sh.o[2]), pb, decide, comp, ntot, ncell);
-                    continue;
-                }
-            }
-            // ---- pairs and clip jobs of the candidates
-            if (nk > 0) {
-                unsigned used;
-                int nq;
-                R tol;
-                if constexpr (F64) tol = ldg4(fpl, b).w;
-                else tol = sh.X[1].w;
-                if constexpr (F64) nq = pf_pairs64(sh, nt, nk, tol, acc, used, wk);
+        bool comp = p.comp;
+        int last = -1;
+        pf_stencil(m, a, sh, p, part, ls, comp, acc, wk, [&](int nq, unsigned used, R tol) {
+            if (last == PF_FAIL) return;
+            const int nt = p.nt, nprism = nt / 3;
+            // the jobs, as a batch of the queue (a warp that found no
+            // room once adds nothing more: the counter stays near the
+            // capacity, far from overflowing its halves)
+            const int nu = __popc(used);
+            const PfLayout<R> L(nprism, nu, nq);
+            unsigned off = PF_NONE;
+            int bi = -1;
+            if (lane == 0 && !full) {
+                const unsigned long long old = atomicAdd(q.ctr, (1ull << 32) | L.end);
+                off = (unsigned)old;
+                bi = (int)(old >> 32);
+                if (bi >= q.bcap) bi = -1;
+                else if (off > q.cap || L.end > q.cap - off) { q.boff[bi] = PF_NONE; bi = -1; }
                 else {
-                    R kb[6];
-#pragma unroll
-                    for (int i = 0; i < 6; ++i) kb[i] = lane < nk ? sh.Kb[lane][i] : R(0);
-                    nq = mx_pairs(sh, nt, nk, kb, tol, sh.X[0].w, acc, used, wk);
+                    q.boff[bi] = off;
+                    q.bnext[bi] = -1;
+                    if (last < 0) q.head[unit].x = bi;
+                    else q.bnext[last] = bi;
                 }
-                if (nq > 0 && head != PF_FAIL) {
-                    // the jobs, as a batch of the queue (a warp that found no
-                    // room once adds nothing more: the counter stays near the
-                    // capacity, far from overflowing its halves)
-                    const int nu = __popc(used);
-                    const PfLayout<R> L(nprism, nu, nq);
-                    unsigned off = PF_NONE;
-                    int bi = -1;
-                    if (lane == 0 && !full) {
-                        const unsigned long long old = atomicAdd(q.ctr, (1ull << 32) | L.end);
-                        off = (unsigned)old;
-                        bi = (int)(old >> 32);
-                        if (bi >= q.bcap) bi = -1;
-                        else if (off > q.cap || L.end > q.cap - off) { q.boff[bi] = PF_NONE; bi = -1; }
-                        else { q.boff[bi] = off; q.bnext[bi] = head; }
-                    }
-                    if (used >> lane & 1u) sh.Kmap[__popc(used & lt)] = (unsigned char)lane;
-                    __syncwarp();  // the map and the job codes are read by other lanes below
-                    const R sg = lane < nt ? sh.Tsg[lane] : R(0);
-                    const unsigned pos = __ballot_sync(0xffffffffu, sg > R(0)), neg = __ballot_sync(0xffffffffu, sg < R(0));
-                    off = __shfl_sync(0xffffffffu, off, 0);
-                    bi = __shfl_sync(0xffffffffu, bi, 0);
-                    head = bi < 0 ? PF_FAIL : bi;
-                    full = bi < 0;
-                    if (bi >= 0) {
-                        uint4 *ob = q.arena + off;
-                        if (lane == 0) {
-                            ob[0] = make_uint4((unsigned)nq | (unsigned)nu << 16 | (unsigned)nprism << 24, pos, neg, 0u);
-                            if constexpr (F64) {
-                                const DBits t = dbits(tol);
-                                const float4 lo = sh.X[0], hi = sh.X[1];
-                                const float box[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
-                                ob[1] = make_uint4(t.lo, (unsigned)t.hi, __float_as_uint(drop_slack(box)), 0u);
-                            } else ob[1] = make_uint4(__float_as_uint(tol), 0u, 0u, 0u);
-                        }
-                        const uint4 *ps = reinterpret_cast<const uint4 *>(sh.P6);
-                        for (unsigned i = lane; i < nprism * 5 * L.RW; i += 32) ob[L.P + i] = ps[i];
-                        R4<R> *ok = reinterpret_cast<R4<R> *>(ob + L.K);
-                        for (int i = lane; i < nu * 5; i += 32) {
-                            const int k = sh.Kmap[i / 5], c = i % 5;
-                            ok[i] = sh.Kp[k][c];
-                        }
-                        if (lane < nu) reinterpret_cast<R *>(ob + L.W)[lane] = sh.Kw[sh.Kmap[lane]];
-                        auto code = [&](int i) -> unsigned {  // candidates renumbered among those used
-                            if (i >= nq) return 0u;
-                            const unsigned v = sh.Q[i], k = v >> 5 & 31;
-                            return (v & ~(31u << 5)) | (unsigned)__popc(used & ((1u << k) - 1u)) << 5;
-                        };
-                        unsigned *oq = reinterpret_cast<unsigned *>(ob + L.Q);
-                        for (int i = lane; 2 * i < nq; i += 32) oq[i] = code(2 * i) | code(2 * i + 1) << 16;
-                    }
-                }
-                nk = 0;
-                __syncwarp();
             }
-            if (cdone && cnt == 0 && sc >= s1) break;
-        }
+            if (used >> lane & 1u) sh.Kmap[__popc(used & lt)] = (unsigned char)lane;
+            __syncwarp();  // the map and the job codes are read by other lanes below
+            const R sg = lane < nt ? sh.Tsg[lane] : R(0);
+            const unsigned pos = __ballot_sync(0xffffffffu, sg > R(0)), neg = __ballot_sync(0xffffffffu, sg < R(0));
+            off = __shfl_sync(0xffffffffu, off, 0);
+            bi = __shfl_sync(0xffffffffu, bi, 0);
+            last = bi < 0 ? PF_FAIL : bi;
+            full = bi < 0;
+            if (bi >= 0) {
+                uint4 *ob = q.arena + off;
+                if (lane == 0) {
+                    ob[0] = make_uint4((unsigned)nq | (unsigned)nu << 16 | (unsigned)nprism << 24, pos, neg, 0u);
+                    if constexpr (F64) {
+                        const DBits t = dbits(tol);
+                        ob[1] = make_uint4(t.lo, (unsigned)t.hi, __float_as_uint(pf_drop(sh)), 0u);
+                    } else ob[1] = make_uint4(__float_as_uint(tol), 0u, 0u, 0u);
+                }
+                const uint4 *ps = reinterpret_cast<const uint4 *>(sh.P6);
+                for (unsigned i = lane; i < nprism * 5 * L.RW; i += 32) ob[L.P + i] = ps[i];
+                R4<R> *ok = reinterpret_cast<R4<R> *>(ob + L.K);
+                for (int i = lane; i < nu * 5; i += 32) {
+                    const int k = sh.Kmap[i / 5], c = i % 5;
+                    ok[i] = sh.Kp[k][c];
+                }
+                if (lane < nu) reinterpret_cast<R *>(ob + L.W)[lane] = sh.Kw[sh.Kmap[lane]];
+                auto code = [&](int i) -> unsigned {  // candidates renumbered among those used
+                    if (i >= nq) return 0u;
+                    const unsigned v = sh.Q[i], k = v >> 5 & 31;
+                    return (v & ~(31u << 5)) | (unsigned)__popc(used & ((1u << k) - 1u)) << 5;
+                };
+                unsigned *oq = reinterpret_cast<unsigned *>(ob + L.Q);
+                for (int i = lane; 2 * i < nq; i += 32) oq[i] = code(2 * i) | code(2 * i + 1) << 16;
+            }
+        });
         mx_merge(acc);
         if (lane == 0) {
             put_sum(q.base, unit, acc);
-            q.head[unit] = make_int2(head, comp);
-            if (head == PF_FAIL) q.ovf[atomicAdd(q.novf, 1)] = item;
+            q.head[unit].y = comp;
+            if (last < 0) q.head[unit].x = last;
+            if (last == PF_FAIL) q.ovf[atomicAdd(q.novf, 1)] = unit;
         }
         __syncwarp();
         if (!ahead) {
@@ -1660,6 +1695,17 @@ struct __align__(16) ClipShared : StackShared<R, MX_STACK_> {
     R Tsg[MX_MAXT];
     R Kw[MX_CAND];
 };
+
+// tetrahedron i of the prisms with points P (20 numbers a prism): T0 = a0 a1 a2 b2,
+// T1 = a0 a1 b2 b1, T2 = a0 b0 b1 b2
+template <class R>
+__device__ __forceinline__ RTet<R> prism_tet(const R *P, int i)
+{
+    const int j = i % 3;
+    const R *p = P + 20 * (i / 3);
+    auto at = [&](int k) { return r3(p[k], p[k + 1], p[k + 2]); };
+    return RTet<R>{{at(0), at(j == 2 ? 9 : 3), at(j == 0 ? 6 : j == 1 ? 15 : 12), at(j == 1 ? 12 : 15)}};
+}
 
 template <class R, int ST, class Wk>
 __device__ __forceinline__ void pf_clip_body(const MXArgs &a, const PfQueue &q, ClipShared<R, ST> &sh)
@@ -1688,11 +1734,7 @@ __device__ __forceinline__ void pf_clip_body(const MXArgs &a, const PfQueue &q, 
         for (unsigned i = lane; i < nu * 5 * L.RW; i += 32) kd[i] = ob[L.K + i];
         if (lane < nu) sh.Kw[lane] = reinterpret_cast<const R *>(ob + L.W)[lane];
         if (lane < 3 * nprism) {
-            // T0 = a0 a1 a2 b2, T1 = a0 a1 b2 b1, T2 = a0 b0 b1 b2
-            const int j = lane % 3;
-            const R *p = reinterpret_cast<const R *>(ob + L.P) + 20 * (lane / 3);
-            auto at = [&](int i) { return r3(p[i], p[i + 1], p[i + 2]); };
-            stT(sh.T[lane], RTet<R>{{at(0), at(j == 2 ? 9 : 3), at(j == 0 ? 6 : j == 1 ? 15 : 12), at(j == 1 ? 12 : 15)}});
+            stT(sh.T[lane], prism_tet(reinterpret_cast<const R *>(ob + L.P), lane));
             sh.Tsg[lane] = h0.y >> lane & 1u ? R(1) : h0.z >> lane & 1u ? R(-1) : R(0);
         }
         __syncwarp();
@@ -1706,26 +1748,94 @@ __device__ __forceinline__ void pf_clip_body(const MXArgs &a, const PfQueue &q, 
     wk.flush(a.work, lane);
 }
 
-// V_alpha of the band faces from their parts, in a fixed order
+// V_alpha of a band face from 6 x its volume (rounded step by step: the two
+// callers have to agree to the bit)
+__device__ __forceinline__ void pf_write(const MXArgs &a, int item, double v6, bool comp)
+{
+    const int f = a.list[item];
+    const double v = __dmul_rn(v6, 1.0 / 6.0);
+    a.Va[f] = comp ? fma(a.F[f], a.dt, -v) : v;
+}
+
+// The band faces from their parts, in a fixed order: a unit's batches, then what
+// its pair stage summed.  A lane a unit (the batches are a chain of reads), the
+// units of a face side by side.
 template <class R>
 __device__ __forceinline__ void pf_sums(const MXArgs &a, const PfQueue &q)
 {
-    const int total = *a.count, ls = pf_split(total, q.pair_warps);
-    for (int item = blockIdx.x * blockDim.x + threadIdx.x; item < total; item += gridDim.x * blockDim.x) {
-        double v = 0.0;
-        bool comp = false, fail = false;
-        for (int u = item << ls; u < (item + 1) << ls; ++u) {
-            const int2 h = q.head[u];
-            comp = h.y != 0;
-            fail |= h.x == PF_FAIL;
-            v += get_sum<R>(q.base, u);
-            for (int bi = h.x; bi >= 0; bi = q.bnext[bi]) v += get_sum<R>(q.part, bi);
+    const int total = *a.count, ls = pf_split(total, q.pair_warps), per = 32 >> ls;
+    const int lane = threadIdx.x & 31, part = lane & ((1 << ls) - 1);
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    for (int i0 = warp * per; i0 < total; i0 += nw * per) {
+        const int item = i0 + (lane >> ls);
+        const bool live = item < total;
+        int2 h = make_int2(-1, 0);
+        double w = 0.0, v = 0.0;
+        if (live) {
+            const int u = (item << ls) + part;
+            h = q.head[u];
+            for (int bi = h.x; bi >= 0; bi = q.bnext[bi]) w += get_sum<R>(q.part, bi);
+            w += get_sum<R>(q.base, u);
         }
-        if (fail) continue;
-        const int f = a.list[item];
-        v *= 1.0 / 6.0;
-        a.Va[f] = comp ? a.F[f] * a.dt - v : v;
+        const unsigned fail = __ballot_sync(0xffffffffu, h.x == PF_FAIL) >> (lane - part) & ((1u << (1 << ls)) - 1u);
+        for (int k = 0; k < 1 << ls; ++k) v += __shfl_sync(0xffffffffu, w, lane - part + k);
+        if (live && part == 0 && !fail) pf_write(a, item, v, h.y != 0);
     }
+}
+
+// The faces without room, a warp each: pairs and clips of a unit in turn, the
+// batches as the pair stage forms them and the clips with the clip stage's stack.
+template <class R, int ST>
+struct __align__(16) RedoShared : PairShared<R>, StackShared<R, ST> {
+    static constexpr int MX_STACK = ST;
+};
+__device__ __forceinline__ double lane_sum(const Acc<float> &v) { return (double)v.s + (double)v.c; }
+__device__ __forceinline__ double lane_sum(const Acc<double> &v) { return v.s + v.c; }
+
+template <class R, int ST, class Wk>
+__device__ __forceinline__ void pf_redo(const DevMesh &m, const MXArgs &a, const PfQueue &q, RedoShared<R, ST> &sh)
+{
+    const int lane = threadIdx.x & 31;
+    const int ls = pf_split(*a.count, q.pair_warps), n = *q.novf;
+    auto take = [&]() {
+        int v = 0;
+        if (lane == 0) v = atomicAdd(q.next_ovf, 1);
+        return __shfl_sync(0xffffffffu, v, 0);
+    };
+    Wk wk;
+    unsigned done = 0;
+    for (int i = take(); i < n; i = take()) {
+        const int unit = q.ovf[i], item = unit >> ls;
+        bool other = false;  // (a face is redone once, for its first part without room)
+        for (int u = item << ls; u < unit; ++u) other |= q.head[u].x == PF_FAIL;
+        if (other) continue;
+        ++done;
+        const uint4 rec = lane < 4 ? q.rec[4 * (size_t)item + lane] : make_uint4(0u, 0u, 0u, 0u);
+        const PfFace p = pf_face<R>(rec, sh);
+        pf_poly<R>(m, a, sh, item, p);
+        __syncwarp();
+        double v = 0.0;
+        bool comp = p.comp;
+        for (int part = 0; part < 1 << ls; ++part) {
+            double w = 0.0;
+            Acc<R> acc;
+            WkOff off;  // (its pairs are counted by the pair stage)
+            comp = p.comp;
+            pf_stencil<R>(m, a, sh, p, part, ls, comp, acc, off, [&](int nq, unsigned, R tol) {
+                if (lane < p.nt) stT(sh.T[lane], prism_tet(reinterpret_cast<const R *>(sh.P6), lane));
+                Acc<R> cut;
+                mx_clip(sh, sh.Q, nq, tol, pf_drop<R>(sh), cut, wk);
+                mx_merge(cut);
+                w += lane_sum(cut);
+            });
+            mx_merge(acc);
+            v += w + lane_sum(acc);
+        }
+        if (lane == 0) pf_write(a, item, v, comp);
+        __syncwarp();
+    }
+    if (std::is_same<Wk, WkOn>::value && lane == 0) work_add1(a.work, WK_NOROOM, done);
+    wk.flush(a.work, lane);
 }
 
 // warps per block of the pair launch, and blocks per SM: FP32 3 / 4 / 5 / 6
@@ -1753,21 +1863,16 @@ __global__ void __launch_bounds__(W * 32, pc_resident<R>(W, ST)) k_pf_clip(MXArg
     pf_clip_body<R, ST, Wk>(a, q, reinterpret_cast<ClipShared<R, ST> *>(pf_smem)[threadIdx.x >> 5]);
 }
 
-// (a.items, a.next and a.count describe the faces without room)
-template <class R, class Wk>
-__global__ void __launch_bounds__(64, sizeof(R) == 4 ? 8 : 4) k_pf_finish(DevMesh m, MXArgs a, PfQueue q, const int *count)
+constexpr int PF_FINISH_WARPS = 2;
+template <class R, int ST, class Wk>
+__global__ void __launch_bounds__(32 * PF_FINISH_WARPS, sizeof(R) == 4 ? 8 : 4) k_pf_finish(DevMesh m, MXArgs a, PfQueue q)
 {
     next_kernel();
     previous_kernel();
     extern __shared__ __align__(16) unsigned char pf_smem[];
-    {
-        MXArgs s = a;
-        s.count = count;
-        pf_sums<R>(s, q);
-    }
-    if (*a.count > 0)
-        phase_flux_body<R, MX_STACK_WIDE, true, Wk>(
-            m, a, reinterpret_cast<MXShared<R, MX_STACK_WIDE> *>(pf_smem)[threadIdx.x >> 5]);
+    pf_sums<R>(a, q);
+    if (*q.novf > 0)
+        pf_redo<R, ST, Wk>(m, a, q, reinterpret_cast<RedoShared<R, ST> *>(pf_smem)[threadIdx.x >> 5]);
 }
 
 // geometry of every cell relative to its centre (context creation): face
@@ -1886,8 +1991,8 @@ static MXArgs mx_args(vof_ctx *c, const double *alpha, const double *n, const do
                       const double *Up, const double *F, const double *lambda, double dt, double *Va,
                       const int *list, const int *count, const void *disp, unsigned long long *work)
 {
-    return MXArgs{alpha, n, d, flags, Up, F, lambda, dt, Va, list, count, disp, c->lam_b, c->status, work,
-                  c->fpl, c->cbl, c->ktl, c->m.ctptr, nullptr, nullptr};
+    return MXArgs{alpha, n, d, flags, Up, F, lambda, dt, Va, list, count, disp, c->status, work,
+                  c->fpl, c->cbl, c->ktl, c->m.ctptr};
 }
 
 // the band slots' work queue and counters (zeroed with the step's counters)
@@ -1910,10 +2015,11 @@ static bool pf_smem_form()
 {
     bool ok = pf_smem(k_phase_flux<R, W, Wk>, W * sizeof(MXShared<R, MX_STACK_WIDE>)) &&
               pf_smem(k_pf_pairs<R, Wk>, pp_warps<R>() * sizeof(PairShared<R>)) &&
-              pf_smem(k_pf_finish<R, Wk>, 2 * sizeof(MXShared<R, MX_STACK_WIDE>)) &&
+              pf_smem(k_pf_finish<R, MX_STACK_WIDE, Wk>, PF_FINISH_WARPS * sizeof(RedoShared<R, MX_STACK_WIDE>)) &&
               pf_smem(k_pf_clip<R, 1, MX_STACK_WIDE, Wk>, sizeof(ClipShared<R, MX_STACK_WIDE>));
     if constexpr (sizeof(R) == 4)
-        ok = ok && pf_smem(k_pf_clip<R, 2, MX_STACK_WIDE, Wk>, 2 * sizeof(ClipShared<R, MX_STACK_WIDE>)) &&
+        ok = ok && pf_smem(k_pf_finish<R, MX_STACK_SLIM, Wk>, PF_FINISH_WARPS * sizeof(RedoShared<R, MX_STACK_SLIM>)) &&
+             pf_smem(k_pf_clip<R, 2, MX_STACK_WIDE, Wk>, 2 * sizeof(ClipShared<R, MX_STACK_WIDE>)) &&
              pf_smem(k_pf_clip<R, 3, MX_STACK_WIDE, Wk>, 3 * sizeof(ClipShared<R, MX_STACK_WIDE>)) &&
              pf_smem(k_pf_clip<R, 1, MX_STACK_SLIM, Wk>, sizeof(ClipShared<R, MX_STACK_SLIM>)) &&
              pf_smem(k_pf_clip<R, 2, MX_STACK_SLIM, Wk>, 2 * sizeof(ClipShared<R, MX_STACK_SLIM>)) &&
@@ -1928,12 +2034,19 @@ static int go_clip(const MXArgs &a, const PfQueue &q, int sms, int mult, cudaStr
     return launch_after(k_pf_clip<R, W, ST, Wk>, sms * pc_resident<R>(W, ST) * mult, 32 * W, bytes, s, a, q);
 }
 
+template <class R, int ST, class Wk>
+static int go_finish(vof_ctx *c, const MXArgs &a, const PfQueue &q, int sms, cudaStream_t s)
+{
+    constexpr size_t bytes = PF_FINISH_WARPS * sizeof(RedoShared<R, ST>);
+    return launch_after(k_pf_finish<R, ST, Wk>, sms * 4, 32 * PF_FINISH_WARPS, bytes, s, c->m, a, q);
+}
+
 template <class R, class Wk>
 static int go_list(vof_ctx *c, const MXArgs &a, int sms, cudaStream_t s)
 {
     const int pblocks = sms * pp_resident<R>();
     const PfQueue q = pf_queue(c, pblocks * pp_warps<R>());
-    constexpr size_t pbytes = pp_warps<R>() * sizeof(PairShared<R>), fbytes = 2 * sizeof(MXShared<R, MX_STACK_WIDE>);
+    constexpr size_t pbytes = pp_warps<R>() * sizeof(PairShared<R>);
     k_pf_pairs<R, Wk><<<pblocks, 32 * pp_warps<R>(), pbytes, s>>>(c->m, a, q);
     // launch configuration of the clips (vof_tune): warps per block, stack
     // depth, and grid = SMs x resident blocks x multiplier
@@ -1951,11 +2064,9 @@ static int go_list(vof_ctx *c, const MXArgs &a, int sms, cudaStream_t s)
                                 : go_clip<R, 3, MX_STACK_WIDE, Wk>(a, q, sms, mult, s);
     } else r = go_clip<R, 1, MX_STACK_WIDE, Wk>(a, q, sms, 1, s);
     if (r) return r;
-    MXArgs o = a;
-    o.items = q.ovf;
-    o.count = q.novf;
-    o.next = q.next_ovf;
-    r = launch_after(k_pf_finish<R, Wk>, sms * 4, 64, fbytes, s, c->m, o, q, a.count);
+    if constexpr (sizeof(R) == 4)
+        r = c->pf_stack == 1 ? go_finish<R, MX_STACK_SLIM, Wk>(c, a, q, sms, s) : go_finish<R, MX_STACK_WIDE, Wk>(c, a, q, sms, s);
+    else r = go_finish<R, MX_STACK_WIDE, Wk>(c, a, q, sms, s);
     if (r) return r;
     return cudaGetLastError() == cudaSuccess ? VOF_OK : VOF_ERR_CUDA;
 }

@@ -345,7 +345,8 @@ def vof_count_work(h, on: bool = True):
 
 
 def vof_work_counts(h, reset: bool = True, stream=None):
-    """Counted primitives since the last reset (include/vof.h), by name."""
+    """Counted primitives since the last reset (include/vof.h), by name (reserved:
+    band faces that found no room in the queue of clip jobs)."""
     c = (ctypes.c_ulonglong * len(WORK))()
     _check(lib().vof_work_counts(h, c, int(bool(reset)), _stream(stream)), "vof_work_counts")
     return {k: int(c[i]) for i, k in enumerate(WORK)}

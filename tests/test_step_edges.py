@@ -1,6 +1,7 @@
 """What a step does at its edges: shared memory handed between the lanes of a
 warp, settings changed between batch steps, cells of any aspect ratio,
-NaN fractions, what the positioning's stop leaves of an offset.
+NaN fractions, what the positioning's stop leaves of an offset,
+a band beyond the queue of clip jobs.
 
 FP64 is held to the replay tolerance against the oracle (1e-11).
 """
@@ -187,3 +188,43 @@ def test_fp64_offsets_beyond_the_stop(torch, oracle_lib):
     res = np.array([abs(om.cut_volume(c, n[:, c], d[c]) / vc[c] - a[c]) for c in cells])
     assert res.max() <= 1e-14, res.max()
     ctx.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision", [0, 1])
+def test_no_room_in_the_queue_changes_no_bit(torch, precision):
+    """A step whose band (every face) has more clip jobs than the context's queue
+    holds: the same bits from run to run, and as in a joined mesh
+    with an empty case whose faces make the queue large enough."""
+    from paper_1305_3417_gb300 import vof
+    w = I.make_workload("deform3d", n=16)
+    rest = I.hex_mesh((64, 64, 64))
+    F, U, dt = w.step_inputs(1)
+    a0 = np.random.default_rng(3).uniform(0.05, 0.95, w.mesh.n_cells)
+    joined, off = I.concat_meshes([w.mesh, rest])[:2]
+    ni = w.mesh.n_internal
+    Fj = np.concatenate([F[:ni], np.zeros(rest.n_internal), F[ni:], np.zeros(rest.n_faces - rest.n_internal)])
+    Uj = np.concatenate([U.reshape(3, -1), np.zeros((3, rest.n_cells))], axis=1)
+
+    def run(h, a, u, f):
+        ta, tU, tF = T(torch, a), T(torch, u), T(torch, f)
+        vof.vof_count_work(h)
+        out = []
+        for _ in range(3):
+            t = ta.clone()
+            vof.vof_work_counts(h)
+            vof.vof_advect(h, t, tU, tF, dt)
+            out.append((t[:w.mesh.n_cells].clone(), vof.vof_work_counts(h)))
+        assert vof.vof_status(h) == 0
+        return out
+
+    ctx = vof.VofContext(w.mesh, precision=precision, bound=False)
+    few = run(ctx.h, a0, U, F)
+    ctx.close()
+    b = vof.vof_batch_create(joined, off, precision=precision, bound=False)
+    all_ = run(vof.vof_batch_context(b), np.concatenate([a0, np.zeros(rest.n_cells)]), Uj, Fj)
+    vof.vof_batch_destroy(b)
+    # ("reserved" counts the faces without room)
+    assert all(c["reserved"] > 100 for _, c in few) and all(c["reserved"] == 0 for _, c in all_)
+    for t, _ in few[1:] + all_:
+        assert torch.equal(few[0][0], t)
