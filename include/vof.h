@@ -16,8 +16,9 @@
  *   Every per-step call is asynchronous on `stream` (a cudaStream_t; NULL is
  *   the legacy default stream) and allocates no memory: the context allocates
  *   all of its scratch in vof_create (the largest: the cell tetrahedra's planes,
- *   and the phase flux's queue of clip jobs, 512 bytes per face, 1024 in FP64;
- *   band faces that find no room in it are fluxed more slowly, to the same bits).
+ *   and the phase flux's queue of clip jobs, 512 bytes per face, 1024 in FP64,
+ *   less where that is more than half of the free device memory; band faces
+ *   that find no room in it are fluxed more slowly, to the same bits).
  * - Vectors are structure-of-arrays: x block, then y block, then z block.
  * - Face f of the mesh has points face_pts[face_ptr[f] .. face_ptr[f+1]),
  *   ordered so that the right-hand area vector S_f points from owner[f] to

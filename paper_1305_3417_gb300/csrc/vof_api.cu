@@ -42,7 +42,11 @@ T *dev_alloc(vof_ctx *c, size_t n, int *err)
     if (*err) return nullptr;
     if (c->nbufs >= (int)(sizeof(c->bufs) / sizeof(c->bufs[0]))) { *err = VOF_ERR_CUDA; return nullptr; }
     void *p = nullptr;
-    if (cudaMalloc(&p, std::max<size_t>(n, 1) * sizeof(T)) != cudaSuccess) { *err = VOF_ERR_CUDA; return nullptr; }
+    if (cudaMalloc(&p, std::max<size_t>(n, 1) * sizeof(T)) != cudaSuccess) {
+        cudaGetLastError();  // (not left behind for a launch's check)
+        *err = VOF_ERR_CUDA;
+        return nullptr;
+    }
     c->bufs[c->nbufs++] = p;
     return (T *)p;
 }
@@ -59,6 +63,39 @@ T *dev_copy(vof_ctx *c, const T *h, size_t n, int *err)
 bool finite_pos(double x) { return std::isfinite(x) && x > 0.0; }
 
 }  // namespace
+
+// The phase flux's queue, after everything else.  A band face has about 2.5 KB
+// of clip jobs (twice that in FP64); 512 (1024) bytes per mesh face hold a band
+// of a fifth of the faces, and the floor any band of a small mesh.  It takes half
+// of the free memory at most: the caller's fields, a batch's regions and the
+// buffers of vof_set_gradient and vof_set_guess come after it.  Faces beyond it
+// are fluxed again by the slower third launch, to the same bits, so where memory
+// is short a smaller queue serves too, down to none.
+static int alloc_queue(vof_ctx *c)
+{
+    const size_t unit = 16, per = c->precision == VOF_MIXED ? 512 : 1024, batch = 14;  // units of the smallest batch
+    const size_t entry = 2 * sizeof(int) + sizeof(double);                             // the tables' bytes a batch
+    size_t bytes = std::max(per * (size_t)c->nf, per * (size_t)(1 << 16)), avail = 0, total = 0;
+    bytes = std::min(bytes, unit * ((size_t)1 << 31));
+    if (cudaMemGetInfo(&avail, &total) != cudaSuccess) return VOF_ERR_CUDA;
+    while (bytes + bytes / (unit * batch) * entry > avail / 2) bytes /= 2;
+    for (;; bytes /= 2) {
+        const int n0 = c->nbufs;
+        const size_t nb = bytes / unit / batch;
+        int err = 0;
+        c->pf_arena = dev_alloc<unsigned char>(c, bytes, &err);
+        c->pf_boff = dev_alloc<unsigned>(c, nb, &err);
+        c->pf_bnext = dev_alloc<int>(c, nb, &err);
+        c->pf_part = dev_alloc<double>(c, nb, &err);
+        if (!err) {
+            c->pf_cap = (unsigned)(bytes / unit);
+            c->pf_bcap = (int)nb;
+            return VOF_OK;
+        }
+        while (c->nbufs > n0) cudaFree(c->bufs[--c->nbufs]);
+        if (bytes == 0) return err;
+    }
+}
 
 // regions of the global bounding step, cut into segments (a block's share of
 // the update): a cell a thread on small meshes, so that they spread over the
@@ -538,7 +575,9 @@ int vof_create(const vof_mesh *mesh, const vof_options *opt, vof_ctx **out)
     c->cmark = dev_alloc<unsigned>(c, nc, &err);
     c->counters = dev_alloc<int>(c, CNT_ALLOC, &err);
     c->lam_b = dev_alloc<double>(c, nf, &err);
-    c->disp_b = dev_alloc<double>(c, (size_t)nf * (VOF_MAXFP + 1) * 3, &err);
+    // (band displacements in the form's type)
+    c->disp_b = dev_alloc<unsigned char>(
+        c, (size_t)nf * (VOF_MAXFP + 1) * 3 * (c->precision == VOF_MIXED ? sizeof(float) : sizeof(double)), &err);
     c->it_b = dev_alloc<int>(c, nf, &err);
     c->n = dev_alloc<double>(c, 3 * (size_t)nc, &err);
     c->d = dev_alloc<double>(c, nc, &err);
@@ -565,32 +604,11 @@ int vof_create(const vof_mesh *mesh, const vof_options *opt, vof_ctx **out)
     c->bpflag = dev_alloc<uint8_t>(c, np, &err);
     c->upb = dev_alloc<double>(c, 3 * (size_t)np, &err);
     c->ktl = dev_alloc<unsigned char>(c, e4 * 6 * (size_t)ctptr[nc], &err);
-    if (!err) {
-        // The phase flux's queue: a band face has about 2.5 KB of clip jobs
-        // (twice that in FP64); 512 (1024) bytes per mesh face hold a band of a
-        // fifth of the faces, and the floor any band of a small mesh.  Faces
-        // beyond it are fluxed in the slower one-warp form, so where memory is
-        // short a smaller queue serves too.
-        const size_t unit = 16, per = c->precision == VOF_MIXED ? 512 : 1024;
-        size_t bytes = std::max(per * (size_t)nf, per * (size_t)(1 << 16));
-        bytes = std::min(bytes, unit * ((size_t)1 << 31));
-        void *p = nullptr;
-        while (cudaMalloc(&p, bytes) != cudaSuccess && bytes > (1u << 20)) {
-            cudaGetLastError();
-            p = nullptr;
-            bytes /= 2;
-        }
-        if (!p || c->nbufs >= (int)(sizeof(c->bufs) / sizeof(c->bufs[0]))) err = VOF_ERR_CUDA;
-        else c->bufs[c->nbufs++] = p;
-        c->pf_arena = p;
-        c->pf_cap = (unsigned)(bytes / unit);
-        c->pf_bcap = (int)(bytes / unit / 14);  // the smallest batch
-        // units of work: a band face, or its parts where the band is small
+    {
+        // units of work of the phase flux: a band face, or its parts where the
+        // band is small
         const size_t units = std::max<size_t>(nf, 128 * (size_t)prop.multiProcessorCount);
         c->pf_rec = dev_alloc<BandRec>(c, nf, &err);
-        c->pf_boff = dev_alloc<unsigned>(c, c->pf_bcap, &err);
-        c->pf_bnext = dev_alloc<int>(c, c->pf_bcap, &err);
-        c->pf_part = dev_alloc<double>(c, c->pf_bcap, &err);
         c->pf_base = dev_alloc<double>(c, units, &err);
         c->pf_head = dev_alloc<int2>(c, units, &err);
         c->pf_ovf = dev_alloc<int>(c, units, &err);
@@ -612,6 +630,7 @@ int vof_create(const vof_mesh *mesh, const vof_options *opt, vof_ctx **out)
     {
         const int whole[2] = {0, nc};
         if (!err) err = set_bound_regions(c, whole, 1);
+        if (!err) err = alloc_queue(c);
         if (err) { vof_destroy(c); return err; }
     }
     int r = launch_setup_geometry(c, 0);

@@ -100,7 +100,8 @@ struct vof_ctx {
     uint8_t *pstate;
     int *band, *icell, *viol[2];
     int *counters;               // CNT_ALLOC ints, laid out as CNT_* above
-    double *lam_b, *disp_b;      // per band slot
+    double *lam_b;               // per band slot
+    void *disp_b;                // per band slot, in the form's type
     int *it_b;
     double *n, *d;
     uint8_t *flags;

@@ -1,7 +1,8 @@
 """What a step does at its edges: shared memory handed between the lanes of a
 warp, settings changed between batch steps, cells of any aspect ratio,
 NaN fractions, what the positioning's stop leaves of an offset,
-a band beyond the queue of clip jobs.
+a band beyond the queue of clip jobs,
+a context made where memory is short.
 
 FP64 is held to the replay tolerance against the oracle (1e-11).
 """
@@ -228,3 +229,46 @@ def test_no_room_in_the_queue_changes_no_bit(torch, precision):
     assert all(c["reserved"] > 100 for _, c in few) and all(c["reserved"] == 0 for _, c in all_)
     for t, _ in few[1:] + all_:
         assert torch.equal(few[0][0], t)
+
+
+@pytest.mark.gpu
+def test_context_where_memory_is_short(torch):
+    """With all but a part of what a context likes to take allocated elsewhere, a
+    smaller queue serves: the same step, and memory left for the buffers that the
+    caller and the least-squares gradient take afterwards."""
+    from paper_1305_3417_gb300 import vof
+    w = I.make_workload("deform3d", n=64)
+    F, U, dt = w.step_inputs(1)
+    a0 = np.random.default_rng(3).uniform(0.05, 0.95, w.mesh.n_cells)   # (every face in the band)
+    tF, tU, t0 = T(torch, F), T(torch, U), T(torch, a0)
+
+    def step():
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        ctx = vof.VofContext(w.mesh, precision=1)
+        took = before - torch.cuda.mem_get_info()[0]
+        t = t0.clone()
+        ctx.advect(t, tU, tF, dt)
+        vof.vof_set_gradient(ctx.h, vof.GRAD_LSQ)
+        b = t0.clone()
+        ctx.advect(b, tU, tF, dt)
+        assert ctx.status() == 0
+        ctx.close()
+        return took, t, b
+
+    step()
+    took, t, b = step()
+    queue = 512 * w.mesh.n_faces                # preferred size, and 16 bytes of tables a batch of 224
+    queue += 16 * (queue // 224)
+    # room for the rest, 200 MB for what the step's second half takes, and parts of a queue
+    for part in (0.9, 0.5, 0.0):
+        leave = took - queue + (200 << 20) + int(part * queue)
+        torch.cuda.empty_cache()
+        hog = torch.empty(torch.cuda.mem_get_info()[0] - leave, dtype=torch.uint8, device="cuda")
+        try:
+            less, u, v = step()
+        finally:
+            del hog
+            torch.cuda.empty_cache()
+        assert less < took - queue // 4
+        assert torch.equal(t, u) and torch.equal(b, v)
