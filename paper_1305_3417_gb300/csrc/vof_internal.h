@@ -59,7 +59,7 @@ enum { CNT_BAND = 0, CNT_ICELL, CNT_MAXPOS, CNT_MAXCORR, CNT_FALLBACK, CNT_PFNEX
        // the update group's
        CNT_UPD = 12, CNT_VIOL0 = CNT_UPD, CNT_VIOL1, CNT_BPASS, CNT_BACT0, CNT_BACT1, CNT_NRL0, CNT_NRL1, CNT_LEFT0,
        CNT_LEFT1, CNT_NDL, CNT_UPD_N = CNT_NDL - CNT_UPD + 1, CNT_LEN = 24,
-       CNT_EPOCH = 28 /* kept from step to step */ };
+       CNT_EPOCH = 28 /* kept, moved on before each update group */ };
 enum { CNT_BAR = 32, CNT_BARGEN = 64, CNT_ALLOC = 96 };
 // algorithmic work counted by the step kernels (vof_work_counts): the phase
 // flux's primitives (FP32 in the mixed form, FP64 in the plain one) -- signed

@@ -1361,6 +1361,11 @@ __device__ bool grid_sync(unsigned *count, unsigned *generation, unsigned *statu
     return !gave_up;
 }
 
+// Numbers that a launch may use to mark cells (a pass each) and segments.  They
+// move on where the update group's counters are cleared, before the launch:
+// one whose waits ran out leaves no mark that a later launch takes for its own.
+constexpr unsigned EPOCH_STEP = BOUND_PASSES_MAX + 2;
+
 // The redistribution of a step: passes over the sources and their receivers,
 // the mesh-wide fallback for what no local pass can place (a source none of
 // whose face neighbours is an interface cell with room): the total excess
@@ -1370,7 +1375,7 @@ __device__ bool grid_sync(unsigned *count, unsigned *generation, unsigned *statu
 //
 // A pass has three phases with a barrier after each: sources weigh their
 // receivers and list them, each once (marked with the pass's own number, so the
-// marks need no clearing); receivers gather their requests, scale them and
+// marks need no clearing; EPOCH_STEP); receivers gather their requests, scale them and
 // form their new value; sources take off what was placed while the receivers'
 // values are written.  The phases are chains of a few dependent loads over
 // hundreds of items: barriers, first-time instruction fetches and, where many
@@ -1392,7 +1397,7 @@ struct BoundStep {
     unsigned *mark;              // per cell: the pass that listed it
     unsigned *segmark;           // per segment: the launch that changed it
     int *dl, *ndl;               // changed segments
-    unsigned *epoch;             // numbers used so far
+    const unsigned *epoch;       // the launch's first number less one (EPOCH_STEP apart)
     int *npass, *act, *left;     // passes that moved something; sources with a receiver, sources left, by pass parity
     int *nleft;                  // out: sources left to the fallback
     const int4 *seg;
@@ -1623,7 +1628,6 @@ __global__ void __launch_bounds__(BA_THREADS, 1) k_bound_step(DevMesh m, BoundSt
     stats_block(a.sd, a.nseg, a.counters, a.stats, a.status);
     if (lead) {
         *a.npass = npass;
-        *a.epoch = e0 + (unsigned)npass + 2;
         double gv = 0.0;  // volume the fallback moved (regions where it applied)
         if (nleft > 0)
             for (int r = 0; r < a.nreg; ++r) {
@@ -1659,6 +1663,7 @@ __global__ void k_zero_update(int *cnt)
     const int i = threadIdx.x;
     if (i < CNT_UPD_N) cnt[CNT_UPD + i] = 0;
     if (i == CNT_UPD_N) cnt[CNT_BAR] = 0;
+    if (i == CNT_UPD_N + 1) cnt[CNT_EPOCH] = (int)((unsigned)cnt[CNT_EPOCH] + EPOCH_STEP);
 }
 
 // ============================================== band classification (A2, R9)
@@ -1672,6 +1677,7 @@ __global__ void k_point_state(DevMesh m, const double *__restrict__ alpha, uint8
     int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p < CNT_LEN) cnt[p] = 0;
     if (p == CNT_LEN) cnt[CNT_BAR] = 0;
+    if (p == CNT_LEN + 1) cnt[CNT_EPOCH] = (int)((unsigned)cnt[CNT_EPOCH] + EPOCH_STEP);
     if (p >= m.np) return;
     bool all_e = true, all_f = true;
     const double full = 1.0 - m.eps;

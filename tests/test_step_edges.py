@@ -31,6 +31,24 @@ def test_queue_write_waits_for_its_shared_inputs():
         assert first > stored and "__syncwarp();" in body[stored:first], read
 
 
+def test_marks_move_on_before_the_redistribution():
+    """The numbers that the redistribution marks cells with move on where a
+    step's (an update's) counters are cleared, not at its end, which a launch
+    whose waits ran out does not reach: its marks would be taken for the next
+    step's own and their cells left out.  Read from the source: no wait runs out
+    in a sound step."""
+    src = open(os.path.join(SRC, "vof_kernels.cu")).read()
+
+    def body(name):
+        i = src.index(name)
+        return src[i:src.index("\n}\n", i)]
+    for kernel in ("void k_point_state(", "void k_zero_update("):
+        assert "cnt[CNT_EPOCH]" in body(kernel) and "EPOCH_STEP" in body(kernel)
+    step = body("k_bound_step(DevMesh m, BoundStep a)")
+    assert "*a.epoch" in step and not re.search(r"\*a\.epoch\s*=[^=]", step)
+    assert "EPOCH_STEP = BOUND_PASSES_MAX + 2" in src       # a launch's marks: one a pass, and the segments'
+
+
 @pytest.fixture(scope="module")
 def torch():
     import torch
