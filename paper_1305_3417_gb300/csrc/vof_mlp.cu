@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstdint>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -513,6 +514,7 @@ struct vof_mlp {
     bf *W1t, *W2, *W2t, *W3, *W3t;
     float *part;
     double *lpart;
+    float *y;                              // outputs of a forward pass over its own features
     float *h_loss;                         // pinned host memory that the device writes
     std::vector<void *> bufs;
 };
@@ -601,6 +603,7 @@ int vof_mlp_create(int max_batch, const float *params, int device, vof_mlp **out
     q->W3t = mlp_alloc<bf>(q, HID * OUTP, &ok);
     q->part = mlp_alloc<float>(q, (size_t)q->nblk * NPARAM, &ok);
     q->lpart = mlp_alloc<double>(q, q->nblk, &ok);
+    q->y = mlp_alloc<float>(q, (size_t)max_batch * OUT, &ok);
     ok = ok && cudaMallocHost(&q->h_loss, sizeof(float)) == cudaSuccess &&
          cudaFuncSetAttribute(k_mlp_pass<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(MlpShared)) ==
              cudaSuccess &&
@@ -646,7 +649,14 @@ int vof_mlp_forward(vof_mlp *q, const float *feat, int n, float *out, void *stre
 {
     if (!q || !feat || !out || n < 1 || n > q->max_batch) return VOF_ERR_INVALID_ARG;
     if (cudaSetDevice(q->device) != cudaSuccess) return VOF_ERR_CUDA;
-    return mlp_forward(q, feat, n, out, (cudaStream_t)stream);
+    cudaStream_t s = (cudaStream_t)stream;
+    // out may lie over feat: a block would write rows that another has yet to read
+    const std::uintptr_t f = reinterpret_cast<std::uintptr_t>(feat), o = reinterpret_cast<std::uintptr_t>(out);
+    const size_t fb = sizeof(float) * IN * (size_t)n, ob = sizeof(float) * OUT * (size_t)n;
+    if (o >= f + fb || f >= o + ob) return mlp_forward(q, feat, n, out, s);
+    const int r = mlp_forward(q, feat, n, q->y, s);
+    if (r) return r;
+    return cudaMemcpyAsync(out, q->y, ob, cudaMemcpyDeviceToDevice, s) == cudaSuccess ? VOF_OK : VOF_ERR_CUDA;
 }
 
 int vof_mlp_gradient(vof_mlp *q, const float *feat, const float *target, int n, float *grad, float *loss,

@@ -2,7 +2,7 @@
 warp, settings changed between batch steps, cells of any aspect ratio,
 NaN fractions, what the positioning's stop leaves of an offset,
 a band beyond the queue of clip jobs,
-a context made where memory is short.
+a context made where memory is short, network outputs written over their inputs.
 
 FP64 is held to the replay tolerance against the oracle (1e-11).
 """
@@ -290,3 +290,20 @@ def test_context_where_memory_is_short(torch):
             torch.cuda.empty_cache()
         assert less < took - queue // 4
         assert torch.equal(t, u) and torch.equal(b, v)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("at", [0, 29 * 12801])      # over the first rows, or the last ones
+def test_forward_over_its_own_features(torch, at):
+    """More tiles than blocks; the same bits as into a buffer of its own."""
+    from paper_1305_3417_gb300 import mlp, vof
+    n = 12801
+    net = vof.Mlp(mlp.init_params(3), max_batch=n)
+    feat = torch.rand((n, vof.MLP_IN), generator=torch.Generator().manual_seed(1)).cuda()
+    want = net.forward(feat)
+    flat = feat.reshape(-1).clone()
+    out = flat[at:at + n * vof.MLP_OUT]
+    assert vof.lib().vof_mlp_forward(net.h, vof._ptr(flat), n, vof._ptr(out), vof._stream(None)) == 0
+    torch.cuda.synchronize()
+    assert torch.equal(out.reshape(n, -1), want)
+    net.close()
