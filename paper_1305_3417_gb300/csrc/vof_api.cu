@@ -177,7 +177,6 @@ void vof_destroy(vof_ctx *c)
     free_profile(c);
     for (int i = 0; i < c->nbufs; ++i) cudaFree(c->bufs[i]);
     cudaFree(c->mlp_s0);
-    cudaFree(c->mlp_feat);
     cudaFree(c->mlp_nbr);
     cudaFree(c->mlp_geo);
     if (c->s_copy) cudaStreamDestroy(c->s_copy);

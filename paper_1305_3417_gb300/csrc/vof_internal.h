@@ -171,10 +171,10 @@ struct vof_ctx {
     uint8_t *lcode;  // periodic meshes: translation code of each LSQ neighbour (else null)
     double *grad;
     // learned guess of the positioning (vof_set_guess): the network, offsets by
-    // interface-list position, features
+    // interface-list position
     struct vof_mlp *mlp;
-    float *mlp_s0, *mlp_feat;
-    int mlp_feat_cap;
+    float *mlp_s0;
+    int mlp_s0_cap;
     int *mlp_nbr;                // per cell: 27 lattice-slot cell indices (-1: itself)
     float *mlp_geo;              // per cell: 6 shape numbers
     // counts the changes of what a step's launches hold besides their arguments

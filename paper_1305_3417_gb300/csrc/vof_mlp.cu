@@ -691,26 +691,33 @@ int vof_set_guess(vof_ctx *c, vof_mlp *q)
     if (!c) return VOF_ERR_INVALID_ARG;
     if (cudaSetDevice(c->device) != cudaSuccess) return VOF_ERR_CUDA;
     if (q && q->device != c->device) return VOF_ERR_INVALID_ARG;
-    ++c->cfg_gen;  // (also for the same network again: its weights or buffers may be new ones)
+    // (a buffer that cannot be had leaves the context as it was: the network
+    // attached before keeps its own)
+    auto get = [](void **p, size_t bytes) {
+        if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+        cudaGetLastError();
+        return false;
+    };
     if (q && !c->mlp_nbr) {
-        if (cudaMalloc(&c->mlp_nbr, sizeof(int) * 27 * (size_t)c->nc) != cudaSuccess ||
-            cudaMalloc(&c->mlp_geo, sizeof(float) * 6 * (size_t)c->nc) != cudaSuccess)
+        void *nbr = nullptr, *geo = nullptr;
+        if (!get(&nbr, sizeof(int) * 27 * (size_t)c->nc) || !get(&geo, sizeof(float) * 6 * (size_t)c->nc)) {
+            cudaFree(nbr);
             return VOF_ERR_CUDA;
+        }
+        c->mlp_nbr = static_cast<int *>(nbr);
+        c->mlp_geo = static_cast<float *>(geo);
         k_mlp_tables<<<cdiv(c->nc, 128), 128>>>(c->m, c->mlp_nbr, c->mlp_geo);
         if (cudaDeviceSynchronize() != cudaSuccess) return VOF_ERR_CUDA;
     }
-    if (q && c->mlp_feat_cap < q->max_batch) {
-        // guess and feature buffers for the network's batch (kept until vof_destroy)
+    if (q && c->mlp_s0_cap < q->max_batch) {
+        // offsets for the network's batch (kept until vof_destroy)
+        void *s0 = nullptr;
+        if (!get(&s0, sizeof(float) * (size_t)q->max_batch)) return VOF_ERR_CUDA;
         cudaFree(c->mlp_s0);
-        cudaFree(c->mlp_feat);
-        c->mlp_s0 = nullptr;
-        c->mlp_feat = nullptr;
-        c->mlp_feat_cap = 0;
-        if (cudaMalloc(&c->mlp_s0, sizeof(float) * (size_t)q->max_batch) != cudaSuccess ||
-            cudaMalloc(&c->mlp_feat, sizeof(float) * IN * (size_t)q->max_batch) != cudaSuccess)
-            return VOF_ERR_CUDA;
-        c->mlp_feat_cap = q->max_batch;
+        c->mlp_s0 = static_cast<float *>(s0);
+        c->mlp_s0_cap = q->max_batch;
     }
+    ++c->cfg_gen;  // (also for the same network again: its weights or buffers may be new ones)
     c->mlp = q;
     return VOF_OK;
 }

@@ -2,7 +2,8 @@
 warp, settings changed between batch steps, cells of any aspect ratio,
 NaN fractions, what the positioning's stop leaves of an offset,
 a band beyond the queue of clip jobs,
-a context made where memory is short, network outputs written over their inputs.
+a context made, or a network attached, where memory is short, network outputs
+written over their inputs.
 
 FP64 is held to the replay tolerance against the oracle (1e-11).
 """
@@ -307,3 +308,33 @@ def test_forward_over_its_own_features(torch, at):
     torch.cuda.synchronize()
     assert torch.equal(out.reshape(n, -1), want)
     net.close()
+
+
+@pytest.mark.gpu
+def test_network_that_finds_no_room(torch):
+    """A network whose offsets' buffer cannot be had is refused, and the one
+    attached before goes on as it was."""
+    from paper_1305_3417_gb300 import mlp, vof
+    w = I.make_workload("deform3d", n=16)
+    F, U, dt = w.step_inputs(1)
+    tF, tU, t0 = T(torch, F), T(torch, U), T(torch, w.alpha0)
+    ctx = vof.VofContext(w.mesh, precision=1)
+    nets = [vof.Mlp(mlp.init_params(k), max_batch=b) for k, b in ((1, 1 << 12), (2, 1 << 26))]
+    vof.vof_set_guess(ctx.h, nets[0])
+    a = t0.clone()
+    ctx.advect(a, tU, tF, dt)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - (128 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        with pytest.raises(vof.VofError):
+            vof.vof_set_guess(ctx.h, nets[1])          # 256 MB
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    b = t0.clone()
+    ctx.advect(b, tU, tF, dt)
+    assert ctx.status() == 0 and torch.equal(a, b)
+    ctx.close()
+    for net in nets:
+        net.close()
