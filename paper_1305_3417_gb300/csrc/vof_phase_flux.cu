@@ -1595,11 +1595,11 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
         return lane < 4 && u < units ? q.rec[4 * (size_t)(u >> ls) + lane] : make_uint4(0u, 0u, 0u, 0u);
     };
     Wk wk;
-    bool full = false;
     int unit = __shfl_sync(0xffffffffu, take(), 0);
     uint4 rec = record(unit);
     while (unit < units) {
         const int item = unit >> ls, part = unit & ((1 << ls) - 1);
+        const Wk wk0 = wk;
         const PfFace p = pf_face(rec, sh);
         const int taken = ahead ? take() : 0;
         pf_poly(m, a, sh, item, p);
@@ -1616,14 +1616,14 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
         pf_stencil(m, a, sh, p, part, ls, comp, acc, wk, [&](int nq, unsigned used, R tol) {
             if (last == PF_FAIL) return;
             const int nt = p.nt, nprism = nt / 3;
-            // the jobs, as a batch of the queue (a warp that found no
-            // room once adds nothing more: the counter stays near the
-            // capacity, far from overflowing its halves)
+            // the jobs, as a batch of the queue (a warp that found no room once
+            // takes no more units on: the counter stays near the capacity, far
+            // from overflowing its halves)
             const int nu = __popc(used);
             const PfLayout<R> L(nprism, nu, nq);
             unsigned off = PF_NONE;
             int bi = -1;
-            if (lane == 0 && !full) {
+            if (lane == 0) {
                 const unsigned long long old = atomicAdd(q.ctr, (1ull << 32) | L.end);
                 off = (unsigned)old;
                 bi = (int)(old >> 32);
@@ -1642,8 +1642,9 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
             const unsigned pos = __ballot_sync(0xffffffffu, sg > R(0)), neg = __ballot_sync(0xffffffffu, sg < R(0));
             off = __shfl_sync(0xffffffffu, off, 0);
             bi = __shfl_sync(0xffffffffu, bi, 0);
+            if (bi < 0 && lane == 0 && last >= 0)  // the unit's batches so far are not clipped
+                for (int k = q.head[unit].x; k >= 0; k = q.bnext[k]) q.boff[k] = PF_NONE;
             last = bi < 0 ? PF_FAIL : bi;
-            full = bi < 0;
             if (bi >= 0) {
                 uint4 *ob = q.arena + off;
                 if (lane == 0) {
@@ -1671,6 +1672,7 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
             }
         });
         mx_merge(acc);
+        if (last == PF_FAIL) wk = wk0;  // (done, and counted, again)
         if (lane == 0) {
             put_sum(q.base, unit, acc);
             q.head[unit].y = comp;
@@ -1683,7 +1685,14 @@ __device__ __forceinline__ void pf_pairs_body(const DevMesh &m, const MXArgs &a,
             rec = record(next);
         }
         unit = next;
+        if (last == PF_FAIL) break;
     }
+    // no room in the queue any more: the rest is left to the third launch
+    for (; unit < units; unit = __shfl_sync(0xffffffffu, take(), 0))
+        if (lane == 0) {
+            q.head[unit].x = PF_FAIL;
+            q.ovf[atomicAdd(q.novf, 1)] = unit;
+        }
     next_kernel();
     wk.flush(a.work, lane);
 }
@@ -1814,14 +1823,17 @@ __device__ __forceinline__ void pf_redo(const DevMesh &m, const MXArgs &a, const
         const PfFace p = pf_face<R>(rec, sh);
         pf_poly<R>(m, a, sh, item, p);
         __syncwarp();
+        if (q.head[item << ls].x == PF_FAIL) {  // (else counted by its first part)
+            wk.add(WK_VOL, lane < p.nt);
+            wk.face();
+        }
         double v = 0.0;
         bool comp = p.comp;
         for (int part = 0; part < 1 << ls; ++part) {
             double w = 0.0;
             Acc<R> acc;
-            WkOff off;  // (its pairs are counted by the pair stage)
             comp = p.comp;
-            pf_stencil<R>(m, a, sh, p, part, ls, comp, acc, off, [&](int nq, unsigned, R tol) {
+            pf_stencil<R>(m, a, sh, p, part, ls, comp, acc, wk, [&](int nq, unsigned, R tol) {
                 if (lane < p.nt) stT(sh.T[lane], prism_tet(reinterpret_cast<const R *>(sh.P6), lane));
                 Acc<R> cut;
                 mx_clip(sh, sh.Q, nq, tol, pf_drop<R>(sh), cut, wk);
@@ -1864,8 +1876,9 @@ __global__ void __launch_bounds__(W * 32, pc_resident<R>(W, ST)) k_pf_clip(MXArg
 }
 
 constexpr int PF_FINISH_WARPS = 2;
+template <class R> constexpr int pf_finish_resident() { return sizeof(R) == 4 ? 7 : 3; }  // by its shared memory
 template <class R, int ST, class Wk>
-__global__ void __launch_bounds__(32 * PF_FINISH_WARPS, sizeof(R) == 4 ? 8 : 4) k_pf_finish(DevMesh m, MXArgs a, PfQueue q)
+__global__ void __launch_bounds__(32 * PF_FINISH_WARPS, pf_finish_resident<R>()) k_pf_finish(DevMesh m, MXArgs a, PfQueue q)
 {
     next_kernel();
     previous_kernel();
@@ -2038,7 +2051,7 @@ template <class R, int ST, class Wk>
 static int go_finish(vof_ctx *c, const MXArgs &a, const PfQueue &q, int sms, cudaStream_t s)
 {
     constexpr size_t bytes = PF_FINISH_WARPS * sizeof(RedoShared<R, ST>);
-    return launch_after(k_pf_finish<R, ST, Wk>, sms * 4, 32 * PF_FINISH_WARPS, bytes, s, c->m, a, q);
+    return launch_after(k_pf_finish<R, ST, Wk>, sms * pf_finish_resident<R>(), 32 * PF_FINISH_WARPS, bytes, s, c->m, a, q);
 }
 
 template <class R, class Wk>

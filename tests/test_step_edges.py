@@ -246,8 +246,10 @@ def test_no_room_in_the_queue_changes_no_bit(torch, precision):
     vof.vof_batch_destroy(b)
     # ("reserved" counts the faces without room)
     assert all(c["reserved"] > 100 for _, c in few) and all(c["reserved"] == 0 for _, c in all_)
-    for t, _ in few[1:] + all_:
+    for t, c in few[1:] + all_:
         assert torch.equal(few[0][0], t)
+        # and no face's work is done, or counted, twice
+        assert {k: v for k, v in c.items() if k != "reserved"} == {k: v for k, v in few[0][1].items() if k != "reserved"}
 
 
 @pytest.mark.gpu
