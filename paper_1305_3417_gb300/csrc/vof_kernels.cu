@@ -155,8 +155,8 @@ __global__ void k_point_velocity(DevMesh m, const double *__restrict__ Uc, doubl
 // then the plane offset, the fill function summed over the cell tetrahedra, KL
 // or fewer per lane, each a closed-form cut fraction of its sorted projections.
 //
-// Bound by the FP64 pipe, which issues one warp instruction in 16 cycles on
-// this part whatever the number of active lanes: what counts is FP64 warp
+// Bound by the FP64 pipe, which takes one warp instruction in 64 cycles on each
+// of an SM's four sub-partitions, whatever the number of active lanes: what counts is FP64 warp
 // instructions per cell.  So several cells share a warp, every order and
 // threshold test is taken on the integer pipe from the bit patterns, the
 // tetrahedra's volumes come from the context, and the fill is evaluated
@@ -1062,7 +1062,7 @@ __device__ __forceinline__ double warp_max_bits(double v)
 // A block per segment, a thread per cell.  Bound by HBM (28 B of cell CSR, 16 of
 // alpha, 8 of V a cell, each face's flux once) and, on small meshes, by the chain
 // of dependent loads.  An empty cell without flux costs no FP64 instruction and
-// a full one without flux no division (the FP64 pipe runs at 1/62 of FP32).
+// a full one without flux no division (the FP64 pipe runs at 1/63 of FP32).
 __global__ void __launch_bounds__(UPD_THREADS) k_update(DevMesh m, double *alpha, const double *Va,
                                                         const int4 *__restrict__ seg, int nseg, double *sd,
                                                         uint8_t *seg_mixed, int *viol, int *nviol, unsigned *status)
@@ -1382,9 +1382,12 @@ constexpr unsigned EPOCH_STEP = BOUND_PASSES_MAX + 2;
 // cells are strictly inside, FP64 work on few SMs are the cost.  On meshes up to
 // BOUND_CLUSTER_CELLS the kernel is one cluster of eight blocks with the
 // hardware's cluster barrier, beyond that one block per SM of a cooperative
-// launch (the update and this, 24^3: 38 us; 32^3-based octree 69 in one cluster,
-// 62 over all SMs; 64^3 film 76 / 63; 48^3 tetrahedra, with a fallback, 230 /
-// 143; 128^3 114 / 95).  With four barriers a pass over 608 blocks and two
+// launch: the cluster's barriers are cheaper, and it starts while the update
+// ends, until the cells take more than eight SMs (the update and this, in one
+// cluster / over all SMs: 32^2 disc 33 / 41 us, 24^3 35 / 42, 24^3 film 37 / 46,
+// 16^3 tetrahedra, with a fallback, 71 / 88, 32^3 37 / 47; beyond the line
+// 32^3-based octree 69 / 62, 64^3 film 76 / 63, 48^3 tetrahedra, with a fallback,
+// 230 / 143, 128^3 114 / 95).  With four barriers a pass over 608 blocks and two
 // sweeps over every cell in each step they took 60 us on the 32^2 disc without a
 // source (now 19), 94 at 24^3, 135 on the octree, 117 on the film, 153 at 128^3.
 struct BoundStep {

@@ -90,7 +90,7 @@ template <class R> __device__ __forceinline__ R3<R> ld43(const R4<R> *p, long i)
 // Threshold, sign and order tests of distances (tol >= 0).  FP32: the native
 // compares.  FP64: integer compares of the bit patterns (dbits), the same
 // decisions for every value that is not NaN: this part's FP64 pipe runs at
-// 1/64 of the FP32 rate, and an FP64 compare or min/max holds it as long as
+// 1/63 of the FP32 rate, and an FP64 compare or min/max holds it as long as
 // an FMA.
 __device__ __forceinline__ bool rpos(float v) { return v > 0.0f; }
 __device__ __forceinline__ bool rneg(float v) { return v < 0.0f; }
