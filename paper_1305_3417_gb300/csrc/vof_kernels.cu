@@ -207,7 +207,12 @@ __device__ __forceinline__ double fill_below(const FillTet &q, double d)
     return hiword(u) <= 0 ? 0.0 : f;
 }
 
-// the same in FP32 with its derivative (the cut area over the volume)
+// The same in FP32 with its derivative (the cut area over the volume).  Every
+// form is a sum of terms that are not negative, the one for one vertex above
+// too: 1 - (1-b)(1-e)(1-g) as b + (1-b)(e + (1-e) g), so that the fill's error is
+// relative to the fill and small levels are resolved (one minus a product
+// leaves 6e-8 of the tetrahedron: cells of 1e-9 with a normal along the mesh, whose
+// tetrahedra have three vertices at the bottom, did not converge on it).
 struct FillTetF { float h0, h1, h2, h3, r10, ra, rb, rc, re, r32; };
 
 __device__ __forceinline__ float fill_below(const FillTetF &q, float d, float &df)
@@ -219,7 +224,7 @@ __device__ __forceinline__ float fill_below(const FillTetF &q, float d, float &d
     const float dmid = q.ra * b + a * q.rb + q.ra * b1 * e - a * q.rb * e + a * b1 * q.re - q.ra * c * e +
                        a1 * q.rc * e + a1 * c * q.re;
     const float lx = q.r10 * ab, tx = (y * q.re) * (y * q.rb) * q.r32;
-    const float low = u * lx, top = 1.0f - y * tx;
+    const float low = u * lx, top = fmaf(b1, fmaf(1.0f - e, -z * q.r32, e), b);
     float f = v <= 0.0f ? low : z <= 0.0f ? top : mid;
     df = v <= 0.0f ? 3.0f * lx : z <= 0.0f ? 3.0f * tx : dmid;
     if (y <= 0.0f) { f = 1.0f; df = 0.0f; }
@@ -408,7 +413,8 @@ __device__ __forceinline__ RcCell rc_cell(const DevMesh &m, const double *__rest
             if (!sure) break;
         }
         r.it32 = it;
-        double X = (double)x * range, lo64 = (double)A * range, hi64 = (double)B * range;
+        // (the whole extent as the bracket: nothing that FP32 decided is taken over)
+        double X = (double)x * range, lo64 = 0.0, hi64 = range;
         while (it < POS_MAXIT) {
             double S[4] = {0.0, 0.0, 0.0, 0.0};
             int gap = 0x7fffffff;

@@ -1,6 +1,7 @@
 """What a step does at its edges: shared memory handed between the lanes of a
 warp, settings changed between batch steps, cells of any aspect ratio,
 NaN fractions, what the positioning's stop leaves of an offset,
+wisps in cells along the mesh,
 a band beyond the queue of clip jobs,
 a context made, or a network attached, where memory is short, network outputs
 written over their inputs.
@@ -340,3 +341,46 @@ def test_network_that_finds_no_room(torch):
     ctx.close()
     for net in nets:
         net.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("n", [15, 16])
+def test_wisps_along_the_mesh(torch, oracle_lib, precision, n):
+    """Cells of 1.1e-9 to 1e-3 (and as much below 1) on uniform hexahedra, next to
+    a boundary or to a slab, so that their normals lie along the mesh up to
+    roundings: every offset converges, to the stopping residual of 1e-13 (3e-13
+    with the roundings of both sides)."""
+    from paper_1305_3417_gb300 import vof
+    m = I.hex_mesh((n, n, n), open_sides=("x-", "x+", "y-", "y+", "z-", "z+"))
+    om = oracle_lib.OracleMesh(m)
+    vc = om.geometry()[1]
+    rng = np.random.default_rng(n)
+    ctx = vof.VofContext(m, precision=precision)
+    worst = 0
+    for up in (False, True):
+        for layer in (False, True):
+            a = np.zeros((n, n, n))                     # [z, y, x]
+            if layer:
+                a[:, :, :4] = 1.0
+                a[:, :, 4] = 10.0 ** rng.uniform(-8.9, -3.0, (n, n))
+                a[::2, ::2, 4] = 3e-9
+            else:
+                t = 10.0 ** np.linspace(-8.9, -3.0, 3 * (n // 3) ** 2).reshape(3, n // 3, n // 3)
+                k = 3 * np.arange(n // 3) + 1
+                a[np.ix_(k, k, [0])] = t[0][:, :, None]
+                a[np.ix_(k, [n - 1], k)] = t[1][:, None, :]
+                a[np.ix_([0], k, k)] = t[2][None]
+            a = a.reshape(-1)
+            if up:
+                a = 1.0 - a
+            nn, d, fl, it = (x.cpu().numpy() for x in ctx.reconstruct(T(torch, a)))
+            nn = nn.reshape(3, -1)
+            cells = np.flatnonzero(fl & oracle_lib.ORIENTED)
+            assert cells.size >= 3 * (n // 3) ** 2 - 3
+            assert ctx.status() == 0
+            worst = max(worst, int(it[cells].max()))
+            for c in cells:
+                assert abs(om.cut_volume(c, nn[:, c], d[c]) / vc[c] - a[c]) <= 3e-13
+    assert worst < 60                                   # Alg. 1 ends within 50; Newton well before
+    ctx.close()
