@@ -56,15 +56,14 @@ PF_KERNELS = "k_pf_pairs + k_pf_clip + k_pf_finish"
 # face point indices 20, alpha r/w and volume 8, point data 28)
 BYTES_PER_FACE = 72.0
 
-# DRAM bytes per launch of the mixed phase flux (here of its earlier form, one
-# launch a step; its sources have changed since): dram__bytes_read.sum +
-# dram__bytes_write.sum, mean of the two timed launches of one ncu capture of
-# the default launch shape (ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,
-# gpu__time_duration.sum -k regex:k_phase_flux_mixed -s 3 -c 3 python bench.py
+# DRAM bytes a step of the mixed phase flux (its three launches together):
+# dram__bytes_read.sum + dram__bytes_write.sum, mean of the two timed steps of one
+# ncu capture of the default launch shape (ncu --metrics dram__bytes_read.sum,
+# dram__bytes_write.sum,gpu__time_duration.sum -k regex:k_pf_ python bench.py
 # --steps 2 --warmup 3 --no-tune --no-cpu-baseline --fp64-steps 0 --full-run 0);
-# valid while the kernel's sources hash to the captured digest, else null.
+# valid while the kernels' sources hash to the captured digest, else null.
 TRAFFIC = {
-    ("deform3d", 128, "mixed"): {"bytes": 68.08e6, "sources_sha256": "a46f217f59e4de731bd9a6d310010b01930eabe90b9d14362bd5b68a8c8addaf"},
+    ("deform3d", 128, "mixed"): {"bytes": 232.8e6, "sources_sha256": "4d9053e1368b81ef9aa6c5364f1be9fe2d0977e0d2a074895e8d35da45aadb4a"},
 }
 TRAFFIC_SOURCES = ["paper_1305_3417_gb300/csrc/vof_phase_flux.cu", "paper_1305_3417_gb300/csrc/vof_device.cuh"]
 
@@ -885,7 +884,7 @@ def main():
             if args.skip == 0 else None
         roof = {"kernel": PF_KERNELS, "bound": "alu",
                 "achieved": achieved, "peak": alu / 1e12, "unit": "TFLOP/s", "frac": achieved * 1e12 / alu,
-                "traffic": traffic, "traffic_unit": "bytes per launch (ncu capture)",
+                "traffic": traffic, "traffic_unit": "bytes per step (ncu capture)",
                 "peak_source": f"measured {'FP64' if prec == vof.FP64 else 'FP32'} FMA probe (vof_probe_fma)",
                 "work_per_launch": work, "flops_per_launch": pf}
     else:
