@@ -568,7 +568,7 @@ int vof_create(const vof_mesh *mesh, const vof_options *opt, vof_ctx **out)
     c->pstate = dev_alloc<uint8_t>(c, np, &err);
     c->band = dev_alloc<int>(c, nf, &err);
     c->icell = dev_alloc<int>(c, nc, &err);
-    c->viol[0] = dev_alloc<int>(c, nc, &err);
+    c->viol = dev_alloc<int>(c, nc, &err);
     c->rl = dev_alloc<int>(c, nc, &err);
     c->ra = dev_alloc<double>(c, nc, &err);
     c->cmark = dev_alloc<unsigned>(c, nc, &err);

@@ -98,7 +98,7 @@ struct vof_ctx {
     int nbufs;
     // per-step scratch
     uint8_t *pstate;
-    int *band, *icell, *viol[2];
+    int *band, *icell, *viol;
     int *counters;               // CNT_ALLOC ints, laid out as CNT_* above
     double *lam_b;               // per band slot
     void *disp_b;                // per band slot, in the form's type
@@ -228,7 +228,6 @@ inline int launch_after(void (*kernel)(P...), int grid, int block, size_t smem, 
 int launch_advect(vof_ctx *c, double *alpha, const double *Uc, const double *F, double dt,
                   double *stats, cudaStream_t s,
                   cudaEvent_t wait_before_correct = nullptr);
-int launch_validate(vof_ctx *c, cudaStream_t s, unsigned *bad);
 // ---- phase-flux tables (vof_phase_flux.cu) ----
 int launch_setup_mixed(vof_ctx *c, cudaStream_t s);
 // regions of the global bounding step: region r = cells [reg_cell[r], reg_cell[r+1]) (host array)

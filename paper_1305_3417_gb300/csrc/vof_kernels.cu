@@ -2161,13 +2161,13 @@ static int launch_update_group(vof_ctx *c, double *alpha, const double *Va, cons
 {
     int *cnt = c->counters;
     if (launch_after(k_update, std::min(c->nseg, num_sms(c->device) * 8), UPD_THREADS, 0, s, c->m, alpha, Va, c->seg,
-                     c->nseg, c->sd, c->seg_mixed, c->bound ? c->viol[0] : nullptr, cnt + CNT_VIOL0, c->status))
+                     c->nseg, c->sd, c->seg_mixed, c->bound ? c->viol : nullptr, cnt + CNT_VIOL0, c->status))
         return VOF_ERR_CUDA;
     LAUNCH_CHECK();
     if (!c->bound) {
         return launch_after(k_stats, 1, ST_THREADS, 0, s, c->sd, c->nseg, counters, stats);
     }
-    const BoundStep a{alpha, c->viol[0], cnt + CNT_VIOL0, c->rl, cnt + CNT_NRL0, c->ra, c->bscr, c->cmark, c->segmark,
+    const BoundStep a{alpha, c->viol, cnt + CNT_VIOL0, c->rl, cnt + CNT_NRL0, c->ra, c->bscr, c->cmark, c->segmark,
                       c->dl, cnt + CNT_NDL, reinterpret_cast<unsigned *>(cnt + CNT_EPOCH), cnt + CNT_BPASS,
                       cnt + CNT_BACT0, cnt + CNT_LEFT0, cnt + CNT_VIOL1, c->seg, c->seg_at, c->nseg, c->seg_mixed, c->sd, c->reg_seg,
                       c->nreg, c->reg_tot, counters, stats, reinterpret_cast<unsigned *>(cnt + CNT_BAR),
@@ -2310,11 +2310,5 @@ int launch_advect(vof_ctx *c, double *alpha, const double *Uc, const double *F, 
     MARK(5);
 #undef MARK
     c->launches = launches;
-    return VOF_OK;
-}
-
-int launch_validate(vof_ctx *c, cudaStream_t s, unsigned *bad)
-{
-    (void)c; (void)s; (void)bad;
     return VOF_OK;
 }
